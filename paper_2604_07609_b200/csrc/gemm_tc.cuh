@@ -413,18 +413,26 @@ __device__ __forceinline__ unsigned long long gu_stamp(const DevCtx& c, int laye
 __device__ __forceinline__ int tc_epi_half(int n_mma) { return n_mma >= 128 ? ((n_mma / 16 + 1) / 2) * 16 : n_mma; }
 
 // ---- the GEMM phase -----------------------------------------------------------------------------
-// Shape of one GEMM's pipeline for the current step; every role derives the same numbers.
+// Shape of one GEMM's pipeline for the current step; every role derives the same numbers.  All of it is 32-bit
+// arithmetic and the roles walk their range segment by segment (TcSeg) without dividing: a 64-bit division is a
+// subroutine of a few hundred cycles, and three of them per stage in the single-threaded producers used to set
+// the time of a stage (0.64 us per k-block whatever its bytes; 2.7 TB/s of weights at 256 rows, 43 % tensor pipe).
 struct TcGeom {
   int kblocks, ntiles, passes, box_id, box_rows, load_box, KPS, S;
   int pass_fixed, pdiv;   // one token pass per CTA (or -1), and the passes interleaved in its unit order
   uint32_t b_bytes, stage_bytes;
-  long long u0, u1;
+  int u0, u1;
 };
+// floor(total * b / nb) without the 64-bit product
+__device__ __forceinline__ int tc_share(int total, int nb, int b) {
+  const unsigned q = (unsigned)total / (unsigned)nb, r = (unsigned)total - q * (unsigned)nb;
+  return (int)(q * (unsigned)b + r * (unsigned)b / (unsigned)nb);
+}
 __device__ __forceinline__ TcGeom tc_geom(const DevCtx& c, int T, int N, int K, bool whole_tiles, int nb, int b, int ntiles, bool half_tokens) {
   TcGeom g;
-  g.kblocks = K / 64;
+  g.kblocks = (int)((unsigned)K >> 6);
   g.ntiles = ntiles;   // weight tiles of 128 rows, or pairs of them
-  g.passes = (T + 255) / 256;
+  g.passes = (int)((unsigned)(T + 255) >> 8);
   g.box_id = TC_BOXES - 1;
   if (g.passes == 1) {
     g.box_id = 0;
@@ -438,17 +446,15 @@ __device__ __forceinline__ TcGeom tc_geom(const DevCtx& c, int T, int N, int K, 
   g.load_box = half_tokens ? (g.box_id > 0 ? g.box_id - 1 : 0) : g.box_id;
   g.b_bytes = (uint32_t)(16 << g.load_box) * 128u;
   g.stage_bytes = (uint32_t)g.KPS * (TC_A_BYTES + g.b_bytes);
-  g.S = TC_TILE_BUDGET / (int)g.stage_bytes;
+  g.S = (int)((unsigned)TC_TILE_BUDGET / g.stage_bytes);
   if (g.S > TC_MAX_STAGES) g.S = TC_MAX_STAGES;
-  const long long total = (long long)g.passes * g.ntiles * g.kblocks;
-  g.u0 = total * b / nb;
-  g.u1 = total * (b + 1) / nb;
+  const int total = g.passes * g.ntiles * g.kblocks;
   g.pass_fixed = -1;
   g.pdiv = g.passes;
   if (whole_tiles && g.passes == 1) {
     // every worker gets whole weight tiles (at most one more than its neighbours): no partial sums at all
-    g.u0 = (long long)g.kblocks * ((long long)g.ntiles * b / nb);
-    g.u1 = (long long)g.kblocks * ((long long)g.ntiles * (b + 1) / nb);
+    g.u0 = g.kblocks * tc_share(g.ntiles, nb, b);
+    g.u1 = g.kblocks * tc_share(g.ntiles, nb, b + 1);
     return g;
   }
   // More than 256 token rows: the passes of a weight tile go to neighbouring workers, which walk the
@@ -456,43 +462,67 @@ __device__ __forceinline__ TcGeom tc_geom(const DevCtx& c, int T, int N, int K, 
   // L2 for the others.  One worker doing the passes in turn re-reads it after the whole grid has
   // streamed more than L2 holds in between.
   if (g.passes > 1 && nb >= g.passes) {
-    const int groups = nb / g.passes;
-    const long long units = (long long)g.ntiles * g.kblocks;
+    const int groups = (int)((unsigned)nb / (unsigned)g.passes);
+    const int units = g.ntiles * g.kblocks;
     g.pdiv = 1;
-    if (b < groups * g.passes) {
-      const int grp = b / g.passes;
-      g.pass_fixed = b % g.passes;
-      g.u0 = units * grp / groups;
-      g.u1 = units * (grp + 1) / groups;
+    const int grp = (int)((unsigned)b / (unsigned)g.passes);
+    if (grp < groups) {
+      g.pass_fixed = b - grp * g.passes;
+      g.u0 = tc_share(units, groups, grp);
+      g.u1 = tc_share(units, groups, grp + 1);
     } else {
       g.pass_fixed = 0;
       g.u0 = g.u1 = 0;
     }
+    return g;
   }
   // Few weight tiles (QKV, O, down at decode sizes): give every tile the same whole number of
   // workers, so that no range crosses a tile and each has one partial tile to reduce at the
   // end instead of two.  The longest range grows by (per * nb - total) / nb k-blocks of about
   // 0.4 us each; the saved reduction takes about 0.018 us per token row.
-  const int split = nb / g.ntiles;
+  const int split = (int)((unsigned)nb / (unsigned)g.ntiles);
   if (g.passes == 1 && split >= 2) {
-    const int per = (g.kblocks + split - 1) / split;
-    if (((long long)per * nb - total) * 23 < (long long)T * nb) {
-      if (b < g.ntiles * split) {
-        const int nt = b / split, part = b % split;
-        g.u0 = (long long)nt * g.kblocks + (long long)g.kblocks * part / split;
-        g.u1 = (long long)nt * g.kblocks + (long long)g.kblocks * (part + 1) / split;
+    const int per = (int)((unsigned)(g.kblocks + split - 1) / (unsigned)split);
+    if ((per * nb - total) * 23 < T * nb) {
+      const int nt = (int)((unsigned)b / (unsigned)split), part = b - nt * split;
+      if (nt < g.ntiles) {
+        g.u0 = nt * g.kblocks + (int)((unsigned)(g.kblocks * part) / (unsigned)split);
+        g.u1 = nt * g.kblocks + (int)((unsigned)(g.kblocks * (part + 1)) / (unsigned)split);
       } else {
         g.u0 = g.u1 = 0;
       }
+      return g;
     }
   }
+  g.u0 = tc_share(total, nb, b);
+  g.u1 = tc_share(total, nb, b + 1);
   return g;
 }
-// position of unit u: weight tile and token pass (the k-block is u % kblocks)
-__device__ __forceinline__ int tc_unit_nt(const TcGeom& g, long long u) { return (int)(u / ((long long)g.kblocks * g.pdiv)); }
-__device__ __forceinline__ int tc_unit_pass(const TcGeom& g, long long u) {
-  return g.pass_fixed >= 0 ? g.pass_fixed : (int)((u / g.kblocks) % g.passes);
+// One segment of a worker's range: k-blocks [kb0, kb1) of weight tile nt for token pass `pass`; `left` units
+// remain, this segment's included.
+struct TcSeg {
+  int nt, pass, kb0, kb1, left;
+};
+__device__ __forceinline__ TcSeg tc_seg_first(const TcGeom& g) {
+  TcSeg s;
+  const int q = (int)((unsigned)g.u0 / (unsigned)g.kblocks);
+  s.kb0 = g.u0 - q * g.kblocks;
+  s.nt = (int)((unsigned)q / (unsigned)g.pdiv);
+  s.pass = g.pass_fixed >= 0 ? g.pass_fixed : q - s.nt * g.pdiv;
+  s.left = g.u1 - g.u0;
+  s.kb1 = min(g.kblocks, s.kb0 + s.left);
+  return s;
 }
+__device__ __forceinline__ void tc_seg_next(const TcGeom& g, TcSeg& s) {
+  s.left -= s.kb1 - s.kb0;
+  s.kb0 = 0;
+  s.kb1 = min(g.kblocks, s.left);
+  if (g.pass_fixed >= 0 || ++s.pass == g.pdiv) {
+    if (g.pass_fixed < 0) s.pass = 0;
+    ++s.nt;
+  }
+}
+__device__ __forceinline__ bool tc_seg_is_last(const TcSeg& s) { return s.kb1 - s.kb0 == s.left; }
 // tiles need 1024-byte alignment for the 128-byte swizzle
 __device__ __forceinline__ char* tc_tiles(float* smem_f) {
   const uint32_t raw = smem_u32(smem_f);
@@ -512,36 +542,64 @@ __device__ __forceinline__ void tc_produce_weights(const DevCtx& c, const void* 
   const int row_a0 = (int)w_row0;
   volatile int* dead = &g_tc.dead;
   const uint64_t stream_policy = l2_evict_first();
-  long long u = g.u0;
   int stage = 0;
-  while (u < g.u1) {
-    const long long seg_end = min(g.u1, (u / g.kblocks + 1) * (long long)g.kblocks);
-    const int nk = (int)min((long long)g.KPS, seg_end - u);
-    const int kb = (int)(u % g.kblocks);
-    const int nt = tc_my_tile<PAIR>(tc_unit_nt(g, u), rank);
-    // the n-th fill of a stage waits for its (n-1)-th release
-    if (!mbar_wait(c, &g_tc.empty[stage], ((tc.fill_bits >> stage) & 1u) ^ 1u, dead)) break;
-    tc.fill_bits ^= 1u << stage;
-    char* sa = tiles + (size_t)stage * g.stage_bytes;
-    if constexpr (PAIR) {
-      mbar_expect_tx_cta0(&g_tc.full[stage], (uint32_t)nk * TC_A_BYTES);
-      if (c.w_streaming) {   // tile index inside the whole tensor; one or two consecutive tiles per copy
-        const int tile = (int)(((w_row0 >> 7) + nt) * g.kblocks + kb);
-        tma_pair_load_3d(sa, &maps->ws[which][nk - 1], 0, 0, tile, &g_tc.full[stage], stream_policy);
+  for (TcSeg sg = tc_seg_first(g); sg.left > 0; tc_seg_next(g, sg)) {
+    const int nt = tc_my_tile<PAIR>(sg.nt, rank);
+    const int tile0 = ((int)(w_row0 >> 7) + nt) * g.kblocks;   // streaming layout: tile index inside the whole tensor
+    const char* tile_ptr = reinterpret_cast<const char*>(w) + (size_t)nt * g.kblocks * TC_A_BYTES;
+    for (int kb = sg.kb0; kb < sg.kb1;) {
+      const int nk = min(g.KPS, sg.kb1 - kb);
+      // the n-th fill of a stage waits for its (n-1)-th release
+      if (!mbar_wait(c, &g_tc.empty[stage], ((tc.fill_bits >> stage) & 1u) ^ 1u, dead)) return;
+      tc.fill_bits ^= 1u << stage;
+      char* sa = tiles + (size_t)stage * g.stage_bytes;
+      if constexpr (PAIR) {
+        mbar_expect_tx_cta0(&g_tc.full[stage], (uint32_t)nk * TC_A_BYTES);
+        if (c.w_streaming) {   // one or two consecutive tiles per copy
+          tma_pair_load_3d(sa, &maps->ws[which][nk - 1], 0, 0, tile0 + kb, &g_tc.full[stage], stream_policy);
+        } else {
+          tma_pair_load_2d(sa, map_a, kb * 64, row_a0 + nt * 128, &g_tc.full[stage], stream_policy);
+        }
       } else {
-        tma_pair_load_2d(sa, map_a, kb * 64, row_a0 + nt * 128, &g_tc.full[stage], stream_policy);
+        mbar_expect_tx(&g_tc.full[stage], (uint32_t)nk * TC_A_BYTES);
+        if (c.w_streaming) {  // contiguous tiles, already in the shared-memory operand image
+          tma_bulk_load_hint(sa, tile_ptr + (size_t)kb * TC_A_BYTES, (uint32_t)nk * TC_A_BYTES, &g_tc.full[stage],
+                             stream_policy);
+        } else {
+          tma_load_2d_hint(sa, map_a, kb * 64, row_a0 + nt * 128, &g_tc.full[stage], stream_policy);
+        }
       }
-    } else {
-      mbar_expect_tx(&g_tc.full[stage], (uint32_t)nk * TC_A_BYTES);
-      if (c.w_streaming) {  // contiguous tiles, already in the shared-memory operand image
-        tma_bulk_load_hint(sa, reinterpret_cast<const char*>(w) + ((size_t)nt * g.kblocks + kb) * TC_A_BYTES,
-                           (uint32_t)nk * TC_A_BYTES, &g_tc.full[stage], stream_policy);
-      } else {
-        tma_load_2d_hint(sa, map_a, kb * 64, row_a0 + nt * 128, &g_tc.full[stage], stream_policy);
-      }
+      kb += nk;
+      if (++stage == g.S) stage = 0;
     }
-    u += nk;
-    if (++stage == g.S) stage = 0;
+  }
+}
+
+// Token-tile producer (one thread): the same sequence of stages, nk k-blocks of one segment each.
+template <bool PAIR>
+__device__ __forceinline__ void tc_produce_tokens(const DevCtx& c, const CUtensorMap* map_b, int x_row0, int T, const TcGeom& g,
+                                                  char* tiles, TcState& tc, uint32_t rank) {
+  volatile int* dead = &g_tc.dead;
+  const uint64_t keep_policy = l2_evict_normal();
+  int stage = 0;
+  for (TcSeg sg = tc_seg_first(g); sg.left > 0; tc_seg_next(g, sg)) {
+    // pairs: this CTA's half of the pass is rows [rank * n_mma / 2, + n_mma / 2) (the box may reach further)
+    const int n_mma = (min(256, T - sg.pass * 256) + 15) & ~15;
+    const int row0 = x_row0 + sg.pass * 256 + (PAIR ? (int)rank * (n_mma / 2) : 0);
+    for (int kb = sg.kb0; kb < sg.kb1;) {
+      const int nk = min(g.KPS, sg.kb1 - kb);
+      if (!mbar_wait(c, &g_tc.empty[stage], ((tc.fill_bits >> stage) & 1u) ^ 1u, dead)) return;
+      tc.fill_bits ^= 1u << stage;
+      char* sb = tiles + (size_t)stage * g.stage_bytes + g.KPS * TC_A_BYTES;
+      if constexpr (PAIR) mbar_expect_tx_cta0(&g_tc.full[stage], (uint32_t)nk * g.b_bytes);
+      else mbar_expect_tx(&g_tc.full[stage], (uint32_t)nk * g.b_bytes);
+      for (int j = 0; j < nk; ++j) {
+        if constexpr (PAIR) tma_pair_load_2d(sb + j * g.b_bytes, map_b, (kb + j) * 64, row0, &g_tc.full[stage], keep_policy);
+        else tma_load_2d(sb + j * g.b_bytes, map_b, (kb + j) * 64, row0, &g_tc.full[stage]);
+      }
+      kb += nk;
+      if (++stage == g.S) stage = 0;
+    }
   }
 }
 
@@ -554,37 +612,36 @@ static __device__ __noinline__ void tc_finish_tiles(const DevCtx& c, const GemmA
   constexpr int BATCH = 16;
   __shared__ int s_fin[BATCH];
   __shared__ int s_nfin;
-  __shared__ long long s_next;
+  __shared__ bool s_more;
   // gate/up: with plain rows gate tile j and up tile j + ntiles / 2 share slot j; with interleaved rows one
   // weight tile holds gate and up of 64 features
   const bool two_tiles = a.fix == FIX_SILU && !c.w_streaming;
   const int ntiles_slot = two_tiles ? g.ntiles / 2 : g.ntiles;
   const int need = (two_tiles ? 2 : 1) * g.kblocks;
-  long long u = g.u0;
-  while (u < g.u1) {   // uniform over the CTA
+  TcSeg sg = tc_seg_first(g);   // walked by thread 0
+  bool more = g.u0 < g.u1;
+  while (more) {   // uniform over the CTA
     if (threadIdx.x == 0) {
       int n = 0;
       __threadfence();   // the CTA's partial sums (ordered before by the barrier above) before the counters
-      while (u < g.u1 && n < BATCH) {
-        const long long seg_end = min(g.u1, (u / g.kblocks + 1) * (long long)g.kblocks);
-        const int nt = tc_unit_nt(g, u), pass = tc_unit_pass(g, u);
-        const int units = (int)(seg_end - u);
-        const int tile = nt % ntiles_slot;
-        const int slot = (pass * ntiles_slot + tile) % TILE_CNT_SLOTS;
+      while (sg.left > 0 && n < BATCH) {
+        const int units = sg.kb1 - sg.kb0;
+        const int tile = sg.nt % ntiles_slot;
+        const int slot = (sg.pass * ntiles_slot + tile) % TILE_CNT_SLOTS;
         const int old = atomicAdd(&c.tile_cnt[slot], units);
         if (old + units == need) {
           c.tile_cnt[slot] = 0;   // nobody touches this counter again before the next grid barrier
-          s_fin[n++] = (pass << 16) | tile;
+          s_fin[n++] = (sg.pass << 16) | tile;
         }
-        u = seg_end;
+        tc_seg_next(g, sg);
       }
       if (n > 0) __threadfence();
       s_nfin = n;
-      s_next = u;
+      s_more = sg.left > 0;
     }
     __syncthreads();
     const int n = s_nfin;
-    u = s_next;
+    more = s_more;
     for (int i = 0; i < n; ++i) {
       const int tile = s_fin[i] & 0xffff, pass = s_fin[i] >> 16;
       const int t0 = pass * 256, t1 = min(a.M, t0 + 256);
@@ -618,64 +675,30 @@ static __device__ __noinline__ void phase_gemm_tc(const DevCtx& c, const GemmArg
                      : (which == GEMM_GU && c.E > 0) ? ACT_XG : ACT_XN;
   const CUtensorMap* map_b = &maps->act[act_id][g.load_box];
   char* tiles = tc_tiles(smem_f);
-  const long long u0 = g.u0, u1 = g.u1;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* dead = &g_tc.dead;
 
   if (warp == 0) {
-    if (lane == 0) {
-      tc_produce_weights<PAIR>(c, a.w, a.w_row0, which, g, tiles, tc, rank);
-    }
+    if (lane == 0) tc_produce_weights<PAIR>(c, a.w, a.w_row0, which, g, tiles, tc, rank);
   } else if (warp == 2) {
     // token-tile producer: walks the same sequence of stages (nk k-blocks of one segment each)
-    if (lane == 0) {
-      const int x_row0 = a.x_row0;
-      const uint64_t keep_policy = l2_evict_normal();
-      int stage = 0;
-      long long u = u0;
-      while (u < u1) {
-        const long long seg_end = min(u1, (u / kblocks + 1) * (long long)kblocks);
-        const int nk = (int)min((long long)KPS, seg_end - u);
-        const int kb = (int)(u % kblocks);
-        const int pass = tc_unit_pass(g, u);
-        if (!mbar_wait(c, &g_tc.empty[stage], ((tc.fill_bits >> stage) & 1u) ^ 1u, dead)) break;
-        tc.fill_bits ^= 1u << stage;
-        char* sa = tiles + (size_t)stage * stage_bytes;
-        if constexpr (PAIR) {
-          // this CTA's half of the pass: rows [rank * n_mma / 2, + n_mma / 2) (the box may reach further)
-          const int n_mma = (min(256, T - pass * 256) + 15) & ~15;
-          const int row0 = x_row0 + pass * 256 + (int)rank * (n_mma / 2);
-          mbar_expect_tx_cta0(&g_tc.full[stage], (uint32_t)nk * b_bytes);
-          for (int j = 0; j < nk; ++j)
-            tma_pair_load_2d(sa + KPS * TC_A_BYTES + j * b_bytes, map_b, (kb + j) * 64, row0, &g_tc.full[stage], keep_policy);
-        } else {
-          mbar_expect_tx(&g_tc.full[stage], (uint32_t)nk * b_bytes);
-          for (int j = 0; j < nk; ++j)
-            tma_load_2d(sa + KPS * TC_A_BYTES + j * b_bytes, map_b, (kb + j) * 64, x_row0 + pass * 256, &g_tc.full[stage]);
-        }
-        u += nk;
-        if (++stage == S) stage = 0;
-      }
-    }
+    if (lane == 0) tc_produce_tokens<PAIR>(c, map_b, a.x_row0, T, g, tiles, tc, rank);
   } else if (warp == 1) {
     if (lane == 0 && rank == 0) {   // pairs: CTA 0 issues the MMAs for both
       int stage = 0;
       int abuf = 0;
-      long long u = u0;
-      while (u < u1) {
-        const long long seg_end = min(u1, (u / kblocks + 1) * (long long)kblocks);
-        const int pass = tc_unit_pass(g, u);
-        const int rows = min(256, T - pass * 256);
+      bool ok = true;
+      for (TcSeg sg = tc_seg_first(g); ok && sg.left > 0; tc_seg_next(g, sg)) {
+        const int rows = min(256, T - sg.pass * 256);
         const int n_mma = (rows + 15) & ~15;
         const uint32_t idesc = PAIR ? idesc_bf16_pair(n_mma) : idesc_bf16(n_mma);
         const uint32_t d_tmem = tc.tmem_base + (uint32_t)abuf * 256u;
         if (!mbar_wait(c, &g_tc.acc_empty[abuf], ((tc.acc_mma >> abuf) & 1u) ^ 1u, dead)) break;
         tc.acc_mma ^= 1u << abuf;
         tc_fence_after();
-        bool first = true;
-        bool ok = true;
-        while (u < seg_end) {
-          const int nk = (int)min((long long)KPS, seg_end - u);
+        uint32_t accumulate = 0u;
+        for (int kb = sg.kb0; kb < sg.kb1; kb += KPS) {
+          const int nk = min(KPS, sg.kb1 - kb);
           if (!mbar_wait(c, &g_tc.full[stage], (tc.use_bits >> stage) & 1u, dead)) { ok = false; break; }
           tc.use_bits ^= 1u << stage;
           tc_fence_after();
@@ -686,14 +709,13 @@ static __device__ __noinline__ void phase_gemm_tc(const DevCtx& c, const GemmArg
 #pragma unroll
             for (int k16 = 0; k16 < 4; ++k16) {
               // 16 bf16 = 32 bytes further along K inside the swizzle atom: +2 in 16-byte units
-              if constexpr (PAIR) umma_bf16_pair(d_tmem, da + (uint64_t)(2 * k16), db + (uint64_t)(2 * k16), idesc, (first && k16 == 0) ? 0u : 1u);
-              else umma_bf16(d_tmem, da + (uint64_t)(2 * k16), db + (uint64_t)(2 * k16), idesc, (first && k16 == 0) ? 0u : 1u);
+              if constexpr (PAIR) umma_bf16_pair(d_tmem, da + (uint64_t)(2 * k16), db + (uint64_t)(2 * k16), idesc, accumulate);
+              else umma_bf16(d_tmem, da + (uint64_t)(2 * k16), db + (uint64_t)(2 * k16), idesc, accumulate);
+              accumulate = 1u;
             }
-            first = false;
           }
           if constexpr (PAIR) umma_commit_pair(&g_tc.empty[stage]);
           else umma_commit(&g_tc.empty[stage]);
-          u += nk;
           if (++stage == S) stage = 0;
         }
         if (!ok) break;
@@ -703,10 +725,10 @@ static __device__ __noinline__ void phase_gemm_tc(const DevCtx& c, const GemmArg
         // that completes exactly once per phase has no such ambiguity.
         if constexpr (PAIR) {
           umma_commit_pair(&g_tc.acc_full[abuf]);
-          if (u == u1) umma_commit_pair(&g_tc.acc_last);
+          if (tc_seg_is_last(sg)) umma_commit_pair(&g_tc.acc_last);
         } else {
           umma_commit(&g_tc.acc_full[abuf]);
-          if (u == u1) umma_commit(&g_tc.acc_last);
+          if (tc_seg_is_last(sg)) umma_commit(&g_tc.acc_last);
         }
         abuf ^= 1;
       }
@@ -716,22 +738,18 @@ static __device__ __noinline__ void phase_gemm_tc(const DevCtx& c, const GemmArg
     const TcEpiOut eo{a.out, (size_t)a.ldo, a.row_map, a.row_scale, T, N, ilv_F, act_direct};
     const bool accumulate = a.accumulate != 0;
     int abuf = 0;
-    long long u = u0;
-    while (u < u1) {
-      const long long seg_end = min(u1, (u / kblocks + 1) * (long long)kblocks);
-      const int kb0 = (int)(u % kblocks);
-      const int kb1 = kb0 + (int)(seg_end - u);
-      const int nt = tc_my_tile<PAIR>(tc_unit_nt(g, u), rank);
-      const int pass = tc_unit_pass(g, u);
+    for (TcSeg sg = tc_seg_first(g); sg.left > 0; tc_seg_next(g, sg)) {
+      const int nt = tc_my_tile<PAIR>(sg.nt, rank);
+      const int pass = sg.pass;
       const int rows = min(256, T - pass * 256);
       const int n_mma = (rows + 15) & ~15;
-      const bool plain = (kb0 == 0 && kb1 == kblocks) && !accumulate && eo.row_map == nullptr;
+      const bool plain = (sg.kb0 == 0 && sg.kb1 == kblocks) && !accumulate && eo.row_map == nullptr;
       if (!mbar_wait(c, &g_tc.acc_full[abuf], (tc.acc_epi >> abuf) & 1u, dead)) break;
       tc.acc_epi ^= 1u << abuf;
       tc_fence_after();
       const uint32_t taddr = tc.tmem_base + (uint32_t)abuf * 256u + ((uint32_t)(q * 32) << 16);
       // the upper columns of the CTA's last accumulator are left to warps 0-3
-      const int c_end = (seg_end == u1) ? tc_epi_half(n_mma) : n_mma;
+      const int c_end = tc_seg_is_last(sg) ? tc_epi_half(n_mma) : n_mma;
       if (plain && eo.act != nullptr) {
         tc_epi_silu(eo, taddr, nt * 128 + q * 32 + lane, pass * 256, 0, c_end);
         if (q == 0 && lane == 0 && nt * 128 < N) c.gu_done[pass * ((N + 127) / 128) + nt] = gu_stamp(c, layer);   // read after the grid barrier
@@ -745,33 +763,30 @@ static __device__ __noinline__ void phase_gemm_tc(const DevCtx& c, const GemmArg
         else mbar_arrive(&g_tc.acc_empty[abuf]);
       }
       abuf ^= 1;
-      u = seg_end;
     }
   }
   if (warp < 4) {
     // Producers and the MMA issuer are done once the last MMA is committed: their warps store
     // the upper columns of the last accumulator.
     __syncwarp();
-    if (u0 < u1) {
+    if (g.u0 < g.u1) {
       const uint32_t par = tc.last_bit;
       tc.last_bit ^= 1u;
-      long long last_u = u0;
+      TcSeg sg = tc_seg_first(g);   // the last segment and its accumulator buffer
       int last_abuf = 0;
-      for (long long u = u0; u < u1;) {   // find the last segment and its accumulator buffer
-        last_u = u;
-        u = min(u1, (u / kblocks + 1) * (long long)kblocks);
-        if (u < u1) last_abuf ^= 1;
+      while (!tc_seg_is_last(sg)) {
+        tc_seg_next(g, sg);
+        last_abuf ^= 1;
       }
-      const int kb0 = (int)(last_u % kblocks);
-      const int nt = tc_my_tile<PAIR>(tc_unit_nt(g, last_u), rank);
-      const int pass = tc_unit_pass(g, last_u);
+      const int nt = tc_my_tile<PAIR>(sg.nt, rank);
+      const int pass = sg.pass;
       const int n_mma = (min(256, T - pass * 256) + 15) & ~15;
       const int c_begin = tc_epi_half(n_mma);
       // every thread waits (also when it has no columns to store) so that its parity stays in step
       if (mbar_wait_idle(c, &g_tc.acc_last, par, dead) && c_begin < n_mma) {
         tc_fence_after();
         const TcEpiOut eo{a.out, (size_t)a.ldo, a.row_map, a.row_scale, T, N, ilv_F, act_direct};
-        const bool plain = (kb0 == 0 && (long long)kb0 + (u1 - last_u) == kblocks) && a.accumulate == 0 && eo.row_map == nullptr;
+        const bool plain = (sg.kb0 == 0 && sg.kb1 == kblocks) && a.accumulate == 0 && eo.row_map == nullptr;
         const uint32_t taddr = tc.tmem_base + (uint32_t)last_abuf * 256u + ((uint32_t)(warp * 32) << 16);
         if (plain && eo.act != nullptr) tc_epi_silu(eo, taddr, nt * 128 + warp * 32 + lane, pass * 256, c_begin, n_mma);
         else tc_epi_columns(eo, taddr, nt * 128 + warp * 32 + lane, pass * 256, c_begin, n_mma, plain);
