@@ -789,26 +789,32 @@ static __device__ __noinline__ int silu_pending_units(const unsigned long long* 
   }
   return count;
 }
-// A CTA takes a quarter of a pending unit at a time: 64 rows x 64 features, four items per thread.  The
+// A CTA takes up to a quarter of a pending unit at a time: 64 rows x 64 features, four items per thread.  The
 // loads are asynchronous copies into a staging area in shared memory (each thread reads back only what it
 // copied itself), so four items are in flight per thread without holding registers for them: a body that
 // needs many registers here changes the register allocation of the other phase functions of the loop
 // kernel, to their cost.
+// Token rows per pass of a tensor-core GEMM over T rows: at most 256, a multiple of 16, the passes as even as they go.
+__device__ __forceinline__ int tc_pass_rows(int T) {
+  const unsigned passes = (unsigned)(T + 255) >> 8;
+  return (int)((((unsigned)T + passes - 1u) / passes + 15u) & ~15u);
+}
 constexpr int SILU_STAGE_OFF = 32768 * 4;   // bytes: the staging area follows the list of pending units
 template <typename WT>
 __device__ __noinline__ void silu_mul_pending(float* __restrict__ gu, WT* __restrict__ out, int T, int F, const int* list, int count) {
-  const int tiles = F >> 6;
+  const int tiles = F >> 6, pass_rows = tc_pass_rows(T);
   const int r_in = threadIdx.x >> 4, col = (threadIdx.x & 15) << 2;
   const char* stage = reinterpret_cast<const char*>(list) + SILU_STAGE_OFF + threadIdx.x * 16;   // [8][FWD_THREADS] x 16 bytes
   const uint32_t stage_s = (uint32_t)__cvta_generic_to_shared(stage);
   for (int q = blockIdx.x; q < count * 4; q += gridDim.x) {
     const int unit = list[q >> 2];
     const int pass = unit / tiles, tile = unit - pass * tiles;
-    const int row0 = (pass << 8) + ((q & 3) << 6) + r_in, j = (tile << 6) + col;
+    const int row0 = pass * pass_rows + ((q & 3) << 6) + r_in, j = (tile << 6) + col;
+    const int t_end = min(T, (pass + 1) * pass_rows);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const int t = row0 + 16 * k;
-      if (t < T) {
+      if (t < t_end) {
         const float* src = gu + (size_t)t * 2 * F + j;
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(stage_s + (2 * k) * FWD_THREADS * 16), "l"(src) : "memory");
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(stage_s + (2 * k + 1) * FWD_THREADS * 16), "l"(src + F) : "memory");
@@ -819,7 +825,7 @@ __device__ __noinline__ void silu_mul_pending(float* __restrict__ gu, WT* __rest
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const int t = row0 + 16 * k;
-      if (t < T) {
+      if (t < t_end) {
         const float4 g = *reinterpret_cast<const float4*>(stage + (2 * k) * FWD_THREADS * 16);
         const float4 u = *reinterpret_cast<const float4*>(stage + (2 * k + 1) * FWD_THREADS * 16);
         silu_store<WT>(gu, out, t, j, F, g, u, true);

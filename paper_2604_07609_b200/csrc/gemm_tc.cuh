@@ -34,8 +34,8 @@ namespace blink {
 
 enum GemmWhich : int { GEMM_QKV = 0, GEMM_O, GEMM_GU, GEMM_DOWN, GEMM_LMHEAD, GEMM_KINDS };
 enum ActBuf : int { ACT_XN = 0, ACT_ATTN, ACT_ACT, ACT_XS, ACT_XG, ACT_BUFS };
-constexpr int TC_BOXES = 5;  // token-tile boxes of 16, 32, 64, 128, 256 rows
-constexpr int TC_MAX_STAGES = 8;
+constexpr int TC_BOXES = 32;  // token-tile boxes of 8, 16, .. 256 rows (one 1 KiB group of the operand image each step)
+constexpr int TC_MAX_STAGES = 11;
 constexpr int TC_A_BYTES = 128 * 128;  // 128 weight rows x 64 bf16
 constexpr int TC_TILE_BUDGET = 196608;
 
@@ -103,6 +103,38 @@ __device__ __forceinline__ bool mbar_wait(const DevCtx& c, uint64_t* bar, uint32
     }
   }
   return true;
+}
+
+// One lane of the (converged) warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+// The same wait by a whole warp, with one answer for all of its lanes.  The single-threaded roles of the GEMM
+// (MMA issue, copies) run as converged warps that elect a lane for the issuing instruction: their loop state is
+// then uniform and stays in uniform registers.  As the code of one lane in a diverged branch the MMA issuer took
+// 100 cycles per MMA and 200 per satisfied wait, which made it the limit of every large GEMM.
+static __device__ __noinline__ bool mbar_wait_warp_slow(const DevCtx& c, uint64_t* bar, uint32_t parity) {
+  volatile int* dead = &g_tc.dead;
+  const long long t0 = clock64();
+  unsigned int spins = 0;
+  while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) {
+    if ((++spins & 63u) == 0) {
+      bool stop = *dead != 0;
+      if (!stop && (unsigned long long)(clock64() - t0) > c.barrier_timeout_cycles) {
+        *dead = 1;
+        if ((threadIdx.x & 31) == 0) dev_fail(c, DEV_ERR_PIPE_TIMEOUT);
+        stop = true;
+      }
+      if (__any_sync(0xffffffffu, stop)) return false;
+    }
+  }
+  return true;
+}
+__device__ __forceinline__ bool mbar_wait_warp(const DevCtx& c, uint64_t* bar, uint32_t parity) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  return mbar_wait_warp_slow(c, bar, parity);
 }
 
 __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
@@ -211,15 +243,7 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// arrive (optionally announcing `bytes` of copies) on the barrier at the same shared-memory offset in CTA 0 of the pair
-__device__ __forceinline__ void mbar_expect_tx_cta0(uint64_t* bar, uint32_t bytes) {
-  asm volatile(
-      "{\n\t.reg .b32 ra;\n\t"
-      "mapa.shared::cluster.u32 ra, %0, 0;\n\t"
-      "mbarrier.arrive.expect_tx.shared::cluster.b64 _, [ra], %1;\n\t}" ::"r"(smem_u32(bar)),
-      "r"(bytes)
-      : "memory");
-}
+// arrive on the barrier at the same shared-memory offset in CTA 0 of the pair
 __device__ __forceinline__ void mbar_arrive_cta0(uint64_t* bar) {
   asm volatile(
       "{\n\t.reg .b32 ra;\n\t"
@@ -296,9 +320,11 @@ __device__ __forceinline__ void tc_init(const DevCtx& c, float*, TcState& s) {
   s.fill_bits = s.use_bits = s.acc_mma = s.acc_epi = s.last_bit = 0;
   if (!c.gemm_tc) return;
   if (threadIdx.x == 32) {
-    // pairs: the operands of a stage come from four producers (two per CTA), counted on CTA 0's barrier;
-    // an accumulator is free again when the epilogue warps of both CTAs have drained it
-    for (int i = 0; i < TC_MAX_STAGES; ++i) { mbar_init(&g_tc.full[i], PAIR ? 4 : 2); mbar_init(&g_tc.empty[i], 1); }
+    // pairs: the operands of a stage come from four producers (two per CTA), all counted on CTA 0's barrier,
+    // where CTA 0's two producers announce the bytes of both CTAs (an announcement by CTA 1 would be a remote
+    // arrival on the path of every stage); an accumulator is free again when the epilogue warps of both CTAs
+    // have drained it
+    for (int i = 0; i < TC_MAX_STAGES; ++i) { mbar_init(&g_tc.full[i], 2); mbar_init(&g_tc.empty[i], 1); }
     for (int b = 0; b < 2; ++b) { mbar_init(&g_tc.acc_full[b], 1); mbar_init(&g_tc.acc_empty[b], PAIR ? 8 : 4); }
     mbar_init(&g_tc.acc_last, 1);
     g_tc.dead = 0;
@@ -418,7 +444,7 @@ __device__ __forceinline__ int tc_epi_half(int n_mma) { return n_mma >= 128 ? ((
 // subroutine of a few hundred cycles, and three of them per stage in the single-threaded producers used to set
 // the time of a stage (0.64 us per k-block whatever its bytes; 2.7 TB/s of weights at 256 rows, 43 % tensor pipe).
 struct TcGeom {
-  int kblocks, ntiles, passes, box_id, box_rows, load_box, KPS, S;
+  int kblocks, ntiles, passes, pass_rows, load_box, KPS, S;
   int pass_fixed, pdiv;   // one token pass per CTA (or -1), and the passes interleaved in its unit order
   uint32_t b_bytes, stage_bytes;
   int u0, u1;
@@ -433,18 +459,15 @@ __device__ __forceinline__ TcGeom tc_geom(const DevCtx& c, int T, int N, int K, 
   g.kblocks = (int)((unsigned)K >> 6);
   g.ntiles = ntiles;   // weight tiles of 128 rows, or pairs of them
   g.passes = (int)((unsigned)(T + 255) >> 8);
-  g.box_id = TC_BOXES - 1;
-  if (g.passes == 1) {
-    g.box_id = 0;
-    while ((16 << g.box_id) < T) ++g.box_id;
-  }
-  g.box_rows = 16 << g.box_id;
+  // even passes: the workers of a weight tile's passes take equal shares, so the longest pass sets the time
+  // (520 rows as 3 x 176 instead of 256 + 256 + 8: gate/up of the 8B shape 123 -> 98 us)
+  g.pass_rows = tc_pass_rows(T);
   // A stage holds one k-block, or two when the token tile is small and the weights are stored as
   // contiguous tiles (then one bulk copy brings 32 KiB): fewer, larger copies per producer step.
-  g.KPS = (c.w_streaming && g.box_rows <= 128) ? 2 : 1;
-  // pairs: each CTA stages half of the token rows of a pass (the box that covers n_mma / 2 rows)
-  g.load_box = half_tokens ? (g.box_id > 0 ? g.box_id - 1 : 0) : g.box_id;
-  g.b_bytes = (uint32_t)(16 << g.load_box) * 128u;
+  g.KPS = (c.w_streaming && g.pass_rows <= 128) ? 2 : 1;
+  // the box that covers the token rows this CTA stages: pairs stage half of the rows of a pass each
+  g.load_box = (half_tokens ? g.pass_rows >> 4 : g.pass_rows >> 3) - 1;
+  g.b_bytes = (uint32_t)(8 * (g.load_box + 1)) * 128u;
   g.stage_bytes = (uint32_t)g.KPS * (TC_A_BYTES + g.b_bytes);
   g.S = (int)((unsigned)TC_TILE_BUDGET / g.stage_bytes);
   if (g.S > TC_MAX_STAGES) g.S = TC_MAX_STAGES;
@@ -533,15 +556,15 @@ __device__ __forceinline__ char* tc_tiles(float* smem_f) {
 template <bool PAIR>
 __device__ __forceinline__ int tc_my_tile(int nt_unit, uint32_t rank) { return PAIR ? 2 * nt_unit + (int)rank : nt_unit; }
 
-// Weight producer (one thread): stream the weight tiles of this CTA's range through the ring.
+// Weight producer (one warp): stream the weight tiles of this CTA's range through the ring.
 template <bool PAIR>
 __device__ __forceinline__ void tc_produce_weights(const DevCtx& c, const void* w, long long w_row0, int which,
                                                    const TcGeom& g, char* tiles, TcState& tc, uint32_t rank) {
   const TcMaps* maps = reinterpret_cast<const TcMaps*>(c.tc_maps);
   const CUtensorMap* map_a = &maps->w[which];
   const int row_a0 = (int)w_row0;
-  volatile int* dead = &g_tc.dead;
   const uint64_t stream_policy = l2_evict_first();
+  uint32_t fill_bits = tc.fill_bits;
   int stage = 0;
   for (TcSeg sg = tc_seg_first(g); sg.left > 0; tc_seg_next(g, sg)) {
     const int nt = tc_my_tile<PAIR>(sg.nt, rank);
@@ -550,57 +573,129 @@ __device__ __forceinline__ void tc_produce_weights(const DevCtx& c, const void* 
     for (int kb = sg.kb0; kb < sg.kb1;) {
       const int nk = min(g.KPS, sg.kb1 - kb);
       // the n-th fill of a stage waits for its (n-1)-th release
-      if (!mbar_wait(c, &g_tc.empty[stage], ((tc.fill_bits >> stage) & 1u) ^ 1u, dead)) return;
-      tc.fill_bits ^= 1u << stage;
+      if (!mbar_wait_warp(c, &g_tc.empty[stage], ((fill_bits >> stage) & 1u) ^ 1u)) { tc.fill_bits = fill_bits; return; }
+      fill_bits ^= 1u << stage;
       char* sa = tiles + (size_t)stage * g.stage_bytes;
-      if constexpr (PAIR) {
-        mbar_expect_tx_cta0(&g_tc.full[stage], (uint32_t)nk * TC_A_BYTES);
-        if (c.w_streaming) {   // one or two consecutive tiles per copy
-          tma_pair_load_3d(sa, &maps->ws[which][nk - 1], 0, 0, tile0 + kb, &g_tc.full[stage], stream_policy);
+      if (elect_one()) {
+        if constexpr (PAIR) {
+          if (rank == 0) mbar_expect_tx(&g_tc.full[stage], 2u * (uint32_t)nk * TC_A_BYTES);
+          if (c.w_streaming) {   // one or two consecutive tiles per copy
+            tma_pair_load_3d(sa, &maps->ws[which][nk - 1], 0, 0, tile0 + kb, &g_tc.full[stage], stream_policy);
+          } else {
+            tma_pair_load_2d(sa, map_a, kb * 64, row_a0 + nt * 128, &g_tc.full[stage], stream_policy);
+          }
         } else {
-          tma_pair_load_2d(sa, map_a, kb * 64, row_a0 + nt * 128, &g_tc.full[stage], stream_policy);
-        }
-      } else {
-        mbar_expect_tx(&g_tc.full[stage], (uint32_t)nk * TC_A_BYTES);
-        if (c.w_streaming) {  // contiguous tiles, already in the shared-memory operand image
-          tma_bulk_load_hint(sa, tile_ptr + (size_t)kb * TC_A_BYTES, (uint32_t)nk * TC_A_BYTES, &g_tc.full[stage],
-                             stream_policy);
-        } else {
-          tma_load_2d_hint(sa, map_a, kb * 64, row_a0 + nt * 128, &g_tc.full[stage], stream_policy);
+          mbar_expect_tx(&g_tc.full[stage], (uint32_t)nk * TC_A_BYTES);
+          if (c.w_streaming) {  // contiguous tiles, already in the shared-memory operand image
+            tma_bulk_load_hint(sa, tile_ptr + (size_t)kb * TC_A_BYTES, (uint32_t)nk * TC_A_BYTES, &g_tc.full[stage],
+                               stream_policy);
+          } else {
+            tma_load_2d_hint(sa, map_a, kb * 64, row_a0 + nt * 128, &g_tc.full[stage], stream_policy);
+          }
         }
       }
       kb += nk;
       if (++stage == g.S) stage = 0;
     }
   }
+  tc.fill_bits = fill_bits;
 }
 
-// Token-tile producer (one thread): the same sequence of stages, nk k-blocks of one segment each.
+// Token-tile producer (one warp): the same sequence of stages, nk k-blocks of one segment each.
 template <bool PAIR>
 __device__ __forceinline__ void tc_produce_tokens(const DevCtx& c, const CUtensorMap* map_b, int x_row0, int T, const TcGeom& g,
                                                   char* tiles, TcState& tc, uint32_t rank) {
-  volatile int* dead = &g_tc.dead;
   const uint64_t keep_policy = l2_evict_normal();
+  uint32_t fill_bits = tc.fill_bits;
   int stage = 0;
   for (TcSeg sg = tc_seg_first(g); sg.left > 0; tc_seg_next(g, sg)) {
     // pairs: this CTA's half of the pass is rows [rank * n_mma / 2, + n_mma / 2) (the box may reach further)
-    const int n_mma = (min(256, T - sg.pass * 256) + 15) & ~15;
-    const int row0 = x_row0 + sg.pass * 256 + (PAIR ? (int)rank * (n_mma / 2) : 0);
+    const int n_mma = (min(g.pass_rows, T - sg.pass * g.pass_rows) + 15) & ~15;
+    const int row0 = x_row0 + sg.pass * g.pass_rows + (PAIR ? (int)rank * (n_mma / 2) : 0);
     for (int kb = sg.kb0; kb < sg.kb1;) {
       const int nk = min(g.KPS, sg.kb1 - kb);
-      if (!mbar_wait(c, &g_tc.empty[stage], ((tc.fill_bits >> stage) & 1u) ^ 1u, dead)) return;
-      tc.fill_bits ^= 1u << stage;
+      if (!mbar_wait_warp(c, &g_tc.empty[stage], ((fill_bits >> stage) & 1u) ^ 1u)) { tc.fill_bits = fill_bits; return; }
+      fill_bits ^= 1u << stage;
       char* sb = tiles + (size_t)stage * g.stage_bytes + g.KPS * TC_A_BYTES;
-      if constexpr (PAIR) mbar_expect_tx_cta0(&g_tc.full[stage], (uint32_t)nk * g.b_bytes);
-      else mbar_expect_tx(&g_tc.full[stage], (uint32_t)nk * g.b_bytes);
-      for (int j = 0; j < nk; ++j) {
-        if constexpr (PAIR) tma_pair_load_2d(sb + j * g.b_bytes, map_b, (kb + j) * 64, row0, &g_tc.full[stage], keep_policy);
-        else tma_load_2d(sb + j * g.b_bytes, map_b, (kb + j) * 64, row0, &g_tc.full[stage]);
+      if (elect_one()) {
+        if (!PAIR || rank == 0) mbar_expect_tx(&g_tc.full[stage], (PAIR ? 2u : 1u) * (uint32_t)nk * g.b_bytes);
+        for (int j = 0; j < nk; ++j) {
+          if constexpr (PAIR) tma_pair_load_2d(sb + j * g.b_bytes, map_b, (kb + j) * 64, row0, &g_tc.full[stage], keep_policy);
+          else tma_load_2d(sb + j * g.b_bytes, map_b, (kb + j) * 64, row0, &g_tc.full[stage]);
+        }
       }
       kb += nk;
       if (++stage == g.S) stage = 0;
     }
   }
+  tc.fill_bits = fill_bits;
+}
+
+// MMA issuer (one warp): accumulates the segments of the range in turn, one accumulator buffer each.
+template <bool PAIR>
+__device__ __forceinline__ void tc_issue_mmas(const DevCtx& c, int T, const TcGeom& g, char* tiles, TcState& tc) {
+  const int KPS = g.KPS;
+  const uint64_t desc0 = smem_desc_sw128(smem_u32(tiles));   // stages follow one another: only the address field moves
+  const uint32_t stage_step = g.stage_bytes >> 4, b_off = ((uint32_t)KPS * TC_A_BYTES) >> 4, b_step = g.b_bytes >> 4;
+  uint32_t use_bits = tc.use_bits, acc_mma = tc.acc_mma;
+  int stage = 0;
+  int abuf = 0;
+  bool ok = true;
+  for (TcSeg sg = tc_seg_first(g); ok && sg.left > 0; tc_seg_next(g, sg)) {
+    const int rows = min(g.pass_rows, T - sg.pass * g.pass_rows);
+    const int n_mma = (rows + 15) & ~15;
+    const uint32_t idesc = PAIR ? idesc_bf16_pair(n_mma) : idesc_bf16(n_mma);
+    const uint32_t d_tmem = tc.tmem_base + (uint32_t)abuf * 256u;
+    if (!mbar_wait_warp(c, &g_tc.acc_empty[abuf], ((acc_mma >> abuf) & 1u) ^ 1u)) break;
+    acc_mma ^= 1u << abuf;
+    tc_fence_after();
+    for (int kb = sg.kb0; kb < sg.kb1; kb += KPS) {
+      if (!mbar_wait_warp(c, &g_tc.full[stage], (use_bits >> stage) & 1u)) { ok = false; break; }
+      use_bits ^= 1u << stage;
+      tc_fence_after();
+      const uint64_t da = desc0 + (uint64_t)(stage_step * (uint32_t)stage), db = da + (uint64_t)b_off;
+      const uint32_t more = kb > sg.kb0 ? 1u : 0u;   // the segment's first MMA overwrites the accumulator
+      const bool two = KPS == 2 && kb + 1 < sg.kb1;
+      if (elect_one()) {
+        // 16 bf16 = 32 bytes further along K inside the swizzle atom: +2 in 16-byte units
+#pragma unroll
+        for (int k16 = 0; k16 < 4; ++k16) {
+          if constexpr (PAIR) umma_bf16_pair(d_tmem, da + (uint64_t)(2 * k16), db + (uint64_t)(2 * k16), idesc, k16 ? 1u : more);
+          else umma_bf16(d_tmem, da + (uint64_t)(2 * k16), db + (uint64_t)(2 * k16), idesc, k16 ? 1u : more);
+        }
+        if (two) {
+          const uint64_t da2 = da + (uint64_t)(TC_A_BYTES >> 4), db2 = db + (uint64_t)b_step;
+#pragma unroll
+          for (int k16 = 0; k16 < 4; ++k16) {
+            if constexpr (PAIR) umma_bf16_pair(d_tmem, da2 + (uint64_t)(2 * k16), db2 + (uint64_t)(2 * k16), idesc, 1u);
+            else umma_bf16(d_tmem, da2 + (uint64_t)(2 * k16), db2 + (uint64_t)(2 * k16), idesc, 1u);
+          }
+        }
+        if constexpr (PAIR) umma_commit_pair(&g_tc.empty[stage]);
+        else umma_commit(&g_tc.empty[stage]);
+      }
+      __syncwarp();
+      if (++stage == g.S) stage = 0;
+    }
+    if (!ok) break;
+    // Warps 0-3 take part of the CTA's last accumulator.  They cannot wait on acc_full: a parity
+    // wait tells two consecutive completions apart, not the first use of a buffer in this phase
+    // from its third, and they arrive here long before the epilogue warps.  A barrier of their own
+    // that completes exactly once per phase has no such ambiguity.
+    if (elect_one()) {
+      if constexpr (PAIR) {
+        umma_commit_pair(&g_tc.acc_full[abuf]);
+        if (tc_seg_is_last(sg)) umma_commit_pair(&g_tc.acc_last);
+      } else {
+        umma_commit(&g_tc.acc_full[abuf]);
+        if (tc_seg_is_last(sg)) umma_commit(&g_tc.acc_last);
+      }
+    }
+    __syncwarp();
+    abuf ^= 1;
+  }
+  tc.use_bits = use_bits;
+  tc.acc_mma = acc_mma;
 }
 
 // ---- consumers of finished output tiles -------------------------------------------------------------
@@ -644,7 +739,7 @@ static __device__ __noinline__ void tc_finish_tiles(const DevCtx& c, const GemmA
     more = s_more;
     for (int i = 0; i < n; ++i) {
       const int tile = s_fin[i] & 0xffff, pass = s_fin[i] >> 16;
-      const int t0 = pass * 256, t1 = min(a.M, t0 + 256);
+      const int t0 = pass * g.pass_rows, t1 = min(a.M, t0 + g.pass_rows);
       if (a.fix == FIX_ROPE_KV) fixup_rope_kv<__nv_bfloat16>(c, layer, tile, t0, t1);
       else if (a.fix == FIX_SILU) fixup_silu<__nv_bfloat16>(a.out, reinterpret_cast<__nv_bfloat16*>(a.fix_out), a.N / 2, two_tiles ? tile * 128 : tile * 64, two_tiles ? 128 : 64, t0, t1);
       else fixup_sumsq(a.out, a.ldo, a.N, a.fix_rowss, tile, t0, t1);
@@ -669,8 +764,7 @@ static __device__ __noinline__ void phase_gemm_tc(const DevCtx& c, const GemmArg
                                   (int)blockIdx.x / 2, (n_tiles128 + 1) / 2, true)
                         : tc_geom(c, T, N, K, which == GEMM_LMHEAD && lm_head_whole_tiles(c), (int)gridDim.x, (int)blockIdx.x,
                                   n_tiles128, false);
-  const int kblocks = g.kblocks, KPS = g.KPS, S = g.S;
-  const uint32_t b_bytes = g.b_bytes, stage_bytes = g.stage_bytes;
+  const int kblocks = g.kblocks;
   const int act_id = which == GEMM_O ? ACT_ATTN : which == GEMM_DOWN ? ACT_ACT : which == GEMM_LMHEAD ? ACT_XS
                      : (which == GEMM_GU && c.E > 0) ? ACT_XG : ACT_XN;
   const CUtensorMap* map_b = &maps->act[act_id][g.load_box];
@@ -679,60 +773,11 @@ static __device__ __noinline__ void phase_gemm_tc(const DevCtx& c, const GemmArg
   volatile int* dead = &g_tc.dead;
 
   if (warp == 0) {
-    if (lane == 0) tc_produce_weights<PAIR>(c, a.w, a.w_row0, which, g, tiles, tc, rank);
+    tc_produce_weights<PAIR>(c, a.w, a.w_row0, which, g, tiles, tc, rank);
   } else if (warp == 2) {
-    // token-tile producer: walks the same sequence of stages (nk k-blocks of one segment each)
-    if (lane == 0) tc_produce_tokens<PAIR>(c, map_b, a.x_row0, T, g, tiles, tc, rank);
+    tc_produce_tokens<PAIR>(c, map_b, a.x_row0, T, g, tiles, tc, rank);
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {   // pairs: CTA 0 issues the MMAs for both
-      int stage = 0;
-      int abuf = 0;
-      bool ok = true;
-      for (TcSeg sg = tc_seg_first(g); ok && sg.left > 0; tc_seg_next(g, sg)) {
-        const int rows = min(256, T - sg.pass * 256);
-        const int n_mma = (rows + 15) & ~15;
-        const uint32_t idesc = PAIR ? idesc_bf16_pair(n_mma) : idesc_bf16(n_mma);
-        const uint32_t d_tmem = tc.tmem_base + (uint32_t)abuf * 256u;
-        if (!mbar_wait(c, &g_tc.acc_empty[abuf], ((tc.acc_mma >> abuf) & 1u) ^ 1u, dead)) break;
-        tc.acc_mma ^= 1u << abuf;
-        tc_fence_after();
-        uint32_t accumulate = 0u;
-        for (int kb = sg.kb0; kb < sg.kb1; kb += KPS) {
-          const int nk = min(KPS, sg.kb1 - kb);
-          if (!mbar_wait(c, &g_tc.full[stage], (tc.use_bits >> stage) & 1u, dead)) { ok = false; break; }
-          tc.use_bits ^= 1u << stage;
-          tc_fence_after();
-          const uint32_t sa = smem_u32(tiles + (size_t)stage * stage_bytes);
-          for (int j = 0; j < nk; ++j) {
-            const uint64_t da = smem_desc_sw128(sa + j * TC_A_BYTES);
-            const uint64_t db = smem_desc_sw128(sa + KPS * TC_A_BYTES + j * b_bytes);
-#pragma unroll
-            for (int k16 = 0; k16 < 4; ++k16) {
-              // 16 bf16 = 32 bytes further along K inside the swizzle atom: +2 in 16-byte units
-              if constexpr (PAIR) umma_bf16_pair(d_tmem, da + (uint64_t)(2 * k16), db + (uint64_t)(2 * k16), idesc, accumulate);
-              else umma_bf16(d_tmem, da + (uint64_t)(2 * k16), db + (uint64_t)(2 * k16), idesc, accumulate);
-              accumulate = 1u;
-            }
-          }
-          if constexpr (PAIR) umma_commit_pair(&g_tc.empty[stage]);
-          else umma_commit(&g_tc.empty[stage]);
-          if (++stage == S) stage = 0;
-        }
-        if (!ok) break;
-        // Warps 0-3 take part of the CTA's last accumulator.  They cannot wait on acc_full: a parity
-        // wait tells two consecutive completions apart, not the first use of a buffer in this phase
-        // from its third, and they arrive here long before the epilogue warps.  A barrier of their own
-        // that completes exactly once per phase has no such ambiguity.
-        if constexpr (PAIR) {
-          umma_commit_pair(&g_tc.acc_full[abuf]);
-          if (tc_seg_is_last(sg)) umma_commit_pair(&g_tc.acc_last);
-        } else {
-          umma_commit(&g_tc.acc_full[abuf]);
-          if (tc_seg_is_last(sg)) umma_commit(&g_tc.acc_last);
-        }
-        abuf ^= 1;
-      }
-    }
+    if (rank == 0) tc_issue_mmas<PAIR>(c, T, g, tiles, tc);   // pairs: CTA 0 issues the MMAs for both
   } else if (warp >= 4) {
     const int q = warp & 3;  // TMEM lane quarter this warp may read
     const TcEpiOut eo{a.out, (size_t)a.ldo, a.row_map, a.row_scale, T, N, ilv_F, act_direct};
@@ -741,7 +786,8 @@ static __device__ __noinline__ void phase_gemm_tc(const DevCtx& c, const GemmArg
     for (TcSeg sg = tc_seg_first(g); sg.left > 0; tc_seg_next(g, sg)) {
       const int nt = tc_my_tile<PAIR>(sg.nt, rank);
       const int pass = sg.pass;
-      const int rows = min(256, T - pass * 256);
+      const int t_base = pass * g.pass_rows;
+      const int rows = min(g.pass_rows, T - t_base);
       const int n_mma = (rows + 15) & ~15;
       const bool plain = (sg.kb0 == 0 && sg.kb1 == kblocks) && !accumulate && eo.row_map == nullptr;
       if (!mbar_wait(c, &g_tc.acc_full[abuf], (tc.acc_epi >> abuf) & 1u, dead)) break;
@@ -751,10 +797,10 @@ static __device__ __noinline__ void phase_gemm_tc(const DevCtx& c, const GemmArg
       // the upper columns of the CTA's last accumulator are left to warps 0-3
       const int c_end = tc_seg_is_last(sg) ? tc_epi_half(n_mma) : n_mma;
       if (plain && eo.act != nullptr) {
-        tc_epi_silu(eo, taddr, nt * 128 + q * 32 + lane, pass * 256, 0, c_end);
+        tc_epi_silu(eo, taddr, nt * 128 + q * 32 + lane, t_base, 0, c_end);
         if (q == 0 && lane == 0 && nt * 128 < N) c.gu_done[pass * ((N + 127) / 128) + nt] = gu_stamp(c, layer);   // read after the grid barrier
       } else {
-        tc_epi_columns(eo, taddr, nt * 128 + q * 32 + lane, pass * 256, 0, c_end, plain);
+        tc_epi_columns(eo, taddr, nt * 128 + q * 32 + lane, t_base, 0, c_end, plain);
       }
       tc_fence_before();
       __syncwarp();
@@ -780,7 +826,8 @@ static __device__ __noinline__ void phase_gemm_tc(const DevCtx& c, const GemmArg
       }
       const int nt = tc_my_tile<PAIR>(sg.nt, rank);
       const int pass = sg.pass;
-      const int n_mma = (min(256, T - pass * 256) + 15) & ~15;
+      const int t_base = pass * g.pass_rows;
+      const int n_mma = (min(g.pass_rows, T - t_base) + 15) & ~15;
       const int c_begin = tc_epi_half(n_mma);
       // every thread waits (also when it has no columns to store) so that its parity stays in step
       if (mbar_wait_idle(c, &g_tc.acc_last, par, dead) && c_begin < n_mma) {
@@ -788,8 +835,8 @@ static __device__ __noinline__ void phase_gemm_tc(const DevCtx& c, const GemmArg
         const TcEpiOut eo{a.out, (size_t)a.ldo, a.row_map, a.row_scale, T, N, ilv_F, act_direct};
         const bool plain = (sg.kb0 == 0 && sg.kb1 == kblocks) && a.accumulate == 0 && eo.row_map == nullptr;
         const uint32_t taddr = tc.tmem_base + (uint32_t)last_abuf * 256u + ((uint32_t)(warp * 32) << 16);
-        if (plain && eo.act != nullptr) tc_epi_silu(eo, taddr, nt * 128 + warp * 32 + lane, pass * 256, c_begin, n_mma);
-        else tc_epi_columns(eo, taddr, nt * 128 + warp * 32 + lane, pass * 256, c_begin, n_mma, plain);
+        if (plain && eo.act != nullptr) tc_epi_silu(eo, taddr, nt * 128 + warp * 32 + lane, t_base, c_begin, n_mma);
+        else tc_epi_columns(eo, taddr, nt * 128 + warp * 32 + lane, t_base, c_begin, n_mma, plain);
         tc_fence_before();
       }
     }
@@ -875,7 +922,7 @@ inline int tc_host_setup(TcHost& h, DevCtx& c) {
   const uint64_t rows[ACT_BUFS] = {(uint64_t)c.Tmax, (uint64_t)c.Tmax, RA, (uint64_t)c.MB, c.xg ? RA : (uint64_t)c.Tmax};
   const uint64_t cols[ACT_BUFS] = {(uint64_t)c.d, (uint64_t)c.q_dim, (uint64_t)c.F, (uint64_t)c.d, (uint64_t)c.d};
   for (int b = 0; b < ACT_BUFS; ++b)
-    for (int i = 0; i < TC_BOXES; ++i) ok &= tc_make_map(enc, &hm->act[b][i], bufs[b], rows[b], cols[b], 16u << i, false);
+    for (int i = 0; i < TC_BOXES; ++i) ok &= tc_make_map(enc, &hm->act[b][i], bufs[b], rows[b], cols[b], 8u * (uint32_t)(i + 1), false);
   int rc = 0;
   if (!ok) rc = -7;
   if (rc == 0 && cudaMalloc(&h.d_maps, sizeof(TcMaps)) != cudaSuccess) rc = -6;
