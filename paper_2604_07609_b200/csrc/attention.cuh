@@ -31,14 +31,21 @@ __shared__ int g_att_pre[MAX_BATCH + 1];   // prefix of KV blocks over the decod
 __shared__ int g_att_bslot[MAX_BATCH];
 __shared__ int g_att_nctx[MAX_BATCH];
 __shared__ int g_att_row[MAX_BATCH];
+// the step's scalars: like the arrays above they do not change between layers and are read from memory once per step
+struct AttStep {
+  int n_dec, TT, S, C, npf;
+};
+__shared__ AttStep g_att_step;
 
 // per-thread state that survives from phase to phase (mbarrier parities of the warp's ring)
 struct AttState {
   uint32_t par;
+  int blk;   // CTA-wide decode: the lane's block id of the CTA's first item (the same in all layers of a step)
 };
 
 __device__ __forceinline__ void att_init(const DevCtx& c, AttState& s) {
   s.par = 0;
+  s.blk = 0;
   if (c.dtype != 0 || c.control_only) return;
   if ((threadIdx.x & 31) == 0) {
     for (int i = 0; i < ATT_NS; ++i) mbar_init(&g_att.bar[threadIdx.x >> 5][i], 1);
@@ -86,6 +93,18 @@ __device__ __forceinline__ void dec_seek(DecCursor& cur, int f, int f_end, int n
   cur.g = rem / cur.nkb;
   cur.kb = rem - cur.g * cur.nkb;
 }
+// tiles [b0, b1) of sub-range `id`: S tiles of the flat sequence, or (S == 0) one whole unit
+__device__ __forceinline__ void dec_sub_range(int id, int S, int TT, int Hkv, int& b0, int& b1) {
+  if (S > 0) {
+    b0 = id * S;
+    b1 = min(TT, b0 + S);
+  } else {
+    const int d = id / Hkv, g = id - d * Hkv;
+    const int pre = g_att_pre[d], nkb = g_att_pre[d + 1] - pre;
+    b0 = Hkv * pre + g * nkb;
+    b1 = b0 + nkb;
+  }
+}
 __device__ __forceinline__ void dec_advance(DecCursor& cur, int n_dec, int Hkv) {
   cur.f += 1;
   if (++cur.kb == cur.nkb) {
@@ -114,6 +133,73 @@ __device__ __forceinline__ void mma_bf16_16816(float* d, const uint32_t* a, uint
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// One 16-key tile of a (row, kv head) unit by one warp: scores, online softmax, out += P V (see below).
+template <int HD>
+__device__ __forceinline__ void att_tile_math(uint32_t kt, uint32_t vt, int n_valid, float qscale, const uint32_t (&qf)[HD / 16][2],
+                                              float (&o)[HD / 16][4], float (&m2)[2], float (&l2)[2]) {
+  constexpr int KS = HD / 16, NBOX = HD / 64;
+  const int lane = threadIdx.x & 31;
+  const int gq = lane >> 2;
+  // The matrix loads and MMAs below are issued in program order, so all loads of an operand are
+  // issued before the MMAs that use them, and V is fetched before the softmax arithmetic.
+  uint32_t kf[KS][4];    // A operand of the scores: K tile, keys x dims
+#pragma unroll
+  for (int ks = 0; ks < KS; ++ks) {
+    const int key = (lane & 7) + ((lane >> 3) & 1) * 8;
+    const int ck = ks * 2 + (lane >> 4);
+    const int line = key * NBOX + (ck >> 3);   // 128-byte line of the tile; chunks are swizzled with the line index
+    ldsm_x4(kt + line * 128 + (((ck & 7) ^ (line & 7)) << 4), kf[ks][0], kf[ks][1], kf[ks][2], kf[ks][3]);
+  }
+  uint32_t vf[HD / 16][4];   // A operand of the output: V tile transposed, dims x keys
+#pragma unroll
+  for (int i = 0; i < HD / 16; ++i) {
+    const int key = (lane & 7) + ((lane >> 4) & 1) * 8;
+    const int ck = i * 2 + ((lane >> 3) & 1);
+    const int line = key * NBOX + (ck >> 3);
+    ldsm_x4_t(vt + line * 128 + (((ck & 7) ^ (line & 7)) << 4), vf[i][0], vf[i][1], vf[i][2], vf[i][3]);
+  }
+  // scores^T [16 keys][8 heads]: four accumulators (k-step mod 4) keep the dependent chains short
+  float sacc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) { sacc[i][0] = sacc[i][1] = sacc[i][2] = sacc[i][3] = 0.f; }
+#pragma unroll
+  for (int ks = 0; ks < KS; ++ks) mma_bf16_16816(sacc[ks & 3], kf[ks], qf[ks][0], qf[ks][1]);
+  float sv[4];   // keys gq (0, 1) and gq + 8 (2, 3), heads 2 tq (0, 2) and 2 tq + 1 (1, 3)
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const float v = (sacc[0][e] + sacc[1][e]) + (sacc[2][e] + sacc[3][e]);
+    sv[e] = (gq + (e >> 1) * 8 < n_valid) ? v * qscale : -INFINITY;
+  }
+  // online softmax per head: maxima over the 16 keys live in the lanes with the same tq
+  float mx0 = fmaxf(sv[0], sv[2]), mx1 = fmaxf(sv[1], sv[3]);
+#pragma unroll
+  for (int sh = 4; sh <= 16; sh <<= 1) {
+    mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, sh));
+    mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, sh));
+  }
+  const float mn0 = fmaxf(m2[0], mx0), mn1 = fmaxf(m2[1], mx1);   // finite: key 0 of the tile is always valid
+  if (__any_sync(0xffffffffu, mn0 > m2[0] || mn1 > m2[1])) {
+    const float c0 = fast_ex2(m2[0] - mn0), c1 = fast_ex2(m2[1] - mn1);
+    l2[0] *= c0; l2[1] *= c1;
+#pragma unroll
+    for (int i = 0; i < HD / 16; ++i) { o[i][0] *= c0; o[i][1] *= c1; o[i][2] *= c0; o[i][3] *= c1; }
+  }
+  m2[0] = mn0; m2[1] = mn1;
+  const float p0 = fast_ex2(sv[0] - mn0), p1 = fast_ex2(sv[1] - mn1), p2 = fast_ex2(sv[2] - mn0), p3 = fast_ex2(sv[3] - mn1);
+  l2[0] += p0 + p2;
+  l2[1] += p1 + p3;
+  // P^T as the B operand of the output: transpose the two 8 x 8 (key, head) blocks in registers
+  uint32_t pb0, pb1;
+  {
+    const uint32_t plo = pack_bf2(p0, p1), phi = pack_bf2(p2, p3);
+    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(pb0) : "r"(plo));
+    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(pb1) : "r"(phi));
+  }
+  // out^T += V^T P^T: 16 dims per MMA, one k-step of 16 keys
+#pragma unroll
+  for (int i = 0; i < HD / 16; ++i) mma_bf16_16816(o[i], vf[i], pb0, pb1);
+}
+
 // ---- decode rows: warp-level streaming kernel -------------------------------------------------
 // One warp owns a (row, kv head) unit at a time and walks its 16-key tiles.  A tile's K and V
 // ([16 keys][head_dim] each, contiguous in the pool) arrive through one TMA tile copy with the
@@ -133,11 +219,10 @@ __device__ __noinline__ void attn_decode_stream(const DevCtx& c, int layer, char
   constexpr int REC = NREP * HD + ((2 * NREP + 3) & ~3);  // floats per partial record, 16-byte multiple
   constexpr unsigned FULL = 0xffffffffu;
   static_assert(NREP <= 8, "the group's heads must fit the first eight operand rows");
-  const SchedState* ss = c.ss;
-  const int n_dec = ss->cur_ndec, TT = ss->cur_TT, S = ss->cur_S;
+  const int n_dec = g_att_step.n_dec, TT = g_att_step.TT, S = g_att_step.S;   // S == 0: a sub-range is a unit
   if (TT <= 0) return;
-  const int n_sub = (TT + S - 1) / S;
   const int Hkv = c.Hkv;
+  const int n_sub = S > 0 ? (TT + S - 1) / S : n_dec * Hkv;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int gq = lane >> 2, tq = lane & 3;   // operand row (= head of the group) and column pair
   const bool live = gq < NREP;   // this lane loads the q of head gq
@@ -180,8 +265,7 @@ __device__ __noinline__ void attn_decode_stream(const DevCtx& c, int layer, char
             id = __shfl_sync(FULL, id, 0);
           }
           if (id >= n_sub) { p_done = true; break; }
-          b0 = id * S;
-          b1 = min(TT, id * S + S);
+          dec_sub_range(id, S, TT, Hkv, b0, b1);
           if (b0 < b1) break;
         }
         if (p_done) break;
@@ -212,8 +296,9 @@ __device__ __noinline__ void attn_decode_stream(const DevCtx& c, int layer, char
     while (cc.f == cc.f_end) {   // next non-empty sub-range (the producer already issued a tile of it)
       sub_id = g_att.ids[w][c_k & 7];
       c_k += 1;
-      sub_start = sub_id * S;
-      dec_seek(cc, sub_start, min(TT, sub_start + S), n_dec, Hkv);
+      int sub_end;
+      dec_sub_range(sub_id, S, TT, Hkv, sub_start, sub_end);
+      dec_seek(cc, sub_start, sub_end, n_dec, Hkv);
       in_unit = false;
     }
     const int t_row = g_att_row[cc.d];
@@ -244,64 +329,7 @@ __device__ __noinline__ void attn_decode_stream(const DevCtx& c, int layer, char
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // before TMA refills this stage
       __syncwarp();
     }
-    // The matrix loads and MMAs below are issued in program order, so all loads of an operand are
-    // issued before the MMAs that use them, and V is fetched before the softmax arithmetic.
-    uint32_t kf[KS][4];    // A operand of the scores: K tile, keys x dims
-#pragma unroll
-    for (int ks = 0; ks < KS; ++ks) {
-      const int key = (lane & 7) + ((lane >> 3) & 1) * 8;
-      const int ck = ks * 2 + (lane >> 4);
-      const int line = key * NBOX + (ck >> 3);   // 128-byte line of the tile; chunks are swizzled with the line index
-      ldsm_x4(kt + line * 128 + (((ck & 7) ^ (line & 7)) << 4), kf[ks][0], kf[ks][1], kf[ks][2], kf[ks][3]);
-    }
-    uint32_t vf[HD / 16][4];   // A operand of the output: V tile transposed, dims x keys
-#pragma unroll
-    for (int i = 0; i < HD / 16; ++i) {
-      const int key = (lane & 7) + ((lane >> 4) & 1) * 8;
-      const int ck = i * 2 + ((lane >> 3) & 1);
-      const int line = key * NBOX + (ck >> 3);
-      ldsm_x4_t(vt + line * 128 + (((ck & 7) ^ (line & 7)) << 4), vf[i][0], vf[i][1], vf[i][2], vf[i][3]);
-    }
-    // scores^T [16 keys][8 heads]: four accumulators (k-step mod 4) keep the dependent chains short
-    float sacc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) { sacc[i][0] = sacc[i][1] = sacc[i][2] = sacc[i][3] = 0.f; }
-#pragma unroll
-    for (int ks = 0; ks < KS; ++ks) mma_bf16_16816(sacc[ks & 3], kf[ks], qf[ks][0], qf[ks][1]);
-    float sv[4];   // keys gq (0, 1) and gq + 8 (2, 3), heads 2 tq (0, 2) and 2 tq + 1 (1, 3)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float v = (sacc[0][e] + sacc[1][e]) + (sacc[2][e] + sacc[3][e]);
-      sv[e] = (gq + (e >> 1) * 8 < n_valid) ? v * qscale : -INFINITY;
-    }
-    // online softmax per head: maxima over the 16 keys live in the lanes with the same tq
-    float mx0 = fmaxf(sv[0], sv[2]), mx1 = fmaxf(sv[1], sv[3]);
-#pragma unroll
-    for (int sh = 4; sh <= 16; sh <<= 1) {
-      mx0 = fmaxf(mx0, __shfl_xor_sync(FULL, mx0, sh));
-      mx1 = fmaxf(mx1, __shfl_xor_sync(FULL, mx1, sh));
-    }
-    const float mn0 = fmaxf(m2[0], mx0), mn1 = fmaxf(m2[1], mx1);   // finite: key 0 of the tile is always valid
-    if (__any_sync(FULL, mn0 > m2[0] || mn1 > m2[1])) {
-      const float c0 = fast_ex2(m2[0] - mn0), c1 = fast_ex2(m2[1] - mn1);
-      l2[0] *= c0; l2[1] *= c1;
-#pragma unroll
-      for (int i = 0; i < HD / 16; ++i) { o[i][0] *= c0; o[i][1] *= c1; o[i][2] *= c0; o[i][3] *= c1; }
-    }
-    m2[0] = mn0; m2[1] = mn1;
-    const float p0 = fast_ex2(sv[0] - mn0), p1 = fast_ex2(sv[1] - mn1), p2 = fast_ex2(sv[2] - mn0), p3 = fast_ex2(sv[3] - mn1);
-    l2[0] += p0 + p2;
-    l2[1] += p1 + p3;
-    // P^T as the B operand of the output: transpose the two 8 x 8 (key, head) blocks in registers
-    uint32_t pb0, pb1;
-    {
-      const uint32_t plo = pack_bf2(p0, p1), phi = pack_bf2(p2, p3);
-      asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(pb0) : "r"(plo));
-      asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(pb1) : "r"(phi));
-    }
-    // out^T += V^T P^T: 16 dims per MMA, one k-step of 16 keys
-#pragma unroll
-    for (int i = 0; i < HD / 16; ++i) mma_bf16_16816(o[i], vf[i], pb0, pb1);
+    att_tile_math<HD>(kt, vt, n_valid, qscale, qf, o, m2, l2);
     __syncwarp();  // all reads of this stage are done before it is refilled
     n_consumed += 1;
 
@@ -315,7 +343,7 @@ __device__ __noinline__ void attn_decode_stream(const DevCtx& c, int layer, char
         lt1 += __shfl_xor_sync(FULL, lt1, sh);
       }
       const int us = Hkv * g_att_pre[cc.d] + cc.g * cc.nkb, ue = us + cc.nkb;
-      const int j_first = us / S, j_last = (ue - 1) / S;
+      const int j_first = S > 0 ? us / S : 0, j_last = S > 0 ? (ue - 1) / S : 0;
       const int h0 = 2 * tq;   // this lane's heads: h0, h0 + 1
       if (j_first == j_last) {   // the whole unit was handled here
         __nv_bfloat16* obase = out + (size_t)t_row * c.q_dim + (size_t)(cc.g * NREP) * HD;
@@ -382,6 +410,182 @@ __device__ __noinline__ void attn_decode_stream(const DevCtx& c, int layer, char
       }
     }
     dec_advance(cc, n_dec, Hkv);
+  }
+}
+
+// ---- decode rows: one CTA per part of a unit -----------------------------------------------------------
+// Few (row, kv head) units, as a handful of requests make them: the streaming kernel above gives a unit to one
+// warp, or cuts it and pays a record, a fence, a counter and a merge by one warp for every cut, so that one row of
+// 300 keys took 22 us and one of 4000 keys 51 us per layer, nearly all of it latency.  Here the eight warps of a
+// CTA share a part of a unit (C tiles, no part crosses units): their tiles are in flight at once, their sums are
+// merged in shared memory, and only units of more than C tiles leave records, merged by the whole last CTA.
+constexpr int ATT_NSC = 2;   // ring stages per warp here
+template <int HD, int NREP>
+static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer, char* base, AttState& as) {
+  constexpr int RB = HD * 2;
+  constexpr int TILE = 16 * RB;
+  constexpr int STAGE = 2 * TILE;
+  constexpr int KS = HD / 16;
+  constexpr int REC = NREP * HD + ((2 * NREP + 3) & ~3);
+  constexpr unsigned FULL = 0xffffffffu;
+  __shared__ float s_m[ATT_WARPS][8], s_l[ATT_WARPS][8];
+  __shared__ int s_last;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int gq = lane >> 2, tq = lane & 3;
+  const bool live = gq < NREP;
+  const int n_dec = g_att_step.n_dec, C = g_att_step.C, Hkv = c.Hkv;
+  float* s_o = reinterpret_cast<float*>(base + ATT_WARPS * ATT_NSC * STAGE);   // [warps][NREP][HD]
+  char* ring = base + w * ATT_NSC * STAGE;
+  uint64_t* bars = g_att.bar[w];
+  volatile int* dead = &g_att.dead;
+  const CUtensorMap* kv_map = reinterpret_cast<const CUtensorMap*>(c.kv_map);
+  const __nv_bfloat16* qb = reinterpret_cast<const __nv_bfloat16*>(c.qb);
+  __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(c.attn);
+  const float qscale = c.attn_scale * 1.4426950408889634f;
+  const uint64_t kv_policy = l2_evict_first();
+
+  // items in unit order; prefill tiles of a step sit on the first CTAs, so the decode items start from the last
+  for (int item = (int)gridDim.x - 1 - (int)blockIdx.x; ; item += gridDim.x) {   // uniform over the CTA
+    int d = 0, rest = item, nkb = 0, ns = 1;
+    for (; d < n_dec; ++d) {
+      nkb = g_att_pre[d + 1] - g_att_pre[d];
+      ns = (nkb + C - 1) / C;
+      if (rest < Hkv * ns) break;
+      rest -= Hkv * ns;
+    }
+    if (d >= n_dec) break;
+    const int g = rest / ns, part = rest - g * ns;
+    const int kb0 = part * C, kb1 = min(nkb, kb0 + C);
+    const int n_tiles = kb0 + w < kb1 ? (kb1 - kb0 - w + ATT_WARPS - 1) / ATT_WARPS : 0;   // kb0 + w, + 8, ...
+    const int t_row = g_att_row[d], n_ctx = g_att_nctx[d];
+    const int32_t* table = c.block_table + (size_t)g_att_bslot[d] * c.max_blocks_seq;
+    // block ids of the warp's first 32 tiles, one per lane; the first item's are kept from layer to layer
+    const bool first = item < (int)gridDim.x;
+    int blk = as.blk;
+    if (!(first && layer > 0 && !c.stepped)) {
+      blk = lane < n_tiles ? table[kb0 + w + ATT_WARPS * lane] : 0;
+      if (first) as.blk = blk;
+    }
+    auto issue = [&](int i) {
+      if (i >= 32 && (i & 31) == 0) blk = i + lane < n_tiles ? table[kb0 + w + ATT_WARPS * (i + lane)] : 0;
+      const int b = __shfl_sync(FULL, blk, i & 31);
+      if (lane == 0) {
+        const int s = i % ATT_NSC;
+        mbar_expect_tx(&bars[s], STAGE);
+        tma_load_5d(ring + s * STAGE, kv_map, 0, 0, (b * Hkv + g) * 16, 0, layer, &bars[s], kv_policy);
+      }
+    };
+#pragma unroll
+    for (int i = 0; i < ATT_NSC; ++i)
+      if (i < n_tiles) issue(i);
+    uint32_t qf[KS][2];
+    float o[HD / 16][4];
+    float m2[2] = {-INFINITY, -INFINITY}, l2[2] = {0.f, 0.f};
+    {
+      const __nv_bfloat16* qrow = qb + (size_t)t_row * c.q_dim + (size_t)(g * NREP + (live ? gq : 0)) * HD;
+#pragma unroll
+      for (int ks = 0; ks < KS; ++ks) {
+        qf[ks][0] = live ? *reinterpret_cast<const uint32_t*>(qrow + ks * 16 + 2 * tq) : 0u;
+        qf[ks][1] = live ? *reinterpret_cast<const uint32_t*>(qrow + ks * 16 + 8 + 2 * tq) : 0u;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < HD / 16; ++i) { o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f; }
+    for (int i = 0; i < n_tiles; ++i) {
+      const int s = i % ATT_NSC;
+      if (!__all_sync(FULL, mbar_wait(c, &bars[s], (as.par >> s) & 1u, dead))) break;
+      as.par ^= 1u << s;
+      char* st = ring + s * STAGE;
+      const int n_valid = min(16, n_ctx - (kb0 + w + ATT_WARPS * i) * 16);   // >= 1
+      if (n_valid < 16) {   // the tail of the last block holds whatever the pool held: clear those V rows (0 x NaN)
+        uint4* vg = reinterpret_cast<uint4*>(st + TILE + n_valid * RB);
+        for (int k = lane; k < (16 - n_valid) * RB / 16; k += 32) vg[k] = make_uint4(0u, 0u, 0u, 0u);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+      }
+      att_tile_math<HD>(smem_u32(st), smem_u32(st) + TILE, n_valid, qscale, qf, o, m2, l2);
+      __syncwarp();   // all reads of this stage are done before it is refilled
+      if (i + ATT_NSC < n_tiles) issue(i + ATT_NSC);
+    }
+    // the warp's sums to shared memory
+    float lt0 = l2[0], lt1 = l2[1];
+#pragma unroll
+    for (int sh = 4; sh <= 16; sh <<= 1) {
+      lt0 += __shfl_xor_sync(FULL, lt0, sh);
+      lt1 += __shfl_xor_sync(FULL, lt1, sh);
+    }
+    const int h0 = 2 * tq;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      if (h0 + e < NREP) {
+        if (n_tiles > 0) {
+          float* ow = s_o + ((size_t)w * NREP + h0 + e) * HD;
+#pragma unroll
+          for (int i = 0; i < HD / 16; ++i) {
+            ow[16 * i + gq] = o[i][e];
+            ow[16 * i + 8 + gq] = o[i][2 + e];
+          }
+        }
+        if (gq == 0) { s_m[w][h0 + e] = m2[e]; s_l[w][h0 + e] = e ? lt1 : lt0; }
+      }
+    }
+    __syncthreads();
+    // merge the warps: a thread takes two consecutive dims of a head at a time
+    const int n_warps = min(ATT_WARPS, kb1 - kb0);   // warps 0 .. n_warps - 1 had tiles
+    float* rec = c.att_part + (size_t)item * REC;
+    __nv_bfloat16* obase = out + (size_t)t_row * c.q_dim + (size_t)(g * NREP) * HD;
+    for (int i2 = threadIdx.x; i2 < NREP * HD / 2; i2 += FWD_THREADS) {
+      const int h = i2 * 2 / HD;
+      float M = -INFINITY;
+      for (int k = 0; k < n_warps; ++k) M = fmaxf(M, s_m[k][h]);
+      float2 num = make_float2(0.f, 0.f);
+      float den = 0.f;
+      for (int k = 0; k < n_warps; ++k) {
+        const float f = fast_ex2(s_m[k][h] - M);
+        const float2 a = *reinterpret_cast<const float2*>(s_o + (size_t)k * NREP * HD + i2 * 2);
+        num.x = fmaf(f, a.x, num.x);
+        num.y = fmaf(f, a.y, num.y);
+        den = fmaf(f, s_l[k][h], den);
+      }
+      if (ns == 1) {
+        const float inv = __fdividef(1.0f, den);
+        *reinterpret_cast<uint32_t*>(obase + i2 * 2) = pack_bf2(num.x * inv, num.y * inv);
+      } else {
+        *reinterpret_cast<float2*>(rec + i2 * 2) = num;
+        if ((i2 * 2) % HD == 0) { rec[NREP * HD + h] = M; rec[NREP * HD + NREP + h] = den; }
+      }
+    }
+    if (ns > 1) {
+      const int unit = d * Hkv + g;
+      __threadfence();
+      __syncthreads();
+      if (threadIdx.x == 0) s_last = atomicAdd(&c.att_cnt[unit], 1) == ns - 1;
+      __syncthreads();
+      if (s_last) {   // this CTA delivered the last part: merge in part order (records of a unit are consecutive)
+        __threadfence();
+        const float* r0 = c.att_part + (size_t)(item - part) * REC;
+        for (int i2 = threadIdx.x; i2 < NREP * HD / 2; i2 += FWD_THREADS) {
+          const int h = i2 * 2 / HD;
+          float M = -INFINITY;
+#pragma unroll 8
+          for (int k = 0; k < ns; ++k) M = fmaxf(M, __ldcg(r0 + (size_t)k * REC + NREP * HD + h));
+          float2 num = make_float2(0.f, 0.f);
+          float den = 0.f;
+#pragma unroll 8
+          for (int k = 0; k < ns; ++k) {
+            const float f = fast_ex2(__ldcg(r0 + (size_t)k * REC + NREP * HD + h) - M);
+            const float2 a = __ldcg(reinterpret_cast<const float2*>(r0 + (size_t)k * REC) + i2);
+            num.x = fmaf(f, a.x, num.x);
+            num.y = fmaf(f, a.y, num.y);
+            den = fmaf(f, __ldcg(r0 + (size_t)k * REC + NREP * HD + NREP + h), den);
+          }
+          const float inv = __fdividef(1.0f, den);
+          *reinterpret_cast<uint32_t*>(obase + i2 * 2) = pack_bf2(num.x * inv, num.y * inv);
+        }
+        if (threadIdx.x == 0) c.att_cnt[unit] = 0;
+      }
+    }
+    __syncthreads();   // the sums in shared memory are free for the next item
   }
 }
 
@@ -562,31 +766,40 @@ __device__ __noinline__ void attn_prefill_tile(const DevCtx& c, int layer, int i
 template <int HD>
 constexpr int att_smem_bytes() {
   constexpr int ring = ATT_WARPS * ATT_NS * 2 * 16 * HD * 2 + 1024;   // + alignment slack
+  constexpr int cta = ATT_WARPS * ATT_NSC * 2 * 16 * HD * 2 + ATT_WARPS * 8 * HD * 4 + 1024;   // up to 8 heads per group
   constexpr int tile = 128 * HD * 2 + 2 * 2 * 64 * HD * 2;
-  return ring > tile ? ring : tile;
+  return ring > cta ? (ring > tile ? ring : tile) : (cta > tile ? cta : tile);
 }
 
 template <int HD, int NREP>
 __device__ __forceinline__ void phase_attention_bf16(const DevCtx& c, int layer, float* smem_f, AttState& as) {
-  const SchedState* ss = c.ss;
   char* smem = reinterpret_cast<char*>(smem_f);
-  const int n_pf = ss->cur_npf * c.Hkv;
+  if (layer == 0 || c.stepped) {   // the step's work lists: once per step
+    const SchedState* ss = c.ss;
+    const int n = ss->cur_ndec;
+    if (threadIdx.x == 0) g_att_step = AttStep{n, ss->cur_TT, ss->cur_S, ss->cur_C, ss->cur_npf};
+    for (int i = threadIdx.x; i <= n; i += FWD_THREADS) {
+      g_att_pre[i] = c.dec_kbpre[i];
+      if (i < n) { g_att_bslot[i] = c.dec_bslot[i]; g_att_nctx[i] = c.dec_nctx[i]; g_att_row[i] = c.dec_row[i]; }
+    }
+    __syncthreads();
+  }
+  const int n_pf = g_att_step.npf * c.Hkv;
   for (int u = blockIdx.x; u < n_pf; u += gridDim.x) {
     const int e = u / c.Hkv, g = u % c.Hkv;
     attn_prefill_tile<HD, NREP>(c, layer, c.pf_item[e], c.pf_qb[e], g, smem);
   }
-  const int n_dec = ss->cur_ndec;
+  const int n_dec = g_att_step.n_dec;
   if (n_dec > 0) {
-    __syncthreads();
-    for (int i = threadIdx.x; i <= n_dec; i += FWD_THREADS) {
-      g_att_pre[i] = c.dec_kbpre[i];
-      if (i < n_dec) { g_att_bslot[i] = c.dec_bslot[i]; g_att_nctx[i] = c.dec_nctx[i]; g_att_row[i] = c.dec_row[i]; }
+    if (n_pf > 0) __syncthreads();   // the prefill tiles' shared memory is free
+    if (g_att_step.C > 0) {
+      attn_decode_cta<HD, NREP>(c, layer, tc_tiles(smem_f), as);
+    } else {
+      const int w = threadIdx.x >> 5;
+      constexpr int STAGE = 2 * 16 * HD * 2;
+      char* ring = tc_tiles(smem_f) + w * ATT_NS * STAGE;   // 1024-byte aligned: the tiles are swizzled
+      attn_decode_stream<HD, NREP>(c, layer, ring, as);
     }
-    __syncthreads();
-    const int w = threadIdx.x >> 5;
-    constexpr int STAGE = 2 * 16 * HD * 2;
-    char* ring = tc_tiles(smem_f) + w * ATT_NS * STAGE;   // 1024-byte aligned: the tiles are swizzled
-    attn_decode_stream<HD, NREP>(c, layer, ring, as);
   }
 }
 

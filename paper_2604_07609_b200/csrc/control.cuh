@@ -361,10 +361,12 @@ static __device__ int schedule_step(const DevCtx& c, unsigned long long visible)
   __shared__ int s_trace_ok;
   __shared__ unsigned long long s_ctx, s_kv;
   __shared__ int s_ndec;
+  __shared__ int s_nkb[MAX_BATCH];
+  __shared__ int s_maxkb, s_C, s_Citems;
 
   const uint64_t t_begin = global_timer_ns();
   s_phase[tid] = tid < MB ? c.b_phase[tid] : -1;
-  if (tid == 0) { s_n_admit = 0; s_ctx = 0; s_kv = 0; s_ndec = 0; }
+  if (tid == 0) { s_n_admit = 0; s_ctx = 0; s_kv = 0; s_ndec = 0; s_maxkb = 0; s_C = 0; s_Citems = 0; }
   __syncthreads();
 
   // open a trace record (header is completed later)
@@ -549,6 +551,8 @@ static __device__ int schedule_step(const DevCtx& c, unsigned long long visible)
         c.dec_bslot[dec_idx] = tid;
         c.dec_nctx[dec_idx] = new_len;
         c.dec_kbpre[dec_idx] = kb_pre;
+        s_nkb[dec_idx] = nkb_att;
+        atomicMax(&s_maxkb, nkb_att);
       }
       for (int q = 0; q < n_qb; ++q) {   // heaviest (last) row block first
         c.pf_item[pf_off + q] = item;
@@ -572,6 +576,23 @@ static __device__ int schedule_step(const DevCtx& c, unsigned long long visible)
   if (tid == 0) s_qstart[n_items] = T;
   __threadfence();
   __syncthreads();
+
+  // CTA-wide decode attention for few units: the smallest part size (of 32 candidates from a fair share up, at
+  // least 24 tiles: a cut unit costs a merge through memory, about the time of three tiles per warp) whose parts fit
+  // the grid at once; when none does, units stay whole
+  const int n_ctas = c.n_warps_grid / (CTRL_THREADS / 32);
+  if (tid < 32 && c.dec_row != nullptr && n_dec_att > 0 && n_dec_att * c.Hkv <= 2 * n_ctas) {
+    const int share = max(24, (tot_kb * c.Hkv + n_ctas - 1) / n_ctas);
+    const int C = share + tid * ((share + 7) / 8);
+    int parts = 0;
+    for (int i = 0; i < n_dec_att; ++i) parts += (s_nkb[i] + C - 1) / C;
+    const unsigned fit = __ballot_sync(0xffffffffu, parts * c.Hkv <= n_ctas);
+    const int pick = fit ? __ffs(fit) - 1 : 31;
+    if (tid == pick) {
+      s_C = fit ? C : s_maxkb;
+      s_Citems = fit ? parts * c.Hkv : n_dec_att * c.Hkv;
+    }
+  }
 
   // per-row metadata: token id, position, owning item, KV slot
   // every warp of the grid starts on the sub-range of its own index; the counter hands out the rest
@@ -621,10 +642,23 @@ static __device__ int schedule_step(const DevCtx& c, unsigned long long visible)
       // sub-range made a single 2048-token row take 120 us per layer, most of it the merge
       if (S < 8) S = 8;
       while ((TT + S - 1) / S > c.att_sub_max) S *= 2;   // cannot happen with the sizes set at create
+      // Three ways to run the decode units (estimates in quarters of a tile's time, about 0.8 us of one warp):
+      // the streaming kernel cuts the flat sequence evenly (at least 8 tiles per warp, about 10 tiles' time for the
+      // ends of cut units); whole units per warp need no cuts; a CTA per part shares a unit between eight warps.
+      const int U = n_dec_att * c.Hkv, maxkb = s_maxkb;
+      const long long t_stream = 4 * S * ((((TT + S - 1) / S) + NW - 1) / NW) + 40;
+      const long long t_unit = 4ll * maxkb * ((U + NW - 1) / NW) + 16;
+      int C = 0;
+      if (s_C > 0) {
+        const long long t_cta = ((s_Citems + n_ctas - 1) / n_ctas) * (4ll * ((min(s_C, maxkb) + 7) / 8) + 10) + (s_C < maxkb ? 14 : 0);
+        if (t_cta <= t_stream && t_cta <= t_unit) C = s_C;
+      }
+      if (C == 0 && t_unit < t_stream) S = 0;
       c.dec_kbpre[n_dec_att] = tot_kb;
       ss->cur_ndec = n_dec_att;
       ss->cur_TT = (int)TT;
       ss->cur_S = (int)S;
+      ss->cur_C = C;
       ss->cur_npf = n_pf;
     }
     if (tr) {

@@ -95,7 +95,8 @@ struct SchedState {
   int cur_T, cur_items, cur_rows, cur_decode;
   int cur_ndec;   // attention: requests with one query row in this step
   int cur_TT;     // attention: (row, kv head, KV block) tiles of those rows
-  int cur_S;      // attention: tiles per sub-range of the flat tile sequence
+  int cur_S;      // attention: tiles per sub-range of the flat tile sequence, 0 = a sub-range is a (row, kv head) unit
+  int cur_C;      // attention: > 0: decode units are shared by the warps of a CTA, C tiles per part
   int cur_npf;    // attention: (request, query-row block) units of the multi-row requests
   long long cur_ctx;
   long long cur_kv;
