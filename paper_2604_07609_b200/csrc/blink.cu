@@ -47,7 +47,7 @@ blink_sample_kernel(const float* logits, int rows, int V, const int* top_k, cons
   extern __shared__ __align__(1024) float smem[];
   for (int r = blockIdx.x; r < rows; r += gridDim.x) {
     const int tok = sample_row(logits + (size_t)r * V, V, min(top_k[r], MAX_TOPK), temp[r], top_p ? top_p[r] : 0.f, ticket[r],
-                               gen_index[r], seed[r], smem);
+                               gen_index[r], seed[r], smem, nullptr, nullptr, nullptr);
     if (threadIdx.x == 0) out[r] = tok;
   }
 }
@@ -322,7 +322,11 @@ int step_once(blink_ctx* x) {
           launch_phase(x, ph, l);
         }
       }
-    for (int ph = PH_FNORM; ph <= PH_SAMPLE; ++ph) launch_phase(x, ph, 0);
+    for (int i = 0; i < 5; ++i) {
+      const int ph = output_phase(i);
+      if ((ph == PH_SMAX || ph == PH_SNUC) && !sample_split_rows(x->dc.V)) continue;
+      launch_phase(x, ph, 0);
+    }
   }
   return cudaGetLastError() == cudaSuccess ? BLINK_OK : BLINK_ECUDA;
 }
@@ -745,6 +749,8 @@ int blink_create(const blink_model_cfg* model, const blink_sched_cfg* sched, con
     c.gu_direct = c.w_streaming && c.gemm_tc && c.E == 0 && !c.fused && gu_units <= 32768;
     TRY(dev_alloc(x, &c.gu_done, gu_units));
     TRY(dev_alloc(x, &c.logits, MB * c.V));
+    TRY(dev_alloc(x, &c.cmax, MB * SAMPLE_CHUNKS, false));
+    TRY(dev_alloc(x, &c.nuc_m, MB * 256, false)); TRY(dev_alloc(x, &c.nuc_c, MB * 256, false));
     TRY(dev_alloc(x, &c.rope_cos, (size_t)c.max_pos * (c.hd / 2), false));
     TRY(dev_alloc(x, &c.rope_sin, (size_t)c.max_pos * (c.hd / 2), false));
     std::vector<float> cs((size_t)c.max_pos * (c.hd / 2)), sn(cs.size());

@@ -362,11 +362,11 @@ static __device__ int schedule_step(const DevCtx& c, unsigned long long visible)
   __shared__ unsigned long long s_ctx, s_kv;
   __shared__ int s_ndec;
   __shared__ int s_nkb[MAX_BATCH];
-  __shared__ int s_maxkb, s_C, s_Citems;
+  __shared__ int s_maxkb, s_C, s_Citems, s_nuc;
 
   const uint64_t t_begin = global_timer_ns();
   s_phase[tid] = tid < MB ? c.b_phase[tid] : -1;
-  if (tid == 0) { s_n_admit = 0; s_ctx = 0; s_kv = 0; s_ndec = 0; s_maxkb = 0; s_C = 0; s_Citems = 0; }
+  if (tid == 0) { s_n_admit = 0; s_ctx = 0; s_kv = 0; s_ndec = 0; s_maxkb = 0; s_C = 0; s_Citems = 0; s_nuc = 0; }
   __syncthreads();
 
   // open a trace record (header is completed later)
@@ -544,6 +544,8 @@ static __device__ int schedule_step(const DevCtx& c, unsigned long long visible)
     if (sample) {
       c.row_tok[row] = qstart + take - 1;
       c.row_item[row] = item;
+      const float tp = c.b_topp[tid];
+      if (c.b_topk[tid] <= 0 && tp > 0.f && tp < 1.f) s_nuc = 1;
     }
     if (c.dec_row != nullptr) {
       if (is_dec) {
@@ -622,6 +624,7 @@ static __device__ int schedule_step(const DevCtx& c, unsigned long long visible)
     ss->cur_items = n_items;
     ss->cur_rows = n_rows;
     ss->cur_decode = s_ndec;
+    ss->cur_nuc = s_nuc;
     ss->cur_ctx = (long long)s_ctx;
     ss->cur_kv = (long long)s_kv;
     ss->cur_t_begin = t_begin;

@@ -97,6 +97,7 @@ struct SchedState {
   int cur_TT;     // attention: (row, kv head, KV block) tiles of those rows
   int cur_S;      // attention: tiles per sub-range of the flat tile sequence, 0 = a sub-range is a (row, kv head) unit
   int cur_C;      // attention: > 0: decode units are shared by the warps of a CTA, C tiles per part
+  int cur_nuc;    // some row of the step samples from the nucleus of the whole row
   int cur_npf;    // attention: (request, query-row block) units of the multi-row requests
   long long cur_ctx;
   long long cur_kv;
@@ -204,6 +205,9 @@ struct DevCtx {
   unsigned long long* gu_done;   // [token passes][gate/up weight tiles] stamp (iteration * L + layer + 1, 64 bits: never repeats) of the last such write
   int fused_norm;      // 1: the O and down epilogues add up sum(x^2) per row and the norms are element-wise
   float* logits;  // [MB][V]
+  float* cmax;                 // [MB][1024] maxima of the chunks of a row of logits
+  unsigned long long* nuc_m;   // [MB][256] nucleus rows: weight per bucket of z
+  unsigned int* nuc_c;         // [MB][256]               number of entries
   float *rope_cos, *rope_sin;  // [max_pos][hd/2]
   void* kv_base;               // [L][2][n_blocks][Hkv][bs][hd] operand type
   const void* tc_maps;         // TMA descriptors of the tensor-core path (device memory)

@@ -896,497 +896,6 @@ static __device__ __noinline__ void phase_moe_group(const DevCtx& c, float* smem
   }
 }
 
-// ---- sampling ------------------------------------------------------------------------------
-// Philox4x32-10 (Salmon et al., SC'11): counter-based, so the draw for (ticket, index)
-// does not depend on batch composition.
-__device__ __forceinline__ uint32_t philox4x32_10_word0(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
-                                                        uint32_t k0, uint32_t k1) {
-#pragma unroll
-  for (int r = 0; r < 10; ++r) {
-    const uint32_t hi0 = __umulhi(0xD2511F53u, c0), lo0 = 0xD2511F53u * c0;
-    const uint32_t hi1 = __umulhi(0xCD9E8D57u, c2), lo1 = 0xCD9E8D57u * c2;
-    const uint32_t n0 = hi1 ^ c1 ^ k0, n2 = hi0 ^ c3 ^ k1;
-    c0 = n0; c1 = lo1; c2 = n2; c3 = lo0;
-    k0 += 0x9E3779B9u; k1 += 0xBB67AE85u;
-  }
-  return c0;
-}
-
-// order-preserving map float -> uint32 (larger float => larger key)
-__device__ __forceinline__ uint32_t float_key(float f) {
-  const uint32_t u = __float_as_uint(f);
-  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-
-// ---- top-p (nucleus) arithmetic: Section 4.2 names "Top-P with temperature" as the in-step sampler ----
-// Weights are integers, q = floor(exp(z - z0) * 2^40) with z0 the largest z of the row, so that every
-// sum is exact and no result depends on the order in which a parallel machine adds: the nucleus is
-// the smallest prefix of the order (z desc, index asc) with cum * 2^24 >= P24 * Q (Q = total weight,
-// P24 = round(top_p * 2^24) in [1, 2^24]); the draw is renormalised to its weight M: with the 24-bit
-// uniform x24, the token is the first of the order with cum > (x24 * M) >> 24.
-__device__ __forceinline__ unsigned long long nucleus_weight(float z, float z0) {
-  return __double2ull_rd(exp((double)z - (double)z0) * 1099511627776.0);
-}
-__device__ __forceinline__ unsigned long long nucleus_p24(float top_p) {
-  long long p = (long long)rint((double)top_p * 16777216.0);
-  return (unsigned long long)(p < 1 ? 1 : (p > 16777216 ? 16777216 : p));
-}
-// ceil(p24 * Q / 2^24): the weight the nucleus has to reach (Q < 2^58, p24 <= 2^24)
-__device__ __forceinline__ unsigned long long nucleus_need(unsigned long long p24, unsigned long long Q) {
-  unsigned long long lo = p24 * Q, hi = __umul64hi(p24, Q);
-  const unsigned long long lo2 = lo + 16777215ull;
-  if (lo2 < lo) hi += 1;
-  return (hi << 40) | (lo2 >> 24);
-}
-// (x24 * M) >> 24
-__device__ __forceinline__ unsigned long long nucleus_target(unsigned long long x24, unsigned long long M) {
-  return (__umul64hi(x24, M) << 40) | ((x24 * M) >> 24);
-}
-
-// Shared state of the whole-row nucleus search (one CTA per row).
-constexpr int NUC_CAND = 1024;
-struct NucShared {
-  unsigned long long m0[256];   // level 0: weight per bucket of z (linear in z between the row's min and max)
-  unsigned int c0[256];         //          and number of entries
-  unsigned long long m[256];    // deeper levels: buckets linear in the float key inside [klo, khi]
-  unsigned int cn[256];
-  unsigned long long acc;       // weight of everything ahead of the current member set in the order
-  unsigned long long res_cum;   // result: cumulative weight up to and including the entry found
-  unsigned int klo, khi, cnt;
-  int b0, first, done, res_idx, n;
-  float zmin, scale;
-  unsigned int chunk_cnt[FWD_THREADS];
-};
-__device__ __forceinline__ int nuc_bucket0(float z, float zmin, float scale) {
-  const int b = (int)((z - zmin) * scale);
-  return b < 0 ? 0 : (b > 255 ? 255 : b);
-}
-
-// First entry of the order (z desc, index asc) whose cumulative weight exceeds t (t < total weight).
-// The member set starts as one level-0 bucket and is narrowed 256-fold per pass over the row (buckets
-// over the float-key interval of the set) until it fits the candidate buffer, which is then ranked
-// exactly.  A set that cannot be narrowed (more than NUC_CAND equal values) is resolved by index.
-static __device__ __noinline__ void nucleus_locate(NucShared& st, const float* lg, int V, float temp, float z0,
-                                                   unsigned long long t, float* s_cz, int* s_ci, float* s_sz, int* s_si) {
-  const int tid = threadIdx.x;
-  if (tid == 0) {
-    unsigned long long acc = 0;
-    int b = 255;
-    for (; b > 0; --b) {
-      if (acc + st.m0[b] > t) break;
-      acc += st.m0[b];
-    }
-    st.b0 = b; st.acc = acc; st.cnt = st.c0[b]; st.klo = 0u; st.khi = 0xffffffffu; st.first = 1; st.done = 0;
-  }
-  __syncthreads();
-  const float zmin = st.zmin, scale = st.scale;
-  for (int level = 0; level < 8; ++level) {   // a level divides the key interval by 256: four suffice
-    const int b0 = st.b0;
-    const unsigned int klo = st.klo, khi = st.khi;
-    if (st.cnt <= (unsigned)NUC_CAND) {
-      // ---- gather the members, rank them exactly, walk the cumulative weights ----
-      if (tid == 0) st.n = 0;
-      __syncthreads();
-      for (int i = tid; i < V; i += FWD_THREADS) {
-        const float z = __fdiv_rn(lg[i], temp);
-        const unsigned int key = float_key(z);
-        if (nuc_bucket0(z, zmin, scale) == b0 && key >= klo && key <= khi) {
-          const int p = atomicAdd(&st.n, 1);
-          if (p < NUC_CAND) { s_cz[p] = z; s_ci[p] = i; }
-        }
-      }
-      __syncthreads();
-      const int nc = min(st.n, NUC_CAND);
-      for (int a = tid; a < nc; a += FWD_THREADS) {
-        const float za = s_cz[a];
-        const int ia = s_ci[a];
-        int rank = 0;
-        for (int j = 0; j < nc; ++j) {
-          const float zj = s_cz[j];
-          rank += (zj > za) || (zj == za && s_ci[j] < ia);
-        }
-        s_sz[rank] = za; s_si[rank] = ia;
-      }
-      __syncthreads();
-      if (tid == 0) {
-        unsigned long long cum = st.acc;
-        int pick = nc > 0 ? s_si[nc - 1] : 0;
-        for (int j = 0; j < nc; ++j) {
-          cum += nucleus_weight(s_sz[j], z0);
-          if (cum > t) { pick = s_si[j]; break; }
-        }
-        st.res_idx = pick; st.res_cum = cum; st.done = 1;
-      }
-      __syncthreads();
-      return;
-    }
-    if (st.first) {   // key interval of the level-0 bucket's members
-      __syncthreads();
-      if (tid == 0) { st.klo = 0xffffffffu; st.khi = 0u; }
-      __syncthreads();
-      for (int i = tid; i < V; i += FWD_THREADS) {
-        const float z = __fdiv_rn(lg[i], temp);
-        if (nuc_bucket0(z, zmin, scale) == b0) {
-          const unsigned int key = float_key(z);
-          atomicMin(&st.klo, key);
-          atomicMax(&st.khi, key);
-        }
-      }
-      __syncthreads();
-      if (tid == 0) st.first = 0;
-      __syncthreads();
-      continue;   // same member set, now with its key interval
-    }
-    if (klo == khi) {
-      // ---- more than NUC_CAND entries with one and the same z: equal weights, ordered by index ----
-      const float z = __uint_as_float((klo & 0x80000000u) ? (klo & 0x7fffffffu) : ~klo);
-      const unsigned long long q0 = nucleus_weight(z, z0);            // > 0: the set's weight exceeds t - acc
-      const unsigned long long jl = q0 > 0 ? (t - st.acc) / q0 : 0;   // entries of the set ahead of the one sought
-      const int ch = (V + FWD_THREADS - 1) / FWD_THREADS;
-      const int i0 = tid * ch, i1 = min(V, i0 + ch);
-      unsigned int mine = 0;
-      for (int i = i0; i < i1; ++i) {
-        const float zi = __fdiv_rn(lg[i], temp);
-        mine += (nuc_bucket0(zi, zmin, scale) == b0 && float_key(zi) == klo) ? 1u : 0u;
-      }
-      st.chunk_cnt[tid] = mine;
-      __syncthreads();
-      unsigned long long before = 0;
-      for (int k = 0; k < tid; ++k) before += st.chunk_cnt[k];
-      if (jl >= before && jl < before + mine) {
-        unsigned long long seen = before;
-        for (int i = i0; i < i1; ++i) {
-          const float zi = __fdiv_rn(lg[i], temp);
-          if (nuc_bucket0(zi, zmin, scale) == b0 && float_key(zi) == klo) {
-            if (seen == jl) { st.res_idx = i; st.res_cum = st.acc + (jl + 1) * q0; st.done = 1; break; }
-            ++seen;
-          }
-        }
-      }
-      __syncthreads();
-      if (tid == 0 && !st.done) { st.res_idx = 0; st.res_cum = st.acc; st.done = 1; }   // cannot happen for t < total
-      __syncthreads();
-      return;
-    }
-    // ---- one more level: 256 buckets over the key interval [klo, khi] ----
-    st.m[tid] = 0ull;
-    st.cn[tid] = 0u;
-    __syncthreads();
-    const unsigned long long W = (unsigned long long)khi - klo + 1ull;
-    for (int i = tid; i < V; i += FWD_THREADS) {
-      const float z = __fdiv_rn(lg[i], temp);
-      const unsigned int key = float_key(z);
-      if (nuc_bucket0(z, zmin, scale) == b0 && key >= klo && key <= khi) {
-        const int b = (int)((((unsigned long long)(key - klo)) << 8) / W);
-        atomicAdd(&st.m[b], nucleus_weight(z, z0));
-        atomicAdd(&st.cn[b], 1u);
-      }
-    }
-    __syncthreads();
-    if (tid == 0) {
-      unsigned long long acc = st.acc;
-      int b = 255;
-      for (; b > 0; --b) {
-        if (acc + st.m[b] > t) break;
-        acc += st.m[b];
-      }
-      st.acc = acc;
-      st.cnt = st.cn[b];
-      // keys of bucket b: (key - klo) * 256 / W == b
-      st.klo = klo + (unsigned int)(((unsigned long long)b * W + 255ull) >> 8);
-      st.khi = klo + (unsigned int)((((unsigned long long)(b + 1) * W + 255ull) >> 8) - 1ull);
-    }
-    __syncthreads();
-  }
-  if (tid == 0 && !st.done) { st.res_idx = 0; st.res_cum = st.acc; st.done = 1; }
-  __syncthreads();
-}
-
-// Top-p over the whole row (no top-k cut): z = logit / T, weights and order as described above.
-// The result is returned by thread 0 (other threads return -1).
-static __device__ __noinline__ int sample_row_nucleus(const float* lg, int V, float temp, float top_p, unsigned long long ticket,
-                                                      int gen_index, unsigned long long seed, float* smem) {
-  __shared__ NucShared st;
-  __shared__ float s_mx[FWD_THREADS / 32], s_mn[FWD_THREADS / 32];
-  const int tid = threadIdx.x;
-  float* s_cz = smem + 256;
-  int* s_ci = reinterpret_cast<int*>(smem + 256 + NUC_CAND);
-  float* s_sz = smem + 256 + 2 * NUC_CAND;
-  int* s_si = reinterpret_cast<int*>(smem + 256 + 3 * NUC_CAND);
-  __syncthreads();
-  // range of the row (z is monotone in the logit, so min and max can be taken on logits)
-  float lmax = -INFINITY, lmin = INFINITY;
-  for (int i = tid; i < V; i += FWD_THREADS) {
-    const float v = lg[i];
-    lmax = fmaxf(lmax, v);
-    lmin = fminf(lmin, v);
-  }
-  lmax = warp_max(lmax);
-  lmin = -warp_max(-lmin);
-  if ((tid & 31) == 0) { s_mx[tid >> 5] = lmax; s_mn[tid >> 5] = lmin; }
-  st.m0[tid] = 0ull;
-  st.c0[tid] = 0u;
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < FWD_THREADS / 32; ++i) { lmax = fmaxf(lmax, s_mx[i]); lmin = fminf(lmin, s_mn[i]); }
-  const float z0 = __fdiv_rn(lmax, temp), zmin = __fdiv_rn(lmin, temp);
-  const float scale = z0 > zmin ? 255.0f / (z0 - zmin) : 0.0f;
-  if (tid == 0) { st.zmin = zmin; st.scale = scale; }
-  // level 0: weights per bucket of z
-  for (int i = tid; i < V; i += FWD_THREADS) {
-    const float z = __fdiv_rn(lg[i], temp);
-    const int b = nuc_bucket0(z, zmin, scale);
-    atomicAdd(&st.m0[b], nucleus_weight(z, z0));
-    atomicAdd(&st.c0[b], 1u);
-  }
-  __syncthreads();
-  __shared__ unsigned long long s_t;
-  if (tid == 0) {
-    unsigned long long Q = 0;
-    for (int b = 0; b < 256; ++b) Q += st.m0[b];
-    s_t = nucleus_need(nucleus_p24(top_p), Q) - 1ull;   // first entry with cum >= need  <=>  cum > need - 1
-  }
-  __syncthreads();
-  nucleus_locate(st, lg, V, temp, z0, s_t, s_cz, s_ci, s_sz, s_si);   // end of the nucleus: its weight is res_cum
-  if (tid == 0) {
-    const uint32_t x = philox4x32_10_word0((uint32_t)ticket, (uint32_t)(ticket >> 32), (uint32_t)gen_index, 0u,
-                                           (uint32_t)seed, (uint32_t)(seed >> 32));
-    s_t = nucleus_target((unsigned long long)(x >> 8), st.res_cum);
-  }
-  __syncthreads();
-  nucleus_locate(st, lg, V, temp, z0, s_t, s_cz, s_ci, s_sz, s_si);
-  const int result = tid == 0 ? st.res_idx : -1;
-  __syncthreads();
-  return result;
-}
-
-// One CTA per sampled row.  Greedy: lowest index among the maxima.  Top-k: z = logit / T
-// (IEEE fp32 divide); the k largest by (z desc, index asc) are found with a radix select
-// on the float keys; weights exp(z - z0) and the inverse-CDF walk run in fp64.
-// The result is returned by thread 0 (other threads return -1).
-static __device__ int sample_row(const float* lg, int V, int top_k, float temp, float top_p, unsigned long long ticket,
-                                 int gen_index, unsigned long long seed, float* smem) {
-  constexpr int CAND_MAX = 1024;
-  const int tid = threadIdx.x;
-  uint32_t* s_hist = reinterpret_cast<uint32_t*>(smem);             // [256]
-  float* s_cz = smem + 256;                                          // [CAND_MAX]
-  int* s_ci = reinterpret_cast<int*>(smem + 256 + CAND_MAX);         // [CAND_MAX]
-  __shared__ float s_bv[FWD_THREADS / 32];
-  __shared__ int s_bi[FWD_THREADS / 32];
-  __shared__ unsigned long long s_prefix, s_mask;
-  __shared__ int s_remaining, s_ncand;
-  __shared__ float s_tz[MAX_TOPK];
-  __shared__ int s_ti[MAX_TOPK];
-  int result = -1;
-  const bool nucleus = top_p > 0.f && top_p < 1.f;   // outside (0, 1): no nucleus cut
-  if (top_k <= 0 && nucleus) return sample_row_nucleus(lg, V, temp, top_p, ticket, gen_index, seed, smem);
-  __syncthreads();
-  if (top_k <= 0) {
-    float bv = -INFINITY;
-    int bi = 0x7fffffff;
-    for (int i = tid; i < V; i += FWD_THREADS) {
-      const float v = lg[i];
-      if (v > bv || (v == bv && i < bi)) { bv = v; bi = i; }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
-    }
-    if ((tid & 31) == 0) { s_bv[tid >> 5] = bv; s_bi[tid >> 5] = bi; }
-    __syncthreads();
-    if (tid == 0) {
-      for (int i = 1; i < FWD_THREADS / 32; ++i)
-        if (s_bv[i] > bv || (s_bv[i] == bv && s_bi[i] < bi)) { bv = s_bv[i]; bi = s_bi[i]; }
-      result = bi;
-    }
-    __syncthreads();
-    return result;
-  }
-  const int k = min(top_k, V);
-  // Fast path.  Every thread takes the maximum of its strided share of the row; the k-th largest
-  // of those 256 maxima, tau, is a lower bound of the k-th largest z of the row (k threads hold an
-  // element >= tau each), so {z >= tau} contains the top k and is usually a few dozen elements.
-  // z = logit / T is monotone in the logit, so the maxima can be taken on logits and divided once.
-  {
-    float* s_tm = smem;   // [FWD_THREADS] thread maxima of z (aliases the histogram, not live yet)
-    float lmax = -INFINITY;
-    const bool vec = (V & 3) == 0 && ((size_t)lg & 15) == 0;
-    if (vec) {
-      const float4* lg4 = reinterpret_cast<const float4*>(lg);
-#pragma unroll 8
-      for (int i = tid; i < V / 4; i += FWD_THREADS) {
-        const float4 v = lg4[i];
-        lmax = fmaxf(fmaxf(lmax, fmaxf(v.x, v.y)), fmaxf(v.z, v.w));
-      }
-    } else {
-      for (int i = tid; i < V; i += FWD_THREADS) lmax = fmaxf(lmax, lg[i]);
-    }
-    const float zmax = __fdiv_rn(lmax, temp);
-    s_tm[tid] = zmax;
-    if (tid == 0) s_ncand = 0;
-    __syncthreads();
-    int rank = 0;
-    for (int j = 0; j < FWD_THREADS; ++j) {
-      const float zj = s_tm[j];
-      rank += (zj > zmax) || (zj == zmax && j < tid);
-    }
-    __syncthreads();
-    if (rank == k - 1) s_tm[0] = zmax;
-    __syncthreads();
-    const float tau = s_tm[0];
-    __syncthreads();
-    if (tau > -INFINITY) {
-      // cheap conservative test on the logit first, the exact one on z for the survivors
-      const float x = tau * temp;
-      const float thr_l = x - fabsf(x) * 9.5367431640625e-7f - 1e-30f;
-      auto consider = [&](float v, int i) {
-        if (v >= thr_l) {
-          const float z = __fdiv_rn(v, temp);
-          if (z >= tau) {
-            const int p = atomicAdd(&s_ncand, 1);
-            if (p < CAND_MAX) { s_cz[p] = z; s_ci[p] = i; }
-          }
-        }
-      };
-      if (vec) {
-        const float4* lg4 = reinterpret_cast<const float4*>(lg);
-#pragma unroll 8
-        for (int i = tid; i < V / 4; i += FWD_THREADS) {
-          const float4 v = lg4[i];
-          if (fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)) >= thr_l) {
-            consider(v.x, 4 * i); consider(v.y, 4 * i + 1); consider(v.z, 4 * i + 2); consider(v.w, 4 * i + 3);
-          }
-        }
-      } else {
-        for (int i = tid; i < V; i += FWD_THREADS) consider(lg[i], i);
-      }
-    }
-    __syncthreads();
-  }
-  const bool fast_ok = s_ncand >= k && s_ncand <= CAND_MAX;
-  __syncthreads();
-  if (!fast_ok) {
-  // Fallback (huge plateaus of equal values, or fewer than k finite thread maxima):
-  // radix select over the composite key (z key, ~index): unique keys, so ties in z
-  // break towards the lower index and the k-th key is exact.  Refine 8 bits at a time
-  // until the set {key >= prefix} (>= k elements by construction) fits the sort buffer.
-  if (tid == 0) { s_prefix = 0; s_mask = 0; s_remaining = k; }
-  __syncthreads();
-  for (int shift = 56; shift >= 0; shift -= 8) {
-    s_hist[tid] = 0;   // FWD_THREADS == 256 bins
-    __syncthreads();
-    const unsigned long long prefix = s_prefix, mask = s_mask;
-    for (int i = tid; i < V; i += FWD_THREADS) {
-      const unsigned long long key =
-          ((unsigned long long)float_key(__fdiv_rn(lg[i], temp)) << 32) | (uint32_t)(~(uint32_t)i);
-      if ((key & mask) == prefix) atomicAdd(&s_hist[(unsigned)(key >> shift) & 255u], 1u);
-    }
-    __syncthreads();
-    if (tid == 0) {
-      const int need = s_remaining;   // how many are still needed from inside the current prefix
-      int bin = 255;
-      uint32_t above = 0;
-      for (; bin > 0; --bin) {
-        if (above + s_hist[bin] >= (uint32_t)need) break;
-        above += s_hist[bin];
-      }
-      s_remaining = need - (int)above;
-      s_prefix = prefix | ((unsigned long long)bin << shift);
-      s_mask = mask | (255ull << shift);
-      // keys >= new prefix: those in strictly higher bins at every level so far, plus this bin
-      s_ncand = (k - s_remaining) + (int)s_hist[bin];
-    }
-    __syncthreads();
-    if (s_ncand <= CAND_MAX) break;
-  }
-  const unsigned long long thr = s_prefix;
-  __syncthreads();
-  if (tid == 0) s_ncand = 0;
-  __syncthreads();
-  for (int i = tid; i < V; i += FWD_THREADS) {
-    const float z = __fdiv_rn(lg[i], temp);
-    const unsigned long long key = ((unsigned long long)float_key(z) << 32) | (uint32_t)(~(uint32_t)i);
-    if (key >= thr) {
-      const int p = atomicAdd(&s_ncand, 1);
-      if (p < CAND_MAX) { s_cz[p] = z; s_ci[p] = i; }
-    }
-  }
-  __syncthreads();
-  }  // fallback
-  const int nc = min(s_ncand, CAND_MAX);
-  // rank every candidate by (z desc, index asc); the k best land at their rank
-  for (int a = tid; a < nc; a += FWD_THREADS) {
-    const float za = s_cz[a];
-    const int ia = s_ci[a];
-    int rank = 0;
-    for (int j = 0; j < nc; ++j) {
-      const float zj = s_cz[j];
-      rank += (zj > za) || (zj == za && s_ci[j] < ia);
-    }
-    if (rank < k) { s_tz[rank] = za; s_ti[rank] = ia; }
-  }
-  __syncthreads();
-  if (tid == 0) {
-    const uint32_t x = philox4x32_10_word0((uint32_t)ticket, (uint32_t)(ticket >> 32), (uint32_t)gen_index, 0u,
-                                           (uint32_t)seed, (uint32_t)(seed >> 32));
-    const int kk = min(k, nc);
-    if (nucleus) {
-      // nucleus inside the k candidates (already in the order), integer weights
-      unsigned long long Q = 0;
-      for (int j = 0; j < kk; ++j) Q += nucleus_weight(s_tz[j], s_tz[0]);
-      const unsigned long long need = nucleus_need(nucleus_p24(top_p), Q);
-      unsigned long long M = 0;
-      int m = 0;
-      for (; m < kk; ++m) {
-        M += nucleus_weight(s_tz[m], s_tz[0]);
-        if (M >= need) { ++m; break; }
-      }
-      const unsigned long long target = nucleus_target((unsigned long long)(x >> 8), M);
-      unsigned long long cum = 0;
-      int pick = s_ti[m - 1];
-      for (int j = 0; j < m; ++j) {
-        cum += nucleus_weight(s_tz[j], s_tz[0]);
-        if (cum > target) { pick = s_ti[j]; break; }
-      }
-      result = pick;
-    } else {
-      const double u = (double)(x >> 8) * (1.0 / 16777216.0);
-      double total = 0.0;
-      for (int j = 0; j < kk; ++j) total += exp((double)s_tz[j] - (double)s_tz[0]);
-      const double target = u * total;
-      double accum = 0.0;
-      int pick = s_ti[kk - 1];
-      for (int j = 0; j < kk; ++j) {
-        accum += exp((double)s_tz[j] - (double)s_tz[0]);
-        if (accum > target) { pick = s_ti[j]; break; }
-      }
-      result = pick;
-    }
-  }
-  __syncthreads();
-  return result;
-}
-
-static __device__ __noinline__ void phase_sample(const DevCtx& c, float* smem) {
-  const int R = c.ss->cur_rows;
-  const int V = c.V;
-  const int tid = threadIdx.x;
-  const unsigned long long rows_before = c.ss->sample_rows_total;
-  for (int r = blockIdx.x; r < R; r += gridDim.x) {
-    const float* lg = c.logits + (size_t)r * V;
-    const int item = c.row_item[r];
-    const int b = c.it_bslot[item];
-    if (c.logits_capture != nullptr && (long long)(rows_before + r) < c.capture_rows) {
-      float* dst = c.logits_capture + (size_t)(rows_before + r) * V;
-      for (int i = tid; i < V; i += FWD_THREADS) dst[i] = lg[i];
-    }
-    const int tok = sample_row(lg, V, min(c.b_topk[b], MAX_TOPK), c.b_temp[b], c.b_topp[b], (unsigned long long)c.b_ticket[b],
-                               c.b_generated[b], c.b_seed[b], smem);
-    if (tid == 0) c.row_sampled[r] = tok;
-  }
-}
-constexpr int SAMPLE_SMEM_FLOATS = 256 + 4 * 1024;
-
 }  // namespace blink
+
+#include "sampler.cuh"

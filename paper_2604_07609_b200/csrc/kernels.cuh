@@ -101,6 +101,8 @@ __device__ __forceinline__ void run_phase(const DevCtx& c, int phase, int layer,
       GemmArgs a{c.xs, c.w_base + c.w_off[9], c.logits, c.ss->cur_rows, c.V, c.d, c.V, 0};
       gemm_dispatch<WT, PAIR>(c, a, GEMM_LMHEAD, 0, smem, tc);
     } break;
+    case PH_SMAX: phase_sample_max(c); break;
+    case PH_SNUC: phase_sample_weights(c, smem); break;
     case PH_SAMPLE: phase_sample(c, smem); break;
     default: break;
   }
@@ -137,7 +139,11 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) blink_loop_kernel(const __grid
         run_phase<WT, HD, NREP, PAIR>(c, ph, layer, sub, smem, tc, as, T);
         if (!barrier) return;
         ok = grid_barrier(c, gen);
-        if (timed) { const uint64_t t = global_timer_ns(); c.ss->cur_phase_ns[ph] += t - t_prev; t_prev = t; }
+        if (timed) {   // the parts of sampling share a timer
+          const uint64_t t = global_timer_ns();
+          c.ss->cur_phase_ns[ph >= PH_SMAX ? (int)PH_SAMPLE : ph] += t - t_prev;
+          t_prev = t;
+        }
       };
       for (int layer = 0; layer < c.L && ok; ++layer) {
         for (int ph = PH_NORM1; ph <= PH_DOWN && ok; ++ph) {
@@ -149,7 +155,15 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) blink_loop_kernel(const __grid
           }
         }
       }
-      for (int ph = PH_FNORM; ph <= PH_SAMPLE && ok; ++ph) step_phase(ph, 0, 0);
+      // the output part; long rows are prepared for sampling by all CTAs, rows that sample from a whole-row nucleus
+      // with one more pass over the logits
+      const bool split = sample_split_rows(c.V);
+      const bool nuc = split && __ldcg(&c.ss->cur_nuc) != 0;
+      for (int i = 0; i < 5 && ok; ++i) {
+        const int ph = output_phase(i);
+        if ((ph == PH_SMAX && !split) || (ph == PH_SNUC && !nuc)) continue;
+        step_phase(ph, 0, 0);
+      }
       if (!ok) break;
     } else if (!grid_barrier(c, gen)) break;
   }
