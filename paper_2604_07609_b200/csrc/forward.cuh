@@ -318,8 +318,7 @@ static __device__ __noinline__ void phase_final_norm(const DevCtx& c) {
     norm_row_cta<WT>(c, c.h + (size_t)c.row_tok[r] * c.d, nullptr, g, out + (size_t)r * c.d, s_red);
 }
 
-// ---- CUDA-core reference GEMM: out[t][n] (+)= sum_k x[t][k] * w[n][k], fp32 accumulate.
-// 64x64 output tile, BK = 16, 4x4 outputs per thread.  Deterministic (no split-K).
+// ---- dense contractions ------------------------------------------------------------------
 enum GemmFix : int {
   FIX_NONE = 0,
   FIX_ROPE_KV,  // QKV: RoPE on q and k, q -> 16-bit attention operand, k and v -> paged pool; the tile is cleared
@@ -346,66 +345,82 @@ struct GemmArgs {
   float* fix_rowss = nullptr;// FIX_SUMSQ: per-row sums of squares to add to
 };
 
-template <typename WT>
-static __device__ __noinline__ void phase_gemm_simt(const GemmArgs& a) {
-  constexpr int BM = 64, BN = 64, BK = 16;
-  __shared__ float xs[BK][BM + 4];
-  __shared__ float ws[BK][BN + 4];
+// Sums of NV values over the 32 lanes by halving exchange: lane l ends with the sum of value (l * NV) / 32.
+template <int NV>
+__device__ __forceinline__ float warp_sum_many(float (&v)[NV]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int n = NV, o = 16; o > 0; o >>= 1) {
+    if (n > 1) {
+      n >>= 1;
+      const bool up = (lane & o) != 0;
+#pragma unroll
+      for (int i = 0; i < NV / 2; ++i) {
+        if (i < n) {
+          const float send = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
+          v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+      }
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    }
+  }
+  return v[0];
+}
+// One warp: GR token rows x NC output features, the 32 lanes side by side along K (four elements each), so that all
+// loads of 256 elements of K are in flight at once.  The reference shapes are small (a few dozen rows, K of 256 to
+// 1024): with 64 x 64 tiles and 16 elements of K per step only 4 to 64 CTAs had work and every step waited for
+// its own loads (27 us for K = 256, 98 us for K = 1024 at 8 rows; now 3 and 5).
+constexpr int SIMT_GR = 8;
+template <typename WT, int NC>
+__device__ __forceinline__ void gemm_simt_tasks(const GemmArgs& a) {
   const WT* X = reinterpret_cast<const WT*>(a.x);
   const WT* W = reinterpret_cast<const WT*>(a.w);
-  const int tiles_m = (a.M + BM - 1) / BM, tiles_n = (a.N + BN - 1) / BN;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;  // 16 x 16 threads
-  const int lrow = threadIdx.x >> 2, lk = (threadIdx.x & 3) * 4;
-  for (int tile = blockIdx.x; tile < tiles_m * tiles_n; tile += gridDim.x) {
-    const int tm = tile % tiles_m, tn = tile / tiles_m;
-    const int m0 = tm * BM, n0 = tn * BN;
-    float acc[4][4];
+  const int lane = threadIdx.x & 31;
+  const int groups_n = (a.N + NC - 1) / NC, groups_m = (a.M + SIMT_GR - 1) / SIMT_GR;
+  const int nw = gridDim.x * (FWD_THREADS / 32);
+  for (int task = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; task < groups_m * groups_n; task += nw) {
+    const int gm = task / groups_n, gn = task - gm * groups_n;
+    const int m0 = gm * SIMT_GR, n0 = gn * NC;
+    float acc[SIMT_GR * NC];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < SIMT_GR * NC; ++i) acc[i] = 0.f;
+#pragma unroll 2
+    for (int k = lane * 4; k < a.K; k += 128) {
+      float4 w[NC], x[SIMT_GR];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-    for (int k0 = 0; k0 < a.K; k0 += BK) {
-      {
-        const int m = m0 + lrow, n = n0 + lrow;
+      for (int j = 0; j < NC; ++j) w[j] = load4<WT>(W + (size_t)min(n0 + j, a.N - 1) * a.K + k);   // clamped: rows past the end repeat
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int k = k0 + lk + e;
-          xs[lk + e][lrow] = (m < a.M && k < a.K) ? OpType<WT>::to_f(X[(size_t)m * a.K + k]) : 0.f;
-          ws[lk + e][lrow] = (n < a.N && k < a.K) ? OpType<WT>::to_f(W[(size_t)n * a.K + k]) : 0.f;
+      for (int i = 0; i < SIMT_GR; ++i) x[i] = load4<WT>(X + (size_t)min(m0 + i, a.M - 1) * a.K + k);
+#pragma unroll
+      for (int i = 0; i < SIMT_GR; ++i)
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+          float& s = acc[i * NC + j];
+          s = fmaf(x[i].x, w[j].x, s); s = fmaf(x[i].y, w[j].y, s); s = fmaf(x[i].z, w[j].z, s); s = fmaf(x[i].w, w[j].w, s);
         }
-      }
-      __syncthreads();
-#pragma unroll
-      for (int k = 0; k < BK; ++k) {
-        float xv[4], wv[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) xv[i] = xs[k][ty * 4 + i];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) wv[j] = ws[k][tx * 4 + j];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(xv[i], wv[j], acc[i][j]);
-      }
-      __syncthreads();
     }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int m = m0 + ty * 4 + i;
-      if (m >= a.M) continue;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int n = n0 + tx * 4 + j;
-        if (n >= a.N) continue;
-        if (a.row_map != nullptr) {
-          atomicAdd(a.out + (size_t)a.row_map[m] * a.ldo + n, a.row_scale[m] * acc[i][j]);
-        } else {
-          float* o = a.out + (size_t)m * a.ldo + n;
-          *o = a.accumulate ? (*o + acc[i][j]) : acc[i][j];
-        }
+    const float v = warp_sum_many<SIMT_GR * NC>(acc);
+    constexpr int LPV = 32 / (SIMT_GR * NC);   // lanes that hold the same sum
+    const int idx = lane / LPV, m = m0 + idx / NC, n = n0 + idx % NC;
+    if (lane % LPV == 0 && m < a.M && n < a.N) {
+      if (a.row_map != nullptr) {
+        atomicAdd(a.out + (size_t)a.row_map[m] * a.ldo + n, a.row_scale[m] * v);
+      } else {
+        float* o = a.out + (size_t)m * a.ldo + n;
+        *o = a.accumulate ? (*o + v) : v;
       }
     }
   }
+}
+// CUDA-core GEMM: out[t][n] (+)= sum_k x[t][k] * w[n][k], fp32 accumulate, deterministic (no split over CTAs).  Four
+// features per warp load 12 vectors for 128 multiplications; fewer when the tasks would not fill the warps of the grid.
+template <typename WT>
+static __device__ __noinline__ void phase_gemm_simt(const GemmArgs& a) {
+  const long long rows = (a.M + SIMT_GR - 1) / SIMT_GR, warps = (long long)gridDim.x * (FWD_THREADS / 32);
+  if (rows * a.N >= 4 * warps) gemm_simt_tasks<WT, 4>(a);
+  else if (rows * a.N >= 2 * warps) gemm_simt_tasks<WT, 2>(a);
+  else gemm_simt_tasks<WT, 1>(a);
 }
 
 // ---- RoPE (rotate-half pairing) on q and k, then K/V into the paged pool --------------
