@@ -33,7 +33,7 @@ __shared__ int g_att_nctx[MAX_BATCH];
 __shared__ int g_att_row[MAX_BATCH];
 // the step's scalars: like the arrays above they do not change between layers and are read from memory once per step
 struct AttStep {
-  int n_dec, TT, S, C, npf;
+  int n_dec, TT, S, C, npf, fuse;
 };
 __shared__ AttStep g_att_step;
 
@@ -419,7 +419,11 @@ __device__ __noinline__ void attn_decode_stream(const DevCtx& c, int layer, char
 // 300 keys took 22 us and one of 4000 keys 51 us per layer, nearly all of it latency.  Here the eight warps of a
 // CTA share a part of a unit (C tiles, no part crosses units): their tiles are in flight at once, their sums are
 // merged in shared memory, and only units of more than C tiles leave records, merged by the whole last CTA.
+// In steps of at most 16 rows without prompt rows this kernel also takes over RoPE and the K/V write (a phase and a grid
+// barrier less): every CTA rotates the queries it needs, and the warp that meets a unit's last tile computes the new key
+// and value row, writes it to the pool and into its copy of the tile.
 constexpr int ATT_NSC = 2;   // ring stages per warp here
+constexpr int ATT_CTA_OFF = 65536;   // the space before it may be receiving weights of the O projection already
 template <int HD, int NREP>
 static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer, char* base, AttState& as) {
   constexpr int RB = HD * 2;
@@ -434,8 +438,11 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer, 
   const int gq = lane >> 2, tq = lane & 3;
   const bool live = gq < NREP;
   const int n_dec = g_att_step.n_dec, C = g_att_step.C, Hkv = c.Hkv;
-  float* s_o = reinterpret_cast<float*>(base + ATT_WARPS * ATT_NSC * STAGE);   // [warps][NREP][HD]
   char* ring = base + w * ATT_NSC * STAGE;
+  float* s_o = reinterpret_cast<float*>(base);   // a warp's sums [NREP][HD] go where its ring stages were
+  constexpr int S_O = ATT_NSC * STAGE / 4;       // floats from one warp's sums to the next
+  static_assert(NREP * HD * 4 <= ATT_NSC * STAGE, "a warp's sums exceed its stages");
+  const bool fuse = g_att_step.fuse != 0;
   uint64_t* bars = g_att.bar[w];
   volatile int* dead = &g_att.dead;
   const CUtensorMap* kv_map = reinterpret_cast<const CUtensorMap*>(c.kv_map);
@@ -481,7 +488,60 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer, 
     uint32_t qf[KS][2];
     float o[HD / 16][4];
     float m2[2] = {-INFINITY, -INFINITY}, l2[2] = {0.f, 0.f};
-    {
+    // this warp meets the unit's last tile: the new key and value row is its business
+    const bool newest = fuse && n_tiles > 0 && kb0 + w + ATT_WARPS * (n_tiles - 1) == nkb - 1;
+    uint2 new_k = make_uint2(0u, 0u), new_v = make_uint2(0u, 0u);
+    if (fuse) {
+      constexpr int H2 = HD / 2;
+      const int pos = n_ctx - 1;
+      const float* row = c.qkv + (size_t)t_row * c.qkv_dim;
+      const float* qrow = row + (size_t)(g * NREP + (live ? gq : 0)) * HD;
+      const float* cs = c.rope_cos + (size_t)pos * H2;
+      const float* sn = c.rope_sin + (size_t)pos * H2;
+      float4 kx = make_float4(0.f, 0.f, 0.f, 0.f), vx = kx, kc = kx, ks4 = kx;
+      const int d0 = (lane * 4) & (HD - 1);   // four dims of the new row (HD 64: the upper lanes repeat the lower ones)
+      if (newest) {
+        kx = __ldcg(reinterpret_cast<const float4*>(row + c.q_dim + g * HD + d0));
+        vx = __ldcg(reinterpret_cast<const float4*>(row + c.q_dim + c.kv_dim + g * HD + d0));
+        kc = *reinterpret_cast<const float4*>(cs + (d0 & (H2 - 1)));
+        ks4 = *reinterpret_cast<const float4*>(sn + (d0 & (H2 - 1)));
+      }
+#pragma unroll
+      for (int ks = 0; ks < KS / 2; ++ks) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int i = ks * 16 + e * 8 + 2 * tq;   // rotation pair (i, i + HD / 2)
+          const float2 a = __ldcg(reinterpret_cast<const float2*>(qrow + i)), b = __ldcg(reinterpret_cast<const float2*>(qrow + i + H2));
+          const float2 cc = *reinterpret_cast<const float2*>(cs + i), ss = *reinterpret_cast<const float2*>(sn + i);
+          // the same fused forms as the RoPE phase
+          const uint32_t lo = pack_bf2(fmaf(a.x, cc.x, -__fmul_rn(b.x, ss.x)), fmaf(a.y, cc.y, -__fmul_rn(b.y, ss.y)));
+          const uint32_t hi = pack_bf2(fmaf(b.x, cc.x, __fmul_rn(a.x, ss.x)), fmaf(b.y, cc.y, __fmul_rn(a.y, ss.y)));
+          qf[ks][e] = live ? lo : 0u;
+          qf[ks + KS / 2][e] = live ? hi : 0u;
+        }
+      }
+      if (newest) {   // uniform over the warp
+        float4 px;
+        constexpr int PL = HD / 8;   // lanes between the two halves of a pair
+        px.x = __shfl_xor_sync(FULL, kx.x, PL); px.y = __shfl_xor_sync(FULL, kx.y, PL);
+        px.z = __shfl_xor_sync(FULL, kx.z, PL); px.w = __shfl_xor_sync(FULL, kx.w, PL);
+        float4 y;
+        if (d0 < H2) {
+          y = make_float4(fmaf(kx.x, kc.x, -__fmul_rn(px.x, ks4.x)), fmaf(kx.y, kc.y, -__fmul_rn(px.y, ks4.y)),
+                          fmaf(kx.z, kc.z, -__fmul_rn(px.z, ks4.z)), fmaf(kx.w, kc.w, -__fmul_rn(px.w, ks4.w)));
+        } else {
+          y = make_float4(fmaf(kx.x, kc.x, __fmul_rn(px.x, ks4.x)), fmaf(kx.y, kc.y, __fmul_rn(px.y, ks4.y)),
+                          fmaf(kx.z, kc.z, __fmul_rn(px.z, ks4.z)), fmaf(kx.w, kc.w, __fmul_rn(px.w, ks4.w)));
+        }
+        new_k = make_uint2(pack_bf2(y.x, y.y), pack_bf2(y.z, y.w));
+        new_v = make_uint2(pack_bf2(vx.x, vx.y), pack_bf2(vx.z, vx.w));
+        const int b = table[nkb - 1];
+        if (lane * 4 < HD) {
+          *reinterpret_cast<uint2*>(kv_tile<__nv_bfloat16>(c, layer, 0, b, g) + (size_t)(pos & 15) * HD + d0) = new_k;
+          *reinterpret_cast<uint2*>(kv_tile<__nv_bfloat16>(c, layer, 1, b, g) + (size_t)(pos & 15) * HD + d0) = new_v;
+        }
+      }
+    } else {
       const __nv_bfloat16* qrow = qb + (size_t)t_row * c.q_dim + (size_t)(g * NREP + (live ? gq : 0)) * HD;
 #pragma unroll
       for (int ks = 0; ks < KS; ++ks) {
@@ -503,6 +563,15 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer, 
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
       }
+      if (newest && i == n_tiles - 1) {   // the copy holds what the pool held before the row was written
+        if (lane * 4 < HD) {
+          const int d0 = lane * 4, line = ((n_ctx - 1) & 15) * (HD / 64) + (d0 >> 6);
+          char* dst = st + line * 128 + ((((d0 & 63) >> 3) ^ (line & 7)) << 4) + (d0 & 7) * 2;
+          *reinterpret_cast<uint2*>(dst) = new_k;
+          *reinterpret_cast<uint2*>(dst + TILE) = new_v;
+        }
+        __syncwarp();
+      }
       att_tile_math<HD>(smem_u32(st), smem_u32(st) + TILE, n_valid, qscale, qf, o, m2, l2);
       __syncwarp();   // all reads of this stage are done before it is refilled
       if (i + ATT_NSC < n_tiles) issue(i + ATT_NSC);
@@ -519,7 +588,7 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer, 
     for (int e = 0; e < 2; ++e) {
       if (h0 + e < NREP) {
         if (n_tiles > 0) {
-          float* ow = s_o + ((size_t)w * NREP + h0 + e) * HD;
+          float* ow = s_o + w * S_O + (h0 + e) * HD;
 #pragma unroll
           for (int i = 0; i < HD / 16; ++i) {
             ow[16 * i + gq] = o[i][e];
@@ -542,7 +611,7 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer, 
       float den = 0.f;
       for (int k = 0; k < n_warps; ++k) {
         const float f = fast_ex2(s_m[k][h] - M);
-        const float2 a = *reinterpret_cast<const float2*>(s_o + (size_t)k * NREP * HD + i2 * 2);
+        const float2 a = *reinterpret_cast<const float2*>(s_o + k * S_O + i2 * 2);
         num.x = fmaf(f, a.x, num.x);
         num.y = fmaf(f, a.y, num.y);
         den = fmaf(f, s_l[k][h], den);
@@ -585,7 +654,9 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer, 
         if (threadIdx.x == 0) c.att_cnt[unit] = 0;
       }
     }
-    __syncthreads();   // the sums in shared memory are free for the next item
+    // the sums are free for the next item, and before copies land there again
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
   }
 }
 
@@ -766,7 +837,7 @@ __device__ __noinline__ void attn_prefill_tile(const DevCtx& c, int layer, int i
 template <int HD>
 constexpr int att_smem_bytes() {
   constexpr int ring = ATT_WARPS * ATT_NS * 2 * 16 * HD * 2 + 1024;   // + alignment slack
-  constexpr int cta = ATT_WARPS * ATT_NSC * 2 * 16 * HD * 2 + ATT_WARPS * 8 * HD * 4 + 1024;   // up to 8 heads per group
+  constexpr int cta = ATT_CTA_OFF + ATT_WARPS * ATT_NSC * 2 * 16 * HD * 2 + 1024;
   constexpr int tile = 128 * HD * 2 + 2 * 2 * 64 * HD * 2;
   return ring > cta ? (ring > tile ? ring : tile) : (cta > tile ? cta : tile);
 }
@@ -777,7 +848,7 @@ __device__ __forceinline__ void phase_attention_bf16(const DevCtx& c, int layer,
   if (layer == 0 || c.stepped) {   // the step's work lists: once per step
     const SchedState* ss = c.ss;
     const int n = ss->cur_ndec;
-    if (threadIdx.x == 0) g_att_step = AttStep{n, ss->cur_TT, ss->cur_S, ss->cur_C, ss->cur_npf};
+    if (threadIdx.x == 0) g_att_step = AttStep{n, ss->cur_TT, ss->cur_S, ss->cur_C, ss->cur_npf, ss->cur_fuse};
     for (int i = threadIdx.x; i <= n; i += FWD_THREADS) {
       g_att_pre[i] = c.dec_kbpre[i];
       if (i < n) { g_att_bslot[i] = c.dec_bslot[i]; g_att_nctx[i] = c.dec_nctx[i]; g_att_row[i] = c.dec_row[i]; }
@@ -793,7 +864,7 @@ __device__ __forceinline__ void phase_attention_bf16(const DevCtx& c, int layer,
   if (n_dec > 0) {
     if (n_pf > 0) __syncthreads();   // the prefill tiles' shared memory is free
     if (g_att_step.C > 0) {
-      attn_decode_cta<HD, NREP>(c, layer, tc_tiles(smem_f), as);
+      attn_decode_cta<HD, NREP>(c, layer, tc_tiles(smem_f) + ATT_CTA_OFF, as);
     } else {
       const int w = threadIdx.x >> 5;
       constexpr int STAGE = 2 * 16 * HD * 2;

@@ -23,6 +23,7 @@
 #include "dev_ctx.cuh"
 #include "forward.cuh"
 #include "gemm_tc.cuh"
+#include "gemm_dec.cuh"
 #include "attention.cuh"
 #include "kernel_set.h"
 
@@ -827,6 +828,7 @@ int blink_create(const blink_model_cfg* model, const blink_sched_cfg* sched, con
       pick_kernels();
     }
   }
+  dec_host_setup(c, x->pair, x->grid);
   const void* loop_fn = x->ks.loop;
   const void* ph_fn = x->ks.phase;
   if (!loop_fn || !ph_fn) return fail(BLINK_EINVAL);

@@ -97,6 +97,7 @@ struct SchedState {
   int cur_TT;     // attention: (row, kv head, KV block) tiles of those rows
   int cur_S;      // attention: tiles per sub-range of the flat tile sequence, 0 = a sub-range is a (row, kv head) unit
   int cur_C;      // attention: > 0: decode units are shared by the warps of a CTA, C tiles per part
+  int cur_fuse;   // small decode step: the attention applies RoPE and writes K and V itself
   int cur_nuc;    // some row of the step samples from the nucleus of the whole row
   int cur_npf;    // attention: (request, query-row block) units of the multi-row requests
   long long cur_ctx;
@@ -140,6 +141,7 @@ struct DevCtx {
   int control_only, start_paused, stepped, gemm_tc;
   int policy;        // BLINK_POLICY_*: chunked prefill, or whole-prompt prefill steps that pause decoding
   int n_warps_grid;  // warps of the whole grid (attention work split)
+  int dec_small, dec_mid;   // decode-sized steps (up to 16, up to 128 rows) take the GEMMs with prefetched weights
   int w_streaming;   // GEMM matrices are stored as contiguous pre-swizzled 128 x 64 tiles
   long long iteration_budget;
   unsigned long long idle_exit_cycles, barrier_timeout_cycles;

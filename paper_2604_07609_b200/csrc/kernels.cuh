@@ -9,6 +9,7 @@
 #include "control.cuh"
 #include "dev_ctx.cuh"
 #include "forward.cuh"
+#include "gemm_dec.cuh"
 #include "gemm_tc.cuh"
 #include "kernel_set.h"
 
@@ -21,11 +22,72 @@ __device__ __forceinline__ void gemm_dispatch(const DevCtx& c, const GemmArgs& a
   else phase_gemm_simt<WT>(a);
 }
 
-// `T` = rows of the step (read once per step by the caller: it does not change between phases)
+// What the phases of a step depend on besides the layer: read once per step, it does not change between phases.
+struct StepInfo {
+  int T, R;      // rows of the step, rows that sample
+  bool dec;      // decode-sized: the GEMMs of gemm_dec.cuh
+  bool small;    // of at most 16 rows: norms, SwiGLU and final norm run inside those GEMMs
+  bool fuse;     // RoPE and the K/V write run inside the attention
+  bool att_cta;  // the attention phase leaves the first half of the weight ring alone
+};
+template <typename WT, bool PAIR>
+__device__ __forceinline__ StepInfo step_info(const DevCtx& c) {
+  StepInfo s;
+  const SchedState* ss = c.ss;
+  s.T = __ldcg(&ss->cur_T);
+  s.R = __ldcg(&ss->cur_rows);
+  const int C = __ldcg(&ss->cur_C), npf = __ldcg(&ss->cur_npf), fuse = __ldcg(&ss->cur_fuse);
+  if constexpr (sizeof(WT) == 2) {
+    s.small = dec_small(c, s.T);
+    s.dec = dec_step(c, s.T);
+    s.fuse = fuse != 0;
+    s.att_cta = C > 0 && npf == 0;
+    if (s.dec) {
+      dec_geometry<PAIR>(c, s.T, s.R);
+      __syncthreads();
+    }
+  } else {
+    s.small = s.dec = s.fuse = s.att_cta = false;
+  }
+  return s;
+}
+// Phases that a step does not have because others do their work.
+__device__ __forceinline__ bool phase_absorbed(const DevCtx& c, const StepInfo& st, int ph) {
+  if (c.fused) return ph == PH_ROPE || ph == PH_SILU;   // done by the epilogues of the QKV and gate/up GEMMs
+  if (ph == PH_ROPE) return st.fuse;
+  if (!st.small) return false;
+  return ph == PH_NORM1 || ph == PH_FNORM || (c.E == 0 && (ph == PH_NORM2 || ph == PH_SILU));
+}
+// The GEMM phases of a decode-sized step; false when the phase is none of them.  `chain`: weights of the GEMM that
+// follows may be fetched ahead (not when every phase is a launch of its own).
+template <bool PAIR>
+__device__ __forceinline__ bool run_phase_dec(const DevCtx& c, const StepInfo& st, int phase, int layer, float* smem, TcState& tc,
+                                              DecState& ds, bool chain) {
+  int which, next = -1, pre = DEC_STAGES;
+  switch (phase) {
+    case PH_QKV: which = GEMM_QKV; next = GEMM_O; pre = st.att_cta ? ATT_CTA_OFF / DEC_STAGE_BYTES : 0; break;
+    case PH_O: which = GEMM_O; next = c.E == 0 ? GEMM_GU : -1; break;
+    case PH_GU: if (c.E > 0) return false; which = GEMM_GU; next = GEMM_DOWN; break;
+    case PH_DOWN:
+      if (c.E > 0) return false;
+      which = GEMM_DOWN;
+      next = layer + 1 < c.L ? GEMM_QKV : st.R > 0 ? GEMM_LMHEAD : -1;
+      break;
+    case PH_LMHEAD: which = GEMM_LMHEAD; break;
+    default: return false;
+  }
+  phase_gemm_dec<PAIR>(c, which, layer, st.T, st.R, chain ? next : -1, pre, smem, tc, ds);
+  return true;
+}
+
 template <typename WT, int HD, int NREP, bool PAIR>
-__device__ __forceinline__ void run_phase(const DevCtx& c, int phase, int layer, int sub, float* smem, TcState& tc,
-                                          AttState& as, int T) {
+__device__ __forceinline__ void run_phase(const DevCtx& c, const StepInfo& st, int phase, int layer, int sub, float* smem,
+                                          TcState& tc, AttState& as, DecState& ds, bool chain) {
   const size_t esz = sizeof(WT);
+  const int T = st.T;
+  if constexpr (sizeof(WT) == 2) {
+    if (st.dec && run_phase_dec<PAIR>(c, st, phase, layer, smem, tc, ds, chain)) return;
+  }
   switch (phase) {
     case PH_NORM1:
       if (c.fused_norm && layer > 0) phase_norm_apply<WT>(c, layer, 0, T);
@@ -118,6 +180,9 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) blink_loop_kernel(const __grid
   tc_init<PAIR>(c, smem, tc);
   AttState as;
   att_init(c, as);
+  DecState ds;
+  dec_init<PAIR>(c, ds);
+  if constexpr (PAIR) cluster_sync_all();   // the other CTA's barriers exist before they are signalled
   while (true) {
     if (blockIdx.x == 0) control_phase(c, launch_iters);
     if (!grid_barrier(c, gen)) break;
@@ -128,15 +193,15 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) blink_loop_kernel(const __grid
       // the barrier that closes it); recorded only when per-iteration statistics are kept
       const bool timed = c.stats_cap > 0 && blockIdx.x == 0 && threadIdx.x == 0;
       uint64_t t_prev = timed ? global_timer_ns() : 0;
-      const int T = __ldcg(&c.ss->cur_T);   // fixed for the whole step: one L2 read instead of one per phase
+      const StepInfo st = step_info<WT, PAIR>(c);
       auto step_phase = [&](int ph, int layer, int sub) {
-        if (c.fused && (ph == PH_ROPE || ph == PH_SILU)) return;   // done by the epilogues of the QKV and gate/up GEMMs
+        if (phase_absorbed(c, st, ph)) return;
         // The experts' GEMMs are independent of one another (own weights, own gathered rows; the down
         // projections add into the residual rows with reductions): one grid barrier after the last
         // expert, none in between, so every CTA streams its share of all experts back to back.  (With
         // fused epilogues the barriers stay: their tile counters are per GEMM.)
         const bool barrier = !(c.E > 0 && !c.fused && (ph == PH_GU || ph == PH_DOWN) && sub + 1 < c.E);
-        run_phase<WT, HD, NREP, PAIR>(c, ph, layer, sub, smem, tc, as, T);
+        run_phase<WT, HD, NREP, PAIR>(c, st, ph, layer, sub, smem, tc, as, ds, true);
         if (!barrier) return;
         ok = grid_barrier(c, gen);
         if (timed) {   // the parts of sampling share a timer
@@ -167,6 +232,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) blink_loop_kernel(const __grid
       if (!ok) break;
     } else if (!grid_barrier(c, gen)) break;
   }
+  dec_drain<PAIR>(c, ds, PAIR ? cluster_ctarank() : 0u);
   tc_fini<PAIR>(c, tc);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     const int aborted = *(volatile int*)&c.ss->abort_flag;
@@ -184,7 +250,12 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) blink_phase_kernel(const __gri
   tc_init<PAIR>(c, smem, tc);
   AttState as;
   att_init(c, as);
-  run_phase<WT, HD, NREP, PAIR>(c, phase, layer, sub, smem, tc, as, c.ss->cur_T);
+  DecState ds;
+  dec_init<PAIR>(c, ds);
+  if constexpr (PAIR) cluster_sync_all();
+  else __syncthreads();
+  const StepInfo st = step_info<WT, PAIR>(c);
+  if (!phase_absorbed(c, st, phase)) run_phase<WT, HD, NREP, PAIR>(c, st, phase, layer, sub, smem, tc, as, ds, false);
   tc_fini<PAIR>(c, tc);
 }
 
