@@ -179,48 +179,43 @@ __device__ __forceinline__ void norm_row_cta(const DevCtx& c, float* hrow, const
   }
 }
 
-// Rows of a CTA in turn, the next row on its way (asynchronous copies into shared memory, each thread reads
-// back only what it copied itself) while the current one is summed and scaled: with several rows per CTA
-// (steps of more rows than SMs) the phase is a chain of row latencies otherwise.  The copies hold no
-// registers.  NV = d / 1024 16-byte vectors per thread.
+// Two rows of a CTA at a time, one by each half of its threads (NV = d / 512 16-byte vectors per thread, all of a row's
+// loads in flight at once, the gains held in registers).  With one row per CTA in turn a 500-row step had four rounds
+// of load latency and reduction (9 us at d = 4096 although the next row was prefetched); this form has two.
 template <typename WT, int NV>
-static __device__ __noinline__ void norm_rows_pipelined(const DevCtx& c, const float* g, WT* out, int T, float* s_red, float* smem) {
-  constexpr int d = NV * 1024;
-  int t = blockIdx.x;
+static __device__ __noinline__ void norm_rows_halves(const float* __restrict__ h, const float* __restrict__ g, WT* __restrict__ out, int T,
+                                                     float eps) {
+  constexpr int d = NV * 512;
+  __shared__ float s_half[2][2][4];
+  const int half = threadIdx.x >> 7, tid = threadIdx.x & 127;
+  // rows are dealt to the first halves of all CTAs, then to the second halves
+  int t = half * gridDim.x + blockIdx.x;
   if (t >= T) return;
-  const char* stage = reinterpret_cast<const char*>(smem) + threadIdx.x * 16;   // [NV][FWD_THREADS] x 16 bytes
-  const uint32_t stage_s = (uint32_t)__cvta_generic_to_shared(stage);
-  const float* src = c.h + (size_t)t * d + threadIdx.x * 4;
+  float4 gg[NV];
 #pragma unroll
-  for (int k = 0; k < NV; ++k)
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(stage_s + k * FWD_THREADS * 16), "l"(src + k * FWD_THREADS * 4) : "memory");
-  asm volatile("cp.async.commit_group;" ::: "memory");
+  for (int k = 0; k < NV; ++k) gg[k] = __ldg(reinterpret_cast<const float4*>(g + (k * 128 + tid) * 4));
+  int buf = 0;
 #pragma unroll 1
-  for (; t < T; t += gridDim.x) {
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    float4 cur[NV];
+  for (; t < T; t += 2 * gridDim.x) {
+    const float* src = h + (size_t)t * d + tid * 4;
+    float4 v[NV];
 #pragma unroll
-    for (int k = 0; k < NV; ++k) cur[k] = *reinterpret_cast<const float4*>(stage + k * FWD_THREADS * 16);
-    if (t + (int)gridDim.x < T) {
-      src += (size_t)gridDim.x * d;
-#pragma unroll
-      for (int k = 0; k < NV; ++k)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(stage_s + k * FWD_THREADS * 16), "l"(src + k * FWD_THREADS * 4) : "memory");
-      asm volatile("cp.async.commit_group;" ::: "memory");
-    }
+    for (int k = 0; k < NV; ++k) v[k] = __ldcg(reinterpret_cast<const float4*>(src + k * 512));
     float ss = 0.f;
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {  // fixed order, the same as norm_row_cta
-      ss = fmaf(cur[k].x, cur[k].x, ss); ss = fmaf(cur[k].y, cur[k].y, ss); ss = fmaf(cur[k].z, cur[k].z, ss); ss = fmaf(cur[k].w, cur[k].w, ss);
+    for (int k = 0; k < NV; ++k) {   // fixed order
+      ss = fmaf(v[k].x, v[k].x, ss); ss = fmaf(v[k].y, v[k].y, ss); ss = fmaf(v[k].z, v[k].z, ss); ss = fmaf(v[k].w, v[k].w, ss);
     }
-    ss = block_sum(ss, s_red);
-    const float inv = rsqrtf(ss * (1.0f / (float)d) + c.rms_eps);
-    WT* orow = out + (size_t)t * d + threadIdx.x * 4;
+    ss = warp_sum(ss);
+    if ((tid & 31) == 0) s_half[half][buf][tid >> 5] = ss;
+    asm volatile("bar.sync %0, 128;" ::"r"(half + 1) : "memory");   // two buffers: one barrier per row
+    ss = (s_half[half][buf][0] + s_half[half][buf][1]) + (s_half[half][buf][2] + s_half[half][buf][3]);
+    buf ^= 1;
+    const float inv = rsqrtf(ss * (1.0f / (float)d) + eps);
+    WT* orow = out + (size_t)t * d + tid * 4;
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      const float4 gg = *reinterpret_cast<const float4*>(g + (k * FWD_THREADS + threadIdx.x) * 4);
-      store4<WT>(orow + k * FWD_THREADS * 4, cur[k].x * inv * gg.x, cur[k].y * inv * gg.y, cur[k].z * inv * gg.z, cur[k].w * inv * gg.w);
-    }
+    for (int k = 0; k < NV; ++k)
+      store4<WT>(orow + k * 512, v[k].x * inv * gg[k].x, v[k].y * inv * gg[k].y, v[k].z * inv * gg[k].z, v[k].w * inv * gg[k].w);
   }
 }
 
@@ -239,9 +234,9 @@ static __device__ __noinline__ void phase_norm(const DevCtx& c, int layer, int w
       c.rowss_b[i] = 0.f;
     }
   const float* wr = (which == 1 && c.E > 0) ? wptr_f(c, 5) + (size_t)layer * c.E * c.d : nullptr;
-  if (wr == nullptr && !(which == 0 && layer == 0) && T > (int)gridDim.x && (c.d == 4096 || c.d == 2048)) {
-    if (c.d == 4096) norm_rows_pipelined<WT, 4>(c, g, out, T, s_red, smem);
-    else norm_rows_pipelined<WT, 2>(c, g, out, T, s_red, smem);
+  if (wr == nullptr && !(which == 0 && layer == 0) && (c.d == 4096 || c.d == 2048)) {
+    if (c.d == 4096) norm_rows_halves<WT, 8>(c.h, g, out, T, c.rms_eps);
+    else norm_rows_halves<WT, 4>(c.h, g, out, T, c.rms_eps);
     return;
   }
   for (int t = blockIdx.x; t < T; t += gridDim.x) {
@@ -432,57 +427,66 @@ __device__ __forceinline__ WT* kv_tile(const DevCtx& c, int layer, int kv, int b
          ((((size_t)layer * 2 + kv) * c.n_blocks + block) * c.Hkv + head) * tile;
 }
 
+// One warp: four rounds of heads of one row (a lane owns four consecutive rotation pairs i .. i+3, i+half .. i+half+3 of
+// a head; 32 lanes cover 2 heads of 128 or 4 of 64).  Position and table entries are read once per task and all loads
+// are in flight before the first use; a thread per (row, head, quad) with its own index arithmetic, position and table
+// loads took 16 us for 500 rows of the 8B shape (31 MB through L2).
 template <typename WT>
 static __device__ __noinline__ void phase_rope_kv(const DevCtx& c, int layer) {
-  // one thread: four consecutive rotation pairs (i .. i+3, i+half .. i+half+3) of one head of one row
+  constexpr int U = 4;
   const int T = c.ss->cur_T;
-  const int half = c.hd / 2, quads = half / 4;
-  const int heads = c.Hq + 2 * c.Hkv;
-  const int total = T * heads * quads;   // < 2^31
-#pragma unroll 2
-  for (int idx = blockIdx.x * FWD_THREADS + threadIdx.x; idx < total; idx += gridDim.x * FWD_THREADS) {
-    const int i = (idx % quads) * 4;
-    const int hh = (idx / quads) % heads;
-    const int t = idx / (quads * heads);
-    float* row = c.qkv + (size_t)t * c.qkv_dim + (size_t)hh * c.hd;
-    const float4 x1 = *reinterpret_cast<const float4*>(row + i), x2 = *reinterpret_cast<const float4*>(row + i + half);
-    if (hh < c.Hq + c.Hkv) {
-      const int pos = c.tok_pos[t];
-      const float4 cs = *reinterpret_cast<const float4*>(c.rope_cos + (size_t)pos * half + i);
-      const float4 sn = *reinterpret_cast<const float4*>(c.rope_sin + (size_t)pos * half + i);
-      // explicit fused forms: every instance of this code rounds the same way
+  const int hd = c.hd, half = hd >> 1;
+  const int lanes = half >> 2, per_round = 32 / lanes;   // lanes per head, heads per round
+  const int heads = c.Hq + 2 * c.Hkv, rot_heads = c.Hq + c.Hkv;
+  const int per_task = per_round * U, tasks_row = (heads + per_task - 1) / per_task;
+  const int lane = threadIdx.x & 31;
+  const int sub = lane / lanes, i = (lane - sub * lanes) * 4;
+  const int total = T * tasks_row, step = gridDim.x * (FWD_THREADS / 32);
+#pragma unroll 1
+  for (int task = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; task < total; task += step) {
+    const int t = (int)((unsigned)task / (unsigned)tasks_row), h0 = (task - t * tasks_row) * per_task + sub;
+    float* row = c.qkv + (size_t)t * c.qkv_dim + i;
+    float4 x1[U], x2[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int hh = min(h0 + u * per_round, heads - 1);   // past the end: the last head again (not stored)
+      x1[u] = __ldcg(reinterpret_cast<const float4*>(row + hh * hd));
+      x2[u] = __ldcg(reinterpret_cast<const float4*>(row + hh * hd + half));
+    }
+    const int pos = c.tok_pos[t], sm = c.tok_slotmap[t];
+    const float4 cs = *reinterpret_cast<const float4*>(c.rope_cos + (size_t)pos * half + i);
+    const float4 sn = *reinterpret_cast<const float4*>(c.rope_sin + (size_t)pos * half + i);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int hh = h0 + u * per_round;
+      if (hh >= heads) break;
+      float4 y1 = x1[u], y2 = x2[u];
+      if (hh < rot_heads) {   // explicit fused forms: every instance of this code rounds the same way
 #define BLINK_ROT1(a, b, cc, ss_) fmaf((a), (cc), -__fmul_rn((b), (ss_)))
 #define BLINK_ROT2(a, b, cc, ss_) fmaf((b), (cc), __fmul_rn((a), (ss_)))
-      const float4 y1 = make_float4(BLINK_ROT1(x1.x, x2.x, cs.x, sn.x), BLINK_ROT1(x1.y, x2.y, cs.y, sn.y),
-                                    BLINK_ROT1(x1.z, x2.z, cs.z, sn.z), BLINK_ROT1(x1.w, x2.w, cs.w, sn.w));
-      const float4 y2 = make_float4(BLINK_ROT2(x1.x, x2.x, cs.x, sn.x), BLINK_ROT2(x1.y, x2.y, cs.y, sn.y),
-                                    BLINK_ROT2(x1.z, x2.z, cs.z, sn.z), BLINK_ROT2(x1.w, x2.w, cs.w, sn.w));
+        y1 = make_float4(BLINK_ROT1(x1[u].x, x2[u].x, cs.x, sn.x), BLINK_ROT1(x1[u].y, x2[u].y, cs.y, sn.y),
+                         BLINK_ROT1(x1[u].z, x2[u].z, cs.z, sn.z), BLINK_ROT1(x1[u].w, x2[u].w, cs.w, sn.w));
+        y2 = make_float4(BLINK_ROT2(x1[u].x, x2[u].x, cs.x, sn.x), BLINK_ROT2(x1[u].y, x2[u].y, cs.y, sn.y),
+                         BLINK_ROT2(x1[u].z, x2[u].z, cs.z, sn.z), BLINK_ROT2(x1[u].w, x2[u].w, cs.w, sn.w));
 #undef BLINK_ROT1
 #undef BLINK_ROT2
-      if (hh < c.Hq) {
-        if constexpr (sizeof(WT) == 2) {   // 16-bit path: q is an operand of the attention contraction
-          WT* qd = reinterpret_cast<WT*>(c.qb) + (size_t)t * c.q_dim + (size_t)hh * c.hd;
-          store4<WT>(qd + i, y1.x, y1.y, y1.z, y1.w);
-          store4<WT>(qd + i + half, y2.x, y2.y, y2.z, y2.w);
-        } else {
-          *reinterpret_cast<float4*>(row + i) = y1;
-          *reinterpret_cast<float4*>(row + i + half) = y2;
-        }
-      } else {
-        const int sm = c.tok_slotmap[t];
-        WT* dst = kv_tile<WT>(c, layer, 0, sm / c.bs, hh - c.Hq) + (size_t)(sm % c.bs) * c.hd;
-        store4<WT>(dst + i, y1.x, y1.y, y1.z, y1.w);
-        store4<WT>(dst + i + half, y2.x, y2.y, y2.z, y2.w);
       }
-    } else {
-      const int sm = c.tok_slotmap[t];
-      WT* dst = kv_tile<WT>(c, layer, 1, sm / c.bs, hh - c.Hq - c.Hkv) + (size_t)(sm % c.bs) * c.hd;
-      store4<WT>(dst + i, x1.x, x1.y, x1.z, x1.w);
-      store4<WT>(dst + i + half, x2.x, x2.y, x2.z, x2.w);
-    }
-    if (c.gemm_tc) {   // the split-K GEMM of the next layer adds partial sums into this buffer: leave it cleared
-      *reinterpret_cast<float4*>(row + i) = make_float4(0.f, 0.f, 0.f, 0.f);
-      *reinterpret_cast<float4*>(row + i + half) = make_float4(0.f, 0.f, 0.f, 0.f);
+      float* src = row + hh * hd;
+      if (sizeof(WT) != 2 && hh < c.Hq) {   // fp32 mode: the attention reads q from this buffer
+        *reinterpret_cast<float4*>(src) = y1;
+        *reinterpret_cast<float4*>(src + half) = y2;
+        continue;
+      }
+      WT* dst;
+      if (hh < c.Hq) dst = reinterpret_cast<WT*>(c.qb) + (size_t)t * c.q_dim + hh * hd + i;   // operand of the attention contraction
+      else dst = kv_tile<WT>(c, layer, hh < rot_heads ? 0 : 1, sm / c.bs, hh - (hh < rot_heads ? c.Hq : rot_heads)) +
+                 (size_t)(sm % c.bs) * hd + i;
+      store4<WT>(dst, y1.x, y1.y, y1.z, y1.w);
+      store4<WT>(dst + half, y2.x, y2.y, y2.z, y2.w);
+      if (c.gemm_tc) {   // the split-K GEMM of the next layer adds partial sums into this buffer: leave it cleared
+        *reinterpret_cast<float4*>(src) = make_float4(0.f, 0.f, 0.f, 0.f);
+        *reinterpret_cast<float4*>(src + half) = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
     }
   }
 }
@@ -819,34 +823,51 @@ template <typename WT>
 __device__ __noinline__ void silu_mul_pending(float* __restrict__ gu, WT* __restrict__ out, int T, int F, const int* list, int count) {
   const int tiles = F >> 6, pass_rows = tc_pass_rows(T);
   const int r_in = threadIdx.x >> 4, col = (threadIdx.x & 15) << 2;
-  const char* stage = reinterpret_cast<const char*>(list) + SILU_STAGE_OFF + threadIdx.x * 16;   // [8][FWD_THREADS] x 16 bytes
+  const char* stage = reinterpret_cast<const char*>(list) + SILU_STAGE_OFF + threadIdx.x * 16;   // [2][8][FWD_THREADS] x 16 bytes
   const uint32_t stage_s = (uint32_t)__cvta_generic_to_shared(stage);
-  for (int q = blockIdx.x; q < count * 4; q += gridDim.x) {
+  constexpr int BUF = 8 * FWD_THREADS * 16;
+  auto where = [&](int q, int& row0, int& j, int& t_end) {
     const int unit = list[q >> 2];
     const int pass = unit / tiles, tile = unit - pass * tiles;
-    const int row0 = pass * pass_rows + ((q & 3) << 6) + r_in, j = (tile << 6) + col;
-    const int t_end = min(T, (pass + 1) * pass_rows);
+    row0 = pass * pass_rows + ((q & 3) << 6) + r_in;
+    j = (tile << 6) + col;
+    t_end = min(T, (pass + 1) * pass_rows);
+  };
+  auto fetch = [&](int q, int buf) {
+    int row0, j, t_end;
+    where(q, row0, j, t_end);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const int t = row0 + 16 * k;
       if (t < t_end) {
         const float* src = gu + (size_t)t * 2 * F + j;
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(stage_s + (2 * k) * FWD_THREADS * 16), "l"(src) : "memory");
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(stage_s + (2 * k + 1) * FWD_THREADS * 16), "l"(src + F) : "memory");
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(stage_s + buf * BUF + (2 * k) * FWD_THREADS * 16), "l"(src) : "memory");
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(stage_s + buf * BUF + (2 * k + 1) * FWD_THREADS * 16), "l"(src + F) : "memory");
       }
     }
+  };
+  // the next piece is on its way while the current one is worked on (every thread reads back what it copied itself)
+  int q = blockIdx.x, buf = 0;
+  if (q < count * 4) fetch(q, 0);
+  asm volatile("cp.async.commit_group;" ::: "memory");
+#pragma unroll 1
+  for (; q < count * 4; q += gridDim.x, buf ^= 1) {
+    if (q + (int)gridDim.x < count * 4) fetch(q + gridDim.x, buf ^ 1);
     asm volatile("cp.async.commit_group;" ::: "memory");
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    int row0, j, t_end;
+    where(q, row0, j, t_end);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const int t = row0 + 16 * k;
       if (t < t_end) {
-        const float4 g = *reinterpret_cast<const float4*>(stage + (2 * k) * FWD_THREADS * 16);
-        const float4 u = *reinterpret_cast<const float4*>(stage + (2 * k + 1) * FWD_THREADS * 16);
+        const float4 g = *reinterpret_cast<const float4*>(stage + buf * BUF + (2 * k) * FWD_THREADS * 16);
+        const float4 u = *reinterpret_cast<const float4*>(stage + buf * BUF + (2 * k + 1) * FWD_THREADS * 16);
         silu_store<WT>(gu, out, t, j, F, g, u, true);
       }
     }
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 // The GEMM writes activations itself only in steps of more than one token pass: there its epilogue hides
 // behind the tensor-core work of the next tile, while at decode sizes the GEMM is bound by the weight
