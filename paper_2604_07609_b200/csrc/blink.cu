@@ -30,7 +30,8 @@
 namespace blink {
 
 // ---- stepped mode ----------------------------------------------------------------------
-__global__ void __launch_bounds__(CTRL_THREADS, 1) blink_control_kernel(const __grid_constant__ DevCtx c, int post_only) {
+__global__ void __launch_bounds__(CTRL_THREADS, 1) blink_control_kernel(const __grid_constant__ DevCtx param, int post_only) {
+  const DevCtx& c = ctx_to_shared(param);
   if (post_only) {
     if (c.ss->pending_post) post_step(c);
     if (threadIdx.x == 0) c.ss->cmd = CMD_NONE;

@@ -13,6 +13,19 @@
 
 namespace blink {
 
+// The kernels work on a copy of their parameter block in shared memory.  The phase functions take the block by
+// reference, and through a reference the parameter space is read like global memory: by way of L1, which every grid
+// barrier's acquire empties, so that each phase began with round trips to L2 for its own sizes and pointers.
+__shared__ DevCtx g_ctx;
+__device__ __forceinline__ const DevCtx& ctx_to_shared(const DevCtx& param) {
+  static_assert(sizeof(DevCtx) % 4 == 0, "copied by words");
+  const uint32_t* src = reinterpret_cast<const uint32_t*>(&param);
+  uint32_t* dst = reinterpret_cast<uint32_t*>(&g_ctx);
+  for (int i = threadIdx.x; i < (int)(sizeof(DevCtx) / 4); i += blockDim.x) dst[i] = src[i];
+  __syncthreads();
+  return g_ctx;
+}
+
 // ---- memory-ordering helpers ------------------------------------------------------
 __device__ __forceinline__ uint64_t ld_acquire_sys_u64(const volatile uint64_t* p) {
   uint64_t v;

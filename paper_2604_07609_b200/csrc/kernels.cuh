@@ -172,8 +172,9 @@ __device__ __forceinline__ void run_phase(const DevCtx& c, const StepInfo& st, i
 
 // ---- persistent loop -----------------------------------------------------------------
 template <typename WT, int HD, int NREP, bool PAIR>
-__global__ void __launch_bounds__(FWD_THREADS, 1) blink_loop_kernel(const __grid_constant__ DevCtx c) {
+__global__ void __launch_bounds__(FWD_THREADS, 1) blink_loop_kernel(const __grid_constant__ DevCtx param) {
   extern __shared__ __align__(1024) float smem[];
+  const DevCtx& c = ctx_to_shared(param);
   unsigned long long gen = 0;   // arrivals this CTA expects at its next grid barrier
   long long launch_iters = 0;
   TcState tc;
@@ -243,8 +244,9 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) blink_loop_kernel(const __grid
 }
 
 template <typename WT, int HD, int NREP, bool PAIR>
-__global__ void __launch_bounds__(FWD_THREADS, 1) blink_phase_kernel(const __grid_constant__ DevCtx c, int phase, int layer, int sub) {
+__global__ void __launch_bounds__(FWD_THREADS, 1) blink_phase_kernel(const __grid_constant__ DevCtx param, int phase, int layer, int sub) {
   extern __shared__ __align__(1024) float smem[];
+  const DevCtx& c = ctx_to_shared(param);
   if (c.ss->cmd != CMD_RUN) return;
   TcState tc;
   tc_init<PAIR>(c, smem, tc);
