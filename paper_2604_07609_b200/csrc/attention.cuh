@@ -37,15 +37,12 @@ struct AttStep {
 };
 __shared__ AttStep g_att_step;
 
-// per-thread state that survives from phase to phase (mbarrier parities of the warp's ring)
-struct AttState {
-  uint32_t par;
-  int blk;   // CTA-wide decode: the lane's block id of the CTA's first item (the same in all layers of a step)
-};
+__shared__ uint32_t g_att_par[ATT_WARPS];   // mbarrier parities of the warps' rings
+__shared__ int g_att_blk[FWD_THREADS];      // CTA-wide decode: the lane's block id of the CTA's first item (the same in all layers of a step)
 
-__device__ __forceinline__ void att_init(const DevCtx& c, AttState& s) {
-  s.par = 0;
-  s.blk = 0;
+__device__ __forceinline__ void att_init(const DevCtx& c) {
+  g_att_blk[threadIdx.x] = 0;
+  if ((threadIdx.x & 31) == 0) g_att_par[threadIdx.x >> 5] = 0u;
   if (c.dtype != 0 || c.control_only) return;
   if ((threadIdx.x & 31) == 0) {
     for (int i = 0; i < ATT_NS; ++i) mbar_init(&g_att.bar[threadIdx.x >> 5][i], 1);
@@ -210,7 +207,7 @@ __device__ __forceinline__ void att_tile_math(uint32_t kt, uint32_t vt, int n_va
 // slots at about half the HBM bandwidth; this form needs about 110.  Softmax statistics stay in
 // fp32 registers and are combined with shuffles.
 template <int HD, int NREP>
-__device__ __noinline__ void attn_decode_stream(const DevCtx& c, int layer, char* ring, AttState& as) {
+__device__ __noinline__ void attn_decode_stream(const DevCtx& c, int layer, char* ring) {
   constexpr int RB = HD * 2;         // bytes per key row
   constexpr int NBOX = HD / 64;      // 64-column boxes per tile row (128-byte swizzle span)
   constexpr int TILE = 16 * RB;      // bytes of one K (or V) tile of a (block, kv head)
@@ -236,6 +233,7 @@ __device__ __noinline__ void attn_decode_stream(const DevCtx& c, int layer, char
   const uint32_t ring_s = smem_u32(ring);
   const uint64_t kv_policy = l2_evict_first();   // the cache is read once per step
 
+  uint32_t par = g_att_par[w];
   int n_issued = 0, n_consumed = 0, p_k = 0, c_k = 0;
   bool p_done = false, first_fetch = true;
   DecCursor pc{0, 0, 0, 0, 0, 1}, cc{0, 0, 0, 0, 0, 1};
@@ -317,8 +315,8 @@ __device__ __noinline__ void attn_decode_stream(const DevCtx& c, int layer, char
       for (int i = 0; i < HD / 16; ++i) { o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f; }
     }
     const int s = n_consumed % ATT_NS;
-    if (!__all_sync(FULL, mbar_wait(c, &bars[s], (as.par >> s) & 1u, dead))) break;  // uniform exit
-    as.par ^= 1u << s;
+    if (!__all_sync(FULL, mbar_wait(c, &bars[s], (par >> s) & 1u, dead))) break;  // uniform exit
+    par ^= 1u << s;
     const uint32_t kt = ring_s + s * STAGE, vt = kt + TILE;
     const int key0 = cc.kb * 16;
     const int n_valid = min(16, n_ctx - key0);   // >= 1
@@ -411,6 +409,8 @@ __device__ __noinline__ void attn_decode_stream(const DevCtx& c, int layer, char
     }
     dec_advance(cc, n_dec, Hkv);
   }
+  __syncwarp();
+  if (lane == 0) g_att_par[w] = par;
 }
 
 // ---- decode rows: one CTA per part of a unit -----------------------------------------------------------
@@ -425,7 +425,7 @@ __device__ __noinline__ void attn_decode_stream(const DevCtx& c, int layer, char
 constexpr int ATT_NSC = 2;   // ring stages per warp here
 constexpr int ATT_CTA_OFF = 65536;   // the space before it may be receiving weights of the O projection already
 template <int HD, int NREP>
-static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer, char* base, AttState& as) {
+static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer, char* base) {
   constexpr int RB = HD * 2;
   constexpr int TILE = 16 * RB;
   constexpr int STAGE = 2 * TILE;
@@ -450,6 +450,7 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer, 
   __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(c.attn);
   const float qscale = c.attn_scale * 1.4426950408889634f;
   const uint64_t kv_policy = l2_evict_first();
+  uint32_t par = g_att_par[w];
 
   // items in unit order; prefill tiles of a step sit on the first CTAs, so the decode items start from the last
   for (int item = (int)gridDim.x - 1 - (int)blockIdx.x; ; item += gridDim.x) {   // uniform over the CTA
@@ -468,10 +469,10 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer, 
     const int32_t* table = c.block_table + (size_t)g_att_bslot[d] * c.max_blocks_seq;
     // block ids of the warp's first 32 tiles, one per lane; the first item's are kept from layer to layer
     const bool first = item < (int)gridDim.x;
-    int blk = as.blk;
+    int blk = g_att_blk[threadIdx.x];
     if (!(first && layer > 0 && !c.stepped)) {
       blk = lane < n_tiles ? table[kb0 + w + ATT_WARPS * lane] : 0;
-      if (first) as.blk = blk;
+      if (first) g_att_blk[threadIdx.x] = blk;
     }
     auto issue = [&](int i) {
       if (i >= 32 && (i & 31) == 0) blk = i + lane < n_tiles ? table[kb0 + w + ATT_WARPS * (i + lane)] : 0;
@@ -553,8 +554,8 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer, 
     for (int i = 0; i < HD / 16; ++i) { o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f; }
     for (int i = 0; i < n_tiles; ++i) {
       const int s = i % ATT_NSC;
-      if (!__all_sync(FULL, mbar_wait(c, &bars[s], (as.par >> s) & 1u, dead))) break;
-      as.par ^= 1u << s;
+      if (!__all_sync(FULL, mbar_wait(c, &bars[s], (par >> s) & 1u, dead))) break;
+      par ^= 1u << s;
       char* st = ring + s * STAGE;
       const int n_valid = min(16, n_ctx - (kb0 + w + ATT_WARPS * i) * 16);   // >= 1
       if (n_valid < 16) {   // the tail of the last block holds whatever the pool held: clear those V rows (0 x NaN)
@@ -658,6 +659,7 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer, 
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
   }
+  if (lane == 0) g_att_par[w] = par;
 }
 
 // ---- prefill-chunk rows: tensor-core tile kernel ---------------------------------------------------
@@ -843,7 +845,7 @@ constexpr int att_smem_bytes() {
 }
 
 template <int HD, int NREP>
-__device__ __forceinline__ void phase_attention_bf16(const DevCtx& c, int layer, float* smem_f, AttState& as) {
+__device__ __forceinline__ void phase_attention_bf16(const DevCtx& c, int layer, float* smem_f) {
   char* smem = reinterpret_cast<char*>(smem_f);
   if (layer == 0 || c.stepped) {   // the step's work lists: once per step
     const SchedState* ss = c.ss;
@@ -864,12 +866,12 @@ __device__ __forceinline__ void phase_attention_bf16(const DevCtx& c, int layer,
   if (n_dec > 0) {
     if (n_pf > 0) __syncthreads();   // the prefill tiles' shared memory is free
     if (g_att_step.C > 0) {
-      attn_decode_cta<HD, NREP>(c, layer, tc_tiles(smem_f) + ATT_CTA_OFF, as);
+      attn_decode_cta<HD, NREP>(c, layer, tc_tiles(smem_f) + ATT_CTA_OFF);
     } else {
       const int w = threadIdx.x >> 5;
       constexpr int STAGE = 2 * 16 * HD * 2;
       char* ring = tc_tiles(smem_f) + w * ATT_NS * STAGE;   // 1024-byte aligned: the tiles are swizzled
-      attn_decode_stream<HD, NREP>(c, layer, ring, as);
+      attn_decode_stream<HD, NREP>(c, layer, ring);
     }
   }
 }

@@ -17,11 +17,13 @@ namespace blink {
 // reference, and through a reference the parameter space is read like global memory: by way of L1, which every grid
 // barrier's acquire empties, so that each phase began with round trips to L2 for its own sizes and pointers.
 __shared__ DevCtx g_ctx;
+__shared__ unsigned long long g_bar_target;   // arrivals the CTA expects at its next grid barrier, zero when the kernel starts
 __device__ __forceinline__ const DevCtx& ctx_to_shared(const DevCtx& param) {
   static_assert(sizeof(DevCtx) % 4 == 0, "copied by words");
   const uint32_t* src = reinterpret_cast<const uint32_t*>(&param);
   uint32_t* dst = reinterpret_cast<uint32_t*>(&g_ctx);
   for (int i = threadIdx.x; i < (int)(sizeof(DevCtx) / 4); i += blockDim.x) dst[i] = src[i];
+  if (threadIdx.x == 0) g_bar_target = 0ull;
   __syncthreads();
   return g_ctx;
 }
@@ -67,13 +69,13 @@ __device__ __forceinline__ unsigned long long ld_acquire_gpu_u64(const unsigned 
 
 // Grid-wide barrier with a bounded wait: every CTA adds one to a monotone counter (reset by the
 // host before each launch) and waits until it reaches the next multiple of the grid size.
-// Returns false when the loop must unwind (time-out here or abort raised elsewhere).  `target`
-// is the caller's private running total (thread 0 of each CTA keeps it).
+// Returns false when the loop must unwind (time-out here or abort raised elsewhere).  g_bar_target
+// is the CTA's running total.  Out of line: one copy of the code for all phases.
 __device__ __forceinline__ void fence_proxy_async_global() {
   asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 
-__device__ __forceinline__ bool grid_barrier(const DevCtx& c, unsigned long long& target) {
+static __device__ __noinline__ bool grid_barrier(const DevCtx& c) {
   __shared__ int s_ok;
   // Buffers written with ordinary stores in one phase (normed rows, K/V rows, attention output, ...)
   // are read by TMA / bulk copies (the async proxy) in a later phase: every thread orders its
@@ -83,7 +85,8 @@ __device__ __forceinline__ bool grid_barrier(const DevCtx& c, unsigned long long
   if (threadIdx.x == 0) {
     int ok = 1;
     SchedState* ss = c.ss;
-    target += gridDim.x;
+    const unsigned long long target = g_bar_target + gridDim.x;
+    g_bar_target = target;
     // release at gpu scope is cumulative: the stores of the CTA's other threads, ordered before this
     // point by the barrier above, are covered without a separate fence
     asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(&ss->bar_ctr) : "memory");

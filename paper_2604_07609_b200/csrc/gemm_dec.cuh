@@ -32,16 +32,17 @@ struct DecShared {
 };
 __shared__ __align__(8) DecShared g_dec;
 
-// per-thread bookkeeping (parities), see TcState
+// per-warp bookkeeping (parities), see TcState
 struct DecState {
   uint32_t fill_a, use_a, fill_b, use_b, made, loaded;
   int pre;   // weight producer: stages of the coming GEMM that are already on their way
 };
 
+__shared__ DecState g_dec_state[FWD_THREADS / 32];
+
 template <bool PAIR>
-__device__ __forceinline__ void dec_init(const DevCtx& c, DecState& s) {
-  s.fill_a = s.use_a = s.fill_b = s.use_b = s.made = s.loaded = 0;
-  s.pre = 0;
+__device__ __forceinline__ void dec_init(const DevCtx& c) {
+  if ((threadIdx.x & 31) == 0) g_dec_state[threadIdx.x >> 5] = DecState{0u, 0u, 0u, 0u, 0u, 0u, 0};
   if (!c.gemm_tc) return;
   if (threadIdx.x == 32) {
     for (int i = 0; i < DEC_STAGES; ++i) { mbar_init(&g_dec.a_full[i], 1); mbar_init(&g_dec.a_empty[i], 1); }
@@ -54,8 +55,9 @@ __device__ __forceinline__ void dec_init(const DevCtx& c, DecState& s) {
 // The loop may be abandoned between two GEMMs: wait (bounded) for weights that are still on their way into this CTA's
 // shared memory.  Run by warp 0 of every CTA, before the cluster's last barrier.
 template <bool PAIR>
-__device__ __forceinline__ void dec_drain(const DevCtx& c, DecState& s, uint32_t rank) {
-  if (!c.gemm_tc || (threadIdx.x >> 5) != 0 || s.pre == 0) return;
+__device__ __forceinline__ void dec_drain(const DevCtx& c, uint32_t rank) {
+  if (!c.gemm_tc || (threadIdx.x >> 5) != 0) return;
+  const DecState s = g_dec_state[0];
   if (!PAIR || rank == 0) {   // all bytes of a pair are counted in CTA 0
     const long long t0 = clock64();
     for (int i = 0; i < s.pre; ++i)
@@ -86,9 +88,9 @@ __device__ __forceinline__ void dec_geometry(const DevCtx& c, int T, int R) {
 }
 
 // Weight producer (warp 0): stage-sized pieces [first, first + count) of this CTA's range of a GEMM; piece i goes to
-// stage i % DEC_STAGES.  Returns the number of pieces issued.
+// stage i % DEC_STAGES.  Returns the number of pieces issued, and in the low four bits the new parities.
 template <bool PAIR>
-static __device__ __noinline__ int dec_fill_weights(const DevCtx& c, const TcGeom& g, int which, int layer, char* tiles, DecState& s,
+static __device__ __noinline__ int dec_fill_weights(const DevCtx& c, const TcGeom& g, int which, int layer, char* tiles, uint32_t fill_a,
                                                     uint32_t rank, int first, int count) {
   const TcMaps* maps = reinterpret_cast<const TcMaps*>(c.tc_maps);
   const uint64_t policy = l2_evict_first();
@@ -102,10 +104,10 @@ static __device__ __noinline__ int dec_fill_weights(const DevCtx& c, const TcGeo
     int kb = sg.kb0;
     if (first > i) { kb += 2 * (first - i); i = first; }
     for (; kb < sg.kb1; kb += 2, ++i) {
-      if (i >= first + count) return issued;
+      if (i >= first + count) return (issued << 4) | (int)fill_a;
       const int nk = min(2, sg.kb1 - kb), stage = i % DEC_STAGES;
-      if (!mbar_wait_warp(c, &g_dec.a_empty[stage], ((s.fill_a >> stage) & 1u) ^ 1u)) return issued;
-      s.fill_a ^= 1u << stage;
+      if (!mbar_wait_warp(c, &g_dec.a_empty[stage], ((fill_a >> stage) & 1u) ^ 1u)) return (issued << 4) | (int)fill_a;
+      fill_a ^= 1u << stage;
       char* sa = tiles + stage * DEC_STAGE_BYTES;
       if (elect_one()) {
         uint64_t* bar = &g_dec.a_full[stage];
@@ -130,7 +132,7 @@ static __device__ __noinline__ int dec_fill_weights(const DevCtx& c, const TcGeo
       ++issued;
     }
   }
-  return issued;
+  return (issued << 4) | (int)fill_a;
 }
 
 // ---- token operands made by the CTA --------------------------------------------------------------------------
@@ -402,7 +404,7 @@ __device__ __forceinline__ void dec_load_tokens(const DevCtx& c, const DecPhase&
 // stages may be filled before it starts.
 template <bool PAIR>
 static __device__ __noinline__ void phase_gemm_dec(const DevCtx& c, int which, int layer, int T, int R, int next_which, int next_pre,
-                                                   float* smem_f, TcState& tc, DecState& s) {
+                                                   float* smem_f) {
   const TcGeom g = g_dec.g[which];
   const bool small = dec_small(c, T);
   DecPhase p;
@@ -414,6 +416,13 @@ static __device__ __noinline__ void phase_gemm_dec(const DevCtx& c, int which, i
   const uint32_t rank = PAIR ? cluster_ctarank() : 0u;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   char* tiles = tc_tiles(smem_f);
+  TcState tc = g_tc_state[warp];
+  DecState s = g_dec_state[warp];
+  auto fill = [&](int w, int l, int from, int count) {   // (warp 0)
+    const int r = dec_fill_weights<PAIR>(c, g_dec.g[w], w, l, tiles, s.fill_a, rank, from, count);
+    s.fill_a = (uint32_t)r & 15u;
+    return r >> 4;
+  };
   // Small steps have no phases that clear what the split-K GEMMs add into: gate/up rows (read by the down projection of
   // the layer before) are cleared in the QKV and LM head phases, QKV rows (read by the attention) in the O phase, and in
   // the last of those the logits, where the LM head splits K.
@@ -426,7 +435,7 @@ static __device__ __noinline__ void phase_gemm_dec(const DevCtx& c, int which, i
   int first = 0;
   if (warp == 0) {   // whatever the phase before could not bring yet
     first = s.pre;
-    if (first < DEC_STAGES) first += dec_fill_weights<PAIR>(c, g_dec.g[which], which, layer, tiles, s, rank, first, DEC_STAGES - first);
+    if (first < DEC_STAGES) first += fill(which, layer, first, DEC_STAGES - first);
     s.pre = 0;
   }
   if (p.made) {
@@ -447,10 +456,9 @@ static __device__ __noinline__ void phase_gemm_dec(const DevCtx& c, int which, i
   }
 
   if (warp == 0) {
-    dec_fill_weights<PAIR>(c, g_dec.g[which], which, layer, tiles, s, rank, first, 0x40000000);
+    fill(which, layer, first, 0x4000000);
     if (next_which >= 0 && *(volatile int*)&g_tc.dead == 0) {
-      const int nl = next_which == GEMM_QKV ? layer + 1 : layer;
-      s.pre = dec_fill_weights<PAIR>(c, g_dec.g[next_which], next_which, nl, tiles, s, rank, 0, next_pre);
+      s.pre = fill(next_which, next_which == GEMM_QKV ? layer + 1 : layer, 0, next_pre);
     }
   } else if (warp == 2) {
     if (!p.made) dec_load_tokens<PAIR>(c, p, g, tiles, s, rank);
@@ -504,6 +512,10 @@ static __device__ __noinline__ void phase_gemm_dec(const DevCtx& c, int which, i
   if (g.u0 < g.u1) {
     if (p.made) s.made ^= 1u;
     if (p.loaded) s.loaded ^= 1u;
+  }
+  if (lane == 0) {
+    g_tc_state[warp] = tc;
+    g_dec_state[warp] = s;
   }
   __syncthreads();
 }

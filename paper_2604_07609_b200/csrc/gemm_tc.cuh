@@ -39,9 +39,10 @@ constexpr int TC_MAX_STAGES = 11;
 constexpr int TC_A_BYTES = 128 * 128;  // 128 weight rows x 64 bf16
 constexpr int TC_TILE_BUDGET = 196608;
 
-// Per-thread pipeline bookkeeping that survives from one GEMM phase to the next (the
+// Per-warp pipeline bookkeeping that survives from one GEMM phase to the next (the
 // mbarriers are initialised once per kernel).  Bit s of a mask is the parity of the next
-// phase to wait for on barrier s; only the thread that owns a role uses its masks.
+// phase to wait for on barrier s; only the warp that owns a role uses its masks.  Kept in shared memory between
+// phases (a phase works on a copy in registers): on the stack of the loop kernel it was read back from L2.
 struct TcState {
   uint32_t tmem_base;
   uint32_t fill_bits;   // producer: stages filled so far, parity per stage
@@ -58,6 +59,7 @@ struct TcShared {
   int dead;
 };
 __shared__ __align__(8) TcShared g_tc;
+__shared__ TcState g_tc_state[FWD_THREADS / 32];
 
 struct TcHost {
   void* d_maps = nullptr;
@@ -353,10 +355,11 @@ __device__ __forceinline__ bool mbar_wait_idle(const DevCtx& c, uint64_t* bar, u
 
 // ---- TMEM allocation for the life of the kernel ---------------------------------------------
 template <bool PAIR>
-__device__ __forceinline__ void tc_init(const DevCtx& c, float*, TcState& s) {
+__device__ __forceinline__ void tc_init(const DevCtx& c) {
+  TcState s;
   s.tmem_base = 0;
   s.fill_bits = s.use_bits = s.acc_mma = s.acc_epi = s.last_bit = 0;
-  if (!c.gemm_tc) return;
+  if (!c.gemm_tc) return;   // (uniform over the grid)
   if (threadIdx.x == 32) {
     // pairs: the operands of a stage come from four producers (two per CTA), all counted on CTA 0's barrier,
     // where CTA 0's two producers announce the bytes of both CTAs (an announcement by CTA 1 would be a remote
@@ -382,17 +385,20 @@ __device__ __forceinline__ void tc_init(const DevCtx& c, float*, TcState& s) {
   if constexpr (PAIR) cluster_sync_all();   // both CTAs' barriers exist before either touches the other's
   tc_fence_after();
   s.tmem_base = *(volatile uint32_t*)&g_tc.tmem;
+  if ((threadIdx.x & 31) == 0) g_tc_state[threadIdx.x >> 5] = s;
+  __syncthreads();
 }
 template <bool PAIR>
-__device__ __forceinline__ void tc_fini(const DevCtx& c, TcState& s) {
+__device__ __forceinline__ void tc_fini(const DevCtx& c) {
+  const uint32_t tmem_base = c.gemm_tc ? g_tc_state[0].tmem_base : 0u;
   if (!c.gemm_tc) return;
   tc_fence_before();
   __syncthreads();
   if constexpr (PAIR) cluster_sync_all();   // the other CTA no longer signals into this one's shared memory
   if (threadIdx.x < 32) {
     tc_fence_after();
-    if constexpr (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(s.tmem_base) : "memory");
-    else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(s.tmem_base) : "memory");
+    if constexpr (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");
+    else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");
   }
 }
 
@@ -787,7 +793,7 @@ static __device__ __noinline__ void tc_finish_tiles(const DevCtx& c, const GemmA
 }
 
 template <bool PAIR>
-static __device__ __noinline__ void phase_gemm_tc(const DevCtx& c, const GemmArgs& a, int which, int layer, float* smem_f, TcState& tc) {
+static __device__ __noinline__ void phase_gemm_tc(const DevCtx& c, const GemmArgs& a, int which, int layer, float* smem_f) {
   const int T = a.M, N = a.N, K = a.K;
   if (T <= 0) return;  // uniform over the grid
   // gate/up on the streaming layout: weight rows are interleaved (gate f, up f, ...), and in a dense model
@@ -809,6 +815,7 @@ static __device__ __noinline__ void phase_gemm_tc(const DevCtx& c, const GemmArg
   char* tiles = tc_tiles(smem_f);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* dead = &g_tc.dead;
+  TcState tc = g_tc_state[warp];
 
   if (warp == 0) {
     tc_produce_weights<PAIR>(c, a.w, a.w_row0, which, g, tiles, tc, rank);
@@ -879,6 +886,8 @@ static __device__ __noinline__ void phase_gemm_tc(const DevCtx& c, const GemmArg
       }
     }
   }
+  __syncwarp();
+  if (lane == 0) g_tc_state[warp] = tc;
   __syncthreads();
   if constexpr (!PAIR) {
     if (a.fix != FIX_NONE) tc_finish_tiles(c, a, g, layer);

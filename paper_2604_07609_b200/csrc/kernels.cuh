@@ -16,41 +16,27 @@
 namespace blink {
 
 template <typename WT, bool PAIR>
-__device__ __forceinline__ void gemm_dispatch(const DevCtx& c, const GemmArgs& a, int which, int layer, float* smem,
-                                              TcState& tc) {
-  if (c.gemm_tc) phase_gemm_tc<PAIR>(c, a, which, layer, smem, tc);
+__device__ __forceinline__ void gemm_dispatch(const DevCtx& c, const GemmArgs& a, int which, int layer, float* smem) {
+  if (c.gemm_tc) phase_gemm_tc<PAIR>(c, a, which, layer, smem);
   else phase_gemm_simt<WT>(a);
 }
 
-// What the phases of a step depend on besides the layer: read once per step, it does not change between phases.
+// What the phases of a step depend on besides the layer: made once per step, kept in shared memory.
 struct StepInfo {
   int T, R;      // rows of the step, rows that sample
   bool dec;      // decode-sized: the GEMMs of gemm_dec.cuh
   bool small;    // of at most 16 rows: norms, SwiGLU and final norm run inside those GEMMs
   bool fuse;     // RoPE and the K/V write run inside the attention
+  bool nuc;      // some row samples from the nucleus of its whole row
   bool att_cta;  // the attention phase leaves the first half of the weight ring alone
 };
-template <typename WT, bool PAIR>
-__device__ __forceinline__ StepInfo step_info(const DevCtx& c) {
-  StepInfo s;
-  const SchedState* ss = c.ss;
-  s.T = __ldcg(&ss->cur_T);
-  s.R = __ldcg(&ss->cur_rows);
-  const int C = __ldcg(&ss->cur_C), npf = __ldcg(&ss->cur_npf), fuse = __ldcg(&ss->cur_fuse);
-  if constexpr (sizeof(WT) == 2) {
-    s.small = dec_small(c, s.T);
-    s.dec = dec_step(c, s.T);
-    s.fuse = fuse != 0;
-    s.att_cta = C > 0 && npf == 0;
-    if (s.dec) {
-      dec_geometry<PAIR>(c, s.T, s.R);
-      __syncthreads();
-    }
-  } else {
-    s.small = s.dec = s.fuse = s.att_cta = false;
-  }
-  return s;
-}
+__shared__ StepInfo g_step;
+// The phases of a layer and of the output part, in order, for the current step: phase | expert << 8 | PLAN_BARRIER when a
+// grid barrier closes it.
+constexpr int PLAN_BARRIER = 1 << 16, PLAN_MAX = 2 * MAX_EXPERTS + 12;
+__shared__ int g_plan[2][PLAN_MAX], g_plan_n[2];
+__shared__ unsigned long long g_phase_ns[N_PHASE_TIMERS];   // device time per phase kind of the open step (CTA 0)
+__shared__ unsigned long long g_phase_t;                    // when the last phase ended
 // Phases that a step does not have because others do their work.
 __device__ __forceinline__ bool phase_absorbed(const DevCtx& c, const StepInfo& st, int ph) {
   if (c.fused) return ph == PH_ROPE || ph == PH_SILU;   // done by the epilogues of the QKV and gate/up GEMMs
@@ -58,11 +44,74 @@ __device__ __forceinline__ bool phase_absorbed(const DevCtx& c, const StepInfo& 
   if (!st.small) return false;
   return ph == PH_NORM1 || ph == PH_FNORM || (c.E == 0 && (ph == PH_NORM2 || ph == PH_SILU));
 }
+// (one thread)
+__device__ __forceinline__ void make_plan(const DevCtx& c, const StepInfo& st) {
+  int n = 0;
+  for (int ph = PH_NORM1; ph <= PH_DOWN; ++ph) {
+    if (phase_absorbed(c, st, ph)) continue;
+    if (c.E > 0 && (ph == PH_GU || ph == PH_DOWN)) {
+      if (ph == PH_GU) g_plan[0][n++] = PH_MOE_GROUP | PLAN_BARRIER;   // routing lists and gathered rows first
+      // The experts' GEMMs are independent of one another (own weights, own gathered rows; the down projections add
+      // into the residual rows with reductions): one grid barrier after the last expert, none in between, so every
+      // CTA streams its share of all experts back to back.  (With fused epilogues the barriers stay: their tile
+      // counters are per GEMM.)
+      for (int e = 0; e < c.E; ++e) g_plan[0][n++] = ph | e << 8 | (c.fused || e + 1 == c.E ? PLAN_BARRIER : 0);
+    } else {
+      g_plan[0][n++] = ph | PLAN_BARRIER;
+    }
+  }
+  g_plan_n[0] = n;
+  // the output part; long rows are prepared for sampling by all CTAs, rows that sample from a whole-row nucleus with one
+  // more pass over the logits
+  n = 0;
+  for (int i = 0; i < 5; ++i) {
+    const int ph = output_phase(i);
+    if (phase_absorbed(c, st, ph) || ((ph == PH_SMAX || ph == PH_SNUC) && !sample_split_rows(c.V)) || (ph == PH_SNUC && !st.nuc)) continue;
+    g_plan[1][n++] = ph | PLAN_BARRIER;
+  }
+  g_plan_n[1] = n;
+}
+template <typename WT, bool PAIR>
+static __device__ __noinline__ void step_begin(const DevCtx& c) {
+  StepInfo s;
+  const SchedState* ss = c.ss;
+  s.T = __ldcg(&ss->cur_T);
+  s.R = __ldcg(&ss->cur_rows);
+  s.nuc = __ldcg(&ss->cur_nuc) != 0;
+  const int C = __ldcg(&ss->cur_C), npf = __ldcg(&ss->cur_npf), fuse = __ldcg(&ss->cur_fuse);
+  if constexpr (sizeof(WT) == 2) {
+    s.small = dec_small(c, s.T);
+    s.dec = dec_step(c, s.T);
+    s.fuse = fuse != 0;
+    s.att_cta = C > 0 && npf == 0;
+    if (s.dec) dec_geometry<PAIR>(c, s.T, s.R);
+  } else {
+    s.small = s.dec = s.fuse = s.att_cta = false;
+  }
+  if (threadIdx.x < N_PHASE_TIMERS) g_phase_ns[threadIdx.x] = 0ull;
+  if (threadIdx.x == 0) {
+    g_step = s;
+    make_plan(c, s);
+    g_phase_t = global_timer_ns();
+  }
+  __syncthreads();
+}
+// The grid barrier that closes a phase.  CTA 0 keeps a device time per phase kind (a phase's time includes this
+// barrier), recorded when per-iteration statistics are kept.
+__device__ __forceinline__ bool end_phase(const DevCtx& c, int ph) {
+  const bool ok = grid_barrier(c);
+  if (c.stats_cap > 0 && blockIdx.x == 0 && threadIdx.x == 0) {
+    const unsigned long long t = global_timer_ns();
+    g_phase_ns[ph >= PH_SMAX ? (int)PH_SAMPLE : ph] += t - g_phase_t;   // the parts of sampling share a timer
+    g_phase_t = t;
+  }
+  return ok;
+}
 // The GEMM phases of a decode-sized step; false when the phase is none of them.  `chain`: weights of the GEMM that
 // follows may be fetched ahead (not when every phase is a launch of its own).
 template <bool PAIR>
-__device__ __forceinline__ bool run_phase_dec(const DevCtx& c, const StepInfo& st, int phase, int layer, float* smem, TcState& tc,
-                                              DecState& ds, bool chain) {
+__device__ __forceinline__ bool run_phase_dec(const DevCtx& c, const StepInfo& st, int phase, int layer, float* smem,
+                                              bool chain) {
   int which, next = -1, pre = DEC_STAGES;
   switch (phase) {
     case PH_QKV: which = GEMM_QKV; next = GEMM_O; pre = st.att_cta ? ATT_CTA_OFF / DEC_STAGE_BYTES : 0; break;
@@ -76,17 +125,17 @@ __device__ __forceinline__ bool run_phase_dec(const DevCtx& c, const StepInfo& s
     case PH_LMHEAD: which = GEMM_LMHEAD; break;
     default: return false;
   }
-  phase_gemm_dec<PAIR>(c, which, layer, st.T, st.R, chain ? next : -1, pre, smem, tc, ds);
+  phase_gemm_dec<PAIR>(c, which, layer, st.T, st.R, chain ? next : -1, pre, smem);
   return true;
 }
 
 template <typename WT, int HD, int NREP, bool PAIR>
-__device__ __forceinline__ void run_phase(const DevCtx& c, const StepInfo& st, int phase, int layer, int sub, float* smem,
-                                          TcState& tc, AttState& as, DecState& ds, bool chain) {
+__device__ __forceinline__ void run_phase(const DevCtx& c, int phase, int layer, int sub, float* smem, bool chain) {
   const size_t esz = sizeof(WT);
+  const StepInfo& st = g_step;
   const int T = st.T;
   if constexpr (sizeof(WT) == 2) {
-    if (st.dec && run_phase_dec<PAIR>(c, st, phase, layer, smem, tc, ds, chain)) return;
+    if (st.dec && run_phase_dec<PAIR>(c, st, phase, layer, smem, chain)) return;
   }
   switch (phase) {
     case PH_NORM1:
@@ -98,11 +147,11 @@ __device__ __forceinline__ void run_phase(const DevCtx& c, const StepInfo& st, i
                  c.qkv_dim, 0};
       a.w_row0 = (long long)layer * c.qkv_dim;
       if (c.fused) a.fix = FIX_ROPE_KV;
-      gemm_dispatch<WT, PAIR>(c, a, GEMM_QKV, layer, smem, tc);
+      gemm_dispatch<WT, PAIR>(c, a, GEMM_QKV, layer, smem);
     } break;
     case PH_ROPE: phase_rope_kv<WT>(c, layer); break;
     case PH_ATTN:
-      if constexpr (sizeof(WT) == 2) phase_attention_bf16<HD, NREP>(c, layer, smem, as);
+      if constexpr (sizeof(WT) == 2) phase_attention_bf16<HD, NREP>(c, layer, smem);
       else phase_attention<WT, HD, NREP>(c, layer, smem);
 
       break;
@@ -110,7 +159,7 @@ __device__ __forceinline__ void run_phase(const DevCtx& c, const StepInfo& st, i
       GemmArgs a{c.attn, c.w_base + c.w_off[2] + (size_t)layer * c.d * c.q_dim * esz, c.h, T, c.d, c.q_dim, c.d, 1};
       a.w_row0 = (long long)layer * c.d;
       if (c.fused_norm) { a.fix = FIX_SUMSQ; a.fix_rowss = c.rowss_a; }
-      gemm_dispatch<WT, PAIR>(c, a, GEMM_O, layer, smem, tc);
+      gemm_dispatch<WT, PAIR>(c, a, GEMM_O, layer, smem);
     } break;
     case PH_NORM2:
       if (c.fused_norm) phase_norm_apply<WT>(c, layer, 1, T);
@@ -121,7 +170,7 @@ __device__ __forceinline__ void run_phase(const DevCtx& c, const StepInfo& st, i
         GemmArgs a{c.xn, c.w_base + c.w_off[3] + (size_t)layer * 2 * c.F * c.d * esz, c.gu, T, 2 * c.F, c.d, 2 * c.F, 0};
         a.w_row0 = (long long)layer * 2 * c.F;
         if (c.fused) { a.fix = FIX_SILU; a.fix_out = c.act; }
-        gemm_dispatch<WT, PAIR>(c, a, GEMM_GU, layer, smem, tc);
+        gemm_dispatch<WT, PAIR>(c, a, GEMM_GU, layer, smem);
       } else {
         // expert `sub` on the rows routed to it (gathered, contiguous from moe_off[sub])
         const int off = c.moe_off[sub], cnt = c.moe_off[sub + 1] - off;
@@ -131,7 +180,7 @@ __device__ __forceinline__ void run_phase(const DevCtx& c, const StepInfo& st, i
         a.x_row0 = off;
         a.w_row0 = we * 2 * c.F;
         if (c.fused) { a.fix = FIX_SILU; a.fix_out = reinterpret_cast<char*>(c.act) + (size_t)off * c.F * esz; }
-        gemm_dispatch<WT, PAIR>(c, a, GEMM_GU, layer, smem, tc);
+        gemm_dispatch<WT, PAIR>(c, a, GEMM_GU, layer, smem);
       }
     } break;
     case PH_SILU:
@@ -142,7 +191,7 @@ __device__ __forceinline__ void run_phase(const DevCtx& c, const StepInfo& st, i
         GemmArgs a{c.act, c.w_base + c.w_off[4] + (size_t)layer * c.d * c.F * esz, c.h, T, c.d, c.F, c.d, 1};
         a.w_row0 = (long long)layer * c.d;
         if (c.fused_norm) { a.fix = FIX_SUMSQ; a.fix_rowss = c.rowss_b; }
-        gemm_dispatch<WT, PAIR>(c, a, GEMM_DOWN, layer, smem, tc);
+        gemm_dispatch<WT, PAIR>(c, a, GEMM_DOWN, layer, smem);
       } else {
         const int off = c.moe_off[sub], cnt = c.moe_off[sub + 1] - off;
         const long long we = (long long)layer * c.E + sub;
@@ -152,7 +201,7 @@ __device__ __forceinline__ void run_phase(const DevCtx& c, const StepInfo& st, i
         a.w_row0 = we * c.d;
         a.row_map = c.moe_tok + off;     // result row i belongs to token moe_tok[off + i], weighted by its gate
         a.row_scale = c.moe_gate + off;
-        gemm_dispatch<WT, PAIR>(c, a, GEMM_DOWN, layer, smem, tc);
+        gemm_dispatch<WT, PAIR>(c, a, GEMM_DOWN, layer, smem);
       }
     } break;
     case PH_MOE_GROUP: phase_moe_group<WT>(c, smem); break;
@@ -161,7 +210,7 @@ __device__ __forceinline__ void run_phase(const DevCtx& c, const StepInfo& st, i
       break;
     case PH_LMHEAD: {
       GemmArgs a{c.xs, c.w_base + c.w_off[9], c.logits, c.ss->cur_rows, c.V, c.d, c.V, 0};
-      gemm_dispatch<WT, PAIR>(c, a, GEMM_LMHEAD, 0, smem, tc);
+      gemm_dispatch<WT, PAIR>(c, a, GEMM_LMHEAD, 0, smem);
     } break;
     case PH_SMAX: phase_sample_max(c); break;
     case PH_SNUC: phase_sample_weights(c, smem); break;
@@ -175,66 +224,35 @@ template <typename WT, int HD, int NREP, bool PAIR>
 __global__ void __launch_bounds__(FWD_THREADS, 1) blink_loop_kernel(const __grid_constant__ DevCtx param) {
   extern __shared__ __align__(1024) float smem[];
   const DevCtx& c = ctx_to_shared(param);
-  unsigned long long gen = 0;   // arrivals this CTA expects at its next grid barrier
   long long launch_iters = 0;
-  TcState tc;
-  tc_init<PAIR>(c, smem, tc);
-  AttState as;
-  att_init(c, as);
-  DecState ds;
-  dec_init<PAIR>(c, ds);
+  tc_init<PAIR>(c);
+  att_init(c);
+  dec_init<PAIR>(c);
   if constexpr (PAIR) cluster_sync_all();   // the other CTA's barriers exist before they are signalled
+  else __syncthreads();
   while (true) {
     if (blockIdx.x == 0) control_phase(c, launch_iters);
-    if (!grid_barrier(c, gen)) break;
+    if (!grid_barrier(c)) break;
     if (*(volatile int*)&c.ss->cmd != CMD_RUN) break;
     if (!c.control_only) {
       bool ok = true;
-      // CTA 0 keeps a per-phase-kind device time of the open iteration (a phase's time includes
-      // the barrier that closes it); recorded only when per-iteration statistics are kept
-      const bool timed = c.stats_cap > 0 && blockIdx.x == 0 && threadIdx.x == 0;
-      uint64_t t_prev = timed ? global_timer_ns() : 0;
-      const StepInfo st = step_info<WT, PAIR>(c);
-      auto step_phase = [&](int ph, int layer, int sub) {
-        if (phase_absorbed(c, st, ph)) return;
-        // The experts' GEMMs are independent of one another (own weights, own gathered rows; the down
-        // projections add into the residual rows with reductions): one grid barrier after the last
-        // expert, none in between, so every CTA streams its share of all experts back to back.  (With
-        // fused epilogues the barriers stay: their tile counters are per GEMM.)
-        const bool barrier = !(c.E > 0 && !c.fused && (ph == PH_GU || ph == PH_DOWN) && sub + 1 < c.E);
-        run_phase<WT, HD, NREP, PAIR>(c, st, ph, layer, sub, smem, tc, as, ds, true);
-        if (!barrier) return;
-        ok = grid_barrier(c, gen);
-        if (timed) {   // the parts of sampling share a timer
-          const uint64_t t = global_timer_ns();
-          c.ss->cur_phase_ns[ph >= PH_SMAX ? (int)PH_SAMPLE : ph] += t - t_prev;
-          t_prev = t;
+      step_begin<WT, PAIR>(c);
+      // Everything that a phase needs is in shared memory: this loop keeps its counters and nothing else, so that no
+      // spilled register of it lies between the end of one phase and the beginning of the next.
+      for (int layer = 0; layer <= c.L && ok; ++layer) {   // the output part follows the last layer
+        const int part = layer == c.L;
+        for (int i = 0; i < g_plan_n[part] && ok; ++i) {
+          const int todo = g_plan[part][i];
+          run_phase<WT, HD, NREP, PAIR>(c, todo & 255, layer, (todo >> 8) & 255, smem, true);
+          if (todo & PLAN_BARRIER) ok = end_phase(c, todo & 255);
         }
-      };
-      for (int layer = 0; layer < c.L && ok; ++layer) {
-        for (int ph = PH_NORM1; ph <= PH_DOWN && ok; ++ph) {
-          if (c.E > 0 && (ph == PH_GU || ph == PH_DOWN)) {
-            if (ph == PH_GU) step_phase(PH_MOE_GROUP, layer, 0);   // routing lists and gathered rows first
-            for (int e = 0; e < c.E && ok; ++e) step_phase(ph, layer, e);
-          } else {
-            step_phase(ph, layer, 0);
-          }
-        }
-      }
-      // the output part; long rows are prepared for sampling by all CTAs, rows that sample from a whole-row nucleus
-      // with one more pass over the logits
-      const bool split = sample_split_rows(c.V);
-      const bool nuc = split && __ldcg(&c.ss->cur_nuc) != 0;
-      for (int i = 0; i < 5 && ok; ++i) {
-        const int ph = output_phase(i);
-        if ((ph == PH_SMAX && !split) || (ph == PH_SNUC && !nuc)) continue;
-        step_phase(ph, 0, 0);
       }
       if (!ok) break;
-    } else if (!grid_barrier(c, gen)) break;
+      if (c.stats_cap > 0 && blockIdx.x == 0 && threadIdx.x < N_PHASE_TIMERS) c.ss->cur_phase_ns[threadIdx.x] = g_phase_ns[threadIdx.x];
+    } else if (!grid_barrier(c)) break;
   }
-  dec_drain<PAIR>(c, ds, PAIR ? cluster_ctarank() : 0u);
-  tc_fini<PAIR>(c, tc);
+  dec_drain<PAIR>(c, PAIR ? cluster_ctarank() : 0u);
+  tc_fini<PAIR>(c);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     const int aborted = *(volatile int*)&c.ss->abort_flag;
     __threadfence_system();
@@ -248,17 +266,14 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) blink_phase_kernel(const __gri
   extern __shared__ __align__(1024) float smem[];
   const DevCtx& c = ctx_to_shared(param);
   if (c.ss->cmd != CMD_RUN) return;
-  TcState tc;
-  tc_init<PAIR>(c, smem, tc);
-  AttState as;
-  att_init(c, as);
-  DecState ds;
-  dec_init<PAIR>(c, ds);
+  tc_init<PAIR>(c);
+  att_init(c);
+  dec_init<PAIR>(c);
   if constexpr (PAIR) cluster_sync_all();
   else __syncthreads();
-  const StepInfo st = step_info<WT, PAIR>(c);
-  if (!phase_absorbed(c, st, phase)) run_phase<WT, HD, NREP, PAIR>(c, st, phase, layer, sub, smem, tc, as, ds, false);
-  tc_fini<PAIR>(c, tc);
+  step_begin<WT, PAIR>(c);
+  if (!phase_absorbed(c, g_step, phase)) run_phase<WT, HD, NREP, PAIR>(c, phase, layer, sub, smem, false);
+  tc_fini<PAIR>(c);
 }
 
 // `pair`: the variant whose GEMMs run on CTA pairs (tcgen05 cta_group::2; launched with clusters of two).
