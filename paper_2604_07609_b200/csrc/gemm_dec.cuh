@@ -138,9 +138,15 @@ static __device__ __noinline__ int dec_fill_weights(const DevCtx& c, const TcGeo
 // ---- token operands made by the CTA --------------------------------------------------------------------------
 // Slot i of the operand holds the k-block of the i-th unit of the CTA's range (a range longer than K wraps round), so
 // a CTA makes only the k-blocks it will use.  Inside a slot: 8 rows of 128 bytes, 16-byte chunks swizzled by the row.
+// Of a pair, CTA r makes the rows of tokens r, r + 2, r + 4, ..: column j of the accumulator then belongs to token
+// dec_token(j), and a step of few rows is halved between the two.
 struct DecSlots {
   int kb_first, kblocks, n, bytes;   // first k-block, k-blocks of K, slots, bytes of a slot
 };
+template <bool PAIR>
+__device__ __forceinline__ int dec_token(int j) { return PAIR ? ((j & 7) << 1) | (j >> 3) : j; }
+template <bool PAIR>
+__device__ __forceinline__ int dec_rows_here(int rows, uint32_t rank) { return PAIR ? (rows - (int)rank + 1) >> 1 : rows; }
 template <bool PAIR>
 __device__ __forceinline__ DecSlots dec_slots(const TcGeom& g) {
   DecSlots d;
@@ -165,8 +171,7 @@ static __device__ __noinline__ void dec_make_normed(const DevCtx& c, int which, 
   __shared__ float s_ss[2][WARPS][8];
   const int tid = threadIdx.x;
   const int d = c.d;
-  const int t0 = PAIR ? (int)rank * 8 : 0;
-  const int n_here = min(PAIR ? 8 : 16, rows - t0);
+  const int n_here = dec_rows_here<PAIR>(rows, rank);
   const bool embed = which == GEMM_QKV && layer == 0;
   const bool live = tid * 4 < d;   // d = 256: the first two warps
   const float* g = which == GEMM_QKV ? wptr_f(c, 6) + (size_t)layer * d : which == GEMM_GU ? wptr_f(c, 7) + (size_t)layer * d
@@ -183,7 +188,7 @@ static __device__ __noinline__ void dec_make_normed(const DevCtx& c, int which, 
     float ss[RP];
 #pragma unroll
     for (int q = 0; q < RP; ++q) {
-      const int t = t0 + min(r0 + q, n_here - 1);   // past the end: the last row again
+      const int r = min(r0 + q, n_here - 1), t = PAIR ? 2 * r + (int)rank : r;   // past the end: the last row again
       if (embed) {
         const __nv_bfloat16* e = wptr<__nv_bfloat16>(c, 0) + (size_t)c.tok_id[t] * d + tid * 4;
 #pragma unroll
@@ -219,11 +224,12 @@ static __device__ __noinline__ void dec_make_normed(const DevCtx& c, int which, 
           const float inv = rsqrtf(tot * inv_d + c.rms_eps);
           char* row = bt + (r >> 3) * 1024 + (r & 7) * 128 + (((col >> 3) ^ (r & 7)) << 4) + (col & 7) * 2;
           // the embedding row also goes into the residual stream, by one CTA
-          const bool keep = embed && (int)blockIdx.x == (PAIR ? 2 * (r & 7) + (int)rank : r);
+          const int t = PAIR ? 2 * r + (int)rank : r;
+          const bool keep = embed && (int)blockIdx.x == t;
 #pragma unroll
           for (int k = 0; k < NV; ++k) {
             const float4 x = v[q][k];
-            if (keep) *reinterpret_cast<float4*>(c.h + (size_t)(t0 + r) * d + tid * 4 + k * 1024) = x;
+            if (keep) *reinterpret_cast<float4*>(c.h + (size_t)t * d + tid * 4 + k * 1024) = x;
             const int slot = dec_slot_of(sl, k * 16 + (tid >> 4));
             if (slot < sl.n)
               store4<__nv_bfloat16>(reinterpret_cast<__nv_bfloat16*>(row + slot * sl.bytes), x.x * inv * gg[k].x, x.y * inv * gg[k].y,
@@ -238,8 +244,7 @@ static __device__ __noinline__ void dec_make_normed(const DevCtx& c, int which, 
 template <bool PAIR>
 static __device__ __noinline__ void dec_make_silu(const DevCtx& c, int rows, const DecSlots sl, char* bt, uint32_t rank) {
   constexpr int U = 2;
-  const int t0 = PAIR ? (int)rank * 8 : 0;
-  const int nr = min(PAIR ? 8 : 16, rows - t0);
+  const int nr = dec_rows_here<PAIR>(rows, rank);
   const int per_row = sl.n * 8, total = nr * per_row;   // items of 8 features
   for (int base = FWD_THREADS - 1 - threadIdx.x; base < total; base += U * FWD_THREADS) {   // warp 0, busy with the weights, last
     float4 g[U][2], u[U][2];
@@ -251,7 +256,7 @@ static __device__ __noinline__ void dec_make_silu(const DevCtx& c, int rows, con
       const int slot = q >> 3, c8 = q & 7;
       int kb = sl.kb_first + slot;
       if (kb >= sl.kblocks) kb -= sl.kblocks;
-      const float* src = c.gu + (size_t)(t0 + r) * 2 * c.F + kb * 64 + c8 * 8;
+      const float* src = c.gu + (size_t)(PAIR ? 2 * r + (int)rank : r) * 2 * c.F + kb * 64 + c8 * 8;
       dst[k] = slot * sl.bytes + (r >> 3) * 1024 + (r & 7) * 128 + ((c8 ^ (r & 7)) << 4);
       g[k][0] = __ldcg(reinterpret_cast<const float4*>(src));
       g[k][1] = __ldcg(reinterpret_cast<const float4*>(src) + 1);
@@ -400,6 +405,23 @@ __device__ __forceinline__ void dec_load_tokens(const DevCtx& c, const DecPhase&
   }
 }
 
+// The 16 columns of an accumulator whose token operand was made by the CTAs -> out
+template <bool PAIR>
+__device__ __forceinline__ void dec_epi_made(const TcEpiOut& e, uint32_t taddr, int n, bool plain) {
+  float v[16];
+  tmem_ld16(taddr, v);
+  if (n >= e.N) return;
+  float* o = e.out + (e.ilv_F ? (n & 1) * e.ilv_F + (n >> 1) : n);
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    const int t = dec_token<PAIR>(j);
+    if (t < e.T) {
+      if (plain) o[(size_t)t * e.ldo] = v[j];
+      else red_add_f32(o + (size_t)t * e.ldo, v[j]);
+    }
+  }
+}
+
 // One GEMM of a decode-sized step.  `next_which` (or -1): the GEMM whose weights follow; `next_pre`: how many of its
 // stages may be filled before it starts.
 template <bool PAIR>
@@ -498,7 +520,8 @@ static __device__ __noinline__ void phase_gemm_dec(const DevCtx& c, int which, i
       tc.acc_epi ^= 1u << abuf;
       tc_fence_after();
       const uint32_t taddr = tc.tmem_base + (uint32_t)abuf * 256u + ((uint32_t)(q * 32) << 16);
-      tc_epi_columns(eo, taddr, nt * 128 + q * 32 + lane, 0, 0, n_mma, plain);
+      if (p.made) dec_epi_made<PAIR>(eo, taddr, nt * 128 + q * 32 + lane, plain);
+      else tc_epi_columns(eo, taddr, nt * 128 + q * 32 + lane, 0, 0, n_mma, plain);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) {
