@@ -112,34 +112,42 @@ static __device__ __noinline__ bool grid_barrier(const DevCtx& c) {
   return s_ok != 0;
 }
 
-// Exclusive prefix sum over the 256 threads of the control CTA; *total gets the sum.
-__device__ __forceinline__ int block_exscan(int v, int* total) {
-  __shared__ int s_warp[CTRL_THREADS / 32];
-  __shared__ int s_total;
+// Exclusive prefix sums of N values over the 256 threads of the control CTA, all at once (two barriers; one scan after
+// another took 0.4 us each, nine of them in a step); tot gets the sums, v the prefixes.
+template <int N>
+__device__ __forceinline__ void block_exscan(int (&v)[N], int (&tot)[N]) {
+  constexpr int W = CTRL_THREADS / 32;
+  __shared__ __align__(16) int s_scan[N][W];
+  static_assert(W == 8, "a row of warp sums is two 16-byte vectors");
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  int x = v;
+  int x[N];
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    int y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  __syncthreads();  // protects s_warp / s_total from the previous call
-  if (lane == 31) s_warp[w] = x;
-  __syncthreads();
-  if (w == 0) {
-    int t = lane < CTRL_THREADS / 32 ? s_warp[lane] : 0;
-    int z = t;
+  for (int n = 0; n < N; ++n) x[n] = v[n];
 #pragma unroll
-    for (int o = 1; o < 8; o <<= 1) {
-      int y = __shfl_up_sync(0xffffffffu, z, o);
-      if (lane >= o) z += y;
+  for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+    for (int n = 0; n < N; ++n) {
+      const int y = __shfl_up_sync(0xffffffffu, x[n], o);
+      if (lane >= o) x[n] += y;
     }
-    if (lane < CTRL_THREADS / 32) s_warp[lane] = z - t;
-    if (lane == CTRL_THREADS / 32 - 1) s_total = z;
-  }
+  __syncthreads();   // the previous call's sums have been read
+  if (lane == 31)
+#pragma unroll
+    for (int n = 0; n < N; ++n) s_scan[n][w] = x[n];
   __syncthreads();
-  *total = s_total;
-  return x - v + s_warp[w];
+#pragma unroll
+  for (int n = 0; n < N; ++n) {
+    const int4 a = *reinterpret_cast<const int4*>(&s_scan[n][0]), b = *reinterpret_cast<const int4*>(&s_scan[n][4]);
+    const int p[W] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    int before = 0, all = 0;
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+      if (i < w) before += p[i];
+      all += p[i];
+    }
+    v[n] = x[n] - v[n] + before;
+    tot[n] = all;
+  }
 }
 
 __device__ __forceinline__ int32_t fake_token(unsigned long long ticket, int gen, int vocab) {
@@ -160,10 +168,17 @@ static __device__ void post_step(const DevCtx& c) {
   int32_t* rec_post = c.trace + ss->cur_post;
   __shared__ unsigned long long s_ptok;
   __shared__ int s_need_sum;
+  // the host's cancel marks are a round trip to host memory away: asked for first, looked at after the rest
+  int cslot = 0;
+  uint32_t cmark = 0u;
+  if (c.cancel != nullptr && tid < c.MB && c.b_phase[tid] != PHASE_FREE) {
+    cslot = c.b_slot[tid];
+    cmark = ld_relaxed_sys_u32(&c.cancel[cslot]);
+  }
   if (tid == 0) { s_ptok = 0; s_need_sum = 0; }
   __syncthreads();
 
-  int fin = 0, nfree = 0, b = -1, row = -1;
+  int fin = 0, nfree = 0, b = -1, row = -1, out_slot = -1, out_gen = 0;
   long long ticket = 0;
   if (tid < n_items) {
     b = c.it_bslot[tid];
@@ -190,8 +205,8 @@ static __device__ void post_step(const DevCtx& c) {
       c.slot_hot[slot].generated = gen + 1;
       if (phase == PHASE_PREFILL) c.b_phase[b] = PHASE_DECODE;
       c.slot_hot[slot].state = fin ? SLOT_DECODE_COMPLETED : SLOT_DECODE_PROCESSING;
-      __threadfence_system();
-      c.out_count[slot] = (uint32_t)(gen + 1) | (fin ? 0x80000000u : 0u);
+      out_slot = slot;
+      out_gen = gen + 1;
       if (tr) { rec_post[2 * row] = b; rec_post[2 * row + 1] = sampled; }
       if (fin) {
         nfree = c.b_have[b];
@@ -199,10 +214,10 @@ static __device__ void post_step(const DevCtx& c) {
       }
     }
   }
-  int tot_fin, tot_free;
-  const int fin_idx = block_exscan(fin, &tot_fin);
-  const int free_off = block_exscan(nfree, &tot_free);
   const int top = ss->free_top;
+  int sc[2] = {fin, nfree}, sc_tot[2];
+  block_exscan(sc, sc_tot);
+  const int fin_idx = sc[0], free_off = sc[1], tot_fin = sc_tot[0], tot_free = sc_tot[1];
   if (fin) {
     if (tr) rec_post[2 * n_rows + fin_idx] = (int32_t)ticket;
     for (int j = 0; j < nfree; ++j) {
@@ -213,24 +228,28 @@ static __device__ void post_step(const DevCtx& c) {
     c.b_have[b] = 0;
     c.b_phase[b] = PHASE_FREE;
   }
+  if (out_slot >= 0) {   // (the writes above have had the time of the scans to reach the host)
+    __threadfence_system();
+    c.out_count[out_slot] = (uint32_t)out_gen | (fin ? 0x80000000u : 0u);
+  }
   __syncthreads();
   // Cancellation (an early exit the host asks for): every request that is still live after the step's
   // own completions and whose slot carries the host's cancel mark is retired here, in ascending batch
   // slot, exactly as at a normal end: blocks pushed back in logical order, reservation released.
-  int cfin = 0, cfree = 0, cslot = 0;
+  int cfin = 0, cfree = 0;
   long long cticket = 0;
-  if (c.cancel != nullptr && tid < c.MB && c.b_phase[tid] != PHASE_FREE) {
-    cslot = c.b_slot[tid];
-    if (ld_relaxed_sys_u32(&c.cancel[cslot]) != 0u) {
-      cfin = 1;
-      cfree = c.b_have[tid];
-      cticket = c.b_ticket[tid];
-      atomicAdd(&s_need_sum, c.b_need[tid]);
-    }
+  if (cmark != 0u && c.b_phase[tid] != PHASE_FREE) {
+    cfin = 1;
+    cfree = c.b_have[tid];
+    cticket = c.b_ticket[tid];
+    atomicAdd(&s_need_sum, c.b_need[tid]);
   }
-  int tot_cfin, tot_cfree;
-  const int cfin_idx = block_exscan(cfin, &tot_cfin);
-  const int cfree_off = block_exscan(cfree, &tot_cfree);
+  int cfin_idx = 0, cfree_off = 0, tot_cfin = 0, tot_cfree = 0;
+  if (__syncthreads_or(cfin)) {
+    int cs[2] = {cfin, cfree}, cs_tot[2];
+    block_exscan(cs, cs_tot);
+    cfin_idx = cs[0]; cfree_off = cs[1]; tot_cfin = cs_tot[0]; tot_cfree = cs_tot[1];
+  }
   if (cfin) {
     if (tr) rec_post[2 * n_rows + tot_fin + tot_free + cfin_idx] = (int32_t)cticket;
     for (int j = 0; j < cfree; ++j) {
@@ -298,47 +317,50 @@ static __device__ void post_step(const DevCtx& c) {
 }
 
 // ---- stand-in for the frontend's RDMA write: pinned submit area -> HBM ring --------------
+// (a warp per request: entry and prompt are reads from host memory, a microsecond or two each)
 static __device__ void ingress(const DevCtx& c, unsigned long long tail) {
   SchedState* ss = c.ss;
-  const int tid = threadIdx.x;
-  for (unsigned long long e = ss->seen; e < tail; ++e) {
-    const SubEntry* en = &c.sub_q[e % (unsigned long long)c.n_slots];
-    const uint32_t slot = en->slot;
-    const uint32_t np = en->n_prompt;
-    const uint32_t flags = en->flags;
-    if (slot >= (uint32_t)c.n_slots || np > (uint32_t)c.max_prompt || en->ticket != e) {
-      if (tid == 0) dev_fail(c, DEV_ERR_BAD_INDEX);
+  const int tid = threadIdx.x, lane = tid & 31;
+  const unsigned long long seen = ss->seen;
+  for (unsigned long long e = seen + (unsigned)(tid >> 5); e < tail; e += CTRL_THREADS / 32) {
+    const SubEntry en = c.sub_q[e % (unsigned long long)c.n_slots];
+    const uint32_t slot = en.slot, np = en.n_prompt;
+    if (slot >= (uint32_t)c.n_slots || np > (uint32_t)c.max_prompt || en.max_new > (uint32_t)c.max_new || en.ticket != e) {
+      if (lane == 0) dev_fail(c, DEV_ERR_BAD_INDEX);
       break;
     }
-    const int32_t* src = c.sub_tokens + (size_t)slot * c.max_prompt;
-    int32_t* dst = c.in_arena + (size_t)slot * c.max_prompt;
-    for (uint32_t i = tid; i < np; i += CTRL_THREADS) dst[i] = src[i];
-    if (flags & REQ_FLAG_FORCED) {
-      const int32_t* fs = c.sub_forced + (size_t)slot * c.max_new;
-      int32_t* fd = c.forced_arena + (size_t)slot * c.max_new;
-      for (uint32_t i = tid; i < en->max_new; i += CTRL_THREADS) fd[i] = fs[i];
-    }
-    if (tid == 0) {
+    auto copy = [&](int32_t* dst, const int32_t* src, uint32_t n) {
+      for (uint32_t i0 = 0; i0 < n; i0 += 256) {   // eight words per lane on their way at a time
+        int32_t v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = src[min(i0 + 32u * k + lane, n - 1u)];
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          if (i0 + 32u * k + lane < n) dst[i0 + 32u * k + lane] = v[k];
+      }
+    };
+    copy(c.in_arena + (size_t)slot * c.max_prompt, c.sub_tokens + (size_t)slot * c.max_prompt, np);
+    if (en.flags & REQ_FLAG_FORCED)
+      copy(c.forced_arena + (size_t)slot * c.max_new, c.sub_forced + (size_t)slot * c.max_new, en.max_new);
+    if (lane == 0) {
       SlotCold& cold = c.slot_cold[slot];
-      cold.ticket = en->ticket;
-      cold.max_new = en->max_new;
-      cold.top_k = en->top_k;
-      cold.temperature = en->temperature;
-      cold.eos_id = en->eos_id;
-      cold.seed = en->seed;
-      cold.user_tag = en->user_tag;
-      cold.flags = flags;
-      cold.top_p = en->top_p;
+      cold.ticket = en.ticket;
+      cold.max_new = en.max_new;
+      cold.top_k = en.top_k;
+      cold.temperature = en.temperature;
+      cold.eos_id = en.eos_id;
+      cold.seed = en.seed;
+      cold.user_tag = en.user_tag;
+      cold.flags = en.flags;
+      cold.top_p = en.top_p;
       SlotHot& hot = c.slot_hot[slot];
       hot.n_prompt = np;
       hot.generated = 0;
       hot.arena_off = slot;
     }
-    __syncthreads();  // payload before the state flip
-    if (tid == 0) {
-      __threadfence();
-      c.slot_hot[slot].state = SLOT_PREFILL_PENDING;
-    }
+    __threadfence();   // payload before the state flip
+    __syncwarp();
+    if (lane == 0) c.slot_hot[slot].state = SLOT_PREFILL_PENDING;
   }
   __syncthreads();
   if (tid == 0) ss->seen = tail;
@@ -390,37 +412,52 @@ static __device__ int schedule_step(const DevCtx& c, unsigned long long visible)
   if (trace_on(c)) hdr = ss->trace_pos;
   int32_t* rec = c.trace + (hdr >= 0 ? hdr : 0);
 
-  // 1. FCFS admission (serial: one decision depends on the previous one)
-  if (tid == 0) {
-    int n_admit = 0;
-    int reserved = ss->reserved;
-    int cursor = 0;
-    unsigned long long na = ss->next_admit;
-    // worst-case space check for the admitted section is done with the rest below
-    while (na < visible) {
-      const uint32_t slot = c.ticket_to_slot[na % (unsigned long long)c.n_slots];
-      if (slot >= (uint32_t)c.n_slots || c.slot_cold[slot].ticket != na ||
-          c.slot_hot[slot].state != SLOT_PREFILL_PROCESSING) {
-        dev_fail(c, DEV_ERR_TICKET_TABLE);
-        break;
+  // 1. FCFS admission.  The decisions are serial (each depends on the one before), what they need is read and what they
+  // cause is written by all threads.
+  const unsigned long long na = ss->next_admit;
+  const int n_cand = (int)min(visible - na, (unsigned long long)MB);
+  if (n_cand > 0) {   // uniform over the CTA
+    uint32_t slot = 0;
+    int P = 0;
+    SlotCold cold;
+    if (tid < n_cand) {
+      slot = c.ticket_to_slot[(na + tid) % (unsigned long long)c.n_slots];
+      bool bad = slot >= (uint32_t)c.n_slots;
+      if (!bad) {
+        cold = c.slot_cold[slot];
+        P = (int)c.slot_hot[slot].n_prompt;
+        bad = cold.ticket != na + tid || c.slot_hot[slot].state != SLOT_PREFILL_PROCESSING;
       }
-      const int P = (int)c.slot_hot[slot].n_prompt;
-      const SlotCold cold = c.slot_cold[slot];
-      const int N = (int)cold.max_new;
-      const int need = (P + N - 1 + c.bs - 1) / c.bs;
-      while (cursor < MB && s_phase[cursor] != PHASE_FREE) ++cursor;
-      if (cursor >= MB || reserved + need > c.n_blocks) break;  // head of line blocks
-      const int b = cursor;
-      s_phase[b] = PHASE_PREFILL;
+      s_qstart[tid] = bad ? -1 : (P + (int)cold.max_new - 1 + c.bs - 1) / c.bs;   // blocks needed
+    }
+    __syncthreads();
+    if (tid == 0) {
+      int n = 0, reserved = ss->reserved, cursor = 0;
+      for (; n < n_cand; ++n) {
+        const int need = s_qstart[n];
+        if (need < 0) { dev_fail(c, DEV_ERR_TICKET_TABLE); break; }
+        while (cursor < MB && s_phase[cursor] != PHASE_FREE) ++cursor;
+        if (cursor >= MB || reserved + need > c.n_blocks) break;  // head of line blocks
+        s_phase[cursor] = PHASE_PREFILL;
+        s_item_b[n] = cursor;
+        reserved += need;
+      }
+      ss->next_admit = na + n;
+      ss->reserved = reserved;
+      s_n_admit = n;
+    }
+    __syncthreads();
+    if (tid < s_n_admit) {
+      const int b = s_item_b[tid];
       c.b_phase[b] = PHASE_PREFILL;
-      c.b_ticket[b] = (long long)na;
+      c.b_ticket[b] = (long long)(na + tid);
       c.b_slot[b] = (int)slot;
       c.b_P[b] = P;
-      c.b_N[b] = N;
+      c.b_N[b] = (int)cold.max_new;
       c.b_prefilled[b] = 0;
       c.b_generated[b] = 0;
       c.b_have[b] = 0;
-      c.b_need[b] = need;
+      c.b_need[b] = s_qstart[tid];
       c.b_last[b] = 0;
       c.b_eos[b] = cold.eos_id;
       c.b_topk[b] = (int)cold.top_k;
@@ -428,20 +465,14 @@ static __device__ int schedule_step(const DevCtx& c, unsigned long long visible)
       c.b_topp[b] = cold.top_p;
       c.b_seed[b] = cold.seed;
       c.b_flags[b] = (int)cold.flags;
-      reserved += need;
-      if (hdr >= 0 && hdr + TRACE_HDR_WORDS + 2 * (n_admit + 1) <= c.trace_cap) {
-        rec[TRACE_HDR_WORDS + 2 * n_admit] = (int32_t)na;
-        rec[TRACE_HDR_WORDS + 2 * n_admit + 1] = b;
+      if (hdr >= 0 && hdr + TRACE_HDR_WORDS + 2 * (tid + 1) <= c.trace_cap) {
+        rec[TRACE_HDR_WORDS + 2 * tid] = (int32_t)(na + tid);
+        rec[TRACE_HDR_WORDS + 2 * tid + 1] = b;
       }
-      ++n_admit;
-      ++na;
     }
-    ss->next_admit = na;
-    ss->reserved = reserved;
-    s_n_admit = n_admit;
     __threadfence();
+    __syncthreads();
   }
-  __syncthreads();
   const int n_admit = s_n_admit;
 
   // 2. compose
@@ -494,26 +525,20 @@ static __device__ int schedule_step(const DevCtx& c, unsigned long long visible)
   const int new_len = start + take;
   const int want = f ? (new_len + c.bs - 1) / c.bs - have : 0;
   const int sample = f && (phase == PHASE_DECODE || new_len == P);
-  int n_items, T, n_alloc, n_rows;
-  const int item = block_exscan(f, &n_items);
-  const int qstart = block_exscan(take, &T);
-  const int aoff = block_exscan(want, &n_alloc);
-  const int row = block_exscan(sample, &n_rows);
-  // blocks that post_step may free at most, and tickets that may end (completions and cancellations),
-  // for the trace space check
-  int tot_may_free, n_live;
-  block_exscan(phase != PHASE_FREE ? have + want : 0, &tot_may_free);
-  block_exscan(phase != PHASE_FREE ? 1 : 0, &n_live);
   // attention work lists: single-row requests stream their KV blocks, multi-row requests are
   // cut into blocks of 128 / n_rep query rows
   const int q_rows = 128 / c.n_rep;
   const int is_dec = f && take == 1;
   const int nkb_att = is_dec ? (new_len + c.bs - 1) / c.bs : 0;
   const int n_qb = (f && take > 1) ? (take + q_rows - 1) / q_rows : 0;
-  int n_dec_att, tot_kb, n_pf;
-  const int dec_idx = block_exscan(is_dec, &n_dec_att);
-  const int kb_pre = block_exscan(nkb_att, &tot_kb);
-  const int pf_off = block_exscan(n_qb, &n_pf);
+  // (the last two: blocks that post_step may free at most, and tickets that may end, by completion or
+  // cancellation, for the trace space check)
+  int sc[9] = {f, take, want, sample, is_dec, nkb_att, n_qb, phase != PHASE_FREE ? have + want : 0, phase != PHASE_FREE ? 1 : 0};
+  int sc_tot[9];
+  block_exscan(sc, sc_tot);
+  const int item = sc[0], qstart = sc[1], aoff = sc[2], row = sc[3], dec_idx = sc[4], kb_pre = sc[5], pf_off = sc[6];
+  const int n_items = sc_tot[0], T = sc_tot[1], n_alloc = sc_tot[2], n_rows = sc_tot[3], n_dec_att = sc_tot[4], tot_kb = sc_tot[5],
+            n_pf = sc_tot[6], tot_may_free = sc_tot[7], n_live = sc_tot[8];
 
   if (T == 0) return 0;  // uniform: every thread sees the same T
 
@@ -721,12 +746,15 @@ static __device__ __noinline__ void control_phase(const DevCtx& c, long long& la
   while (true) {
     if (tid == 0) {
       int cmd = CMD_NONE;
-      if (ld_relaxed_sys_u32(&c.mbox->stop)) { cmd = CMD_EXIT; ss->exit_reason = 2; }
+      // both words are in host memory: one round trip for the two
+      const uint32_t stop = ld_relaxed_sys_u32(&c.mbox->stop);
+      const unsigned long long sub_tail = ld_acquire_sys_u64(&c.mbox->sub_tail);
+      if (stop) { cmd = CMD_EXIT; ss->exit_reason = 2; }
       else if (*(volatile int*)&ss->abort_flag) { cmd = CMD_EXIT; ss->exit_reason = 5; }
       else if (c.iteration_budget > 0 && launch_iters >= c.iteration_budget) { cmd = CMD_EXIT; ss->exit_reason = 3; }
       unsigned long long tail = ss->seen;
       const int started = !c.start_paused || ld_relaxed_sys_u32(&c.mbox->start);
-      if (cmd == CMD_NONE && started) tail = ld_acquire_sys_u64(&c.mbox->sub_tail);
+      if (cmd == CMD_NONE && started) tail = sub_tail;
       s_cmd = cmd;
       s_tail = tail;
       s_started = started;
@@ -737,8 +765,10 @@ static __device__ __noinline__ void control_phase(const DevCtx& c, long long& la
     const bool started = s_started != 0;
     int T = 0;
     if (started) {
-      if (tail > ss->seen) ingress(c, tail);
-      scan_and_claim(c);
+      if (tail > ss->seen) {   // slots become pending here and nowhere else
+        ingress(c, tail);
+        scan_and_claim(c);
+      }
       T = schedule_step(c, ss->seen);
     }
     __syncthreads();
