@@ -75,41 +75,40 @@ __device__ __forceinline__ void fence_proxy_async_global() {
   asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 
+// Arrival and wait of the CTA, by one thread after a barrier of the threads whose stores it stands for.
+__device__ __forceinline__ bool grid_arrive_and_wait(const DevCtx& c) {
+  SchedState* ss = c.ss;
+  const unsigned long long target = g_bar_target + gridDim.x;
+  g_bar_target = target;
+  // release at gpu scope is cumulative: the stores of the CTA's other threads, ordered before this
+  // point by the barrier before, are covered without a separate fence
+  asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(&ss->bar_ctr) : "memory");
+  long long t0 = 0;
+  unsigned int polls = 0;
+  while (ld_acquire_gpu_u64(&ss->bar_ctr) < target) {
+    if ((++polls & 63u) == 0) {
+      if (*(volatile int*)&ss->abort_flag) return false;
+      if (t0 == 0) t0 = clock64();
+      if ((unsigned long long)(clock64() - t0) > c.barrier_timeout_cycles) {
+        dev_fail(c, DEV_ERR_BARRIER_TIMEOUT);
+        return false;
+      }
+      if (polls > 4096u) __nanosleep(200);
+    }
+  }
+  return *(volatile int*)&ss->abort_flag == 0;
+}
+__shared__ int g_bar_ok;
 static __device__ __noinline__ bool grid_barrier(const DevCtx& c) {
-  __shared__ int s_ok;
   // Buffers written with ordinary stores in one phase (normed rows, K/V rows, attention output, ...)
   // are read by TMA / bulk copies (the async proxy) in a later phase: every thread orders its
   // stores against that proxy before it arrives, and again before it issues copies afterwards.
   fence_proxy_async_global();
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int ok = 1;
-    SchedState* ss = c.ss;
-    const unsigned long long target = g_bar_target + gridDim.x;
-    g_bar_target = target;
-    // release at gpu scope is cumulative: the stores of the CTA's other threads, ordered before this
-    // point by the barrier above, are covered without a separate fence
-    asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(&ss->bar_ctr) : "memory");
-    long long t0 = 0;
-    unsigned int polls = 0;
-    while (ld_acquire_gpu_u64(&ss->bar_ctr) < target) {
-      if ((++polls & 63u) == 0) {
-        if (*(volatile int*)&ss->abort_flag) { ok = 0; break; }
-        if (t0 == 0) t0 = clock64();
-        if ((unsigned long long)(clock64() - t0) > c.barrier_timeout_cycles) {
-          dev_fail(c, DEV_ERR_BARRIER_TIMEOUT);
-          ok = 0;
-          break;
-        }
-        if (polls > 4096u) __nanosleep(200);
-      }
-    }
-    if (*(volatile int*)&ss->abort_flag) ok = 0;
-    s_ok = ok;
-  }
+  if (threadIdx.x == 0) g_bar_ok = grid_arrive_and_wait(c) ? 1 : 0;
   __syncthreads();
   fence_proxy_async_global();
-  return s_ok != 0;
+  return g_bar_ok != 0;
 }
 
 // Exclusive prefix sums of N values over the 256 threads of the control CTA, all at once (two barriers; one scan after

@@ -299,7 +299,7 @@ __device__ __forceinline__ void dec_issue_mmas(const DevCtx& c, const DecPhase& 
   const int slots = min(g.u1 - g.u0, g.kblocks);
   if (g.u0 < g.u1) {
     if (p.made) {
-      if (!mbar_wait_warp_cluster(c, &g_dec.b_made, s.made & 1u)) return;
+      if (!mbar_wait_warp(c, &g_dec.b_made, s.made & 1u)) return;
     } else if (p.loaded) {
       if (!mbar_wait_warp(c, &g_dec.b_loaded, s.loaded & 1u)) return;
     }
@@ -422,6 +422,19 @@ __device__ __forceinline__ void dec_epi_made(const TcEpiOut& e, uint32_t taddr, 
   }
 }
 
+// The grid barrier after a GEMM of a decode-sized step.  Warp 0 may still be bringing weights of the next GEMM (it has
+// nothing in memory that the grid waits for): the others arrive without it.
+static __device__ __noinline__ bool dec_barrier(const DevCtx& c) {
+  if (threadIdx.x >= 32) {
+    fence_proxy_async_global();
+    asm volatile("bar.sync 3, %0;" ::"n"(FWD_THREADS - 32) : "memory");
+    if (threadIdx.x == 32) g_bar_ok = grid_arrive_and_wait(c) ? 1 : 0;
+  }
+  __syncthreads();
+  fence_proxy_async_global();
+  return g_bar_ok != 0;
+}
+
 // One GEMM of a decode-sized step.  `next_which` (or -1): the GEMM whose weights follow; `next_pre`: how many of its
 // stages may be filled before it starts.
 template <bool PAIR>
@@ -472,16 +485,17 @@ static __device__ __noinline__ void phase_gemm_dec(const DevCtx& c, int which, i
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // read by the MMAs next
     __syncthreads();
     if (threadIdx.x == 0 && g.u0 < g.u1) {
-      if constexpr (PAIR) mbar_arrive_cta0_cluster(&g_dec.b_made);
+      // (an arrival with release at cluster scope waits for every outstanding store: 1.1 us a phase; the proxy fence
+      // of the writers and the barrier above order their shared-memory writes before the MMAs of the pair)
+      if constexpr (PAIR) mbar_arrive_cta0(&g_dec.b_made);
       else mbar_arrive(&g_dec.b_made);
     }
   }
 
   if (warp == 0) {
     fill(which, layer, first, 0x4000000);
-    if (next_which >= 0 && *(volatile int*)&g_tc.dead == 0) {
+    if (next_which >= 0 && *(volatile int*)&g_tc.dead == 0)
       s.pre = fill(next_which, next_which == GEMM_QKV ? layer + 1 : layer, 0, next_pre);
-    }
   } else if (warp == 2) {
     if (!p.made) dec_load_tokens<PAIR>(c, p, g, tiles, s, rank);
   } else if (warp == 1) {
@@ -540,7 +554,7 @@ static __device__ __noinline__ void phase_gemm_dec(const DevCtx& c, int which, i
     g_tc_state[warp] = tc;
     g_dec_state[warp] = s;
   }
-  __syncthreads();
+  __syncwarp();   // (the grid barrier that follows brings the warps together)
 }
 
 // ---- host side: which steps may take this path --------------------------------------------------------------

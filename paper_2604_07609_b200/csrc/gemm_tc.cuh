@@ -268,29 +268,6 @@ __device__ __forceinline__ void mbar_arrive_cta0(uint64_t* bar) {
       "mbarrier.arrive.shared::cluster.b64 _, [ra];\n\t}" ::"r"(smem_u32(bar))
       : "memory");
 }
-// the same by threads whose shared-memory writes the other CTA's MMAs are going to read
-__device__ __forceinline__ void mbar_arrive_cta0_cluster(uint64_t* bar) {
-  asm volatile(
-      "{\n\t.reg .b32 ra;\n\t"
-      "mapa.shared::cluster.u32 ra, %0, 0;\n\t"
-      "mbarrier.arrive.release.cluster.shared::cluster.b64 _, [ra];\n\t}" ::"r"(smem_u32(bar))
-      : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ bool mbar_wait_warp_cluster(const DevCtx& c, uint64_t* bar, uint32_t parity) {
-  if (!mbar_wait_warp(c, bar, parity)) return false;
-  return __all_sync(0xffffffffu, mbar_try_wait_cluster(bar, parity));   // complete: only the acquire at cluster scope
-}
 // Tile copies of a pair: the bytes are counted on CTA 0's barrier (the CTA bit of the barrier's address is
 // cleared), whichever CTA of the pair issues the copy and receives the data.
 constexpr uint32_t PAIR_CTA0_MASK = 0xFEFFFFFFu;

@@ -96,10 +96,42 @@ static __device__ __noinline__ void step_begin(const DevCtx& c) {
   }
   __syncthreads();
 }
+// The GEMM whose weights the producer may fetch while the grid waits at the end of `phase` (-1: none), and how many stages
+// of them: the attention between QKV and O leaves half of the ring alone at most.
+__device__ __forceinline__ int dec_next_gemm(const DevCtx& c, const StepInfo& st, int phase, int layer, int& count) {
+  count = DEC_STAGES;
+  if (!st.dec) return -1;
+  if (phase == PH_QKV) { count = ATT_CTA_OFF / DEC_STAGE_BYTES; return st.att_cta ? GEMM_O : -1; }
+  if (c.E > 0) return -1;
+  if (phase == PH_O) return GEMM_GU;
+  if (phase == PH_GU) return GEMM_DOWN;
+  if (phase == PH_DOWN) return layer + 1 < c.L ? GEMM_QKV : st.R > 0 ? GEMM_LMHEAD : -1;
+  return -1;
+}
+
+// The GEMM phases of a decode-sized step; false when the phase is none of them.  `chain`: weights of the GEMM that
+// follows may be fetched ahead (not when every phase is a launch of its own).
+template <bool PAIR>
+__device__ __forceinline__ bool run_phase_dec(const DevCtx& c, const StepInfo& st, int phase, int layer, float* smem, bool chain) {
+  int which;
+  switch (phase) {
+    case PH_QKV: which = GEMM_QKV; break;
+    case PH_O: which = GEMM_O; break;
+    case PH_GU: if (c.E > 0) return false; which = GEMM_GU; break;
+    case PH_DOWN: if (c.E > 0) return false; which = GEMM_DOWN; break;
+    case PH_LMHEAD: which = GEMM_LMHEAD; break;
+    default: return false;
+  }
+  int count;
+  const int next = chain ? dec_next_gemm(c, st, phase, layer, count) : -1;
+  phase_gemm_dec<PAIR>(c, which, layer, st.T, st.R, next, count, smem);
+  return true;
+}
 // The grid barrier that closes a phase.  CTA 0 keeps a device time per phase kind (a phase's time includes this
 // barrier), recorded when per-iteration statistics are kept.
 __device__ __forceinline__ bool end_phase(const DevCtx& c, int ph) {
-  const bool ok = grid_barrier(c);
+  const bool gemm = ph == PH_QKV || ph == PH_O || ph == PH_GU || ph == PH_DOWN;
+  const bool ok = g_step.dec && gemm ? dec_barrier(c) : grid_barrier(c);
   if (c.stats_cap > 0 && blockIdx.x == 0 && threadIdx.x == 0) {
     const unsigned long long t = global_timer_ns();
     g_phase_ns[ph >= PH_SMAX ? (int)PH_SAMPLE : ph] += t - g_phase_t;   // the parts of sampling share a timer
@@ -107,28 +139,6 @@ __device__ __forceinline__ bool end_phase(const DevCtx& c, int ph) {
   }
   return ok;
 }
-// The GEMM phases of a decode-sized step; false when the phase is none of them.  `chain`: weights of the GEMM that
-// follows may be fetched ahead (not when every phase is a launch of its own).
-template <bool PAIR>
-__device__ __forceinline__ bool run_phase_dec(const DevCtx& c, const StepInfo& st, int phase, int layer, float* smem,
-                                              bool chain) {
-  int which, next = -1, pre = DEC_STAGES;
-  switch (phase) {
-    case PH_QKV: which = GEMM_QKV; next = GEMM_O; pre = st.att_cta ? ATT_CTA_OFF / DEC_STAGE_BYTES : 0; break;
-    case PH_O: which = GEMM_O; next = c.E == 0 ? GEMM_GU : -1; break;
-    case PH_GU: if (c.E > 0) return false; which = GEMM_GU; next = GEMM_DOWN; break;
-    case PH_DOWN:
-      if (c.E > 0) return false;
-      which = GEMM_DOWN;
-      next = layer + 1 < c.L ? GEMM_QKV : st.R > 0 ? GEMM_LMHEAD : -1;
-      break;
-    case PH_LMHEAD: which = GEMM_LMHEAD; break;
-    default: return false;
-  }
-  phase_gemm_dec<PAIR>(c, which, layer, st.T, st.R, chain ? next : -1, pre, smem);
-  return true;
-}
-
 template <typename WT, int HD, int NREP, bool PAIR>
 __device__ __forceinline__ void run_phase(const DevCtx& c, int phase, int layer, int sub, float* smem, bool chain) {
   const size_t esz = sizeof(WT);
