@@ -1,0 +1,104 @@
+"""The data path at the sizes where its kernels change over: decode steps around 16 and 128 rows, units of the decode
+attention that are cut or not, token passes, rows of logits around chunk and split limits."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_util import compare_with_oracle, gpu_run_forced
+from oracle import sampler as S
+from paper_2604_07609_b200 import binding as B
+from synth import make_weights
+from synth.configs import ModelCfg, SchedCfg
+from synth.workload import Request
+
+pytestmark = pytest.mark.gpu
+
+# four query heads per kv head: the shape that runs its GEMMs on CTA pairs
+MODELS = {1024: ModelCfg(2, 1024, 8, 2, 128, 1024, 4096), 2048: ModelCfg(1, 2048, 16, 4, 64, 768, 4096),
+          4096: ModelCfg(1, 4096, 8, 2, 128, 640, 1024)}
+
+
+def _requests(prompts, new, vocab, seed=11, **how):
+    rng = np.random.default_rng(seed)
+    return [Request(ticket=t, arrival_s=0.0, prompt=rng.integers(0, vocab, size=p, dtype=np.int64).astype(np.int32), max_new=new,
+                    seed=seed + t, user_tag=t, **how) for t, p in enumerate(prompts)]
+
+
+def _check(model, prompts, new, chunk, layout=B.WEIGHTS_ROW_MAJOR, relative=True):
+    """The bound of the large shapes: two correct evaluations that round at different places are N apart on these inputs.
+    Without `relative` the absolute bound of the small shapes alone."""
+    sched = SchedCfg(max_batch=len(prompts), prefill_chunk_tokens=chunk, n_slots=256, max_prompt=max(prompts), max_new=new,
+                     n_blocks=sum((p + new + 15) // 16 for p in prompts))
+    return compare_with_oracle(model, sched, _requests(prompts, new, model.vocab), make_weights(model, 5, "cpu", random_gains=True),
+                               2e-2, noise_relative=relative, oracle_dtype=np.float32, weights_layout=layout)
+
+
+@pytest.mark.parametrize("d", [1024, 2048, 4096])
+@pytest.mark.parametrize("rows", [1, 2, 3, 15, 16, 17])
+def test_small_decode_steps(rows, d):
+    r = _check(MODELS[d], [3 + (7 * i) % 30 for i in range(rows)], 4, 512,
+               B.WEIGHTS_STREAMING if d != 1024 else B.WEIGHTS_ROW_MAJOR)
+    assert any(int(n) == rows for n in r["its"]["n_decode"])
+
+
+@pytest.mark.parametrize("rows", [127, 128, 129])
+def test_decode_steps_around_128_rows(rows):
+    r = _check(MODELS[1024], [2 + i % 5 for i in range(rows)], 3, 512)
+    assert any(int(n) == rows for n in r["its"]["n_decode"])
+
+
+@pytest.mark.parametrize("prompts", [[15], [16], [383], [384, 1], [1500, 17, 800], [401] * 5], ids=str)
+def test_decode_attention_units_whole_and_cut(prompts):
+    _check(MODELS[2048], prompts, 3, 512, B.WEIGHTS_STREAMING)
+
+
+@pytest.mark.parametrize("tokens", [257, 300, 512, 513])
+def test_prefill_steps_of_several_token_passes(tokens):
+    # 6144 QKV rows: 24 pairs of weight tiles, which three token passes divide evenly over 74 pairs of CTAs
+    model = ModelCfg(1, 512, 32, 8, 128, 256, 1024)
+    # Every sampled row attends to hundreds of keys whose probabilities the prefill kernel rounds to bf16, a rounding
+    # point that neither oracle has: relative error 2^-9 / sqrt(3) per key on top of the others, which puts the rms 2 %
+    # above the distance between the oracles (1.70e-3 | 1.66e-3, max 6.6e-3).  d = 512 makes logits of sigma 0.45, for
+    # which the absolute bound of the small shapes, 2e-2, holds.
+    r = _check(model, [tokens], 2, 1024, B.WEIGHTS_STREAMING, relative=False)
+    assert r["err_plain"] <= 2e-2
+    assert int(r["its"]["n_tokens"][0]) == tokens
+
+
+@pytest.mark.parametrize("V", [2, 5, 1023, 4099, 32768, 32772, 65540, (1 << 20) + 4])
+def test_sampler_rows_around_chunk_limits(V):
+    rng = np.random.default_rng(V)
+    rows = 9
+    logits = (rng.normal(size=(rows, V)) * 1.3).astype(np.float32)
+    logits[3, V // 2:] = logits[3].max() + 1.0   # a plateau that ends with the row
+    logits[4] = 0.5
+    top_k = np.array([0, min(50, V), 0, 7, 0, 0, 1, 64, 0], dtype=np.int32)
+    top_p = np.array([0, 0, 0.9, 0.5, 0.7, 0.999, 0, 0.3, 0.05], dtype=np.float32)
+    temp, ticket = np.full(rows, 0.8, np.float32), np.arange(rows, dtype=np.uint64)
+    gen, seed = np.arange(rows, dtype=np.int32), np.full(rows, 99, np.uint64)
+    got = B.blink_sample_top_p(torch.from_numpy(logits).cuda(), top_k, temp, top_p, ticket, gen, seed)
+    for r in range(rows):
+        assert int(got[r]) == S.sample(logits[r], int(top_k[r]), 0.8, r, r, 99, float(top_p[r])), (V, r)
+
+
+@pytest.mark.parametrize("V", [32768, 36864, 40004])
+def test_sampling_inside_the_loop_equals_the_oracle_on_the_loops_own_logits(V):
+    """Rows of more than 32768 entries are prepared by all CTAs (maxima, nucleus weights): greedy, top-k, nucleus and both
+    together in one batch; the oracle's sampler on the captured rows gives the tokens, bit for bit."""
+    model = ModelCfg(1, 256, 4, 4, 64, 256, V, dtype="fp32")
+    sched = SchedCfg(max_batch=8, prefill_chunk_tokens=64, n_slots=16, max_prompt=16, max_new=6, n_blocks=32)
+    reqs = _requests([4, 5, 6, 7, 8, 9], 6, V)
+    how = [(0, 0.0), (50, 0.0), (0, 0.9), (0, 0.5), (40, 0.8), (0, 0.99)]
+    for r, (k, p) in zip(reqs, how):
+        r.top_k, r.top_p, r.temperature = k, p, 0.8
+    trace, toks, logits, _ = gpu_run_forced(model, sched, reqs, make_weights(model, 5, "cpu"), None)
+    slot_ticket, row, n = {}, 0, {t: 0 for t in range(len(reqs))}
+    for rec in trace:   # row r of the capture is the r-th sampled row since the start
+        slot_ticket.update({b: t for t, b in rec["admitted"]})
+        for b, tok in rec["sampled"]:
+            q = reqs[slot_ticket[b]]
+            want = S.sample(logits[row], q.top_k, q.temperature, q.ticket, n[q.ticket], q.seed, q.top_p)
+            assert tok == want == toks[q.ticket][n[q.ticket]], (q.ticket, n[q.ticket])
+            n[q.ticket] += 1
+            row += 1
+    assert row == 36
