@@ -813,11 +813,10 @@ static __device__ __noinline__ int silu_pending_units(const unsigned long long* 
 // copied itself), so four items are in flight per thread without holding registers for them: a body that
 // needs many registers here changes the register allocation of the other phase functions of the loop
 // kernel, to their cost.
-// Token rows per pass of a tensor-core GEMM over T rows: at most 256, a multiple of 16, the passes as even as they go.
-__device__ __forceinline__ int tc_pass_rows(int T) {
-  const unsigned passes = (unsigned)(T + 255) >> 8;
-  return (int)((((unsigned)T + passes - 1u) / passes + 15u) & ~15u);
-}
+// Token rows per pass of a tensor-core GEMM over T rows in `passes` passes of at most 256: a multiple of 16, the passes
+// as even as they go.
+__device__ __forceinline__ int tc_pass_rows(int T, int passes) { return (int)((((unsigned)T + (unsigned)passes - 1u) / (unsigned)passes + 15u) & ~15u); }
+__device__ __forceinline__ int tc_pass_rows(int T) { return tc_pass_rows(T, (int)((unsigned)(T + 255) >> 8)); }
 constexpr int SILU_STAGE_OFF = 32768 * 4;   // bytes: the staging area follows the list of pending units
 template <typename WT>
 __device__ __noinline__ void silu_mul_pending(float* __restrict__ gu, WT* __restrict__ out, int T, int F, const int* list, int count) {

@@ -83,7 +83,7 @@ __device__ __forceinline__ void dec_geometry(const DevCtx& c, int T, int R) {
     const int tiles = (N + 127) / 128;
     g_dec.g[which] = tc_geom(c, max(rows, 1), N, dec_k(c, which), which == GEMM_LMHEAD && lm_head_whole_tiles(c),
                              PAIR ? (int)gridDim.x / 2 : (int)gridDim.x, PAIR ? (int)blockIdx.x / 2 : (int)blockIdx.x,
-                             PAIR ? (tiles + 1) / 2 : tiles, PAIR);
+                             PAIR ? (tiles + 1) / 2 : tiles, PAIR, 1);
   }
 }
 

@@ -475,14 +475,31 @@ __device__ __forceinline__ int tc_share(int total, int nb, int b) {
   const unsigned q = (unsigned)total / (unsigned)nb, r = (unsigned)total - q * (unsigned)nb;
   return (int)(q * (unsigned)b + r * (unsigned)b / (unsigned)nb);
 }
-__device__ __forceinline__ TcGeom tc_geom(const DevCtx& c, int T, int N, int K, bool whole_tiles, int nb, int b, int ntiles, bool half_tokens) {
+// Token passes of a GEMM over T > 256 rows: as few as there can be, or one more where the workers of a pass then divide the
+// weight tiles evenly (no partial tiles to add up: the results are stored plainly) and the estimate is shorter.  In ns:
+// a k-block takes 40 + 1.65 per row, adding up a partial tile 20 per row, a third of that when it is stored.  QKV of the
+// 8B shape in 2 | 3 passes: 300 rows 23.8 | 21.3 us, 494 rows 27.1 | 25.6.  An extra pass elsewhere lost (1B shape,
+// 550 rows, 3 | 4: 13.8 | 16.1 us), and O and down add to the residual in any case.
+__device__ __forceinline__ int tc_passes(int T, int kblocks, int ntiles, int nb, bool accumulate) {
+  const int least = (int)((unsigned)(T + 255) >> 8), more = least + 1;
+  if (least < 2 || more > nb || accumulate) return least;
+  const int rows = tc_pass_rows(T, least), rows1 = tc_pass_rows(T, more);
+  const int groups = (int)((unsigned)nb / (unsigned)least), groups1 = (int)((unsigned)nb / (unsigned)more);
+  if (least * rows1 >= T) return least;   // the last pass would be empty
+  if ((unsigned)ntiles % (unsigned)groups1 != 0u || (unsigned)ntiles % (unsigned)groups == 0u) return least;
+  const int units = ntiles * kblocks;
+  return (int)((unsigned)units / (unsigned)groups1) * (40 + rows1 * 33 / 20) + 6 * rows1 <
+                 (int)((unsigned)units / (unsigned)groups) * (40 + rows * 33 / 20) + 20 * rows ? more : least;
+}
+__device__ __forceinline__ TcGeom tc_geom(const DevCtx& c, int T, int N, int K, bool whole_tiles, int nb, int b, int ntiles, bool half_tokens,
+                                          int passes) {
   TcGeom g;
   g.kblocks = (int)((unsigned)K >> 6);
   g.ntiles = ntiles;   // weight tiles of 128 rows, or pairs of them
-  g.passes = (int)((unsigned)(T + 255) >> 8);
+  g.passes = passes;
   // even passes: the workers of a weight tile's passes take equal shares, so the longest pass sets the time
   // (520 rows as 3 x 176 instead of 256 + 256 + 8: gate/up of the 8B shape 123 -> 98 us)
-  g.pass_rows = tc_pass_rows(T);
+  g.pass_rows = tc_pass_rows(T, passes);
   // A stage holds one k-block, or two when the token tile is small and the weights are stored as
   // contiguous tiles (then one bulk copy brings 32 KiB): fewer, larger copies per producer step.
   g.KPS = (c.w_streaming && g.pass_rows <= 128) ? 2 : 1;
@@ -781,10 +798,11 @@ static __device__ __noinline__ void phase_gemm_tc(const DevCtx& c, const GemmArg
   const uint32_t rank = PAIR ? cluster_ctarank() : 0u;
   const int n_tiles128 = (N + 127) / 128;
   // workers are CTAs, or CTA pairs that take two weight tiles at a time
-  const TcGeom g = PAIR ? tc_geom(c, T, N, K, which == GEMM_LMHEAD && lm_head_whole_tiles(c), (int)gridDim.x / 2,
-                                  (int)blockIdx.x / 2, (n_tiles128 + 1) / 2, true)
-                        : tc_geom(c, T, N, K, which == GEMM_LMHEAD && lm_head_whole_tiles(c), (int)gridDim.x, (int)blockIdx.x,
-                                  n_tiles128, false);
+  const int nb = PAIR ? (int)gridDim.x / 2 : (int)gridDim.x, ntiles = PAIR ? (n_tiles128 + 1) / 2 : n_tiles128;
+  // the SwiGLU phase knows the gate/up GEMM's units by the fewest passes
+  const int passes = which == GEMM_GU ? (int)((unsigned)(T + 255) >> 8) : tc_passes(T, (int)((unsigned)K >> 6), ntiles, nb, a.accumulate != 0);
+  const TcGeom g = tc_geom(c, T, N, K, which == GEMM_LMHEAD && lm_head_whole_tiles(c), nb, PAIR ? (int)blockIdx.x / 2 : (int)blockIdx.x,
+                           ntiles, PAIR, passes);
   const int kblocks = g.kblocks;
   const int act_id = which == GEMM_O ? ACT_ATTN : which == GEMM_DOWN ? ACT_ACT : which == GEMM_LMHEAD ? ACT_XS
                      : (which == GEMM_GU && c.E > 0) ? ACT_XG : ACT_XN;
