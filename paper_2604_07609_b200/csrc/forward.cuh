@@ -36,6 +36,28 @@ __device__ __forceinline__ float warp_max(float v) {
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
+// Sums of NV values over the 32 lanes by halving exchange: lane l ends with the sum of value (l * NV) / 32.
+template <int NV>
+__device__ __forceinline__ float warp_sum_many(float (&v)[NV]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int n = NV, o = 16; o > 0; o >>= 1) {
+    if (n > 1) {
+      n >>= 1;
+      const bool up = (lane & o) != 0;
+#pragma unroll
+      for (int i = 0; i < NV / 2; ++i) {
+        if (i < n) {
+          const float send = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
+          v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+      }
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    }
+  }
+  return v[0];
+}
 __device__ __forceinline__ float block_sum(float v, float* s_red /*[8]*/) {
   v = warp_sum(v);
   __syncthreads();
@@ -134,45 +156,57 @@ __device__ __forceinline__ void norm_row_cta(const DevCtx& c, float* hrow, const
   if (wr != nullptr) {
     // Router of the routed-expert FFN on the normed row in fp32 (not its 16-bit copy): logits over
     // the E experts, top-k by (logit desc, expert id asc), weights = softmax restricted to the chosen.
+    // Eight experts at a time, their weights for a vector of the row on the way together (expert by expert, each with a
+    // reduction of its own, a row took 10 us).
     __shared__ float s_rl[FWD_THREADS / 32][MAX_EXPERTS];
     const int E = c.E;
-    for (int e = 0; e < E; ++e) {
-      float p = 0.f;
+    for (int e0 = 0; e0 < E; e0 += 8) {
+      float p[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) p[j] = 0.f;
 #pragma unroll
       for (int k = 0; k < NORM_MAXV; ++k) {
         const int i = (k * FWD_THREADS + threadIdx.x) * 4;
         if (i < d) {
-          const float4 w4 = *reinterpret_cast<const float4*>(wr + (size_t)e * d + i);
-          p = fmaf(v[k].x, w4.x, p); p = fmaf(v[k].y, w4.y, p); p = fmaf(v[k].z, w4.z, p); p = fmaf(v[k].w, w4.w, p);
+          float4 w4[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) w4[j] = *reinterpret_cast<const float4*>(wr + (size_t)min(e0 + j, E - 1) * d + i);   // past the end: the last again
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            p[j] = fmaf(v[k].x, w4[j].x, p[j]); p[j] = fmaf(v[k].y, w4[j].y, p[j]); p[j] = fmaf(v[k].z, w4[j].z, p[j]); p[j] = fmaf(v[k].w, w4[j].w, p[j]);
+          }
         }
       }
-      p = warp_sum(p);
-      if ((threadIdx.x & 31) == 0) s_rl[threadIdx.x >> 5][e] = p;
+      const float t = warp_sum_many<8>(p);   // lanes 4 j .. 4 j + 3 hold expert e0 + j
+      const int e = e0 + ((threadIdx.x & 31) >> 2);
+      if ((threadIdx.x & 3) == 0 && e < E) s_rl[threadIdx.x >> 5][e] = t;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      float lg[MAX_EXPERTS];
-      for (int e = 0; e < E; ++e) {
-        float t = 0.f;
-        for (int w = 0; w < FWD_THREADS / 32; ++w) t += s_rl[w][e];
-        lg[e] = t;
-      }
-      int sel[MAX_EXPERTS];
-      float den = 0.f, top = 0.f;
+    if (threadIdx.x < 32) {   // a lane per expert
+      const int lane = threadIdx.x;
+      float lg = 0.f;
+      if (lane < E)
+        for (int w = 0; w < FWD_THREADS / 32; ++w) lg += s_rl[w][lane];
+      bool open = lane < E;   // not chosen yet
+      float den = 0.f, top = 0.f, mine = 0.f;
+      int place = -1;
       for (int j = 0; j < c.topE; ++j) {
-        int best = -1;
-        for (int e = 0; e < E; ++e) {
-          bool taken = false;
-          for (int q = 0; q < j; ++q) taken |= sel[q] == e;
-          if (!taken && (best < 0 || lg[e] > lg[best])) best = e;   // ties keep the lower id
+        float bv = open ? lg : -INFINITY;
+        int bi = open ? lane : 32;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
+          const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+          if (oi < 32 && (bi == 32 || ov > bv || (ov == bv && oi < bi))) { bv = ov; bi = oi; }   // ties keep the lower id
         }
-        sel[j] = best;
-        if (j == 0) top = lg[best];
-        den += expf(lg[best] - top);
+        if (j == 0) top = bv;
+        const float ex = expf(bv - top);
+        den += ex;
+        if (lane == bi) { open = false; place = j; mine = ex; }
       }
-      for (int j = 0; j < c.topE; ++j) {
-        c.moe_sel[(size_t)row_index * c.topE + j] = sel[j];
-        c.moe_wt[(size_t)row_index * c.topE + j] = expf(lg[sel[j]] - top) / den;
+      if (place >= 0) {
+        c.moe_sel[(size_t)row_index * c.topE + place] = lane;
+        c.moe_wt[(size_t)row_index * c.topE + place] = mine / den;
       }
     }
     __syncthreads();
@@ -340,28 +374,6 @@ struct GemmArgs {
   float* fix_rowss = nullptr;// FIX_SUMSQ: per-row sums of squares to add to
 };
 
-// Sums of NV values over the 32 lanes by halving exchange: lane l ends with the sum of value (l * NV) / 32.
-template <int NV>
-__device__ __forceinline__ float warp_sum_many(float (&v)[NV]) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int n = NV, o = 16; o > 0; o >>= 1) {
-    if (n > 1) {
-      n >>= 1;
-      const bool up = (lane & o) != 0;
-#pragma unroll
-      for (int i = 0; i < NV / 2; ++i) {
-        if (i < n) {
-          const float send = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
-          v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-        }
-      }
-    } else {
-      v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
-    }
-  }
-  return v[0];
-}
 // One warp: GR token rows x NC output features, the 32 lanes side by side along K (four elements each), so that all
 // loads of 256 elements of K are in flight at once.  The reference shapes are small (a few dozen rows, K of 256 to
 // 1024): with 64 x 64 tiles and 16 elements of K per step only 4 to 64 CTAs had work and every step waited for
@@ -894,11 +906,19 @@ static __device__ __noinline__ void phase_moe_group(const DevCtx& c, float* smem
   const int A = T * K;   // assignments
   __shared__ int s_off[MAX_EXPERTS + 1];
   int* s_tok = reinterpret_cast<int*>(smem);          // [A] token of each gathered row
+  // the choices as bytes behind it, where they fit: every warp walks all of them for each of its experts, and a walk
+  // over memory waits for every 32 (25 us for 960 choices)
+  unsigned char* s_sel = reinterpret_cast<unsigned char*>(s_tok + A);
+  const bool staged = c.gemm_tc && A <= 32768;        // (the GEMM rings are larger than 5 x 32768 bytes)
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   // counts, then offsets
   if (threadIdx.x <= E) s_off[threadIdx.x] = 0;
   __syncthreads();
-  for (int a = threadIdx.x; a < A; a += FWD_THREADS) atomicAdd(&s_off[c.moe_sel[a] + 1], 1);
+  for (int a = threadIdx.x; a < A; a += FWD_THREADS) {
+    const int e = c.moe_sel[a];
+    if (staged) s_sel[a] = (unsigned char)e;
+    atomicAdd(&s_off[e + 1], 1);
+  }
   __syncthreads();
   if (threadIdx.x == 0)
     for (int e = 0; e < E; ++e) s_off[e + 1] += s_off[e];
@@ -908,7 +928,7 @@ static __device__ __noinline__ void phase_moe_group(const DevCtx& c, float* smem
     int base = s_off[e];
     for (int a0 = 0; a0 < A; a0 += 32) {
       const int a = a0 + lane;
-      const bool mine = a < A && c.moe_sel[a] == e;
+      const bool mine = a < A && (staged ? (int)s_sel[a] : c.moe_sel[a]) == e;
       const unsigned m = __ballot_sync(0xffffffffu, mine);
       if (mine) {
         const int pos = base + __popc(m & ((1u << lane) - 1u));
@@ -927,7 +947,14 @@ static __device__ __noinline__ void phase_moe_group(const DevCtx& c, float* smem
   for (int r = blockIdx.x * (FWD_THREADS / 32) + w; r < A; r += gridDim.x * (FWD_THREADS / 32)) {
     const uint4* src = reinterpret_cast<const uint4*>(xn + (size_t)s_tok[r] * c.d);
     uint4* dst = reinterpret_cast<uint4*>(xg + (size_t)r * c.d);
-    for (int i = lane; i < vec_per_row; i += 32) dst[i] = src[i];
+    for (int i0 = 0; i0 < vec_per_row; i0 += 256) {   // eight vectors per lane on their way at a time
+      uint4 v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[k] = src[min(i0 + 32 * k + lane, vec_per_row - 1)];
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (i0 + 32 * k + lane < vec_per_row) dst[i0 + 32 * k + lane] = v[k];
+    }
   }
 }
 
