@@ -9,6 +9,7 @@
 #include <string.h>
 #include <time.h>
 
+#include <algorithm>
 #include <atomic>
 #include <chrono>
 #include <cmath>
@@ -123,11 +124,12 @@ uint64_t now_ns() {
   return (uint64_t)ts.tv_sec * 1000000000ull + (uint64_t)ts.tv_nsec;
 }
 
-// Pause of a host wait that began at `t0`: the first half millisecond spins (the token or the exit is usually that near, and
-// a sleep of 20 us takes 70 to 100 with the kernel's timer slack: with sleeps alone a pass of one short request of the
-// smallest shape spent 150 of its 1130 us in them), then sleeps of `us`.
-void wait_pause(uint64_t t0, int us) {
-  if (now_ns() - t0 < 500000ull) {
+// Pause of a host wait: spin where what is waited for is near, else sleep `us`.  A sleep of 20 us takes 70 to 100 with the
+// kernel's timer slack: with sleeps alone a pass of one short request of the smallest shape spent 150 of its 1130 us in
+// them.  A thread that always spins is a hog on a busy host and is held back there (submissions 4 ms late instead of
+// 0.3), so it does so only while tokens come every few hundred microseconds.
+void wait_pause(bool spin, int us) {
+  if (spin) {
 #if defined(__x86_64__)
     for (int i = 0; i < 16; ++i) __builtin_ia32_pause();   // about a microsecond: other callers get the lock
 #else
@@ -203,6 +205,7 @@ struct blink_ctx {
   int hint = 0;
   uint64_t next_ticket = 0;
   std::atomic<int64_t> launches{0};
+  uint64_t event_last_ns = 0, event_gap_ns = 1000000;   // running mean of the time between tokens seen by blink_poll, at most 1 ms
   int64_t bytes_to_device = 0, bytes_from_device = 0;
   int64_t clock_offset = 0;
   bool final_stop = false;
@@ -948,9 +951,10 @@ int blink_submit(blink_ctx* x, const blink_request* r, uint64_t* ticket_out) {
 int blink_poll(blink_ctx* x, blink_token_event* out, int max_events, int timeout_us) {
   if (!x || !out || max_events < 1) return BLINK_EINVAL;
   const DevCtx& c = x->dc;
-  const uint64_t t0 = now_ns(), deadline = t0 + (uint64_t)(timeout_us > 0 ? timeout_us : 0) * 1000ull;
+  const uint64_t deadline = now_ns() + (uint64_t)(timeout_us > 0 ? timeout_us : 0) * 1000ull;
   while (true) {
     int n = 0;
+    bool spin;
     {
       std::lock_guard<std::mutex> g(x->mu);
       const int prc = pump(x);
@@ -989,9 +993,14 @@ int blink_poll(blink_ctx* x, blink_token_event* out, int max_events, int timeout
           ++it;
         }
       }
+      if (n > 0) {
+        x->event_gap_ns = (x->event_gap_ns + std::min<uint64_t>(t_now - x->event_last_ns, 1000000ull)) / 2;
+        x->event_last_ns = t_now;
+      }
+      spin = x->event_gap_ns < 300000ull && t_now - x->event_last_ns < 500000ull;
     }
     if (n > 0 || now_ns() >= deadline) return n;
-    wait_pause(t0, 20);
+    wait_pause(spin, 20);
   }
 }
 
@@ -1057,7 +1066,7 @@ int blink_stop(blink_ctx* x, int final, int timeout_ms) {
     if (q == cudaSuccess) break;
     if (q != cudaErrorNotReady) return BLINK_ECUDA;
     if (now_ns() >= deadline) return BLINK_ETIMEDOUT;
-    wait_pause(t0, 50);
+    wait_pause(now_ns() - t0 < 500000ull, 50);
   }
   return BLINK_OK;
 }
