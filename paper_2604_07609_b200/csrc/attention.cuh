@@ -209,7 +209,6 @@ __device__ __forceinline__ void att_tile_math(uint32_t kt, uint32_t vt, int n_va
 template <int HD, int NREP>
 __device__ __noinline__ void attn_decode_stream(const DevCtx& c, int layer, char* ring) {
   constexpr int RB = HD * 2;         // bytes per key row
-  constexpr int NBOX = HD / 64;      // 64-column boxes per tile row (128-byte swizzle span)
   constexpr int TILE = 16 * RB;      // bytes of one K (or V) tile of a (block, kv head)
   constexpr int STAGE = 2 * TILE;
   constexpr int KS = HD / 16;        // k-steps of Q K^T
@@ -281,7 +280,7 @@ __device__ __noinline__ void attn_decode_stream(const DevCtx& c, int layer, char
       const int blk = __shfl_sync(FULL, p_blk, pc.kb & 31);
       if (lane == 0) {
         const int s = n_issued % ATT_NS;
-        // one copy brings the K tile and the V tile: box {64 dims, NBOX halves, 16 keys, K and V, this layer}
+        // one copy brings the K tile and the V tile: box {64 dims, HD / 64 halves, 16 keys, K and V, this layer}
         mbar_expect_tx(&bars[s], STAGE);
         tma_load_5d(ring + s * STAGE, kv_map, 0, 0, (blk * Hkv + pc.g) * 16, 0, layer, &bars[s], kv_policy);
       }

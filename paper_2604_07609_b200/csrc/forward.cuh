@@ -256,7 +256,7 @@ static __device__ __noinline__ void norm_rows_halves(const float* __restrict__ h
 // ---- RMSNorm of the residual rows into the operand buffer; layer 0 gathers the
 // embedding first.
 template <typename WT>
-static __device__ __noinline__ void phase_norm(const DevCtx& c, int layer, int which /*0: norm1, 1: norm2*/, float* smem) {
+static __device__ __noinline__ void phase_norm(const DevCtx& c, int layer, int which /*0: norm1, 1: norm2*/) {
   __shared__ float s_red[FWD_THREADS / 32];
   const int T = c.ss->cur_T;
   const float* g = wptr_f(c, which == 0 ? 6 : 7) + (size_t)layer * c.d;

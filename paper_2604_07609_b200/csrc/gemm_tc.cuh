@@ -17,8 +17,8 @@
 // token rows the passes of a weight tile go to neighbouring CTAs that walk the same range at the
 // same time (the tile comes from HBM once, from L2 for the other passes).
 //
-// Warp roles in the 256-thread CTA: warp 0 = weight producer (one lane), warp 2 = token-tile
-// producer (one lane), warp 1 = MMA issuer (one lane), warps 4..7 = epilogue (TMEM -> registers
+// Warp roles in the 256-thread CTA: warp 0 = weight producer, warp 2 = token-tile producer, warp 1 = MMA issuer (each a
+// whole warp that elects a lane for the issuing instruction), warps 4..7 = epilogue (TMEM -> registers
 // -> global), two accumulator buffers of 256 TMEM columns so the epilogue of one segment
 // overlaps the MMAs of the next; warps 0..3 store half of the CTA's last accumulator.
 // Every wait is bounded: on a time-out the CTA records DEV_ERR_PIPE_TIMEOUT, raises the
@@ -171,13 +171,6 @@ __device__ __forceinline__ void tma_load_3d_hint(void* smem_dst, const CUtensorM
       "l"(map), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar)), "l"(policy)
       : "memory");
 }
-// the same tiles into L2 only
-__device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int x, int y, int z) {
-  asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global [%0, {%1, %2, %3}];" ::"l"(map), "r"(x), "r"(y), "r"(z) : "memory");
-}
-__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int x, int y) {
-  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global [%0, {%1, %2}];" ::"l"(map), "r"(x), "r"(y) : "memory");
-}
 __device__ __forceinline__ void tma_bulk_load_hint(void* smem_dst, const void* src, uint32_t bytes, uint64_t* bar,
                                                    uint64_t policy) {
   asm volatile(
@@ -187,12 +180,6 @@ __device__ __forceinline__ void tma_bulk_load_hint(void* smem_dst, const void* s
       : "memory");
 }
 
-__device__ __forceinline__ void tma_bulk_load(void* smem_dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_u32(smem_dst)),
-               "l"(src), "r"(bytes), "r"(smem_u32(bar))
-               : "memory");
-}
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
