@@ -10,6 +10,7 @@
 #pragma once
 #include "../../include/blink.h"
 #include "dev_ctx.cuh"
+#include "mailbox.h"
 
 namespace blink {
 
@@ -39,6 +40,17 @@ __device__ __forceinline__ uint32_t ld_relaxed_sys_u32(const volatile uint32_t* 
   asm volatile("ld.relaxed.sys.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
+__device__ __forceinline__ uint32_t ld_acquire_sys_u32(const volatile uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.acquire.sys.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+struct MailboxWords {   // see read_mailbox
+  const Mailbox* m;
+  __device__ __forceinline__ uint32_t stop_relaxed() const { return ld_relaxed_sys_u32(&m->stop); }
+  __device__ __forceinline__ uint32_t start_acquire() const { return ld_acquire_sys_u32(&m->start); }
+  __device__ __forceinline__ uint64_t sub_tail_acquire() const { return ld_acquire_sys_u64(&m->sub_tail); }
+};
 __device__ __forceinline__ uint64_t global_timer_ns() {
   uint64_t t;
   asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
@@ -734,18 +746,14 @@ static __device__ __noinline__ void control_phase(const DevCtx& c, long long& la
   while (true) {
     if (tid == 0) {
       int cmd = CMD_NONE;
-      // both words are in host memory: one round trip for the two
-      const uint32_t stop = ld_relaxed_sys_u32(&c.mbox->stop);
-      const unsigned long long sub_tail = ld_acquire_sys_u64(&c.mbox->sub_tail);
-      if (stop) { cmd = CMD_EXIT; ss->exit_reason = 2; }
+      MailboxWords words{c.mbox};
+      const MailboxView mail = read_mailbox(words, c.start_paused && launch_iters == 0);   // (a launch that has run a step has seen the start)
+      if (mail.stop) { cmd = CMD_EXIT; ss->exit_reason = 2; }
       else if (*(volatile int*)&ss->abort_flag) { cmd = CMD_EXIT; ss->exit_reason = 5; }
       else if (c.iteration_budget > 0 && launch_iters >= c.iteration_budget) { cmd = CMD_EXIT; ss->exit_reason = 3; }
-      unsigned long long tail = ss->seen;
-      const int started = !c.start_paused || ld_relaxed_sys_u32(&c.mbox->start);
-      if (cmd == CMD_NONE && started) tail = sub_tail;
       s_cmd = cmd;
-      s_tail = tail;
-      s_started = started;
+      s_tail = cmd == CMD_NONE && mail.started ? mail.tail : ss->seen;
+      s_started = mail.started;
     }
     __syncthreads();
     if (s_cmd == CMD_EXIT) break;
