@@ -131,6 +131,28 @@ __device__ __forceinline__ void sample_chunk_maxima(const float* lg, int V, int 
 // longer than a warp's span.
 __host__ __device__ __forceinline__ bool sample_split_rows(int V) { return V > 32768 && V <= SAMPLE_WARP_SPAN * SAMPLE_CHUNKS; }
 
+// The lowest index whose value under `z` (monotone) is `top`, the largest of the row; the whole CTA, all threads get the
+// answer.  NaN is never the largest, so a row of NaN alone has none: token 0.
+template <typename F>
+__device__ __forceinline__ int sample_first_max(const float* lg, int V, int cl, const float* s_cmax, float top, F z) {
+  constexpr int NONE = 0x7fffffff;
+  __shared__ int s_chunk, s_pick;
+  __syncthreads();
+  if (threadIdx.x == 0) { s_chunk = NONE; s_pick = NONE; }
+  __syncthreads();
+  int i0 = 0, i1 = V;
+  if (top > -INFINITY) {   // (else the maximum of a chunk of NaN looks like a member)
+    for (int i = threadIdx.x; i < (V + cl - 1) / cl; i += FWD_THREADS)
+      if (z(s_cmax[i]) == top) { atomicMin(&s_chunk, i); break; }
+    __syncthreads();
+    if (s_chunk != NONE) { i0 = s_chunk * cl; i1 = min(V, i0 + cl); }
+  }
+  for (int i = i0 + threadIdx.x; i < i1; i += FWD_THREADS)
+    if (z(lg[i]) == top) { atomicMin(&s_pick, i); break; }
+  __syncthreads();
+  return s_pick == NONE ? 0 : s_pick;
+}
+
 // all CTAs: chunk maxima of every sampled row; nucleus weights start at zero
 static __device__ __noinline__ void phase_sample_max(const DevCtx& c) {
   const int R = c.ss->cur_rows, V = c.V;
@@ -539,7 +561,7 @@ static __device__ int sample_row(const float* lg, int V, int top_k, float temp, 
   float* s_cmax = smem + 256 + 4 * CAND_MAX;                         // [SAMPLE_CHUNKS]
   __shared__ float s_red[FWD_THREADS / 32];
   __shared__ unsigned long long s_prefix, s_mask;
-  __shared__ int s_remaining, s_ncand, s_chunk, s_pick, s_nlist;
+  __shared__ int s_remaining, s_ncand, s_nlist;
   __shared__ float s_tz[MAX_TOPK];
   __shared__ int s_ti[MAX_TOPK];
   __shared__ double s_tw[MAX_TOPK];
@@ -560,7 +582,7 @@ static __device__ int sample_row(const float* lg, int V, int top_k, float temp, 
       if ((tid & 31) == 0) s_cmax[ch] = m;
     }
   }
-  if (tid == 0) { s_ncand = 0; s_chunk = 0x7fffffff; s_pick = 0x7fffffff; }
+  if (tid == 0) s_ncand = 0;
   __syncthreads();
   // maximum over the chunks of this thread (tid, tid + 256, ...)
   float lmax = -INFINITY;
@@ -568,16 +590,8 @@ static __device__ int sample_row(const float* lg, int V, int top_k, float temp, 
   if (top_k <= 0) {
     const float gmax = block_max(lmax, s_red);
     if (nucleus) return sample_row_nucleus(lg, V, cl, s_cmax, gmax, temp, top_p, ticket, gen_index, seed, smem, nm, nc_);
-    for (int i = tid; i < nch; i += FWD_THREADS)
-      if (s_cmax[i] == gmax) { atomicMin(&s_chunk, i); break; }
-    __syncthreads();
-    const int i1 = s_chunk == 0x7fffffff ? 0 : min(V, (s_chunk + 1) * cl);
-    for (int i = s_chunk * cl + tid; i < i1; i += FWD_THREADS)
-      if (lg[i] == gmax) { atomicMin(&s_pick, i); break; }
-    __syncthreads();
-    if (tid == 0) result = s_pick == 0x7fffffff ? 0 : s_pick;
-    __syncthreads();
-    return result;
+    const int pick = sample_first_max(lg, V, cl, s_cmax, gmax, [](float v) { return v; });
+    return tid == 0 ? pick : -1;
   }
   const int k = min(top_k, V);
   // Fast path.  The k-th largest of the 256 per-thread maxima, tau, is a lower bound of the k-th largest z of the row

@@ -102,3 +102,29 @@ def test_sampling_inside_the_loop_equals_the_oracle_on_the_loops_own_logits(V):
             n[q.ticket] += 1
             row += 1
     assert row == 36
+
+
+def _sample(logits, top_k, top_p, temp=0.8):
+    """The sampler on rows that lie inside a larger buffer of -inf."""
+    rows, V = logits.shape
+    buf = torch.full((1024 + rows * V + 1024,), float("-inf"), device="cuda")
+    buf[1024:1024 + rows * V] = torch.from_numpy(logits).cuda().reshape(-1)
+    x = buf[1024:1024 + rows * V].view(rows, V)
+    return [int(t) for t in B.blink_sample_top_p(x, np.full(rows, top_k, np.int32), np.full(rows, temp, np.float32),
+                                                 np.full(rows, top_p, np.float32), np.arange(rows, dtype=np.uint64),
+                                                 np.zeros(rows, np.int32), np.full(rows, 3, np.uint64))]
+
+
+@pytest.mark.parametrize("V", [5, 4096, 40004, 140000])
+def test_greedy_rows_with_nan_and_infinities(V):
+    rng = np.random.default_rng(V)
+    x = rng.normal(size=(6, V)).astype(np.float32)
+    x[0] = np.nan                      # nothing to choose from: token 0
+    x[1] = -np.inf
+    x[2, 1:] = np.nan                  # one number
+    x[3, V // 2] = x[3, V - 1] = np.inf
+    x[4, ::2] = np.nan                 # NaN is never the largest
+    x[5] = np.nan
+    x[5, V - 1] = -np.inf              # -inf is larger than no number at all
+    want = [0, 0, 0, V // 2, int(np.nanargmax(x[4])), V - 1]
+    assert _sample(x, 0, 0.0) == want
