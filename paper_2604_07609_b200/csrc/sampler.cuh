@@ -504,6 +504,7 @@ static __device__ __noinline__ int sample_row_nucleus(const float* lg, int V, in
                                                       const unsigned int* nc) {
   __shared__ NucShared st;
   __shared__ unsigned long long s_t;
+  __shared__ bool s_none;
   const int tid = threadIdx.x;
   float* s_cz = smem + 256;
   int* s_ci = reinterpret_cast<int*>(smem + 256 + SAMPLE_CAND);
@@ -530,9 +531,16 @@ static __device__ __noinline__ int sample_row_nucleus(const float* lg, int V, in
     for (int k = 0; k < 8; ++k) Q += st.m0[tid * 8 + k];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) Q += __shfl_xor_sync(0xffffffffu, Q, o);
-    if (tid == 0) s_t = nucleus_need(nucleus_p24(top_p), Q) - 1ull;   // first entry with cum >= need  <=>  cum > need - 1
+    if (tid == 0) {
+      s_none = Q == 0ull;
+      s_t = nucleus_need(nucleus_p24(top_p), Q) - 1ull;   // first entry with cum >= need  <=>  cum > need - 1
+    }
   }
   __syncthreads();
+  if (s_none) {   // the largest z is infinite or there is no number in the row: no distance to it has a weight
+    const int pick = sample_first_max(lg, V, cl, s_cmax, z0, [&](float v) { return __fdiv_rn(v, temp); });
+    return tid == 0 ? pick : -1;
+  }
   nucleus_locate(st, lg, V, cl, s_cmax, temp, z0, s_t, s_cz, s_ci, s_sz, s_si);   // end of the nucleus: its weight is res_cum
   if (tid == 0) {
     const uint32_t x = philox4x32_10_word0((uint32_t)ticket, (uint32_t)(ticket >> 32), (uint32_t)gen_index, 0u,

@@ -128,3 +128,21 @@ def test_greedy_rows_with_nan_and_infinities(V):
     x[5, V - 1] = -np.inf              # -inf is larger than no number at all
     want = [0, 0, 0, V // 2, int(np.nanargmax(x[4])), V - 1]
     assert _sample(x, 0, 0.0) == want
+
+
+@pytest.mark.parametrize("V", [5, 4096, 40004, 140000])
+def test_nucleus_rows_without_a_finite_largest_value(V):
+    """exp(z - z0) has no value there: the first of the largest is the nucleus, token 0 when there is no number."""
+    rng = np.random.default_rng(V)
+    x = rng.normal(size=(5, V)).astype(np.float32)
+    x[0] = np.nan
+    x[1] = -np.inf
+    x[2, V - 2] = np.inf
+    x[3, V // 2] = x[3, V // 2 + 1] = np.inf
+    x[4] = np.nan
+    x[4, V - 1] = -np.inf
+    assert _sample(x, 0, 0.9) == [0, 0, V - 2, V // 2, V - 1]
+    y = np.abs(rng.normal(size=(1, V))).astype(np.float32) + 1   # a temperature so small that every z overflows
+    assert _sample(y, 0, 0.9, temp=1e-39) == [0]
+    y[0, 0] = -1
+    assert _sample(y, 0, 0.9, temp=1e-39) == [1]
