@@ -695,10 +695,11 @@ static __device__ int sample_row(const float* lg, int V, int top_k, float temp, 
   for (int a = tid; a < nc; a += FWD_THREADS) {
     const float za = s_cz[a];
     const int ia = s_ci[a];
+    const uint32_t ka = float_key(za + 0.f);   // keys, so that NaN has a place too: every rank below nc is taken once
     int rank = 0;
     for (int j = 0; j < nc; ++j) {
-      const float zj = s_cz[j];
-      rank += (zj > za) || (zj == za && s_ci[j] < ia);
+      const uint32_t kj = float_key(s_cz[j] + 0.f);   // (-0 counts as 0)
+      rank += (kj > ka) || (kj == ka && s_ci[j] < ia);
     }
     if (rank < k) { s_tz[rank] = za; s_ti[rank] = ia; }
   }

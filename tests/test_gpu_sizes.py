@@ -146,3 +146,14 @@ def test_nucleus_rows_without_a_finite_largest_value(V):
     assert _sample(y, 0, 0.9, temp=1e-39) == [0]
     y[0, 0] = -1
     assert _sample(y, 0, 0.9, temp=1e-39) == [1]
+
+
+@pytest.mark.parametrize("top_p", [0.0, 0.9])
+@pytest.mark.parametrize("V", [5, 4096, 40004])
+def test_top_k_rows_with_nan_answer_the_same_member_of_the_row_each_time(V, top_p):
+    x = np.full((3, V), np.nan, np.float32)
+    x[1, 1:3] = [0.5, -0.5]
+    x[2, : V // 2] = 0.25
+    first = _sample(x, min(50, V), top_p)
+    assert all(0 <= t < V for t in first)
+    assert all(_sample(x, min(50, V), top_p) == first for _ in range(3))
