@@ -299,7 +299,7 @@ __device__ __forceinline__ void dec_issue_mmas(const DevCtx& c, const DecPhase& 
   const int slots = min(g.u1 - g.u0, g.kblocks);
   if (g.u0 < g.u1) {
     if (p.made) {
-      if (!mbar_wait_warp(c, &g_dec.b_made, s.made & 1u)) return;
+      if (!(PAIR ? mbar_wait_warp_acquire(c, &g_dec.b_made, s.made & 1u) : mbar_wait_warp(c, &g_dec.b_made, s.made & 1u))) return;
     } else if (p.loaded) {
       if (!mbar_wait_warp(c, &g_dec.b_loaded, s.loaded & 1u)) return;
     }
@@ -485,9 +485,7 @@ static __device__ __noinline__ void phase_gemm_dec(const DevCtx& c, int which, i
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // read by the MMAs next
     __syncthreads();
     if (threadIdx.x == 0 && g.u0 < g.u1) {
-      // (an arrival with release at cluster scope waits for every outstanding store: 1.1 us a phase; the proxy fence
-      // of the writers and the barrier above order their shared-memory writes before the MMAs of the pair)
-      if constexpr (PAIR) mbar_arrive_cta0(&g_dec.b_made);
+      if constexpr (PAIR) mbar_arrive_cta0_release(&g_dec.b_made);   // the MMAs that read this CTA's half are issued by CTA 0
       else mbar_arrive(&g_dec.b_made);
     }
   }

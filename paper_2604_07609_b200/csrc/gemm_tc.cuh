@@ -255,6 +255,30 @@ __device__ __forceinline__ void mbar_arrive_cta0(uint64_t* bar) {
       "mbarrier.arrive.shared::cluster.b64 _, [ra];\n\t}" ::"r"(smem_u32(bar))
       : "memory");
 }
+// The same by a thread that stands for ordinary shared-memory stores of its CTA which the other CTA's MMAs are going to
+// read (ordered before it by a barrier of the CTA), and the wait on the other side.  Release and acquire are at cluster
+// scope and restricted to shared memory: a full release at cluster scope waits for every store to global memory too.
+__device__ __forceinline__ void mbar_arrive_cta0_release(uint64_t* bar) {
+  asm volatile(
+      "{\n\t.reg .b32 ra;\n\t"
+      "mapa.shared::cluster.u32 ra, %0, 0;\n\t"
+      "fence.release.sync_restrict::shared::cta.cluster;\n\t"
+      "mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [ra];\n\t}" ::"r"(smem_u32(bar))
+      : "memory");
+}
+__device__ __forceinline__ bool mbar_wait_warp_acquire(const DevCtx& c, uint64_t* bar, uint32_t parity) {
+  if (!mbar_wait_warp(c, bar, parity)) return false;
+  uint32_t ok;   // complete: once more as the read that the fence turns into an acquire
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "fence.acquire.sync_restrict::shared::cluster.cluster;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return __all_sync(0xffffffffu, ok != 0u);
+}
 // Tile copies of a pair: the bytes are counted on CTA 0's barrier (the CTA bit of the barrier's address is
 // cleared), whichever CTA of the pair issues the copy and receives the data.
 constexpr uint32_t PAIR_CTA0_MASK = 0xFEFFFFFFu;

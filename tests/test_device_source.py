@@ -1,0 +1,31 @@
+"""Orderings that a run cannot show to be there: checked in the text of the kernels."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2604_07609_b200", "csrc")
+
+
+def _text(name):
+    return open(os.path.join(CSRC, name)).read()
+
+
+def _body(text, name):
+    start = re.search(r"\b%s\([^;{]*\{" % name, text).end()
+    depth, i = 1, start
+    while depth:
+        depth += {"{": 1, "}": -1}.get(text[i], 0)
+        i += 1
+    return text[start:i]
+
+
+def test_a_token_operand_made_by_a_pair_is_handed_over_at_cluster_scope():
+    """CTA 1 writes its half with ordinary stores, CTA 0 issues the MMAs that read it: a release and an acquire whose scope
+    holds both CTAs have to lie between (an arrival without a scope releases to its own CTA only)."""
+    dec, tc = _text("gemm_dec.cuh"), _text("gemm_tc.cuh")
+    arrive = re.search(r"if constexpr \(PAIR\) (\w+)\(&g_dec\.b_made\)", dec).group(1)
+    wait = re.search(r"PAIR \? (\w+)\(c, &g_dec\.b_made", dec)
+    assert wait, "pairs wait for the made operand with a wait of their own"
+    out, back = _body(tc, arrive), _body(tc, wait.group(1))
+    assert re.search(r"arrive\.release\.cluster|fence\.(release\.sync_restrict::shared::cta|acq_rel)\.cluster.*arrive\.relaxed\.cluster", out, re.S), arrive
+    assert re.search(r"try_wait\.parity\.acquire\.cluster|try_wait\.parity\.relaxed\.cluster.*fence\.(acquire\.sync_restrict::shared::cluster|acq_rel)\.cluster",
+                     back, re.S), wait.group(1)
