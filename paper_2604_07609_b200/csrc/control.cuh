@@ -738,10 +738,10 @@ static __device__ __noinline__ void control_phase(const DevCtx& c, long long& la
   const int tid = threadIdx.x;
   __shared__ int s_cmd;
   __shared__ int s_started;
-  __shared__ int s_abort;
+  __shared__ int s_leave;
   __shared__ unsigned long long s_tail;
   if (ss->pending_post) post_step(c);
-  long long idle_t0 = clock64();
+  const long long idle_t0 = clock64();   // (thread 0 compares)
   unsigned int spins = 0;
   while (true) {
     if (tid == 0) {
@@ -774,22 +774,16 @@ static __device__ __noinline__ void control_phase(const DevCtx& c, long long& la
       __syncthreads();
       break;
     }
-    // one thread reads the flag (another CTA may raise it at any time) so that the whole CTA
-    // takes the same branch
-    if (tid == 0) s_abort = *(volatile int*)&ss->abort_flag;
+    // One thread reads the flag (another CTA may raise it at any time) and the clock, so that the whole CTA takes the
+    // same branch: with a clock of its own every warp may pass the limit in another turn, the barriers of the CTA then
+    // no longer match and the kernel does not end.  Idle: poll the submit mailbox, leave the GPU when nothing comes.
+    if (tid == 0) {
+      const int reason = *(volatile int*)&ss->abort_flag ? 5 : !c.stepped && (unsigned long long)(clock64() - idle_t0) > c.idle_exit_cycles ? 4 : 0;
+      if (reason) { s_cmd = CMD_EXIT; ss->exit_reason = reason; }
+      s_leave = reason != 0 || c.stepped;   // (stepped: CMD_NONE)
+    }
     __syncthreads();
-    if (s_abort) {
-      if (tid == 0) { s_cmd = CMD_EXIT; ss->exit_reason = 5; }
-      __syncthreads();
-      break;
-    }
-    if (c.stepped) break;  // CMD_NONE
-    // idle: poll the submit mailbox, leave the GPU when nothing comes
-    if ((unsigned long long)(clock64() - idle_t0) > c.idle_exit_cycles) {
-      if (tid == 0) { s_cmd = CMD_EXIT; ss->exit_reason = 4; }
-      __syncthreads();
-      break;
-    }
+    if (s_leave) break;
     if (++spins > 16) __nanosleep(1000);
     __syncthreads();
   }

@@ -29,3 +29,10 @@ def test_a_token_operand_made_by_a_pair_is_handed_over_at_cluster_scope():
     assert re.search(r"arrive\.release\.cluster|fence\.(release\.sync_restrict::shared::cta|acq_rel)\.cluster.*arrive\.relaxed\.cluster", out, re.S), arrive
     assert re.search(r"try_wait\.parity\.acquire\.cluster|try_wait\.parity\.relaxed\.cluster.*fence\.(acquire\.sync_restrict::shared::cluster|acq_rel)\.cluster",
                      back, re.S), wait.group(1)
+
+
+def test_the_control_cta_leaves_by_one_threads_clock():
+    """Threads that each compare their own clock leave the idle loop in different turns, and the CTA's barriers no longer match."""
+    body = _body(_text("control.cuh"), "control_phase")
+    by_thread_0 = "".join(re.findall(r"if \(tid == 0\) \{.*?\n    \}", body, re.S))
+    assert body.count("- idle_t0") == by_thread_0.count("- idle_t0") == 1
