@@ -35,6 +35,7 @@ __shared__ StepInfo g_step;
 // grid barrier closes it.
 constexpr int PLAN_BARRIER = 1 << 16, PLAN_MAX = 2 * MAX_EXPERTS + 12;
 __shared__ int g_plan[2][PLAN_MAX], g_plan_n[2];
+static_assert(N_PHASE_TIMERS <= 32, "copied by one warp");
 __shared__ unsigned long long g_phase_ns[N_PHASE_TIMERS];   // device time per phase kind of the open step (CTA 0)
 __shared__ unsigned long long g_phase_t;                    // when the last phase ended
 // Phases that a step does not have because others do their work.
@@ -258,7 +259,10 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) blink_loop_kernel(const __grid
         }
       }
       if (!ok) break;
-      if (c.stats_cap > 0 && blockIdx.x == 0 && threadIdx.x < N_PHASE_TIMERS) c.ss->cur_phase_ns[threadIdx.x] = g_phase_ns[threadIdx.x];
+      if (c.stats_cap > 0 && blockIdx.x == 0 && threadIdx.x < 32) {
+        __syncwarp();   // thread 0 has added the last phase after the barrier
+        if (threadIdx.x < N_PHASE_TIMERS) c.ss->cur_phase_ns[threadIdx.x] = g_phase_ns[threadIdx.x];
+      }
     } else if (!grid_barrier(c)) break;
   }
   dec_drain<PAIR>(c, PAIR ? cluster_ctarank() : 0u);

@@ -32,3 +32,24 @@ def test_many_idle_exits_in_a_row():
         assert st.loop_state == B.LOOP_EXIT_IDLE and st.device_status == 0 and st.launches >= n
     finally:
         assert eng.blink_destroy() == B.BLINK_OK
+
+
+def test_phase_times_of_every_step_hold_its_last_phase():
+    """One thread adds a phase's time, other lanes copy the array: with no order between the two the last phase of a step,
+    sampling, could miss."""
+    model = ModelCfg(1, 256, 8, 2, 64, 256, 512)
+    sched = SchedCfg(max_batch=2, prefill_chunk_tokens=16, n_slots=4, max_prompt=8, max_new=500, n_blocks=80)
+    kv = torch.zeros(sched.n_blocks * B.kv_bytes_per_block(model, sched.block_size), dtype=torch.uint8, device="cuda")
+    eng = B.Blink(model, sched, make_weights(model, 3, "cpu").cuda(), kv, exec_mode=B.EXEC_MANUAL, stats_iters=1024)
+    try:
+        eng.blink_submit(np.array([1, 2, 3], np.int32), 500)
+        eng.blink_run(499)
+        its = eng.blink_get_iter_stats()
+        assert len(its) == 499
+        phases = its["phase_ns"].astype(np.int64)
+        assert (phases[:, 11] > 0).all()
+        # the phases fill the time from the end of the control plane to the post step, but for the barrier before them
+        spans = (its["t_end_ns"] - its["t_forward_ns"]).astype(np.int64)
+        assert np.median(phases.sum(axis=1) / spans) > 0.8 and (phases.sum(axis=1) <= spans).all()
+    finally:
+        assert eng.blink_destroy() == B.BLINK_OK
