@@ -178,7 +178,9 @@ __device__ __forceinline__ int nuc_bucket(float z, float z0) { return 255 - (int
 __device__ __forceinline__ bool nucleus_row(int top_k, float top_p) { return top_k <= 0 && top_p > 0.f && top_p < 1.f; }
 
 // Weights and counts of elements [i0, i1) into shared memory.  A weight of up to 41 bits is added as four limbs of
-// 11 bits: 32-bit adds into shared memory are native, the 64-bit one is a compare-and-swap loop (2^21 entries fit).
+// 11 bits: 32-bit adds into shared memory are native, the 64-bit one is a compare-and-swap loop.
+constexpr int NUC_LIMB_ENTRIES = 1 << 21;   // so many entries of one bucket fit: 2047 * 2^21 < 2^32
+static_assert(SAMPLE_WARP_SPAN * SAMPLE_CHUNKS <= NUC_LIMB_ENTRIES, "rows prepared by all CTAs are added up in one go");
 struct NucLimbs {
   unsigned int w[4][256];
   unsigned int n[256];
@@ -517,12 +519,18 @@ static __device__ __noinline__ int sample_row_nucleus(const float* lg, int V, in
     st.c0[tid] = __ldcg(nc + tid);
   } else {
     NucLimbs& L = *reinterpret_cast<NucLimbs*>(s_cz);
-    nuc_limbs_clear(L);
-    __syncthreads();
-    nuc_add_range(L, lg, V, 0, V, temp, z0);
-    __syncthreads();
-    st.m0[tid] = nuc_limb_sum(L, tid);
-    st.c0[tid] = L.n[tid];
+    unsigned long long m = 0;
+    unsigned int n = 0;
+    for (int i0 = 0; i0 < V; i0 += NUC_LIMB_ENTRIES) {   // (a thread clears and reads its own bucket)
+      nuc_limbs_clear(L);
+      __syncthreads();
+      nuc_add_range(L, lg, V, i0, min(V - i0, NUC_LIMB_ENTRIES) + i0, temp, z0);
+      __syncthreads();
+      m += nuc_limb_sum(L, tid);
+      n += L.n[tid];
+    }
+    st.m0[tid] = m;
+    st.c0[tid] = n;
   }
   __syncthreads();
   if (tid < 32) {

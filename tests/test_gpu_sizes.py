@@ -157,3 +157,27 @@ def test_top_k_rows_with_nan_answer_the_same_member_of_the_row_each_time(V, top_
     first = _sample(x, min(50, V), top_p)
     assert all(0 <= t < V for t in first)
     assert all(_sample(x, min(50, V), top_p) == first for _ in range(3))
+
+
+@pytest.mark.parametrize("V", [1 << 18, (1 << 18) + 4, (1 << 21) + 36, 2300001])
+def test_nucleus_of_very_long_rows_adds_up_every_weight(V):
+    """Weights are added in limbs of a few bits: a row of equal weights with all limbs nearly full carries the sums as far
+    as they go.  Two values, so the order and the cut have a closed form."""
+    d = np.arange(1, 40001, dtype=np.float32) / 4096          # the drop whose weight has the fullest lower limbs
+    q = np.floor(np.exp(-d.astype(np.float64)) * 2.0 ** 40).astype(np.int64)
+    fill = np.min([(q >> s) & 2047 for s in (0, 11, 22)], axis=0)
+    drop, w = float(d[fill.argmax()]), int(q[fill.argmax()])
+    assert int(fill.max()) > 1900
+    x = np.full((4, V), -drop, np.float32)
+    top = np.array([V - 1, 0, V // 2, 7])
+    x[np.arange(4), top] = 0.0                                # z0, weight 2^40
+    Q = (V - 1) * w + (1 << 40)
+    p24 = int(np.rint(np.float64(np.float32(0.9)) * (1 << 24)))
+    need = -(-p24 * Q // (1 << 24))
+    n = -(-(need - (1 << 40)) // w)                           # entries of the nucleus beside the top one
+    got = _sample(x, 0, 0.9, temp=1.0)
+    for r in range(4):
+        target = ((S.philox_word(r, 0, 3) >> 8) * ((1 << 40) + n * w)) >> 24
+        j = max(0, -(-(target + 1 - (1 << 40)) // w))         # place in the order: 0 is the top entry
+        want = int(top[r]) if j == 0 else int(np.delete(np.arange(V), top[r])[j - 1])
+        assert got[r] == want, (r, got[r], want)
