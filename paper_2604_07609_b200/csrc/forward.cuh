@@ -191,14 +191,19 @@ __device__ __forceinline__ void norm_row_cta(const DevCtx& c, float* hrow, const
       float den = 0.f, top = 0.f, mine = 0.f;
       int place = -1;
       for (int j = 0; j < c.topE; ++j) {
-        float bv = open ? lg : -INFINITY;
-        int bi = open ? lane : 32;
+        // The first open expert, or one with a larger logit.  NaN is larger than nothing and nothing is larger than NaN: it
+        // stays out of the exchange, where it would keep lanes from hearing of one another, unless it is the first.
+        const int first = __ffs(__ballot_sync(0xffffffffu, open)) - 1;
+        const float lg_first = __shfl_sync(0xffffffffu, lg, first);
+        float bv = open && lg == lg ? lg : -INFINITY;
+        int bi = open && lg == lg ? lane : 32;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
           const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
           const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
           if (oi < 32 && (bi == 32 || ov > bv || (ov == bv && oi < bi))) { bv = ov; bi = oi; }   // ties keep the lower id
         }
+        if (lg_first != lg_first) { bv = lg_first; bi = first; }
         if (j == 0) top = bv;
         const float ex = expf(bv - top);
         den += ex;

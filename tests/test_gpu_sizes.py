@@ -8,6 +8,7 @@ from gpu_util import compare_with_oracle, gpu_run_forced
 from oracle import sampler as S
 from paper_2604_07609_b200 import binding as B
 from synth import make_weights
+from synth.weights import TENSOR_NAMES, weight_layout
 from synth.configs import ModelCfg, SchedCfg
 from synth.workload import Request
 
@@ -181,3 +182,29 @@ def test_nucleus_of_very_long_rows_adds_up_every_weight(V):
         j = max(0, -(-(target + 1 - (1 << 40)) // w))         # place in the order: 0 is the top entry
         want = int(top[r]) if j == 0 else int(np.delete(np.arange(V), top[r])[j - 1])
         assert got[r] == want, (r, got[r], want)
+
+
+@pytest.mark.parametrize("broken", [1, 4])
+def test_an_expert_whose_router_logit_is_nan_is_as_good_as_absent(broken):
+    """NaN is larger than nothing: unless it is the first of the list, such an expert is never chosen, and the model
+    answers as the one without it."""
+    model = ModelCfg(2, 256, 4, 4, 64, 256, 512, n_experts=5, top_k_experts=2, dtype="fp32")
+    less = model.with_(n_experts=4)
+    w = make_weights(model, 17, "cpu")
+    (lay, _), (lay_less, total) = weight_layout(model), weight_layout(less)
+    w_less = torch.zeros(total, dtype=torch.uint8)
+    keep = [e for e in range(5) if e != broken]
+    for name in TENSOR_NAMES:
+        (o, shape, dt), (ol, shape_l, _) = lay[name], lay_less[name]
+        t = w[o:o + int(np.prod(shape)) * 4].view(dt).view(shape)
+        t_less = w_less[ol:ol + int(np.prod(shape_l)) * 4].view(dt).view(shape_l)
+        t_less.copy_(t[:, keep] if name in ("wgu", "wd", "wr") else t)
+        if name == "wr":
+            t[:, broken] = float("nan")
+    sched = SchedCfg(max_batch=4, prefill_chunk_tokens=32, n_slots=16, max_prompt=16, max_new=6, n_blocks=32)
+    reqs = _requests([4, 9, 16, 7], 6, model.vocab)
+    forced = {r.ticket: list(range(10 * r.ticket, 10 * r.ticket + 6)) for r in reqs}
+    a = gpu_run_forced(model, sched, reqs, w, forced)
+    b = gpu_run_forced(less, sched, reqs, w_less, forced)
+    assert np.isfinite(b[2]).all() and float(np.abs(b[2]).max()) > 0.1
+    assert float(np.abs(a[2] - b[2]).max()) <= 1e-4    # the bound of the fp32 mode; the experts' sums are added in any order
