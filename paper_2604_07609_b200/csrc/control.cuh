@@ -699,7 +699,7 @@ static __device__ int schedule_step(const DevCtx& c, unsigned long long visible)
       }
       if (C == 0 && t_unit < t_stream) S = 0;
       // a decode step of few rows: the CTA-wide kernel also applies RoPE and writes the new keys and values
-      const int fuse = c.dec_small && T <= 16 && n_pf == 0 && s_C > 0;
+      const int fuse = c.dec_small && T <= DEC_SMALL_ROWS && n_pf == 0 && s_C > 0;
       if (fuse) C = s_C;
       ss->cur_fuse = fuse;
       c.dec_kbpre[n_dec_att] = tot_kb;

@@ -128,6 +128,9 @@ constexpr int MAX_BATCH = 256;
 constexpr int MAX_TOPK = 64;
 constexpr int MAX_EXPERTS = 16;
 constexpr int TILE_CNT_SLOTS = 8192;
+// Steps of up to so many rows run norms, SwiGLU and final norm inside their GEMMs, and RoPE and the K/V write inside the
+// attention; the scheduler and the phases go by the same limit (a step of the one without the other would lose RoPE).
+constexpr int DEC_SMALL_ROWS = 16;
 
 struct DevCtx {
   // model

@@ -17,7 +17,8 @@
 
 namespace blink {
 
-constexpr int DEC_SMALL_ROWS = 16, DEC_MID_ROWS = 128;
+constexpr int DEC_MID_ROWS = 128;
+static_assert(DEC_SMALL_ROWS == 16, "made operands are two groups of eight rows");
 constexpr int DEC_STAGES = 4, DEC_STAGE_BYTES = 2 * TC_A_BYTES;   // two k-blocks of a 128-row weight tile
 constexpr int DEC_B_OFF = DEC_STAGES * DEC_STAGE_BYTES, DEC_B_BYTES = 65536;
 constexpr int DEC_B_STAGES = 8;

@@ -36,3 +36,10 @@ def test_the_control_cta_leaves_by_one_threads_clock():
     body = _body(_text("control.cuh"), "control_phase")
     by_thread_0 = "".join(re.findall(r"if \(tid == 0\) \{.*?\n    \}", body, re.S))
     assert body.count("- idle_t0") == by_thread_0.count("- idle_t0") == 1
+
+
+def test_scheduler_and_phases_go_by_one_row_limit_for_small_steps():
+    """The scheduler decides who applies RoPE, the phases who clears its input: two limits would drop one or the other."""
+    control, dec = _text("control.cuh"), _text("gemm_dec.cuh")
+    assert re.search(r"const int fuse = c\.dec_small && T <= DEC_SMALL_ROWS\b", control)
+    assert re.search(r"bool dec_small\(.*\{ return c\.dec_small && T <= DEC_SMALL_ROWS; \}", dec)
