@@ -184,9 +184,9 @@ def test_nucleus_of_very_long_rows_adds_up_every_weight(V):
         assert got[r] == want, (r, got[r], want)
 
 
-@pytest.mark.parametrize("broken", [1, 4])
+@pytest.mark.parametrize("broken", [2, 4])   # behind two others: with two choices never the first still open
 def test_an_expert_whose_router_logit_is_nan_is_as_good_as_absent(broken):
-    """NaN is larger than nothing: unless it is the first of the list, such an expert is never chosen, and the model
+    """NaN is larger than nothing: unless it is the first still open, such an expert is never chosen, and the model
     answers as the one without it."""
     model = ModelCfg(2, 256, 4, 4, 64, 256, 512, n_experts=5, top_k_experts=2, dtype="fp32")
     less = model.with_(n_experts=4)
