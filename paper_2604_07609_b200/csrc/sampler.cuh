@@ -172,49 +172,73 @@ static __device__ __noinline__ void phase_sample_max(const DevCtx& c) {
 }
 
 // ---- weights of a row per bucket of z -------------------------------------------------------------------
-// Bucket 255 holds z within 28/255 of the row's largest, bucket 0 everything more than 28 below it, whose weight
-// exp(-28) * 2^40 is below one: an entry of weight zero is never the answer, so bucket 0 need not be resolved.
-__device__ __forceinline__ int nuc_bucket(float z, float z0) { return 255 - (int)fminf((z0 - z) * (255.0f / 28.0f), 255.0f); }
+// An entry more than 28 below the largest z has the weight floor(exp(-28) * 2^40) = 0 and is never the answer: bucket 0.
+// Buckets 255 .. 1 divide the distances from 0 to the smaller of 28 and the spread of the row, which is taken from its
+// first entries: what lies further down still has bucket 1.  Over a fixed 28 a row of small or nearly equal logits falls
+// into a few buckets, whose sums every thread then adds to (100 such rows of 32000 entries in a step: 513 us, by their
+// spread 187; of 128256 entries, shared by all CTAs, 1030 and 800).
+constexpr float NUC_SPAN = 28.0f;
+__device__ __forceinline__ int nuc_bucket(float z, float z0, float scale) {
+  const float d = z0 - z;
+  return d <= NUC_SPAN ? 255 - min((int)(d * scale), 254) : 0;
+}
 __device__ __forceinline__ bool nucleus_row(int top_k, float top_p) { return top_k <= 0 && top_p > 0.f && top_p < 1.f; }
 
-// Weights and counts of elements [i0, i1) into shared memory.  A weight of up to 41 bits is added as four limbs of
-// 11 bits: 32-bit adds into shared memory are native, the 64-bit one is a compare-and-swap loop.
-constexpr int NUC_LIMB_ENTRIES = 1 << 21;   // so many entries of one bucket fit: 2047 * 2^21 < 2^32
-static_assert(SAMPLE_WARP_SPAN * SAMPLE_CHUNKS <= NUC_LIMB_ENTRIES, "rows prepared by all CTAs are added up in one go");
+// Weights and counts of elements [i0, i1) into shared memory.  A weight of up to 41 bits is added as three limbs of
+// 14 bits: 32-bit adds into shared memory are native, the 64-bit one is a compare-and-swap loop.  Eight exponentials per
+// thread are worked on before the first add: with a branch after each they wait for one another (20 rows of 32000 normal
+// logits by a CTA each: 420 us, together 150).
+constexpr int NUC_LIMB_BITS = 14;
+constexpr int NUC_LIMB_ENTRIES = 1 << (32 - NUC_LIMB_BITS);   // so many entries of one bucket fit a 32-bit sum
 struct NucLimbs {
-  unsigned int w[4][256];
+  unsigned int w[3][256];
   unsigned int n[256];
 };
-__device__ __forceinline__ void nuc_add_range(NucLimbs& L, const float* lg, int V, int i0, int i1, float temp, float z0) {
+__device__ __forceinline__ void nuc_add_range(NucLimbs& L, const float* lg, int V, int i0, int i1, float temp, float z0, float scale) {
+  constexpr int U = 2;   // vectors per thread whose exponentials are worked on together
   const bool vec = sample_row_vec(lg, V);
-  for (int i = i0 + threadIdx.x * 4; i < i1; i += FWD_THREADS * 4) {
-    const float4 v = vec ? sample_load4<true>(lg, V, i) : sample_load4<false>(lg, V, i);
-    const float e[4] = {v.x, v.y, v.z, v.w};
+  for (int base = i0 + threadIdx.x * 4; base < i1; base += U * FWD_THREADS * 4) {
+    float e[4 * U];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      if (i + k < V) {
-        const float z = __fdiv_rn(e[k], temp);
-        const int b = nuc_bucket(z, z0);
-        if (b == 0) continue;
-        const unsigned long long q = nucleus_weight(z, z0);
+    for (int u = 0; u < U; ++u) {
+      const int i = base + u * FWD_THREADS * 4;
+      const float4 v = vec ? sample_load4<true>(lg, V, i) : sample_load4<false>(lg, V, i);
+      e[4 * u] = v.x; e[4 * u + 1] = v.y; e[4 * u + 2] = v.z; e[4 * u + 3] = v.w;
+    }
+    int b[4 * U];
+    unsigned long long q[4 * U];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const unsigned int limb = (unsigned int)(q >> (11 * j)) & 2047u;
-          if (limb) atomicAdd(&L.w[j][b], limb);
-        }
-        atomicAdd(&L.n[b], 1u);
+    for (int k = 0; k < 4 * U; ++k) {
+      const float z = __fdiv_rn(e[k], temp);
+      b[k] = base + (k >> 2) * FWD_THREADS * 4 + (k & 3) < i1 ? nuc_bucket(z, z0, scale) : 0;
+      q[k] = nucleus_weight(z, z0);
+    }
+#pragma unroll
+    for (int k = 0; k < 4 * U; ++k) {
+      if (b[k]) {
+        atomicAdd(&L.w[0][b[k]], (unsigned int)q[k] & 16383u);
+        atomicAdd(&L.w[1][b[k]], (unsigned int)(q[k] >> NUC_LIMB_BITS) & 16383u);
+        atomicAdd(&L.w[2][b[k]], (unsigned int)(q[k] >> (2 * NUC_LIMB_BITS)));
+        atomicAdd(&L.n[b[k]], 1u);
       }
     }
   }
 }
-__device__ __forceinline__ unsigned long long nuc_limb_sum(const NucLimbs& L, int b) {
-  return (unsigned long long)L.w[0][b] + ((unsigned long long)L.w[1][b] << 11) + ((unsigned long long)L.w[2][b] << 22) +
-         ((unsigned long long)L.w[3][b] << 33);
-}
-__device__ __forceinline__ void nuc_limbs_clear(NucLimbs& L) {
-#pragma unroll
-  for (int j = 0; j < 4; ++j) L.w[j][threadIdx.x] = 0u;
-  L.n[threadIdx.x] = 0u;
+// The whole CTA: weight m and number n of the entries of bucket threadIdx.x among elements [i0, i1).
+__device__ __forceinline__ void nuc_bucket_sums(NucLimbs& L, const float* lg, int V, int i0, int i1, float temp, float z0, float scale,
+                                                unsigned long long& m, unsigned int& n) {
+  const int b = threadIdx.x;
+  m = 0ull;
+  n = 0u;
+  for (; i0 < i1; i0 += NUC_LIMB_ENTRIES) {   // (a thread clears and reads its own bucket)
+    L.w[0][b] = L.w[1][b] = L.w[2][b] = L.n[b] = 0u;
+    __syncthreads();
+    nuc_add_range(L, lg, V, i0, min(i1 - i0, NUC_LIMB_ENTRIES) + i0, temp, z0, scale);
+    __syncthreads();
+    m += (unsigned long long)L.w[0][b] + ((unsigned long long)L.w[1][b] << NUC_LIMB_BITS) +
+         ((unsigned long long)L.w[2][b] << (2 * NUC_LIMB_BITS));
+    n += L.n[b];
+  }
 }
 __device__ __forceinline__ float block_max(float v, float* s_red /*[8]*/) {
   v = warp_max(v);
@@ -225,6 +249,17 @@ __device__ __forceinline__ float block_max(float v, float* s_red /*[8]*/) {
 #pragma unroll
   for (int i = 0; i < FWD_THREADS / 32; ++i) t = fmaxf(t, s_red[i]);
   return t;
+}
+// Buckets per unit of z, the same in every CTA that works on the row.
+__device__ __forceinline__ float nuc_scale(const float* lg, int V, float temp, float z0, float* s_red) {
+  float low = INFINITY;
+  for (int i = threadIdx.x * 4; i < min(V, FWD_THREADS * 4); i += FWD_THREADS * 4)
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (i + k < V) low = fminf(low, lg[i + k]);
+  low = -block_max(-low, s_red);
+  const float spread = fminf(NUC_SPAN, z0 - __fdiv_rn(low, temp));
+  return spread > 0.f ? 254.0f / spread : 0.f;
 }
 __device__ __forceinline__ float sample_row_max(const float* cmax, int n, float* s_red) {
   float m = -INFINITY;
@@ -245,16 +280,16 @@ static __device__ __noinline__ void phase_sample_weights(const DevCtx& c, float*
     const int r = u / parts, part = u - r * parts;
     const int b = c.it_bslot[c.row_item[r]];
     if (!nucleus_row(c.b_topk[b], c.b_topp[b]) || part * len >= V) continue;   // uniform over the CTA
-    __syncthreads();
-    nuc_limbs_clear(L);
     const float temp = c.b_temp[b];
+    const float* lg = c.logits + (size_t)r * V;
     const float z0 = __fdiv_rn(sample_row_max(c.cmax + (size_t)r * SAMPLE_CHUNKS, nch, s_red), temp);
-    nuc_add_range(L, c.logits + (size_t)r * V, V, part * len, min(V, (part + 1) * len), temp, z0);
-    __syncthreads();
-    if (L.n[threadIdx.x]) {
-      const unsigned long long q = nuc_limb_sum(L, threadIdx.x);
-      if (q) atomicAdd(&c.nuc_m[(size_t)r * 256 + threadIdx.x], q);
-      atomicAdd(&c.nuc_c[(size_t)r * 256 + threadIdx.x], L.n[threadIdx.x]);
+    const float scale = nuc_scale(lg, V, temp, z0, s_red);
+    unsigned long long m;
+    unsigned int n;
+    nuc_bucket_sums(L, lg, V, part * len, min(V, (part + 1) * len), temp, z0, scale, m, n);
+    if (n) {
+      if (m) atomicAdd(&c.nuc_m[(size_t)r * 256 + threadIdx.x], m);
+      atomicAdd(&c.nuc_c[(size_t)r * 256 + threadIdx.x], n);
     }
   }
 }
@@ -344,7 +379,7 @@ __device__ __forceinline__ void sample_for_listed(const float* lg, int V, int cl
 // (buckets over the float-key interval of the set) until it fits the candidate buffer, which is then ranked
 // exactly.  A set that cannot be narrowed (more than NUC_CAND equal values) is resolved by index.
 static __device__ __noinline__ void nucleus_locate(NucShared& st, const float* lg, int V, int cl, const float* s_cmax, float temp,
-                                                   float z0, unsigned long long t, float* s_cz, int* s_ci, float* s_sz, int* s_si) {
+                                                   float z0, float scale, unsigned long long t, float* s_cz, int* s_ci, float* s_sz, int* s_si) {
   const int tid = threadIdx.x;
   const int nch = (V + cl - 1) / cl;
   if (tid < 32) {
@@ -360,7 +395,7 @@ static __device__ __noinline__ void nucleus_locate(NucShared& st, const float* l
   for (int level = 0; level < 8; ++level) {   // a level divides the key interval by 256: four suffice
     const unsigned int klo = st.klo, khi = st.khi;
     const int n_list = sample_list_chunks(s_cmax, nch, s_list, &st.n_list,
-                                          [&](float m) { return nuc_bucket(__fdiv_rn(m, temp), z0) >= b0; });
+                                          [&](float m) { return nuc_bucket(__fdiv_rn(m, temp), z0, scale) >= b0; });
     if (st.cnt <= (unsigned)NUC_CAND) {
       // ---- gather the members, rank them exactly, walk the cumulative weights ----
       if (tid == 0) st.n = 0;
@@ -368,7 +403,7 @@ static __device__ __noinline__ void nucleus_locate(NucShared& st, const float* l
       sample_for_listed(lg, V, cl, s_list, n_list, [&](float v, int i) {
         const float z = __fdiv_rn(v, temp);
         const unsigned int key = float_key(z);
-        if (nuc_bucket(z, z0) == b0 && key >= klo && key <= khi) {
+        if (nuc_bucket(z, z0, scale) == b0 && key >= klo && key <= khi) {
           const int p = atomicAdd(&st.n, 1);
           if (p < NUC_CAND) { s_cz[p] = z; s_ci[p] = i; }
         }
@@ -418,7 +453,7 @@ static __device__ __noinline__ void nucleus_locate(NucShared& st, const float* l
       unsigned int lo = 0xffffffffu, hi = 0u;
       sample_for_listed(lg, V, cl, s_list, n_list, [&](float v, int) {
         const float z = __fdiv_rn(v, temp);
-        if (nuc_bucket(z, z0) == b0) {
+        if (nuc_bucket(z, z0, scale) == b0) {
           const unsigned int key = float_key(z);
           lo = min(lo, key);
           hi = max(hi, key);
@@ -440,7 +475,7 @@ static __device__ __noinline__ void nucleus_locate(NucShared& st, const float* l
       unsigned int mine = 0;
       for (int i = i0; i < i1; ++i) {
         const float zi = __fdiv_rn(lg[i], temp);
-        mine += (nuc_bucket(zi, z0) == b0 && float_key(zi) == klo) ? 1u : 0u;
+        mine += (nuc_bucket(zi, z0, scale) == b0 && float_key(zi) == klo) ? 1u : 0u;
       }
       st.chunk_cnt[tid] = mine;
       __syncthreads();
@@ -450,7 +485,7 @@ static __device__ __noinline__ void nucleus_locate(NucShared& st, const float* l
         unsigned long long seen = before;
         for (int i = i0; i < i1; ++i) {
           const float zi = __fdiv_rn(lg[i], temp);
-          if (nuc_bucket(zi, z0) == b0 && float_key(zi) == klo) {
+          if (nuc_bucket(zi, z0, scale) == b0 && float_key(zi) == klo) {
             if (seen == jl) { st.res_idx = i; st.res_cum = st.acc + (jl + 1) * q0; st.done = 1; break; }
             ++seen;
           }
@@ -469,7 +504,7 @@ static __device__ __noinline__ void nucleus_locate(NucShared& st, const float* l
     sample_for_listed(lg, V, cl, s_list, n_list, [&](float v, int) {
       const float z = __fdiv_rn(v, temp);
       const unsigned int key = float_key(z);
-      if (nuc_bucket(z, z0) == b0 && key >= klo && key <= khi) {
+      if (nuc_bucket(z, z0, scale) == b0 && key >= klo && key <= khi) {
         const int b = (int)((((unsigned long long)(key - klo)) << 8) / W);
         atomicAdd(&st.m[b], nucleus_weight(z, z0));
         atomicAdd(&st.cn[b], 1u);
@@ -512,23 +547,17 @@ static __device__ __noinline__ int sample_row_nucleus(const float* lg, int V, in
   int* s_ci = reinterpret_cast<int*>(smem + 256 + SAMPLE_CAND);
   float* s_sz = smem + 256 + 2 * SAMPLE_CAND;
   int* s_si = reinterpret_cast<int*>(smem + 256 + 3 * SAMPLE_CAND);
+  __shared__ float s_red[FWD_THREADS / 32];
   const float z0 = __fdiv_rn(lmax, temp);
+  const float scale = nuc_scale(lg, V, temp, z0, s_red);
   __syncthreads();
   if (nm != nullptr) {
     st.m0[tid] = __ldcg(nm + tid);
     st.c0[tid] = __ldcg(nc + tid);
   } else {
-    NucLimbs& L = *reinterpret_cast<NucLimbs*>(s_cz);
-    unsigned long long m = 0;
-    unsigned int n = 0;
-    for (int i0 = 0; i0 < V; i0 += NUC_LIMB_ENTRIES) {   // (a thread clears and reads its own bucket)
-      nuc_limbs_clear(L);
-      __syncthreads();
-      nuc_add_range(L, lg, V, i0, min(V - i0, NUC_LIMB_ENTRIES) + i0, temp, z0);
-      __syncthreads();
-      m += nuc_limb_sum(L, tid);
-      n += L.n[tid];
-    }
+    unsigned long long m;
+    unsigned int n;
+    nuc_bucket_sums(*reinterpret_cast<NucLimbs*>(s_cz), lg, V, 0, V, temp, z0, scale, m, n);
     st.m0[tid] = m;
     st.c0[tid] = n;
   }
@@ -549,14 +578,14 @@ static __device__ __noinline__ int sample_row_nucleus(const float* lg, int V, in
     const int pick = sample_first_max(lg, V, cl, s_cmax, z0, [&](float v) { return __fdiv_rn(v, temp); });
     return tid == 0 ? pick : -1;
   }
-  nucleus_locate(st, lg, V, cl, s_cmax, temp, z0, s_t, s_cz, s_ci, s_sz, s_si);   // end of the nucleus: its weight is res_cum
+  nucleus_locate(st, lg, V, cl, s_cmax, temp, z0, scale, s_t, s_cz, s_ci, s_sz, s_si);   // end of the nucleus: its weight is res_cum
   if (tid == 0) {
     const uint32_t x = philox4x32_10_word0((uint32_t)ticket, (uint32_t)(ticket >> 32), (uint32_t)gen_index, 0u,
                                            (uint32_t)seed, (uint32_t)(seed >> 32));
     s_t = nucleus_target((unsigned long long)(x >> 8), st.res_cum);
   }
   __syncthreads();
-  nucleus_locate(st, lg, V, cl, s_cmax, temp, z0, s_t, s_cz, s_ci, s_sz, s_si);
+  nucleus_locate(st, lg, V, cl, s_cmax, temp, z0, scale, s_t, s_cz, s_ci, s_sz, s_si);
   const int result = tid == 0 ? st.res_idx : -1;
   __syncthreads();
   return result;

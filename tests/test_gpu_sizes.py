@@ -208,3 +208,21 @@ def test_an_expert_whose_router_logit_is_nan_is_as_good_as_absent(broken):
     b = gpu_run_forced(less, sched, reqs, w_less, forced)
     assert np.isfinite(b[2]).all() and float(np.abs(b[2]).max()) > 0.1
     assert float(np.abs(a[2] - b[2]).max()) <= 1e-4    # the bound of the fp32 mode; the experts' sums are added in any order
+
+
+@pytest.mark.parametrize("V", [1025, 4099, 32000])
+def test_nucleus_of_rows_whose_first_entries_do_not_show_their_spread(V):
+    """The buckets take the spread of a row from its first entries; whatever those are, the answer is the oracle's."""
+    rng = np.random.default_rng(V)
+    x = rng.normal(size=(7, V)).astype(np.float32)
+    x[0] = 3.0 + 1e-4 * x[0]           # nearly equal
+    x[1, :1024] = -np.inf              # the first entries masked
+    x[2, :1024] = 9.0                  # the first entries equal and the largest
+    x[3, :1024] = -9.0                 # the first entries equal and the smallest
+    x[4] = 60.0 * x[4]                 # most entries without a weight
+    x[5, :1024] = 9.0 + 1e-3 * x[5, :1024]
+    x[6] = 2.5                         # all equal
+    for p in (0.05, 0.6, 0.999):
+        got = _sample(x, 0, p)
+        for r in range(len(x)):
+            assert got[r] == S.sample(x[r], 0, 0.8, r, 0, 3, p), (r, p)
