@@ -126,10 +126,14 @@ __device__ __forceinline__ void sample_chunk_maxima(const float* lg, int V, int 
     }
   }
 }
-// Rows whose maxima and weights are taken by all CTAs together.  Up to 32768 entries the row's own CTA is through in
-// the time of the extra phase (a 4096-entry row: 4.7 us alone, 8.1 us with the phase), and beyond 2^20 a chunk is
-// longer than a warp's span.
-__host__ __device__ __forceinline__ bool sample_split_rows(int V) { return V > 32768 && V <= SAMPLE_WARP_SPAN * SAMPLE_CHUNKS; }
+// Rows whose maxima and weights are taken by all CTAs together: those of more than 24576 entries.  Sampling in the loop by
+// the row's own CTA | with the extra phase, us, for greedy and the nucleus at 1, 20 and 100 rows:
+//   16384 entries:  8.8 |  9.1, 8.4 | 8.9, 8.1 | 10.2     62 | 52,  72 | 66,  74 | 82
+//   24576          10.9 |  9.8, 10.5 | 9.3, 10.5 | 12.5  103 | 83, 133 | 118, 137 | 144
+//   28672          12.8 |  9.6, 12.5 | 9.5, 12.5 | 12.7  119 | 97, 155 | 133, 161 | 166
+//   32000          12.9 |  9.6, 12.6 | 9.5, 12.6 | 12.8  134 | 104, 174 | 152, 178 | 187
+// (top-k as greedy, 11 us more.)  Beyond 2^20 a chunk is longer than a warp's span.
+__host__ __device__ __forceinline__ bool sample_split_rows(int V) { return V > 24576 && V <= SAMPLE_WARP_SPAN * SAMPLE_CHUNKS; }
 
 // The lowest index whose value under `z` (monotone) is `top`, the largest of the row; the whole CTA, all threads get the
 // answer.  NaN is never the largest, so a row of NaN alone has none: token 0.

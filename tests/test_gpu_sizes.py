@@ -84,7 +84,7 @@ def test_sampler_rows_around_chunk_limits(V):
 
 @pytest.mark.parametrize("V", [32768, 36864, 40004])
 def test_sampling_inside_the_loop_equals_the_oracle_on_the_loops_own_logits(V):
-    """Rows of more than 32768 entries are prepared by all CTAs (maxima, nucleus weights): greedy, top-k, nucleus and both
+    """Rows of more than 24576 entries are prepared by all CTAs (maxima, nucleus weights): greedy, top-k, nucleus and both
     together in one batch; the oracle's sampler on the captured rows gives the tokens, bit for bit."""
     model = ModelCfg(1, 256, 4, 4, 64, 256, V, dtype="fp32")
     sched = SchedCfg(max_batch=8, prefill_chunk_tokens=64, n_slots=16, max_prompt=16, max_new=6, n_blocks=32)
@@ -226,3 +226,8 @@ def test_nucleus_of_rows_whose_first_entries_do_not_show_their_spread(V):
         got = _sample(x, 0, p)
         for r in range(len(x)):
             assert got[r] == S.sample(x[r], 0, 0.8, r, 0, 3, p), (r, p)
+
+
+@pytest.mark.parametrize("V", [24576, 24580, 32000])
+def test_sampling_inside_the_loop_around_the_limit_of_shared_rows(V):
+    test_sampling_inside_the_loop_equals_the_oracle_on_the_loops_own_logits(V)
