@@ -486,14 +486,17 @@ __device__ __forceinline__ int tc_share(int total, int nb, int b) {
   const unsigned q = (unsigned)total / (unsigned)nb, r = (unsigned)total - q * (unsigned)nb;
   return (int)(q * (unsigned)b + r * (unsigned)b / (unsigned)nb);
 }
-// Token passes of a GEMM over T > 256 rows: as few as there can be, or one more where the workers of a pass then divide the
-// weight tiles evenly (no partial tiles to add up: the results are stored plainly) and the estimate is shorter.  In ns:
-// a k-block takes 40 + 1.65 per row, adding up a partial tile 20 per row, a third of that when it is stored.  QKV of the
-// 8B shape in 2 | 3 passes: 300 rows 23.8 | 21.3 us, 494 rows 27.1 | 25.6.  An extra pass elsewhere lost (1B shape,
-// 550 rows, 3 | 4: 13.8 | 16.1 us), and O and down add to the residual in any case.
-__device__ __forceinline__ int tc_passes(int T, int kblocks, int ntiles, int nb, bool accumulate) {
+// Token passes of the QKV GEMM over T > 256 rows: as few as there can be, or one more where the workers of a pass then
+// divide the weight tiles evenly (no partial tiles to add up: the results are stored plainly) and the estimate is shorter.
+// In ns: a k-block takes 40 + 1.65 per row, adding up a partial tile 20 per row, a third of that when it is stored.  8B
+// shape, fewest | one more, us: 2 | 3 passes 257 rows 22.7 | 20.9, 300 23.3 | 22.2, 352 25.7 | 22.6, 430 28.2 | 26, 494 31 |
+// 26.8; 5 | 6 passes 1100 rows 46.0 | 46.2, 1280 48.2 | 49.8; 8 | 9 passes 2000 rows 74 | 72.6.  An extra pass elsewhere lost
+// (1B shape, 550 rows, 3 | 4: 13.8 | 16.1 us), and O and down add to the residual in any case; the SwiGLU phase knows the
+// gate/up GEMM's units by the fewest passes.  Once per step, by one thread: its divisions at the start of the phase
+// cost every layer 1.3 us (513 rows 25.5 -> 26.9, 900 rows 38.5 -> 40).
+__device__ __forceinline__ int tc_passes(int T, int kblocks, int ntiles, int nb) {
   const int least = (int)((unsigned)(T + 255) >> 8), more = least + 1;
-  if (least < 2 || more > nb || accumulate) return least;
+  if (least < 2 || more > nb) return least;
   const int rows = tc_pass_rows(T, least), rows1 = tc_pass_rows(T, more);
   const int groups = (int)((unsigned)nb / (unsigned)least), groups1 = (int)((unsigned)nb / (unsigned)more);
   if (least * rows1 >= T) return least;   // the last pass would be empty
@@ -810,8 +813,7 @@ static __device__ __noinline__ void phase_gemm_tc(const DevCtx& c, const GemmArg
   const int n_tiles128 = (N + 127) / 128;
   // workers are CTAs, or CTA pairs that take two weight tiles at a time
   const int nb = PAIR ? (int)gridDim.x / 2 : (int)gridDim.x, ntiles = PAIR ? (n_tiles128 + 1) / 2 : n_tiles128;
-  // the SwiGLU phase knows the gate/up GEMM's units by the fewest passes
-  const int passes = which == GEMM_GU ? (int)((unsigned)(T + 255) >> 8) : tc_passes(T, (int)((unsigned)K >> 6), ntiles, nb, a.accumulate != 0);
+  const int passes = a.passes > 0 ? a.passes : (int)((unsigned)(T + 255) >> 8);
   const TcGeom g = tc_geom(c, T, N, K, which == GEMM_LMHEAD && lm_head_whole_tiles(c), nb, PAIR ? (int)blockIdx.x / 2 : (int)blockIdx.x,
                            ntiles, PAIR, passes);
   const int kblocks = g.kblocks;
