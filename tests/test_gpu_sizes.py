@@ -231,3 +231,9 @@ def test_nucleus_of_rows_whose_first_entries_do_not_show_their_spread(V):
 @pytest.mark.parametrize("V", [24576, 24580, 32000])
 def test_sampling_inside_the_loop_around_the_limit_of_shared_rows(V):
     test_sampling_inside_the_loop_equals_the_oracle_on_the_loops_own_logits(V)
+
+
+@pytest.mark.parametrize("rows", [37, 38, 60, 75])
+def test_decode_attention_of_short_units_in_one_round_and_two(rows):
+    # four kv heads: 148 units fill the CTAs once, more take two rounds by CTAs or one by warps; beyond 296 warps only
+    _check(MODELS[2048], [20 + i % 7 for i in range(rows)], 3, 2048, B.WEIGHTS_STREAMING)
