@@ -686,21 +686,22 @@ static __device__ int schedule_step(const DevCtx& c, unsigned long long visible)
       // sub-range made a single 2048-token row take 120 us per layer, most of it the merge
       if (S < 8) S = 8;
       while ((TT + S - 1) / S > c.att_sub_max) S *= 2;   // cannot happen with the sizes set at create
-      // Three ways to run the decode units (estimates in quarters of a tile's time, about 0.8 us of one warp):
-      // the streaming kernel cuts the flat sequence evenly (at least 8 tiles per warp, about 10 tiles' time for the
-      // ends of cut units); whole units per warp need no cuts; a CTA per part shares a unit between eight warps, and a
-      // round of it costs 22 beside its tiles (start, merge in shared memory, two barriers).  8B shape, us a layer,
-      // streaming | whole units | CTA, for rows x keys:
+      // Three ways to run the decode units.  Estimates in units of 0.2 us, fitted to the measurements below: the streaming
+      // kernel cuts the flat sequence evenly, 8 a tile with all warps at work, 52 for the ends of cut units; whole units
+      // per warp need no cuts, a tile 5 with few warps at work and 8 with all; a CTA per part shares a unit between its
+      // eight warps, 6 a tile and 17 a round (start, merge in shared memory, two barriers).
+      // 8B shape, us a layer, streaming | whole units | CTA, for rows x keys:
       //   17 x 40  17.9 | 11.9 | 10.2    17 x 300  26 | 30 | 12.7    17 x 1500  40 | 106 | 24    17 x 4000  70 | 280 | 50
-      //   24 x 40  18.0 | 11.7 | 15.2    24 x 300  26 | 29 | 19.9    24 x 1500  48 | 110 | 42    37 x 40  18.1 | 12.0 | 20.1
-      //   37 x 300  27 | 30 | 25    48 x 40  18.2 | 12.2    48 x 300  28 | 30    100 x 40  20 | 15.5    100 x 900  88 | 91
-      //   200 x 40  26.5 | 24.5    200 x 700  125 | 146    200 of 20 to 1500 keys  88 | 144
+      //   24 x 40  18.0 | 11.7 | 15.2    24 x 300  26 | 29 | 19.9    24 x 1500  48 | 110 | 42    24 x 4000  87 | 285 | 90
+      //   37 x 40  18.1 | 12.0 | 20.1    37 x 300  27 | 30 | 25      37 x 1500  58 | 126 | 52    48 x 40  18.2 | 12.2
+      //   48 x 300  28 | 30    100 x 40  20 | 15.5    100 x 300  41 | 36    100 x 900  88 | 91    200 x 40  26.5 | 24.5
+      //   200 x 300  69 | 68    200 x 700  125 | 146    200 of 20 to 1500 keys  88 | 144
       const int U = n_dec_att * c.Hkv, maxkb = s_maxkb;
-      const long long t_stream = 4 * S * ((((TT + S - 1) / S) + NW - 1) / NW) + 40;
-      const long long t_unit = 4ll * maxkb * ((U + NW - 1) / NW) + 16;
+      const long long t_stream = 8 * S * ((((TT + S - 1) / S) + NW - 1) / NW) + 52;
+      const long long t_unit = maxkb * ((U + NW - 1) / NW) * (5 * NW + 3 * min((long long)U, NW)) / NW + 14;
       int C = 0;
       if (s_C > 0) {
-        const long long t_cta = ((s_Citems + n_ctas - 1) / n_ctas) * (4ll * ((min(s_C, maxkb) + 7) / 8) + 22) + (s_C < maxkb ? 14 : 0);
+        const long long t_cta = ((s_Citems + n_ctas - 1) / n_ctas) * (6ll * ((min(s_C, maxkb) + 7) / 8) + 17) + (s_C < maxkb ? 14 : 0);
         if (t_cta <= t_stream && t_cta <= t_unit) C = s_C;
       }
       if (C == 0 && t_unit < t_stream) S = 0;
