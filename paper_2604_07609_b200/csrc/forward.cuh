@@ -377,7 +377,6 @@ struct GemmArgs {
   int fix = 0;               // FIX_*
   void* fix_out = nullptr;   // FIX_SILU: the activation rows (operand type) matching `out`
   float* fix_rowss = nullptr;// FIX_SUMSQ: per-row sums of squares to add to
-  int passes = 0;            // tensor-core path: token passes, 0 = as few as there can be
 };
 
 // One warp: GR token rows x NC output features, the 32 lanes side by side along K (four elements each), so that all

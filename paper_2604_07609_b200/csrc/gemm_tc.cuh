@@ -60,6 +60,7 @@ struct TcShared {
 };
 __shared__ __align__(8) TcShared g_tc;
 __shared__ TcState g_tc_state[FWD_THREADS / 32];
+__shared__ int g_qkv_passes;   // token passes of the step's QKV GEMMs (tc_passes)
 
 struct TcHost {
   void* d_maps = nullptr;
@@ -813,7 +814,7 @@ static __device__ __noinline__ void phase_gemm_tc(const DevCtx& c, const GemmArg
   const int n_tiles128 = (N + 127) / 128;
   // workers are CTAs, or CTA pairs that take two weight tiles at a time
   const int nb = PAIR ? (int)gridDim.x / 2 : (int)gridDim.x, ntiles = PAIR ? (n_tiles128 + 1) / 2 : n_tiles128;
-  const int passes = a.passes > 0 ? a.passes : (int)((unsigned)(T + 255) >> 8);
+  const int passes = which == GEMM_QKV ? g_qkv_passes : (int)((unsigned)(T + 255) >> 8);
   const TcGeom g = tc_geom(c, T, N, K, which == GEMM_LMHEAD && lm_head_whole_tiles(c), nb, PAIR ? (int)blockIdx.x / 2 : (int)blockIdx.x,
                            ntiles, PAIR, passes);
   const int kblocks = g.kblocks;

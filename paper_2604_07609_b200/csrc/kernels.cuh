@@ -29,7 +29,6 @@ struct StepInfo {
   bool fuse;     // RoPE and the K/V write run inside the attention
   bool nuc;      // some row samples from the nucleus of its whole row
   bool att_cta;  // the attention phase leaves the first half of the weight ring alone
-  int qkv_passes;   // token passes of the QKV GEMM
 };
 __shared__ StepInfo g_step;
 // The phases of a layer and of the output part, in order, for the current step: phase | expert << 8 | PLAN_BARRIER when a
@@ -89,10 +88,10 @@ static __device__ __noinline__ void step_begin(const DevCtx& c) {
     s.att_cta = C > 0 && npf == 0;
     if (s.dec) dec_geometry<PAIR>(c, s.T, s.R);
     const int tiles = (c.qkv_dim + 127) / 128;
-    s.qkv_passes = c.gemm_tc && threadIdx.x == 0 ? tc_passes(s.T, c.d >> 6, PAIR ? (tiles + 1) / 2 : tiles, PAIR ? (int)gridDim.x / 2 : (int)gridDim.x) : 0;
+    if (c.gemm_tc && threadIdx.x == 0)
+      g_qkv_passes = tc_passes(s.T, c.d >> 6, PAIR ? (tiles + 1) / 2 : tiles, PAIR ? (int)gridDim.x / 2 : (int)gridDim.x);
   } else {
     s.small = s.dec = s.fuse = s.att_cta = false;
-    s.qkv_passes = 0;
   }
   if (threadIdx.x < N_PHASE_TIMERS) g_phase_ns[threadIdx.x] = 0ull;
   if (threadIdx.x == 0) {
@@ -162,7 +161,6 @@ __device__ __forceinline__ void run_phase(const DevCtx& c, int phase, int layer,
       GemmArgs a{c.xn, c.w_base + c.w_off[1] + (size_t)layer * c.qkv_dim * c.d * esz, c.qkv, T, c.qkv_dim, c.d,
                  c.qkv_dim, 0};
       a.w_row0 = (long long)layer * c.qkv_dim;
-      a.passes = st.qkv_passes;
       if (c.fused) a.fix = FIX_ROPE_KV;
       gemm_dispatch<WT, PAIR>(c, a, GEMM_QKV, layer, smem);
     } break;
