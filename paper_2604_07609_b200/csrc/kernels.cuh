@@ -34,8 +34,8 @@ __shared__ StepInfo g_step;
 // The phases of a layer and of the output part, in order, for the current step: phase | expert << 8 | PLAN_BARRIER when a
 // grid barrier closes it.
 constexpr int PLAN_BARRIER = 1 << 16, PLAN_MAX = 2 * MAX_EXPERTS + 12;
-__shared__ int g_plan[2][PLAN_MAX], g_plan_n[2];
-__shared__ int g_pos[FWD_THREADS];   // layer << 16 | place in the plan: a copy per thread, so that none waits for another
+__shared__ int g_plan[2][PLAN_MAX];   // each ends with -1
+__shared__ int g_pos[FWD_THREADS];   // layer << 16 | place in the two lists: a copy per thread, so that none waits for another
 static_assert(N_PHASE_TIMERS <= 32, "copied by one warp");
 __shared__ unsigned long long g_phase_ns[N_PHASE_TIMERS];   // device time per phase kind of the open step (CTA 0)
 __shared__ unsigned long long g_phase_t;                    // when the last phase ended
@@ -62,7 +62,7 @@ __device__ __forceinline__ void make_plan(const DevCtx& c, const StepInfo& st) {
       g_plan[0][n++] = ph | PLAN_BARRIER;
     }
   }
-  g_plan_n[0] = n;
+  g_plan[0][n] = -1;
   // the output part; long rows are prepared for sampling by all CTAs, rows that sample from a whole-row nucleus with one
   // more pass over the logits
   n = 0;
@@ -71,7 +71,7 @@ __device__ __forceinline__ void make_plan(const DevCtx& c, const StepInfo& st) {
     if (phase_absorbed(c, st, ph) || ((ph == PH_SMAX || ph == PH_SNUC) && !sample_split_rows(c.V)) || (ph == PH_SNUC && !st.nuc)) continue;
     g_plan[1][n++] = ph | PLAN_BARRIER;
   }
-  g_plan_n[1] = n;
+  g_plan[1][n] = -1;
 }
 template <typename WT, bool PAIR>
 static __device__ __noinline__ void step_begin(const DevCtx& c) {
@@ -257,19 +257,23 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) blink_loop_kernel(const __grid
       // registers of their own for it.  With layer and index in registers the dispatcher spilled 100 / 212 bytes and
       // steps were longer: one row of the 1B shape 774 -> 754 us, of 8 layers of the 8B shape 911 -> 887, 64 rows of 4 layers
       // 914 -> 896, the smallest shape's 8 rows 103.7 -> 101.4.
+      // (Place and entry are two dependent reads; with list length and layer count read beside them the fp32 steps of the
+      // small configuration, which have the most phases, were 2 % longer.)
       volatile int* pos = &g_pos[threadIdx.x];
+      volatile int* plan = &g_plan[0][0];
       *pos = 0;
       while (true) {
-        const int layer = *pos >> 16, i = *pos & 0xffff, part = layer == g_ctx.L;   // the output part follows the last layer
-        if (i >= g_plan_n[part]) {
-          if (part) break;
-          *pos = (layer + 1) << 16;
+        const int at = *pos, todo = plan[at & 0xffff];
+        if (todo < 0) {   // end of the layer: the next one, or the output part, which follows the last
+          const int layer = (at >> 16) + 1, L = g_ctx.L;
+          if (layer > L) break;
+          *pos = layer << 16 | (layer == L ? PLAN_MAX : 0);
           continue;
         }
-        run_phase<WT, HD, NREP, PAIR>(g_ctx, g_plan[part][i] & 255, layer, (g_plan[part][i] >> 8) & 255, smem, true);
-        const int at = *pos, todo = *(volatile int*)&g_plan[(at >> 16) == g_ctx.L][at & 0xffff];
-        *pos = at + 1;
-        if ((todo & PLAN_BARRIER) && !end_phase(g_ctx, todo & 255)) { ok = false; break; }
+        run_phase<WT, HD, NREP, PAIR>(g_ctx, todo & 255, at >> 16, (todo >> 8) & 255, smem, true);
+        const int now = *pos, done = plan[now & 0xffff];
+        *pos = now + 1;
+        if ((done & PLAN_BARRIER) && !end_phase(g_ctx, done & 255)) { ok = false; break; }
       }
       if (!ok) break;
       if (c.stats_cap > 0 && blockIdx.x == 0 && threadIdx.x < 32) {
