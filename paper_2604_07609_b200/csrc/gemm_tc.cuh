@@ -14,7 +14,7 @@
 // covers the whole K of its tile stores its result, a partial one adds it with
 // red.global.add.f32 (the output is zeroed or already holds the residual).  With few n-tiles
 // every tile gets the same whole number of CTAs (one partial tile per CTA); with more than 256
-// token rows the passes of a weight tile go to neighbouring CTAs that walk the same range at the
+// token rows the passes of a weight tile go to CTAs that walk the same range at the
 // same time (the tile comes from HBM once, from L2 for the other passes).
 //
 // Warp roles in the 256-thread CTA: warp 0 = weight producer, warp 2 = token-tile producer, warp 1 = MMA issuer (each a
@@ -219,6 +219,24 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// The same without the wait: nothing may use the registers before tmem_wait_ld() and regs_ready().
+__device__ __forceinline__ void tmem_ld16_async(uint32_t taddr, float* v) {
+  uint32_t* r = reinterpret_cast<uint32_t*>(v);
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, "
+      "[%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void regs_ready(float (&v)[N]) {   // no use of the registers moves in front of this
+#pragma unroll
+  for (int i = 0; i < N; ++i) asm volatile("" : "+f"(v[i]));
+}
+
 // Shared-memory matrix descriptor: K-major tile of rows x 64 bf16 (128-byte rows), 128-byte
 // swizzle, 8-row groups 1024 bytes apart.
 __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr) {
@@ -326,22 +344,6 @@ __device__ __forceinline__ uint32_t idesc_bf16_pair(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
 }
 
-// The same wait for warps that have nothing else to do for most of a phase: sleep between polls.
-__device__ __forceinline__ bool mbar_wait_idle(const DevCtx& c, uint64_t* bar, uint32_t parity, volatile int* dead) {
-  if (*dead) return false;
-  const long long t0 = clock64();
-  while (!mbar_try_wait(bar, parity)) {
-    __nanosleep(200);
-    if (*dead) return false;
-    if ((unsigned long long)(clock64() - t0) > c.barrier_timeout_cycles) {
-      *dead = 1;
-      dev_fail(c, DEV_ERR_PIPE_TIMEOUT);
-      return false;
-    }
-  }
-  return true;
-}
-
 // ---- TMEM allocation for the life of the kernel ---------------------------------------------
 template <bool PAIR>
 __device__ __forceinline__ void tc_init(const DevCtx& c) {
@@ -408,31 +410,39 @@ struct TcEpiOut {
   int ilv_F;               // gate/up rows interleaved in the weight tiles: row n is output column (n & 1) * F + (n >> 1)
   __nv_bfloat16* act;      // non-null: a tile whose sums are complete goes straight to act = silu(gate) * up
 };
-// columns [c_begin, c_end) of an accumulator (token rows t_base + column) -> out; lane = weight row n
-__device__ __forceinline__ void tc_epi_columns(const TcEpiOut& e, uint32_t taddr, int n, int t_base, int c_begin, int c_end,
-                                               bool plain) {
+// Columns [c_begin, c_end) of an accumulator (token rows t_base + column) -> out; lane = weight row n.  The next group of 16 is
+// on its way from TMEM (some 400 cycles) while one is stored.  An SM stores 32 bytes a cycle to L2 and reduces 25, whatever
+// the other SMs do: 128 columns are 4100 or 5200 cycles for eight warps.  plain: stores.  Else reductions, with row_map
+// into mapped rows, scaled.  Met once a phase, beyond the instruction cache: one copy of this code for all warps.
+__device__ __forceinline__ void tc_epi_columns(const TcEpiOut& e, uint32_t taddr, int n, int t_base, int c_begin, int c_end, bool plain) {
+  if (c_begin >= c_end) return;
+  const int n_out = e.ilv_F ? (n & 1) * e.ilv_F + (n >> 1) : n;
+  float next[16];
+  tmem_ld16_async(taddr + (uint32_t)c_begin, next);
+#pragma unroll 1
   for (int c0 = c_begin; c0 < c_end; c0 += 16) {
     float v[16];
-    tmem_ld16(taddr + (uint32_t)c0, v);
-    if (n < e.N) {
-      const int t0 = t_base + c0;
-      const int nv = min(16, e.T - t0);   // token rows of this group that exist
-      const int n_out = e.ilv_F ? (n & 1) * e.ilv_F + (n >> 1) : n;
-      if (e.row_map != nullptr) {
+    tmem_wait_ld();
+    regs_ready(next);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[j] = next[j];
+    if (c0 + 16 < c_end) tmem_ld16_async(taddr + (uint32_t)(c0 + 16), next);
+    const int t0 = t_base + c0;
+    const int nv = n < e.N ? min(16, e.T - t0) : 0;   // token rows of this group that exist
+    if (e.row_map != nullptr) {
+#pragma unroll
+      for (int j = 0; j < 16; ++j)
+        if (j < nv) red_add_f32(e.out + (size_t)e.row_map[t0 + j] * e.ldo + n_out, e.row_scale[t0 + j] * v[j]);
+    } else {
+      float* o = e.out + (size_t)t0 * e.ldo + n_out;
+      if (plain) {
 #pragma unroll
         for (int j = 0; j < 16; ++j)
-          if (j < nv) red_add_f32(e.out + (size_t)e.row_map[t0 + j] * e.ldo + n_out, e.row_scale[t0 + j] * v[j]);
+          if (j < nv) o[(size_t)j * e.ldo] = v[j];
       } else {
-        float* o = e.out + (size_t)t0 * e.ldo + n_out;
-        if (plain) {
 #pragma unroll
-          for (int j = 0; j < 16; ++j)
-            if (j < nv) o[(size_t)j * e.ldo] = v[j];
-        } else {
-#pragma unroll
-          for (int j = 0; j < 16; ++j)
-            if (j < nv) red_add_f32(o + (size_t)j * e.ldo, v[j]);
-        }
+        for (int j = 0; j < 16; ++j)
+          if (j < nv) red_add_f32(o + (size_t)j * e.ldo, v[j]);
       }
     }
   }
@@ -445,6 +455,7 @@ __device__ __forceinline__ void tc_epi_silu(const TcEpiOut& e, uint32_t taddr, i
   const bool even = (n & 1) == 0;
   const int f = n >> 1;
   const int F = e.ilv_F;
+#pragma unroll 1
   for (int c0 = c_begin; c0 < c_end; c0 += 16) {
     float v[16], o[16];
     tmem_ld16(taddr + (uint32_t)c0, v);
@@ -533,17 +544,19 @@ __device__ __forceinline__ TcGeom tc_geom(const DevCtx& c, int T, int N, int K, 
     g.u1 = g.kblocks * tc_share(g.ntiles, nb, b + 1);
     return g;
   }
-  // More than 256 token rows: the passes of a weight tile go to neighbouring workers, which walk the
+  // More than 256 token rows: the passes of a weight tile go to workers of their own, which walk the
   // same (weight tile, k-block) range at the same time, so the tile comes from HBM once and from
   // L2 for the others.  One worker doing the passes in turn re-reads it after the whole grid has
-  // streamed more than L2 holds in between.
+  // streamed more than L2 holds in between.  The workers of a tile lie `groups` apart: as neighbours the steps of three
+  // passes, which run at the power limit, took 2 to 3 % longer at the same number of cycles (gate/up of 515 rows 105 us
+  // against 103, of 619 rows 104 against 102).
   if (g.passes > 1 && nb >= g.passes) {
     const int groups = (int)((unsigned)nb / (unsigned)g.passes);
     const int units = g.ntiles * g.kblocks;
     g.pdiv = 1;
-    const int grp = (int)((unsigned)b / (unsigned)g.passes);
-    if (grp < groups) {
-      g.pass_fixed = b - grp * g.passes;
+    const int pass = (int)((unsigned)b / (unsigned)groups), grp = b - pass * groups;
+    if (pass < g.passes) {
+      g.pass_fixed = pass;
       g.u0 = tc_share(units, groups, grp);
       g.u1 = tc_share(units, groups, grp + 1);
     } else {
@@ -832,67 +845,46 @@ static __device__ __noinline__ void phase_gemm_tc(const DevCtx& c, const GemmArg
     tc_produce_tokens<PAIR>(c, map_b, a.x_row0, T, g, tiles, tc, rank);
   } else if (warp == 1) {
     if (rank == 0) tc_issue_mmas<PAIR>(c, T, g, tiles, tc);   // pairs: CTA 0 issues the MMAs for both
-  } else if (warp >= 4) {
+  }
+  __syncwarp();
+  if (g.u0 < g.u1) {
+    // Warps 4-7 store the accumulators in turn.  Producers and the MMA issuer (warps 0-3) are done once the last MMA is
+    // committed and store the upper columns of the last one.
     const int q = warp & 3;  // TMEM lane quarter this warp may read
+    const bool helper = warp < 4;
     const TcEpiOut eo{a.out, (size_t)a.ldo, a.row_map, a.row_scale, T, N, ilv_F, act_direct};
     const bool accumulate = a.accumulate != 0;
     int abuf = 0;
-    for (TcSeg sg = tc_seg_first(g); sg.left > 0; tc_seg_next(g, sg)) {
+    TcSeg sg = tc_seg_first(g);
+    if (helper)
+      while (!tc_seg_is_last(sg)) {
+        tc_seg_next(g, sg);
+        abuf ^= 1;
+      }
+    for (; sg.left > 0; tc_seg_next(g, sg)) {
       const int nt = tc_my_tile<PAIR>(sg.nt, rank);
-      const int pass = sg.pass;
-      const int t_base = pass * g.pass_rows;
-      const int rows = min(g.pass_rows, T - t_base);
-      const int n_mma = (rows + 15) & ~15;
+      const int t_base = sg.pass * g.pass_rows;
+      const int n_mma = (min(g.pass_rows, T - t_base) + 15) & ~15;
       const bool plain = (sg.kb0 == 0 && sg.kb1 == kblocks) && !accumulate && eo.row_map == nullptr;
-      if (!mbar_wait(c, &g_tc.acc_full[abuf], (tc.acc_epi >> abuf) & 1u, dead)) break;
-      tc.acc_epi ^= 1u << abuf;
+      const bool direct = plain && eo.act != nullptr;
+      // (every thread waits, also when it has no columns to store, so that its parity stays in step)
+      if (!mbar_wait(c, helper ? &g_tc.acc_last : &g_tc.acc_full[abuf], helper ? tc.last_bit & 1u : (tc.acc_epi >> abuf) & 1u, dead)) break;
+      if (helper) tc.last_bit ^= 1u;
+      else tc.acc_epi ^= 1u << abuf;
       tc_fence_after();
       const uint32_t taddr = tc.tmem_base + (uint32_t)abuf * 256u + ((uint32_t)(q * 32) << 16);
-      // the upper columns of the CTA's last accumulator are left to warps 0-3
-      const int c_end = tc_seg_is_last(sg) ? tc_epi_half(n_mma) : n_mma;
-      if (plain && eo.act != nullptr) {
-        tc_epi_silu(eo, taddr, nt * 128 + q * 32 + lane, t_base, 0, c_end);
-        if (q == 0 && lane == 0 && nt * 128 < N) c.gu_done[pass * ((N + 127) / 128) + nt] = gu_stamp(c, layer);   // read after the grid barrier
-      } else {
-        tc_epi_columns(eo, taddr, nt * 128 + q * 32 + lane, t_base, 0, c_end, plain);
-      }
+      const int half = tc_seg_is_last(sg) ? tc_epi_half(n_mma) : n_mma;
+      const int c_begin = helper ? half : 0, c_end = helper ? n_mma : half;
+      if (direct) tc_epi_silu(eo, taddr, nt * 128 + q * 32 + lane, t_base, c_begin, c_end);
+      else tc_epi_columns(eo, taddr, nt * 128 + q * 32 + lane, t_base, c_begin, c_end, plain);
+      if (direct && warp == 4 && lane == 0 && nt * 128 < N) c.gu_done[sg.pass * ((N + 127) / 128) + nt] = gu_stamp(c, layer);   // read after the grid barrier
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) {
+      if (!helper && lane == 0) {
         if constexpr (PAIR) mbar_arrive_cta0(&g_tc.acc_empty[abuf]);   // the MMA issuer sits in CTA 0
         else mbar_arrive(&g_tc.acc_empty[abuf]);
       }
       abuf ^= 1;
-    }
-  }
-  if (warp < 4) {
-    // Producers and the MMA issuer are done once the last MMA is committed: their warps store
-    // the upper columns of the last accumulator.
-    __syncwarp();
-    if (g.u0 < g.u1) {
-      const uint32_t par = tc.last_bit;
-      tc.last_bit ^= 1u;
-      TcSeg sg = tc_seg_first(g);   // the last segment and its accumulator buffer
-      int last_abuf = 0;
-      while (!tc_seg_is_last(sg)) {
-        tc_seg_next(g, sg);
-        last_abuf ^= 1;
-      }
-      const int nt = tc_my_tile<PAIR>(sg.nt, rank);
-      const int pass = sg.pass;
-      const int t_base = pass * g.pass_rows;
-      const int n_mma = (min(g.pass_rows, T - t_base) + 15) & ~15;
-      const int c_begin = tc_epi_half(n_mma);
-      // every thread waits (also when it has no columns to store) so that its parity stays in step
-      if (mbar_wait_idle(c, &g_tc.acc_last, par, dead) && c_begin < n_mma) {
-        tc_fence_after();
-        const TcEpiOut eo{a.out, (size_t)a.ldo, a.row_map, a.row_scale, T, N, ilv_F, act_direct};
-        const bool plain = (sg.kb0 == 0 && sg.kb1 == kblocks) && a.accumulate == 0 && eo.row_map == nullptr;
-        const uint32_t taddr = tc.tmem_base + (uint32_t)last_abuf * 256u + ((uint32_t)(warp * 32) << 16);
-        if (plain && eo.act != nullptr) tc_epi_silu(eo, taddr, nt * 128 + warp * 32 + lane, t_base, c_begin, n_mma);
-        else tc_epi_columns(eo, taddr, nt * 128 + warp * 32 + lane, t_base, c_begin, n_mma, plain);
-        tc_fence_before();
-      }
     }
   }
   __syncwarp();
