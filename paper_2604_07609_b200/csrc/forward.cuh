@@ -508,6 +508,125 @@ static __device__ __noinline__ void phase_rope_kv(const DevCtx& c, int layer) {
   }
 }
 
+// ---- fp32 steps of little work: the element-wise phases inside the GEMMs ------------------------------------
+// A phase of the small configuration is 3 us, nearly all of it the grid barrier and the first round trip to L2, and a layer had
+// nine.  Here the norm's sum of squares is added up beside the products, by every warp for its own rows (x is read anyway;
+// the gains multiply the weights, the row's factor the result), and a warp owns pairs of features, so that it can rotate q and k
+// and write K and V (QKV), or form silu(gate) * up (gate/up), from its own sums: five phases a layer, and no final norm.
+// Steps of the small configuration: 8 rows 97 -> 72 us, 64 to 68 rows 142 -> 120.
+enum FoldMode : int { FOLD_NORM = 0, FOLD_ROPE, FOLD_SILU };
+// A sum of squares more per row and warp is up to half of the multiplications again: worth it while the largest GEMM of the layer
+// has 10^8 of them (3 us of the chip's rate, what the phases cost).
+__device__ __forceinline__ bool fold_step(const DevCtx& c, int T) {
+  return c.dtype != 0 && c.E == 0 && (long long)T * c.d * 2 * c.F <= 100000000ll;
+}
+template <int NC, int MODE>
+__device__ __forceinline__ void gemm_fold_tasks(const DevCtx& c, const float* X, const int32_t* x_rows, const float* __restrict__ W,
+                                                const float* __restrict__ gain, int M, int N, int layer) {
+  constexpr int PAIRS = MODE == FOLD_NORM ? NC : NC / 2;   // results of a task and row
+  constexpr int LPV = 32 / (SIMT_GR * NC);                 // lanes that hold the same sum
+  const int K = c.d, lane = threadIdx.x & 31, half = c.hd >> 1;
+  const int P = MODE == FOLD_NORM ? N : N / 2;
+  const int groups_n = (P + PAIRS - 1) / PAIRS, groups_m = (M + SIMT_GR - 1) / SIMT_GR;
+  const int nw = gridDim.x * (FWD_THREADS / 32);
+  for (int task = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; task < groups_m * groups_n; task += nw) {
+    const int gm = task / groups_n, gn = task - gm * groups_n;
+    const int m0 = gm * SIMT_GR, p0 = gn * PAIRS;
+    const float *w[NC], *x[SIMT_GR];
+#pragma unroll
+    for (int j = 0; j < NC; ++j) {   // clamped: rows past the end repeat
+      const int q = min(p0 + (MODE == FOLD_NORM ? j : j % PAIRS), P - 1);
+      const int n = MODE == FOLD_NORM ? q : MODE == FOLD_SILU ? q + (j < PAIRS ? 0 : P) : q / half * c.hd + q % half + (j < PAIRS ? 0 : half);
+      w[j] = W + (size_t)n * K;
+    }
+#pragma unroll
+    for (int i = 0; i < SIMT_GR; ++i) {
+      const int m = min(m0 + i, M - 1);
+      x[i] = X + (size_t)(x_rows != nullptr ? x_rows[m] : m) * K;
+    }
+    // what this lane's result needs besides, on its way with the first products
+    const int idx = lane / LPV, r = idx / NC, j = idx % NC, m = m0 + r, q = p0 + j;
+    const bool mine = lane % LPV == 0 && m < M && q < P && j < PAIRS;
+    int sm = 0, hh = 0, d0 = 0;
+    float cs = 1.f, sn = 0.f;
+    if (MODE == FOLD_ROPE && mine) {
+      hh = q / half;
+      d0 = q - hh * half;
+      sm = c.tok_slotmap[m];
+      if (hh < c.Hq + c.Hkv) {
+        const size_t at = (size_t)c.tok_pos[m] * half + d0;
+        cs = c.rope_cos[at];
+        sn = c.rope_sin[at];
+      }
+    }
+    float acc[SIMT_GR * NC], ss[SIMT_GR];
+#pragma unroll
+    for (int i = 0; i < SIMT_GR * NC; ++i) acc[i] = 0.f;
+#pragma unroll
+    for (int i = 0; i < SIMT_GR; ++i) ss[i] = 0.f;
+#pragma unroll 2
+    for (int k = lane * 4; k < K; k += 128) {
+      const float4 g = *reinterpret_cast<const float4*>(gain + k);
+      float4 wv[NC], xv[SIMT_GR];
+#pragma unroll
+      for (int t = 0; t < NC; ++t) wv[t] = *reinterpret_cast<const float4*>(w[t] + k);
+#pragma unroll
+      for (int i = 0; i < SIMT_GR; ++i) xv[i] = *reinterpret_cast<const float4*>(x[i] + k);
+#pragma unroll
+      for (int t = 0; t < NC; ++t) wv[t] = make_float4(wv[t].x * g.x, wv[t].y * g.y, wv[t].z * g.z, wv[t].w * g.w);
+#pragma unroll
+      for (int i = 0; i < SIMT_GR; ++i) {
+        ss[i] = fmaf(xv[i].x, xv[i].x, ss[i]); ss[i] = fmaf(xv[i].y, xv[i].y, ss[i]); ss[i] = fmaf(xv[i].z, xv[i].z, ss[i]); ss[i] = fmaf(xv[i].w, xv[i].w, ss[i]);
+#pragma unroll
+        for (int t = 0; t < NC; ++t) {
+          float& s = acc[i * NC + t];
+          s = fmaf(xv[i].x, wv[t].x, s); s = fmaf(xv[i].y, wv[t].y, s); s = fmaf(xv[i].z, wv[t].z, s); s = fmaf(xv[i].w, wv[t].w, s);
+        }
+      }
+    }
+    const float sq = __shfl_sync(0xffffffffu, warp_sum_many<SIMT_GR>(ss), r * (32 / SIMT_GR));
+    const float v = warp_sum_many<SIMT_GR * NC>(acc) * rsqrtf(__fdividef(sq, (float)K) + c.rms_eps);
+    if constexpr (MODE == FOLD_NORM) {
+      if (mine) c.logits[(size_t)m * N + q] = v;
+    } else {
+      const float v2 = __shfl_down_sync(0xffffffffu, v, LPV * PAIRS);   // the second feature of the pair
+      if (!mine) continue;
+      if constexpr (MODE == FOLD_SILU) {
+        reinterpret_cast<float*>(c.act)[(size_t)m * P + q] = __fdividef(v, 1.0f + __expf(-v)) * v2;
+      } else {
+        float y1 = v, y2 = v2;
+        if (hh < c.Hq + c.Hkv) {   // the fused forms of the RoPE phase
+          y1 = fmaf(v, cs, -__fmul_rn(v2, sn));
+          y2 = fmaf(v2, cs, __fmul_rn(v, sn));
+        }
+        float* dst = hh < c.Hq ? c.qkv + (size_t)m * c.qkv_dim + hh * c.hd + d0
+                               : kv_tile<float>(c, layer, hh < c.Hq + c.Hkv ? 0 : 1, sm / c.bs, (hh - c.Hq) % c.Hkv) + (size_t)(sm % c.bs) * c.hd + d0;
+        dst[0] = y1;
+        dst[half] = y2;
+      }
+    }
+  }
+}
+template <int MODE>
+static __device__ __noinline__ void phase_gemm_fold(const DevCtx& c, int layer) {
+  const int M = MODE == FOLD_NORM ? c.ss->cur_rows : c.ss->cur_T;
+  const int N = MODE == FOLD_NORM ? c.V : MODE == FOLD_ROPE ? c.qkv_dim : 2 * c.F;
+  const float* W = MODE == FOLD_NORM ? wptr<float>(c, 9) : wptr<float>(c, MODE == FOLD_ROPE ? 1 : 3) + (size_t)layer * N * c.d;
+  const float* gain = MODE == FOLD_NORM ? wptr_f(c, 8) : wptr_f(c, MODE == FOLD_ROPE ? 6 : 7) + (size_t)layer * c.d;
+  const float* X = c.h;
+  const int32_t* rows = MODE == FOLD_NORM ? c.row_tok : nullptr;
+  if (MODE == FOLD_ROPE && layer == 0) {   // the embedding rows, which also start the residual stream
+    X = wptr<float>(c, 0);
+    rows = c.tok_id;
+    for (int t = blockIdx.x; t < M; t += gridDim.x)
+      for (int i = threadIdx.x * 4; i < c.d; i += FWD_THREADS * 4)
+        *reinterpret_cast<float4*>(c.h + (size_t)t * c.d + i) = *reinterpret_cast<const float4*>(X + (size_t)rows[t] * c.d + i);
+  }
+  const long long groups = (M + SIMT_GR - 1) / SIMT_GR, warps = (long long)gridDim.x * (FWD_THREADS / 32);
+  if (groups * N >= 4 * warps) gemm_fold_tasks<4, MODE>(c, X, rows, W, gain, M, N, layer);
+  else gemm_fold_tasks<2, MODE>(c, X, rows, W, gain, M, N, layer);
+}
+
 // ---- element-wise consumers of finished GEMM output tiles (fused path) ----------------------------
 // A tile is 128 consecutive output features of rows [t0, t1); the eight warps take rows in turn and a
 // lane owns four consecutive features, so every access is one 512-byte line per row.  The fp32 sums

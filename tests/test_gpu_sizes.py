@@ -66,6 +66,15 @@ def test_prefill_steps_of_several_token_passes(tokens):
     assert int(r["its"]["n_tokens"][0]) == tokens
 
 
+@pytest.mark.parametrize("heads", [(4, 2, 64), (2, 2, 128)], ids=str)
+@pytest.mark.parametrize("rows", [1, 7, 9, 190, 191])   # 191 x 256 x 2048 products are above the limit of the folded phases
+def test_fp32_steps_with_and_without_element_wise_phases(rows, heads):
+    model = ModelCfg(2, 256, *heads, 1024, 1004, dtype="fp32")
+    sched = SchedCfg(max_batch=1, prefill_chunk_tokens=512, n_slots=16, max_prompt=rows, max_new=3, n_blocks=(rows + 18) // 16)
+    r = compare_with_oracle(model, sched, _requests([rows], 3, model.vocab), make_weights(model, 5, "cpu", random_gains=True), 1e-4)
+    assert int(r["its"]["n_tokens"][0]) == rows
+
+
 @pytest.mark.parametrize("V", [2, 5, 1023, 4099, 32768, 32772, 65540, (1 << 20) + 4])
 def test_sampler_rows_around_chunk_limits(V):
     rng = np.random.default_rng(V)
