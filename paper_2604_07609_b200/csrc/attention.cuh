@@ -12,8 +12,10 @@
 //   * prefill-chunk rows (several query tokens of one request): a dense contraction, so it
 //     runs on tensor cores (mma.sync m16n8k16, flash-attention style tiling): one CTA per
 //     (request, block of query rows, kv head), 64-key K/V tiles through a double-buffered
-//     cp.async pipeline, scores and probabilities in registers.
+//     cp.async pipeline, scores and probabilities in registers.  Requests of more than a few hundred keys
+//     go to CTA pairs instead where the shape allows (attn_pair.cuh).
 #pragma once
+#include "attn_pair.cuh"
 #include "gemm_tc.cuh"
 
 namespace blink {
@@ -33,7 +35,7 @@ __shared__ int g_att_nctx[MAX_BATCH];
 __shared__ int g_att_row[MAX_BATCH];
 // the step's scalars: like the arrays above they do not change between layers and are read from memory once per step
 struct AttStep {
-  int n_dec, TT, S, C, npf, fuse;
+  int n_dec, TT, S, C, npf, npp, fuse;
 };
 __shared__ AttStep g_att_step;
 
@@ -48,7 +50,11 @@ __device__ __forceinline__ void att_init(const DevCtx& c) {
     for (int i = 0; i < ATT_NS; ++i) mbar_init(&g_att.bar[threadIdx.x >> 5][i], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (threadIdx.x == 0) g_att.dead = 0;
+  if (threadIdx.x == 0) {
+    g_att.dead = 0;
+    ap_init();
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
   __syncthreads();
 }
 
@@ -207,7 +213,9 @@ __device__ __forceinline__ void att_tile_math(uint32_t kt, uint32_t vt, int n_va
 // slots at about half the HBM bandwidth; this form needs about 110.  Softmax statistics stay in
 // fp32 registers and are combined with shuffles.
 template <int HD, int NREP>
-__device__ __noinline__ void attn_decode_stream(const DevCtx& c, int layer, char* ring) {
+static __device__ __noinline__ void attn_decode_stream(const DevCtx& c, int layer) {
+  extern __shared__ __align__(1024) float smem[];
+  char* ring = tc_tiles(smem) + (threadIdx.x >> 5) * (ATT_NS * 2 * 16 * HD * 2);
   constexpr int RB = HD * 2;         // bytes per key row
   constexpr int TILE = 16 * RB;      // bytes of one K (or V) tile of a (block, kv head)
   constexpr int STAGE = 2 * TILE;
@@ -424,7 +432,9 @@ __device__ __noinline__ void attn_decode_stream(const DevCtx& c, int layer, char
 constexpr int ATT_NSC = 2;   // ring stages per warp here
 constexpr int ATT_CTA_OFF = 65536;   // the space before it may be receiving weights of the O projection already
 template <int HD, int NREP>
-static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer, char* base) {
+static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer) {
+  extern __shared__ __align__(1024) float smem[];
+  char* base = tc_tiles(smem) + ATT_CTA_OFF;
   constexpr int RB = HD * 2;
   constexpr int TILE = 16 * RB;
   constexpr int STAGE = 2 * TILE;
@@ -433,6 +443,7 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer, 
   constexpr unsigned FULL = 0xffffffffu;
   __shared__ float s_m[ATT_WARPS][8], s_l[ATT_WARPS][8];
   __shared__ int s_last;
+  __shared__ __align__(16) __nv_bfloat16 s_q[NREP * HD];   // the unit's queries
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int gq = lane >> 2, tq = lane & 3;
   const bool live = gq < NREP;
@@ -491,11 +502,12 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer, 
     // this warp meets the unit's last tile: the new key and value row is its business
     const bool newest = fuse && n_tiles > 0 && kb0 + w + ATT_WARPS * (n_tiles - 1) == nkb - 1;
     uint2 new_k = make_uint2(0u, 0u), new_v = make_uint2(0u, 0u);
+    // The queries by way of shared memory, a thread per rotation pair: with every warp rotating all of them for itself the
+    // code of this was 64 loads long, and met beyond the instruction cache.
     if (fuse) {
       constexpr int H2 = HD / 2;
       const int pos = n_ctx - 1;
       const float* row = c.qkv + (size_t)t_row * c.qkv_dim;
-      const float* qrow = row + (size_t)(g * NREP + (live ? gq : 0)) * HD;
       const float* cs = c.rope_cos + (size_t)pos * H2;
       const float* sn = c.rope_sin + (size_t)pos * H2;
       float4 kx = make_float4(0.f, 0.f, 0.f, 0.f), vx = kx, kc = kx, ks4 = kx;
@@ -507,18 +519,12 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer, 
         ks4 = *reinterpret_cast<const float4*>(sn + (d0 & (H2 - 1)));
       }
 #pragma unroll
-      for (int ks = 0; ks < KS / 2; ++ks) {
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const int i = ks * 16 + e * 8 + 2 * tq;   // rotation pair (i, i + HD / 2)
-          const float2 a = __ldcg(reinterpret_cast<const float2*>(qrow + i)), b = __ldcg(reinterpret_cast<const float2*>(qrow + i + H2));
-          const float2 cc = *reinterpret_cast<const float2*>(cs + i), ss = *reinterpret_cast<const float2*>(sn + i);
-          // the same fused forms as the RoPE phase
-          const uint32_t lo = pack_bf2(fmaf(a.x, cc.x, -__fmul_rn(b.x, ss.x)), fmaf(a.y, cc.y, -__fmul_rn(b.y, ss.y)));
-          const uint32_t hi = pack_bf2(fmaf(b.x, cc.x, __fmul_rn(a.x, ss.x)), fmaf(b.y, cc.y, __fmul_rn(a.y, ss.y)));
-          qf[ks][e] = live ? lo : 0u;
-          qf[ks + KS / 2][e] = live ? hi : 0u;
-        }
+      for (int k = threadIdx.x; k < NREP * H2; k += FWD_THREADS) {
+        const int i = k % H2, at = k / H2 * HD + i;
+        const float x1 = __ldcg(row + g * NREP * HD + at), x2 = __ldcg(row + g * NREP * HD + at + H2), cc = cs[i], ss = sn[i];
+        // the same fused forms as the RoPE phase
+        s_q[at] = __float2bfloat16_rn(fmaf(x1, cc, -__fmul_rn(x2, ss)));
+        s_q[at + H2] = __float2bfloat16_rn(fmaf(x2, cc, __fmul_rn(x1, ss)));
       }
       if (newest) {   // uniform over the warp
         float4 px;
@@ -541,13 +547,16 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer, 
           *reinterpret_cast<uint2*>(kv_tile<__nv_bfloat16>(c, layer, 1, b, g) + (size_t)(pos & 15) * HD + d0) = new_v;
         }
       }
-    } else {
-      const __nv_bfloat16* qrow = qb + (size_t)t_row * c.q_dim + (size_t)(g * NREP + (live ? gq : 0)) * HD;
+    } else if (threadIdx.x < NREP * HD / 8) {
+      reinterpret_cast<uint4*>(s_q)[threadIdx.x] =
+          __ldcg(reinterpret_cast<const uint4*>(qb + (size_t)t_row * c.q_dim + (size_t)g * NREP * HD) + threadIdx.x);
+    }
+    __syncthreads();
+    const uint32_t* qs = reinterpret_cast<const uint32_t*>(s_q + (live ? gq : 0) * HD + 2 * tq);
 #pragma unroll
-      for (int ks = 0; ks < KS; ++ks) {
-        qf[ks][0] = live ? *reinterpret_cast<const uint32_t*>(qrow + ks * 16 + 2 * tq) : 0u;
-        qf[ks][1] = live ? *reinterpret_cast<const uint32_t*>(qrow + ks * 16 + 8 + 2 * tq) : 0u;
-      }
+    for (int ks = 0; ks < KS; ++ks) {
+      qf[ks][0] = live ? qs[ks * 8] : 0u;
+      qf[ks][1] = live ? qs[ks * 8 + 4] : 0u;
     }
 #pragma unroll
     for (int i = 0; i < HD / 16; ++i) { o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f; }
@@ -671,7 +680,7 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32
 // Shared memory: Q [128][HD] then two stages of K [64][HD], V [64][HD]; 16-byte chunks of a row
 // are XOR-swizzled with the row index so that ldmatrix reads are conflict-free.
 template <int HD, int NREP>
-__device__ __noinline__ void attn_prefill_tile(const DevCtx& c, int layer, int item, int qblk, int g, char* smem) {
+static __device__ __noinline__ void attn_prefill_tile(const DevCtx& c, int layer, int item, int qblk, int g, char* smem) {
   constexpr int QROWS = 128 / NREP;
   constexpr int RB = HD * 2;          // bytes per row
   constexpr int CPR = RB / 16;        // 16-byte chunks per row
@@ -843,37 +852,40 @@ constexpr int att_smem_bytes() {
   return ring > cta ? (ring > tile ? ring : tile) : (cta > tile ? cta : tile);
 }
 
-// (out of line: inlined into the dispatcher it cost the decode attention 2 % at 64 and 128 rows)
+// The attention of a step is up to three pieces of work, each an entry of the step's plan of its own: called from a phase
+// function in between, the decode attention is one call deeper and saves 112 registers on its way in instead of 28, 17.8 us
+// a layer instead of 13.8 for 64 rows of 50 keys; with that function inlined into the dispatcher every phase is a little longer
+// (one-row step of the 8B shape 1.2 %).
+enum AttKind : int { ATT_PAIRS = 0, ATT_TILES, ATT_DEC_CTA, ATT_DEC_STREAM };
+
+// The step's work lists: once per step.
+__device__ __forceinline__ void att_lists(const DevCtx& c) {
+  const SchedState* ss = c.ss;
+  const int n = ss->cur_ndec;
+  if (threadIdx.x == 0) g_att_step = AttStep{n, ss->cur_TT, ss->cur_S, ss->cur_C, ss->cur_npf, ss->cur_npp, ss->cur_fuse};
+  for (int i = threadIdx.x; i <= n; i += FWD_THREADS) {
+    g_att_pre[i] = c.dec_kbpre[i];
+    if (i < n) { g_att_bslot[i] = c.dec_bslot[i]; g_att_nctx[i] = c.dec_nctx[i]; g_att_row[i] = c.dec_row[i]; }
+  }
+}
+// The prompt rows that single CTAs take.  (The pairs' units start from the first CTA, these then from the last.)
 template <int HD, int NREP>
-static __device__ __noinline__ void phase_attention_bf16(const DevCtx& c, int layer, float* smem_f) {
-  char* smem = reinterpret_cast<char*>(smem_f);
-  if (layer == 0 || c.stepped) {   // the step's work lists: once per step
-    const SchedState* ss = c.ss;
-    const int n = ss->cur_ndec;
-    if (threadIdx.x == 0) g_att_step = AttStep{n, ss->cur_TT, ss->cur_S, ss->cur_C, ss->cur_npf, ss->cur_fuse};
-    for (int i = threadIdx.x; i <= n; i += FWD_THREADS) {
-      g_att_pre[i] = c.dec_kbpre[i];
-      if (i < n) { g_att_bslot[i] = c.dec_bslot[i]; g_att_nctx[i] = c.dec_nctx[i]; g_att_row[i] = c.dec_row[i]; }
-    }
-    __syncthreads();
-  }
-  const int n_pf = g_att_step.npf * c.Hkv;
-  for (int u = blockIdx.x; u < n_pf; u += gridDim.x) {
+static __device__ __noinline__ void att_tiles(const DevCtx& c, int layer, float* smem_f) {
+  const int n_pp = g_att_step.npp, n_pf = g_att_step.npf * c.Hkv;
+  for (int u = n_pp > 0 ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x; u < n_pf; u += gridDim.x) {
     const int e = u / c.Hkv, g = u % c.Hkv;
-    attn_prefill_tile<HD, NREP>(c, layer, c.pf_item[e], c.pf_qb[e], g, smem);
+    attn_prefill_tile<HD, NREP>(c, layer, c.pf_item[n_pp + e], c.pf_qb[n_pp + e], g, reinterpret_cast<char*>(smem_f));
   }
-  const int n_dec = g_att_step.n_dec;
-  if (n_dec > 0) {
-    if (n_pf > 0) __syncthreads();   // the prefill tiles' shared memory is free
-    if (g_att_step.C > 0) {
-      attn_decode_cta<HD, NREP>(c, layer, tc_tiles(smem_f) + ATT_CTA_OFF);
-    } else {
-      const int w = threadIdx.x >> 5;
-      constexpr int STAGE = 2 * 16 * HD * 2;
-      char* ring = tc_tiles(smem_f) + w * ATT_NS * STAGE;   // 1024-byte aligned: the tiles are swizzled
-      attn_decode_stream<HD, NREP>(c, layer, ring);
-    }
-  }
+  __syncthreads();   // the tiles' shared memory is free
+}
+template <int HD, int NREP, bool PAIR>
+__device__ __forceinline__ void phase_attention_bf16(const DevCtx& c, int layer, int kind, float* smem_f) {
+  char* tiles = tc_tiles(smem_f);   // 1024-byte aligned: the tiles are swizzled
+  if (kind == ATT_DEC_STREAM) attn_decode_stream<HD, NREP>(c, layer);
+  else if (kind == ATT_DEC_CTA) attn_decode_cta<HD, NREP>(c, layer);
+  else if (kind == ATT_TILES) att_tiles<HD, NREP>(c, layer, smem_f);
+  if constexpr (PAIR && HD == 128 && NREP == 4)
+    if (kind == ATT_PAIRS) attn_prefill_pair(c, layer, tiles, g_att_step.npp);
 }
 
 }  // namespace blink

@@ -743,23 +743,28 @@ int blink_create(const blink_model_cfg* model, const blink_sched_cfg* sched, con
       TRY(dev_alloc(x, &c.dec_row, MB)); TRY(dev_alloc(x, &c.dec_bslot, MB)); TRY(dev_alloc(x, &c.dec_nctx, MB));
       TRY(dev_alloc(x, &c.dec_kbpre, MB + 1));
       TRY(dev_alloc(x, &c.pf_item, TM / 16 + MB + 1)); TRY(dev_alloc(x, &c.pf_qb, TM / 16 + MB + 1));
+      TRY(dev_alloc(x, &c.pf_unit, TM / 16 + MB + 1));
       TRY(dev_alloc(x, &c.att_ctr, (size_t)c.L)); TRY(dev_alloc(x, &c.att_cnt, MB * c.Hkv));
       {  // the KV pool as a rank-5 tensor {64 dims, hd/64 halves, n_blocks*Hkv*16 keys, K|V, L}; one box = the
          // K and V tiles of a (layer, block, kv head): {64, hd/64, 16, 2, 1}, 128-byte swizzle
         EncodeTiledFn enc = tc_encode_fn();
         const uint64_t rows = (uint64_t)c.n_blocks * c.Hkv * 16, rb = (uint64_t)c.hd * 2;
         if (!enc || rows > 0x7fffffffull) return fail(BLINK_EINVAL);
-        CUtensorMap hm;
+        CUtensorMap hm[2];
         cuuint64_t dims[5] = {64, (cuuint64_t)(c.hd / 64), rows, 2, (cuuint64_t)c.L};
         cuuint64_t strides[4] = {128, rb, rows * rb, 2 * rows * rb};
         cuuint32_t box[5] = {64, (cuuint32_t)(c.hd / 64), 16, 2, 1};
         cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-        if (enc(&hm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, c.kv_base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+        if (enc(&hm[0], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, c.kv_base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                 CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
           return fail(BLINK_ECUDA);
+        // the same as rows of head_dim (attn_pair.cuh), while their number fits a coordinate
+        hm[1] = hm[0];
+        c.att_pair = c.hd == 128 && rows * 2 * (uint64_t)c.L <= 0x7fffffffull;
+        if (c.att_pair && !tc_make_map(enc, &hm[1], c.kv_base, rows * 2 * (uint64_t)c.L, (uint64_t)c.hd, 16, true)) return fail(BLINK_ECUDA);
         void* dm = nullptr;
-        TRY(dev_alloc(x, reinterpret_cast<char**>(&dm), sizeof(CUtensorMap), false));
-        if (cudaMemcpy(dm, &hm, sizeof(CUtensorMap), cudaMemcpyHostToDevice) != cudaSuccess) return fail(BLINK_ECUDA);
+        TRY(dev_alloc(x, reinterpret_cast<char**>(&dm), sizeof(hm), false));
+        if (cudaMemcpy(dm, hm, sizeof(hm), cudaMemcpyHostToDevice) != cudaSuccess) return fail(BLINK_ECUDA);
         c.kv_map = dm;
       }
       TRY(dev_alloc(x, &c.att_part, (size_t)(2 * c.att_sub_max) * (c.n_rep * c.hd + ((2 * c.n_rep + 3) & ~3)), false));
@@ -851,6 +856,7 @@ int blink_create(const blink_model_cfg* model, const blink_sched_cfg* sched, con
     }
   }
   dec_host_setup(c, x->pair, x->grid);
+  c.att_pair = c.att_pair && x->pair;   // (pairs have four query heads per kv head)
   const void* loop_fn = x->ks.loop;
   const void* ph_fn = x->ks.phase;
   if (!loop_fn || !ph_fn) return fail(BLINK_EINVAL);

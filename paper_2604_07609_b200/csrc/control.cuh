@@ -150,6 +150,13 @@ __device__ __forceinline__ void block_exscan(int (&v)[N], int (&tot)[N]) {
   }
 }
 
+// Query rows that a CTA pair takes at a time, and the requests that go to the pairs: a unit of a pair starts and ends in 7 us
+// where one of a single CTA takes 3, but goes through 128 keys of 64 rows in 2.6 us where that takes 5 for 32.  8B shape,
+// us a layer, single CTAs | pairs, for prompts x rows: 1 x 128 10.9 | 13.1, 1 x 256 16.7 | 15.4, 1 x 400 24.4 | 17, 1 x 512 27.6 |
+// 19, 512 rows behind 3500 keys 177 | 63, 2 x 256 17.5 | 17.4, 3 x 170 15.4 | 17.5, 8 x 64 12.1 | 18.2, 24 x 20 17.0 | 34.2.
+constexpr int ATT_PAIR_ROWS = 64;
+__device__ __forceinline__ bool att_on_pairs(int keys) { return keys > 256; }
+
 __device__ __forceinline__ int32_t fake_token(unsigned long long ticket, int gen, int vocab) {
   // control-only stand-in sampler: a fixed hash of (ticket, index)
   uint32_t x = (uint32_t)(ticket * 2654435761ull + (unsigned long long)gen * 40503ull + 12345ull);
@@ -530,15 +537,17 @@ static __device__ int schedule_step(const DevCtx& c, unsigned long long visible)
   const int q_rows = 128 / c.n_rep;
   const int is_dec = f && take == 1;
   const int nkb_att = is_dec ? (new_len + c.bs - 1) / c.bs : 0;
-  const int n_qb = (f && take > 1) ? (take + q_rows - 1) / q_rows : 0;
-  // (the last two: blocks that post_step may free at most, and tickets that may end, by completion or
+  const bool on_pairs = c.att_pair && take > 1 && att_on_pairs(new_len);
+  const int n_qb = (f && take > 1 && !on_pairs) ? (take + q_rows - 1) / q_rows : 0;
+  const int n_qp = (f && on_pairs) ? (take + ATT_PAIR_ROWS - 1) / ATT_PAIR_ROWS : 0;
+  // (entries 7 and 8: blocks that post_step may free at most, and tickets that may end, by completion or
   // cancellation, for the trace space check)
-  int sc[9] = {f, take, want, sample, is_dec, nkb_att, n_qb, phase != PHASE_FREE ? have + want : 0, phase != PHASE_FREE ? 1 : 0};
-  int sc_tot[9];
+  int sc[10] = {f, take, want, sample, is_dec, nkb_att, n_qb, phase != PHASE_FREE ? have + want : 0, phase != PHASE_FREE ? 1 : 0, n_qp};
+  int sc_tot[10];
   block_exscan(sc, sc_tot);
-  const int item = sc[0], qstart = sc[1], aoff = sc[2], row = sc[3], dec_idx = sc[4], kb_pre = sc[5], pf_off = sc[6];
+  const int item = sc[0], qstart = sc[1], aoff = sc[2], row = sc[3], dec_idx = sc[4], kb_pre = sc[5], pf_off = n_qp > 0 ? sc[9] : sc_tot[9] + sc[6];
   const int n_items = sc_tot[0], T = sc_tot[1], n_alloc = sc_tot[2], n_rows = sc_tot[3], n_dec_att = sc_tot[4], tot_kb = sc_tot[5],
-            n_pf = sc_tot[6], tot_may_free = sc_tot[7], n_live = sc_tot[8];
+            n_pf = sc_tot[6], tot_may_free = sc_tot[7], n_live = sc_tot[8], n_pp = sc_tot[9];
 
   if (T == 0) return 0;  // uniform: every thread sees the same T
 
@@ -597,9 +606,10 @@ static __device__ int schedule_step(const DevCtx& c, unsigned long long visible)
         s_nkb[dec_idx] = nkb_att;
         atomicMax(&s_maxkb, nkb_att);
       }
-      for (int q = 0; q < n_qb; ++q) {   // heaviest (last) row block first
+      for (int q = 0; q < n_qb + n_qp; ++q) {   // (one of the two is zero) heaviest (last) row block first
         c.pf_item[pf_off + q] = item;
-        c.pf_qb[pf_off + q] = n_qb - 1 - q;
+        c.pf_qb[pf_off + q] = n_qb + n_qp - 1 - q;
+        if (n_qp > 0) c.pf_unit[pf_off + q] = make_int4(start, take, qstart, tid);
       }
     }
     if (tr) {
@@ -678,7 +688,7 @@ static __device__ int schedule_step(const DevCtx& c, unsigned long long visible)
       // step the CTAs reach their decode share at different times and smaller sub-ranges (up to 48
       // tiles, the later ones handed out by the counter) even that out.
       const long long NW = c.n_warps_grid;
-      const long long cap = n_pf > 0 ? 48 : 96;
+      const long long cap = n_pf + n_pp > 0 ? 48 : 96;
       const long long k = (TT + cap * NW - 1) / (cap * NW) > 1 ? (TT + cap * NW - 1) / (cap * NW) : 1;
       long long S = (TT + k * NW - 1) / (k * NW);
       // at least 8 tiles per sub-range: a cut costs a partial record, a fence and a counter update (about the time of
@@ -706,7 +716,7 @@ static __device__ int schedule_step(const DevCtx& c, unsigned long long visible)
       }
       if (C == 0 && t_unit < t_stream) S = 0;
       // a decode step of few rows: the CTA-wide kernel also applies RoPE and writes the new keys and values
-      const int fuse = c.dec_small && T <= DEC_SMALL_ROWS && n_pf == 0 && s_C > 0;
+      const int fuse = c.dec_small && T <= DEC_SMALL_ROWS && n_pf + n_pp == 0 && s_C > 0;
       if (fuse) C = s_C;
       ss->cur_fuse = fuse;
       c.dec_kbpre[n_dec_att] = tot_kb;
@@ -715,6 +725,7 @@ static __device__ int schedule_step(const DevCtx& c, unsigned long long visible)
       ss->cur_S = (int)S;
       ss->cur_C = C;
       ss->cur_npf = n_pf;
+      ss->cur_npp = n_pp;
     }
     if (tr) {
       rec[0] = TRACE_MAGIC;

@@ -99,7 +99,8 @@ struct SchedState {
   int cur_C;      // attention: > 0: decode units are shared by the warps of a CTA, C tiles per part
   int cur_fuse;   // small decode step: the attention applies RoPE and writes K and V itself
   int cur_nuc;    // some row of the step samples from the nucleus of the whole row
-  int cur_npf;    // attention: (request, query-row block) units of the multi-row requests
+  int cur_npf;    // attention: (request, query-row block) units of the multi-row requests that single CTAs take
+  int cur_npp;    // attention: units of the multi-row requests that CTA pairs take; they come first in the list
   long long cur_ctx;
   long long cur_kv;
   int cmd;
@@ -144,6 +145,7 @@ struct DevCtx {
   int control_only, start_paused, stepped, gemm_tc;
   int policy;        // BLINK_POLICY_*: chunked prefill, or whole-prompt prefill steps that pause decoding
   int n_warps_grid;  // warps of the whole grid (attention work split)
+  int att_pair;      // prompt attention may run on CTA pairs (attn_pair.cuh)
   int dec_small, dec_mid;   // decode-sized steps (up to 16, up to 128 rows) take the GEMMs with prefetched weights
   int w_streaming;   // GEMM matrices are stored as contiguous pre-swizzled 128 x 64 tiles
   long long iteration_budget;
@@ -181,6 +183,7 @@ struct DevCtx {
   // attention work lists of the step (bf16 path)
   int32_t *dec_row, *dec_bslot, *dec_nctx, *dec_kbpre;          // [MB] (+1 for the prefix) single-row requests
   int32_t *pf_item, *pf_qb;                                     // [Tmax/16 + MB + 1] multi-row tile units
+  int4* pf_unit;                                                // [Tmax/16 + MB + 1] those of CTA pairs: start, rows, first row, batch slot
   int32_t* att_ctr;      // [L] sub-range counters, zeroed every iteration
   int32_t* att_cnt;      // [MB * Hkv] parts delivered per (row, kv head) unit; self-resetting
   float* att_part;       // partial (acc, m, l) records, two per sub-range
@@ -216,7 +219,8 @@ struct DevCtx {
   float *rope_cos, *rope_sin;  // [max_pos][hd/2]
   void* kv_base;               // [L][2][n_blocks][Hkv][bs][hd] operand type
   const void* tc_maps;         // TMA descriptors of the tensor-core path (device memory)
-  const void* kv_map;          // TMA descriptor of the KV pool seen as [rows][head_dim], box 16 x 64 (device memory)
+  const void* kv_map;          // TMA descriptors of the KV pool (device memory): rank 5, box of the K and V tiles of a
+                               // (block, kv head); [rows][head_dim], box of 16 rows x 64 dims
   // diagnostics
   int32_t* trace;
   long long trace_cap;

@@ -12,6 +12,7 @@
 //     (1 KiB per k-block and CTA of a pair).  The rows are a few KiB to read; a phase and its grid barrier cost more;
 //   * steps of 17 to 128 rows bring their token tiles through a second ring by TMA, as gemm_tc.cuh does.
 // Geometry (who computes what) is that of tc_geom, taken once per step for all five GEMMs.
+// Loops of unknown length stay rolled (a quarter less code for the instruction cache of 32 KB; the times are the same).
 #pragma once
 #include "gemm_tc.cuh"
 
@@ -97,6 +98,7 @@ static __device__ __noinline__ int dec_fill_weights(const DevCtx& c, const TcGeo
   const uint64_t policy = l2_evict_first();
   const int row0 = which == GEMM_LMHEAD ? 0 : layer * dec_n(c, which);
   int i = 0, issued = 0;
+#pragma unroll 1
   for (TcSeg sg = tc_seg_first(g); sg.left > 0; tc_seg_next(g, sg)) {
     const int nt = tc_my_tile<PAIR>(sg.nt, rank);
     const int tile0 = ((row0 >> 7) + nt) * g.kblocks;
@@ -104,6 +106,7 @@ static __device__ __noinline__ int dec_fill_weights(const DevCtx& c, const TcGeo
     if (i + pieces <= first) { i += pieces; continue; }
     int kb = sg.kb0;
     if (first > i) { kb += 2 * (first - i); i = first; }
+#pragma unroll 1
     for (; kb < sg.kb1; kb += 2, ++i) {
       if (i >= first + count) return (issued << 4) | (int)fill_a;
       const int nk = min(2, sg.kb1 - kb), stage = i % DEC_STAGES;
@@ -306,11 +309,13 @@ __device__ __forceinline__ void dec_issue_mmas(const DevCtx& c, const DecPhase& 
     }
   }
   int piece = 0, bstage = 0, slot = 0, abuf = 0;
+#pragma unroll 1
   for (TcSeg sg = tc_seg_first(g); sg.left > 0; tc_seg_next(g, sg)) {
     const uint32_t d_tmem = tc.tmem_base + (uint32_t)abuf * 256u;
     if (!mbar_wait_warp(c, &g_tc.acc_empty[abuf], ((tc.acc_mma >> abuf) & 1u) ^ 1u)) return;
     tc.acc_mma ^= 1u << abuf;
     tc_fence_after();
+#pragma unroll 1
     for (int kb = sg.kb0; kb < sg.kb1; kb += 2, ++piece) {
       const int stage = piece % DEC_STAGES;
       const bool two = kb + 1 < sg.kb1;
@@ -377,6 +382,7 @@ __device__ __forceinline__ void dec_load_tokens(const DevCtx& c, const DecPhase&
     const CUtensorMap* map = &maps->act[act_id][PAIR ? 0 : 1];   // 8 or 16 rows
     if (elect_one()) {
       if (!PAIR || rank == 0) mbar_expect_tx(&g_dec.b_loaded, (PAIR ? 2u : 1u) * (uint32_t)(sl.n * sl.bytes));
+#pragma unroll 1
       for (int i = 0, kb = sl.kb_first; i < sl.n; ++i) {
         if constexpr (PAIR) tma_pair_load_2d(bt + i * sl.bytes, map, kb * 64, row0, &g_dec.b_loaded, keep_policy);
         else tma_load_2d(bt + i * sl.bytes, map, kb * 64, row0, &g_dec.b_loaded);
@@ -388,7 +394,9 @@ __device__ __forceinline__ void dec_load_tokens(const DevCtx& c, const DecPhase&
   const CUtensorMap* map = &maps->act[act_id][g.load_box];
   const int nb = min(DEC_B_STAGES, (int)((unsigned)DEC_B_BYTES / (2u * g.b_bytes)));
   int bstage = 0;
+#pragma unroll 1
   for (TcSeg sg = tc_seg_first(g); sg.left > 0; tc_seg_next(g, sg)) {
+#pragma unroll 1
     for (int kb = sg.kb0; kb < sg.kb1; kb += 2) {
       const int nk = min(2, sg.kb1 - kb);
       if (!mbar_wait_warp(c, &g_dec.b_empty[bstage], ((s.fill_b >> bstage) & 1u) ^ 1u)) return;
@@ -504,18 +512,22 @@ static __device__ __noinline__ void phase_gemm_dec(const DevCtx& c, int which, i
     if (small && (which == GEMM_O || which == GEMM_DOWN)) {   // the gains of the coming norm into L2, one line per thread
       const float* gn = which == GEMM_O ? wptr_f(c, 7) + (size_t)layer * c.d
                         : layer + 1 < c.L ? wptr_f(c, 6) + (size_t)(layer + 1) * c.d : wptr_f(c, 8);
+#pragma unroll 1
       for (int i = id * 32; i < c.d; i += n * 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(gn + i));
     }
     if (clear_gu) {
       float4* q = reinterpret_cast<float4*>(c.gu);
+#pragma unroll 1
       for (int i = id; i < T * c.F / 2; i += n) q[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     } else if (which == GEMM_O && small) {
       if (c.ss->cur_fuse) {   // (else the RoPE phase has cleared them)
         float4* q = reinterpret_cast<float4*>(c.qkv);
+#pragma unroll 1
         for (int i = id; i < T * c.qkv_dim / 4; i += n) q[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       }
       if (layer == c.L - 1 && !lm_head_whole_tiles(c)) {
         float4* q = reinterpret_cast<float4*>(c.logits);
+#pragma unroll 1
         for (int i = id; i < R * (c.V / 4); i += n) q[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       }
     }
@@ -526,6 +538,7 @@ static __device__ __noinline__ void phase_gemm_dec(const DevCtx& c, int which, i
     const TcEpiOut eo{out, (size_t)N, nullptr, nullptr, p.rows, N, (which == GEMM_GU && c.w_streaming) ? c.F : 0, nullptr};
     const int n_mma = (p.rows + 15) & ~15;
     int abuf = 0;
+#pragma unroll 1
     for (TcSeg sg = tc_seg_first(g); sg.left > 0; tc_seg_next(g, sg)) {
       const int nt = tc_my_tile<PAIR>(sg.nt, rank);
       const bool plain = sg.kb0 == 0 && sg.kb1 == g.kblocks && !accumulate;

@@ -815,7 +815,7 @@ static __device__ __noinline__ void tc_finish_tiles(const DevCtx& c, const GemmA
 }
 
 template <bool PAIR>
-static __device__ __noinline__ void phase_gemm_tc(const DevCtx& c, const GemmArgs& a, int which, int layer, float* smem_f) {
+__device__ __forceinline__ void phase_gemm_tc(const DevCtx& c, const GemmArgs& a, int which, int layer, float* smem_f) {
   const int T = a.M, N = a.N, K = a.K;
   if (T <= 0) return;  // uniform over the grid
   // gate/up on the streaming layout: weight rows are interleaved (gate f, up f, ...), and in a dense model

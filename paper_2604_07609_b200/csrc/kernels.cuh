@@ -15,12 +15,6 @@
 
 namespace blink {
 
-template <typename WT, bool PAIR>
-__device__ __forceinline__ void gemm_dispatch(const DevCtx& c, const GemmArgs& a, int which, int layer, float* smem) {
-  if (c.gemm_tc) phase_gemm_tc<PAIR>(c, a, which, layer, smem);
-  else phase_gemm_simt<WT>(a);
-}
-
 // What the phases of a step depend on besides the layer: made once per step, kept in shared memory.
 struct StepInfo {
   int T, R;      // rows of the step, rows that sample
@@ -32,9 +26,9 @@ struct StepInfo {
   bool att_cta;  // the attention phase leaves the first half of the weight ring alone
 };
 __shared__ StepInfo g_step;
-// The phases of a layer and of the output part, in order, for the current step: phase | expert << 8 | PLAN_BARRIER when a
+// The phases of a layer and of the output part, in order, for the current step: phase | (expert or AttKind) << 8 | PLAN_BARRIER when a
 // grid barrier closes it.
-constexpr int PLAN_BARRIER = 1 << 16, PLAN_MAX = 2 * MAX_EXPERTS + 12;
+constexpr int PLAN_BARRIER = 1 << 16, PLAN_MAX = 2 * MAX_EXPERTS + 14;
 __shared__ int g_plan[2][PLAN_MAX];   // each ends with -1
 __shared__ int g_pos[FWD_THREADS];   // layer << 16 | place in the two lists: a copy per thread, so that none waits for another
 static_assert(N_PHASE_TIMERS <= 32, "copied by one warp");
@@ -53,7 +47,13 @@ __device__ __forceinline__ void make_plan(const DevCtx& c, const StepInfo& st) {
   int n = 0;
   for (int ph = PH_NORM1; ph <= PH_DOWN; ++ph) {
     if (phase_absorbed(c, st, ph)) continue;
-    if (c.E > 0 && (ph == PH_GU || ph == PH_DOWN)) {
+    if (ph == PH_ATTN && c.dtype == 0) {   // (every step has rows: at least one of the three)
+      const AttStep& a = g_att_step;
+      if (a.npp > 0) g_plan[0][n++] = ph | ATT_PAIRS << 8;
+      if (a.npf > 0) g_plan[0][n++] = ph | ATT_TILES << 8;
+      if (a.n_dec > 0) g_plan[0][n++] = ph | (a.C > 0 ? ATT_DEC_CTA : ATT_DEC_STREAM) << 8;
+      g_plan[0][n - 1] |= PLAN_BARRIER;
+    } else if (c.E > 0 && (ph == PH_GU || ph == PH_DOWN)) {
       if (ph == PH_GU) g_plan[0][n++] = PH_MOE_GROUP | PLAN_BARRIER;   // routing lists and gathered rows first
       // The experts' GEMMs are independent of one another (own weights, own gathered rows; the down projections add
       // into the residual rows with reductions): one grid barrier after the last expert, none in between, so every
@@ -82,7 +82,7 @@ static __device__ __noinline__ void step_begin(const DevCtx& c) {
   s.T = __ldcg(&ss->cur_T);
   s.R = __ldcg(&ss->cur_rows);
   s.nuc = __ldcg(&ss->cur_nuc) != 0;
-  const int C = __ldcg(&ss->cur_C), npf = __ldcg(&ss->cur_npf), fuse = __ldcg(&ss->cur_fuse);
+  const int C = __ldcg(&ss->cur_C), npf = __ldcg(&ss->cur_npf) + __ldcg(&ss->cur_npp), fuse = __ldcg(&ss->cur_fuse);
   if constexpr (sizeof(WT) == 2) {
     s.small = dec_small(c, s.T);
     s.dec = dec_step(c, s.T);
@@ -90,6 +90,7 @@ static __device__ __noinline__ void step_begin(const DevCtx& c) {
     s.fold = false;
     s.att_cta = C > 0 && npf == 0;
     if (s.dec) dec_geometry<PAIR>(c, s.T, s.R);
+    att_lists(c);
     const int tiles = (c.qkv_dim + 127) / 128;
     if (c.gemm_tc && threadIdx.x == 0)
       g_qkv_passes = tc_passes(s.T, c.d >> 6, PAIR ? (tiles + 1) / 2 : tiles, PAIR ? (int)gridDim.x / 2 : (int)gridDim.x);
@@ -148,9 +149,66 @@ __device__ __forceinline__ bool end_phase(const DevCtx& c, int ph) {
   }
   return ok;
 }
+// One GEMM phase.  (A function of its own, arguments and all: built in the dispatcher, the arguments went by way of its stack and
+// it kept registers of its own there.)
+template <typename WT, bool PAIR>
+static __device__ __noinline__ void phase_gemm(const DevCtx& c, int phase, int layer, int sub, float* smem) {
+  const size_t esz = sizeof(WT);
+  const int T = g_step.T;
+  GemmArgs a;
+  int which;
+  if (phase == PH_QKV) {
+    which = GEMM_QKV;
+    a = GemmArgs{c.xn, c.w_base + c.w_off[1] + (size_t)layer * c.qkv_dim * c.d * esz, c.qkv, T, c.qkv_dim, c.d, c.qkv_dim, 0};
+    a.w_row0 = (long long)layer * c.qkv_dim;
+    if (c.fused) a.fix = FIX_ROPE_KV;
+  } else if (phase == PH_O) {
+    which = GEMM_O;
+    a = GemmArgs{c.attn, c.w_base + c.w_off[2] + (size_t)layer * c.d * c.q_dim * esz, c.h, T, c.d, c.q_dim, c.d, 1};
+    a.w_row0 = (long long)layer * c.d;
+    if (c.fused_norm) { a.fix = FIX_SUMSQ; a.fix_rowss = c.rowss_a; }
+  } else if (phase == PH_LMHEAD) {
+    which = GEMM_LMHEAD;
+    a = GemmArgs{c.xs, c.w_base + c.w_off[9], c.logits, g_step.R, c.V, c.d, c.V, 0};
+  } else {
+    // the dense FFN, or expert `sub` on the rows routed to it (gathered, contiguous from moe_off[sub])
+    const int off = c.E > 0 ? c.moe_off[sub] : 0, cnt = c.E > 0 ? c.moe_off[sub + 1] - off : T;
+    const long long we = c.E > 0 ? (long long)layer * c.E + sub : layer;
+    if (phase == PH_GU) {
+      which = GEMM_GU;
+      a = GemmArgs{reinterpret_cast<const char*>(c.E > 0 ? c.xg : c.xn) + (size_t)off * c.d * esz, c.w_base + c.w_off[3] + (size_t)we * 2 * c.F * c.d * esz,
+                   c.gu + (size_t)off * 2 * c.F, cnt, 2 * c.F, c.d, 2 * c.F, 0};
+      a.w_row0 = we * 2 * c.F;
+      if (c.fused) { a.fix = FIX_SILU; a.fix_out = reinterpret_cast<char*>(c.act) + (size_t)off * c.F * esz; }
+    } else {
+      which = GEMM_DOWN;
+      a = GemmArgs{reinterpret_cast<const char*>(c.act) + (size_t)off * c.F * esz, c.w_base + c.w_off[4] + (size_t)we * c.d * c.F * esz, c.h, cnt, c.d, c.F,
+                   c.d, 1};
+      a.w_row0 = we * c.d;
+      if (c.E > 0) {   // result row i belongs to token moe_tok[off + i], weighted by its gate
+        a.row_map = c.moe_tok + off;
+        a.row_scale = c.moe_gate + off;
+      } else if (c.fused_norm) {
+        a.fix = FIX_SUMSQ;
+        a.fix_rowss = c.rowss_b;
+      }
+    }
+    a.x_row0 = off;
+  }
+  if constexpr (PAIR) {   // (on the tensor cores, and without fused epilogues)
+    phase_gemm_tc<PAIR>(c, a, which, layer, smem);
+  } else {
+    if constexpr (sizeof(WT) == 2) {
+      if (c.gemm_tc) {
+        phase_gemm_tc<PAIR>(c, a, which, layer, smem);
+        return;
+      }
+    }
+    phase_gemm_simt<WT>(a);
+  }
+}
 template <typename WT, int HD, int NREP, bool PAIR>
 __device__ __forceinline__ void run_phase(const DevCtx& c, int phase, int layer, int sub, float* smem, bool chain) {
-  const size_t esz = sizeof(WT);
   const StepInfo& st = g_step;
   const int T = st.T;
   if constexpr (sizeof(WT) == 2) {
@@ -165,79 +223,29 @@ __device__ __forceinline__ void run_phase(const DevCtx& c, int phase, int layer,
   }
   switch (phase) {
     case PH_NORM1:
-      if (c.fused_norm && layer > 0) phase_norm_apply<WT>(c, layer, 0, T);
-      else phase_norm<WT>(c, layer, 0);
+      if constexpr (!PAIR)
+        if (c.fused_norm && layer > 0) { phase_norm_apply<WT>(c, layer, 0, T); break; }
+      phase_norm<WT>(c, layer, 0);
       break;
-    case PH_QKV: {
-      GemmArgs a{c.xn, c.w_base + c.w_off[1] + (size_t)layer * c.qkv_dim * c.d * esz, c.qkv, T, c.qkv_dim, c.d,
-                 c.qkv_dim, 0};
-      a.w_row0 = (long long)layer * c.qkv_dim;
-      if (c.fused) a.fix = FIX_ROPE_KV;
-      gemm_dispatch<WT, PAIR>(c, a, GEMM_QKV, layer, smem);
-    } break;
     case PH_ROPE: phase_rope_kv<WT>(c, layer); break;
     case PH_ATTN:
-      if constexpr (sizeof(WT) == 2) phase_attention_bf16<HD, NREP>(c, layer, smem);
+      if constexpr (sizeof(WT) == 2) phase_attention_bf16<HD, NREP, PAIR>(c, layer, sub, smem);
       else phase_attention<WT, HD, NREP>(c, layer, smem);
 
       break;
-    case PH_O: {
-      GemmArgs a{c.attn, c.w_base + c.w_off[2] + (size_t)layer * c.d * c.q_dim * esz, c.h, T, c.d, c.q_dim, c.d, 1};
-      a.w_row0 = (long long)layer * c.d;
-      if (c.fused_norm) { a.fix = FIX_SUMSQ; a.fix_rowss = c.rowss_a; }
-      gemm_dispatch<WT, PAIR>(c, a, GEMM_O, layer, smem);
-    } break;
     case PH_NORM2:
-      if (c.fused_norm) phase_norm_apply<WT>(c, layer, 1, T);
-      else phase_norm<WT>(c, layer, 1);
+      if constexpr (!PAIR)
+        if (c.fused_norm) { phase_norm_apply<WT>(c, layer, 1, T); break; }
+      phase_norm<WT>(c, layer, 1);
       break;
-    case PH_GU: {
-      if (c.E == 0) {
-        GemmArgs a{c.xn, c.w_base + c.w_off[3] + (size_t)layer * 2 * c.F * c.d * esz, c.gu, T, 2 * c.F, c.d, 2 * c.F, 0};
-        a.w_row0 = (long long)layer * 2 * c.F;
-        if (c.fused) { a.fix = FIX_SILU; a.fix_out = c.act; }
-        gemm_dispatch<WT, PAIR>(c, a, GEMM_GU, layer, smem);
-      } else {
-        // expert `sub` on the rows routed to it (gathered, contiguous from moe_off[sub])
-        const int off = c.moe_off[sub], cnt = c.moe_off[sub + 1] - off;
-        const long long we = (long long)layer * c.E + sub;
-        GemmArgs a{reinterpret_cast<const char*>(c.xg) + (size_t)off * c.d * esz, c.w_base + c.w_off[3] + (size_t)we * 2 * c.F * c.d * esz,
-                   c.gu + (size_t)off * 2 * c.F, cnt, 2 * c.F, c.d, 2 * c.F, 0};
-        a.x_row0 = off;
-        a.w_row0 = we * 2 * c.F;
-        if (c.fused) { a.fix = FIX_SILU; a.fix_out = reinterpret_cast<char*>(c.act) + (size_t)off * c.F * esz; }
-        gemm_dispatch<WT, PAIR>(c, a, GEMM_GU, layer, smem);
-      }
-    } break;
     case PH_SILU:
       phase_silu_mul<WT>(c, layer, smem);
       break;
-    case PH_DOWN: {
-      if (c.E == 0) {
-        GemmArgs a{c.act, c.w_base + c.w_off[4] + (size_t)layer * c.d * c.F * esz, c.h, T, c.d, c.F, c.d, 1};
-        a.w_row0 = (long long)layer * c.d;
-        if (c.fused_norm) { a.fix = FIX_SUMSQ; a.fix_rowss = c.rowss_b; }
-        gemm_dispatch<WT, PAIR>(c, a, GEMM_DOWN, layer, smem);
-      } else {
-        const int off = c.moe_off[sub], cnt = c.moe_off[sub + 1] - off;
-        const long long we = (long long)layer * c.E + sub;
-        GemmArgs a{reinterpret_cast<const char*>(c.act) + (size_t)off * c.F * esz, c.w_base + c.w_off[4] + (size_t)we * c.d * c.F * esz,
-                   c.h, cnt, c.d, c.F, c.d, 1};
-        a.x_row0 = off;
-        a.w_row0 = we * c.d;
-        a.row_map = c.moe_tok + off;     // result row i belongs to token moe_tok[off + i], weighted by its gate
-        a.row_scale = c.moe_gate + off;
-        gemm_dispatch<WT, PAIR>(c, a, GEMM_DOWN, layer, smem);
-      }
-    } break;
     case PH_MOE_GROUP: phase_moe_group<WT>(c, smem); break;
     case PH_FNORM:
       phase_final_norm<WT>(c);
       break;
-    case PH_LMHEAD: {
-      GemmArgs a{c.xs, c.w_base + c.w_off[9], c.logits, c.ss->cur_rows, c.V, c.d, c.V, 0};
-      gemm_dispatch<WT, PAIR>(c, a, GEMM_LMHEAD, 0, smem);
-    } break;
+    case PH_QKV: case PH_O: case PH_GU: case PH_DOWN: case PH_LMHEAD: phase_gemm<WT, PAIR>(c, phase, layer, sub, smem); break;
     case PH_SMAX: phase_sample_max(c); break;
     case PH_SNUC: phase_sample_weights(c, smem); break;
     case PH_SAMPLE: phase_sample(c, smem); break;
@@ -314,7 +322,12 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) blink_phase_kernel(const __gri
   if constexpr (PAIR) cluster_sync_all();
   else __syncthreads();
   step_begin<WT, PAIR>(c);
-  if (!phase_absorbed(c, g_step, phase)) run_phase<WT, HD, NREP, PAIR>(c, phase, layer, sub, smem, false);
+  if (phase == PH_ATTN && sizeof(WT) == 2) {   // all of its pieces
+    for (int i = 0; g_plan[0][i] >= 0; ++i)
+      if ((g_plan[0][i] & 255) == PH_ATTN) run_phase<WT, HD, NREP, PAIR>(c, phase, layer, (g_plan[0][i] >> 8) & 255, smem, false);
+  } else if (!phase_absorbed(c, g_step, phase)) {
+    run_phase<WT, HD, NREP, PAIR>(c, phase, layer, sub, smem, false);
+  }
   tc_fini<PAIR>(c);
 }
 

@@ -75,6 +75,42 @@ def test_fp32_steps_with_and_without_element_wise_phases(rows, heads):
     assert int(r["its"]["n_tokens"][0]) == rows
 
 
+# more than 256 keys: prompt attention on CTA pairs, in units of 64 rows and tiles of 128 keys
+@pytest.mark.parametrize("prompts, chunk", [([256], 512), ([257], 512), ([383, 385], 512), ([1026], 512), ([600, 40, 300], 256),
+                                            ([1500, 17, 800], 700)], ids=str)
+def test_prompt_attention_around_units_and_tiles(prompts, chunk):
+    # (the probabilities' rounding of the test above; logits of d = 512)
+    r = _check(ModelCfg(1, 512, 8, 2, 128, 256, 1024), prompts, 2, chunk, B.WEIGHTS_STREAMING, relative=False)
+    assert r["err_plain"] <= 2e-2
+
+
+def test_prompt_attention_of_more_units_than_pairs():
+    # 8 prompts x 5 units x 2 kv heads on 74 pairs, two layers: some pairs have a second unit in every layer
+    _check(ModelCfg(2, 512, 8, 2, 128, 256, 1024), [290, 300, 310, 320, 257, 319, 288, 305], 2, 4096, B.WEIGHTS_STREAMING, relative=False)
+
+
+def test_prompt_attention_leaves_the_pools_old_contents_alone():
+    """Keys and values beyond a request's last token are whatever the pool held, NaN here."""
+    model = ModelCfg(1, 512, 8, 2, 128, 256, 1024)
+    sched = SchedCfg(max_batch=2, prefill_chunk_tokens=512, n_slots=16, max_prompt=512, max_new=2, n_blocks=80)
+    weights = make_weights(model, 5, "cuda")
+    out = []
+    for fill in (0, 0xFF):
+        kv = torch.full((sched.n_blocks * B.kv_bytes_per_block(model, 16),), fill, dtype=torch.uint8, device="cuda")
+        logits = torch.zeros(4, model.vocab, device="cuda")
+        torch.cuda.synchronize()
+        eng = B.Blink(model, sched, weights, kv, exec_mode=B.EXEC_MANUAL, logits_capture=logits)
+        for r in _requests([270, 491], 2, model.vocab):
+            eng.submit_request(r, forced_tokens=np.zeros(2, np.int32))
+        eng.blink_run(4)
+        eng.drain(4)
+        eng.blink_destroy()
+        out.append(logits)
+    assert torch.isfinite(out[1]).all()
+    # split-K sums in another order move a 16-bit rounding here and there: 2^-8 of a value of up to sigma 0.45 x 4
+    assert (out[0] - out[1]).abs().max() <= 2 ** -8 * 1.8
+
+
 @pytest.mark.parametrize("V", [2, 5, 1023, 4099, 32768, 32772, 65540, (1 << 20) + 4])
 def test_sampler_rows_around_chunk_limits(V):
     rng = np.random.default_rng(V)
