@@ -35,7 +35,7 @@ __shared__ int g_att_nctx[MAX_BATCH];
 __shared__ int g_att_row[MAX_BATCH];
 // the step's scalars: like the arrays above they do not change between layers and are read from memory once per step
 struct AttStep {
-  int n_dec, TT, S, C, npf, npp, fuse;
+  int n_dec, TT, S, C, half, npf, npp, fuse;   // (half: the units of C are for half CTAs)
 };
 __shared__ AttStep g_att_step;
 
@@ -425,13 +425,21 @@ static __device__ __noinline__ void attn_decode_stream(const DevCtx& c, int laye
 // warp, or cuts it and pays a record, a fence, a counter and a merge by one warp for every cut, so that one row of
 // 300 keys took 22 us and one of 4000 keys 51 us per layer, nearly all of it latency.  Here the eight warps of a
 // CTA share a part of a unit (C tiles, no part crosses units): their tiles are in flight at once, their sums are
-// merged in shared memory, and only units of more than C tiles leave records, merged by the whole last CTA.
+// merged in shared memory, and only units of more than C tiles leave records, merged by the whole last CTA.  Where there
+// are more units than CTAs, half CTAs take one each instead of CTAs two in turn: 8B shape, us a layer, 20 rows of 160 keys 15.5 ->
+// 12.4, 24 of 300 19.7 -> 15.3, 37 of 100 20.1 -> 15.5, 37 of 300 24.3 -> 19.2.
 // In steps of at most 16 rows without prompt rows this kernel also takes over RoPE and the K/V write (a phase and a grid
 // barrier less): every CTA rotates the queries it needs, and the warp that meets a unit's last tile computes the new key
 // and value row, writes it to the pool and into its copy of the tile.
 constexpr int ATT_NSC = 2;   // ring stages per warp here
 constexpr int ATT_CTA_OFF = 65536;   // the space before it may be receiving weights of the O projection already
-template <int HD, int NREP>
+struct AttCta {
+  float m[ATT_WARPS][8], l[ATT_WARPS][8];   // maxima and sums of the warps
+  int last[2];
+};
+__shared__ AttCta g_att_cta;
+// GW: warps that share a unit, all of the CTA's or half of them (two groups, which go their own ways).
+template <int HD, int NREP, int GW>
 static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer) {
   extern __shared__ __align__(1024) float smem[];
   char* base = tc_tiles(smem) + ATT_CTA_OFF;
@@ -441,15 +449,24 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer) 
   constexpr int KS = HD / 16;
   constexpr int REC = NREP * HD + ((2 * NREP + 3) & ~3);
   constexpr unsigned FULL = 0xffffffffu;
-  __shared__ float s_m[ATT_WARPS][8], s_l[ATT_WARPS][8];
-  __shared__ int s_last;
-  __shared__ __align__(16) __nv_bfloat16 s_q[NREP * HD];   // the unit's queries
+  constexpr int GT = GW * 32, NG = ATT_WARPS / GW;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int grp = NG == 1 ? 0 : w / GW, w0 = grp * GW, wg = w - w0, tg = (int)threadIdx.x - grp * GT;
+  const int n_groups = NG * (int)gridDim.x;
+  auto group_sync = [&]() {
+    if constexpr (NG == 1) __syncthreads();
+    else asm volatile("bar.sync %0, %1;" ::"r"(4 + grp), "n"(GT) : "memory");
+  };
+  float(*s_m)[8] = g_att_cta.m + w0;
+  float(*s_l)[8] = g_att_cta.l + w0;
+  // the unit's queries, in what the control plane uses between the steps
+  static_assert(NG * NREP * HD * 2 <= (int)sizeof(g_ctl), "no room for the queries");
+  __nv_bfloat16* s_q = reinterpret_cast<__nv_bfloat16*>(&g_ctl) + grp * NREP * HD;
   const int gq = lane >> 2, tq = lane & 3;
   const bool live = gq < NREP;
   const int n_dec = g_att_step.n_dec, C = g_att_step.C, Hkv = c.Hkv;
   char* ring = base + w * ATT_NSC * STAGE;
-  float* s_o = reinterpret_cast<float*>(base);   // a warp's sums [NREP][HD] go where its ring stages were
+  float* s_o = reinterpret_cast<float*>(base + w0 * ATT_NSC * STAGE);   // a warp's sums [NREP][HD] go where its ring stages were
   constexpr int S_O = ATT_NSC * STAGE / 4;       // floats from one warp's sums to the next
   static_assert(NREP * HD * 4 <= ATT_NSC * STAGE, "a warp's sums exceed its stages");
   const bool fuse = g_att_step.fuse != 0;
@@ -463,7 +480,7 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer) 
   uint32_t par = g_att_par[w];
 
   // items in unit order; prefill tiles of a step sit on the first CTAs, so the decode items start from the last
-  for (int item = (int)gridDim.x - 1 - (int)blockIdx.x; ; item += gridDim.x) {   // uniform over the CTA
+  for (int item = (int)gridDim.x - 1 - (int)blockIdx.x + grp * (int)gridDim.x; ; item += n_groups) {   // uniform over the group
     int d = 0, rest = item, nkb = 0, ns = 1;
     for (; d < n_dec; ++d) {
       nkb = g_att_pre[d + 1] - g_att_pre[d];
@@ -474,18 +491,18 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer) 
     if (d >= n_dec) break;
     const int g = rest / ns, part = rest - g * ns;
     const int kb0 = part * C, kb1 = min(nkb, kb0 + C);
-    const int n_tiles = kb0 + w < kb1 ? (kb1 - kb0 - w + ATT_WARPS - 1) / ATT_WARPS : 0;   // kb0 + w, + 8, ...
+    const int n_tiles = kb0 + wg < kb1 ? (kb1 - kb0 - wg + GW - 1) / GW : 0;   // kb0 + wg, + GW, ...
     const int t_row = g_att_row[d], n_ctx = g_att_nctx[d];
     const int32_t* table = c.block_table + (size_t)g_att_bslot[d] * c.max_blocks_seq;
     // block ids of the warp's first 32 tiles, one per lane; the first item's are kept from layer to layer
-    const bool first = item < (int)gridDim.x;
+    const bool first = item < n_groups;
     int blk = g_att_blk[threadIdx.x];
     if (!(first && layer > 0 && !c.stepped)) {
-      blk = lane < n_tiles ? table[kb0 + w + ATT_WARPS * lane] : 0;
+      blk = lane < n_tiles ? table[kb0 + wg + GW * lane] : 0;
       if (first) g_att_blk[threadIdx.x] = blk;
     }
     auto issue = [&](int i) {
-      if (i >= 32 && (i & 31) == 0) blk = i + lane < n_tiles ? table[kb0 + w + ATT_WARPS * (i + lane)] : 0;
+      if (i >= 32 && (i & 31) == 0) blk = i + lane < n_tiles ? table[kb0 + wg + GW * (i + lane)] : 0;
       const int b = __shfl_sync(FULL, blk, i & 31);
       if (lane == 0) {
         const int s = i % ATT_NSC;
@@ -500,7 +517,7 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer) 
     float o[HD / 16][4];
     float m2[2] = {-INFINITY, -INFINITY}, l2[2] = {0.f, 0.f};
     // this warp meets the unit's last tile: the new key and value row is its business
-    const bool newest = fuse && n_tiles > 0 && kb0 + w + ATT_WARPS * (n_tiles - 1) == nkb - 1;
+    const bool newest = fuse && n_tiles > 0 && kb0 + wg + GW * (n_tiles - 1) == nkb - 1;
     uint2 new_k = make_uint2(0u, 0u), new_v = make_uint2(0u, 0u);
     // The queries by way of shared memory, a thread per rotation pair: with every warp rotating all of them for itself the
     // code of this was 64 loads long, and met beyond the instruction cache.
@@ -519,7 +536,7 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer) 
         ks4 = *reinterpret_cast<const float4*>(sn + (d0 & (H2 - 1)));
       }
 #pragma unroll
-      for (int k = threadIdx.x; k < NREP * H2; k += FWD_THREADS) {
+      for (int k = tg; k < NREP * H2; k += GT) {
         const int i = k % H2, at = k / H2 * HD + i;
         const float x1 = __ldcg(row + g * NREP * HD + at), x2 = __ldcg(row + g * NREP * HD + at + H2), cc = cs[i], ss = sn[i];
         // the same fused forms as the RoPE phase
@@ -547,11 +564,11 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer) 
           *reinterpret_cast<uint2*>(kv_tile<__nv_bfloat16>(c, layer, 1, b, g) + (size_t)(pos & 15) * HD + d0) = new_v;
         }
       }
-    } else if (threadIdx.x < NREP * HD / 8) {
-      reinterpret_cast<uint4*>(s_q)[threadIdx.x] =
-          __ldcg(reinterpret_cast<const uint4*>(qb + (size_t)t_row * c.q_dim + (size_t)g * NREP * HD) + threadIdx.x);
+    } else if (tg < NREP * HD / 8) {
+      reinterpret_cast<uint4*>(s_q)[tg] =
+          __ldcg(reinterpret_cast<const uint4*>(qb + (size_t)t_row * c.q_dim + (size_t)g * NREP * HD) + tg);
     }
-    __syncthreads();
+    group_sync();
     const uint32_t* qs = reinterpret_cast<const uint32_t*>(s_q + (live ? gq : 0) * HD + 2 * tq);
 #pragma unroll
     for (int ks = 0; ks < KS; ++ks) {
@@ -565,7 +582,7 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer) 
       if (!__all_sync(FULL, mbar_wait(c, &bars[s], (par >> s) & 1u, dead))) break;
       par ^= 1u << s;
       char* st = ring + s * STAGE;
-      const int n_valid = min(16, n_ctx - (kb0 + w + ATT_WARPS * i) * 16);   // >= 1
+      const int n_valid = min(16, n_ctx - (kb0 + wg + GW * i) * 16);   // >= 1
       if (n_valid < 16) {   // the tail of the last block holds whatever the pool held: clear those V rows (0 x NaN)
         uint4* vg = reinterpret_cast<uint4*>(st + TILE + n_valid * RB);
         for (int k = lane; k < (16 - n_valid) * RB / 16; k += 32) vg[k] = make_uint4(0u, 0u, 0u, 0u);
@@ -597,22 +614,22 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer) 
     for (int e = 0; e < 2; ++e) {
       if (h0 + e < NREP) {
         if (n_tiles > 0) {
-          float* ow = s_o + w * S_O + (h0 + e) * HD;
+          float* ow = s_o + wg * S_O + (h0 + e) * HD;
 #pragma unroll
           for (int i = 0; i < HD / 16; ++i) {
             ow[16 * i + gq] = o[i][e];
             ow[16 * i + 8 + gq] = o[i][2 + e];
           }
         }
-        if (gq == 0) { s_m[w][h0 + e] = m2[e]; s_l[w][h0 + e] = e ? lt1 : lt0; }
+        if (gq == 0) { s_m[wg][h0 + e] = m2[e]; s_l[wg][h0 + e] = e ? lt1 : lt0; }
       }
     }
-    __syncthreads();
+    group_sync();
     // merge the warps: a thread takes two consecutive dims of a head at a time
-    const int n_warps = min(ATT_WARPS, kb1 - kb0);   // warps 0 .. n_warps - 1 had tiles
+    const int n_warps = min(GW, kb1 - kb0);   // the first n_warps of the group had tiles
     float* rec = c.att_part + (size_t)item * REC;
     __nv_bfloat16* obase = out + (size_t)t_row * c.q_dim + (size_t)(g * NREP) * HD;
-    for (int i2 = threadIdx.x; i2 < NREP * HD / 2; i2 += FWD_THREADS) {
+    for (int i2 = tg; i2 < NREP * HD / 2; i2 += GT) {
       const int h = i2 * 2 / HD;
       float M = -INFINITY;
       for (int k = 0; k < n_warps; ++k) M = fmaxf(M, s_m[k][h]);
@@ -636,13 +653,13 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer) 
     if (ns > 1) {
       const int unit = d * Hkv + g;
       __threadfence();
-      __syncthreads();
-      if (threadIdx.x == 0) s_last = atomicAdd(&c.att_cnt[unit], 1) == ns - 1;
-      __syncthreads();
-      if (s_last) {   // this CTA delivered the last part: merge in part order (records of a unit are consecutive)
+      group_sync();
+      if (tg == 0) g_att_cta.last[grp] = atomicAdd(&c.att_cnt[unit], 1) == ns - 1;
+      group_sync();
+      if (g_att_cta.last[grp]) {   // this group delivered the last part: merge in part order (records of a unit are consecutive)
         __threadfence();
         const float* r0 = c.att_part + (size_t)(item - part) * REC;
-        for (int i2 = threadIdx.x; i2 < NREP * HD / 2; i2 += FWD_THREADS) {
+        for (int i2 = tg; i2 < NREP * HD / 2; i2 += GT) {
           const int h = i2 * 2 / HD;
           float M = -INFINITY;
 #pragma unroll 8
@@ -660,12 +677,12 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer) 
           const float inv = __fdividef(1.0f, den);
           *reinterpret_cast<uint32_t*>(obase + i2 * 2) = pack_bf2(num.x * inv, num.y * inv);
         }
-        if (threadIdx.x == 0) c.att_cnt[unit] = 0;
+        if (tg == 0) c.att_cnt[unit] = 0;
       }
     }
     // the sums are free for the next item, and before copies land there again
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
+    group_sync();
   }
   if (lane == 0) g_att_par[w] = par;
 }
@@ -856,13 +873,13 @@ constexpr int att_smem_bytes() {
 // function in between, the decode attention is one call deeper and saves 112 registers on its way in instead of 28, 17.8 us
 // a layer instead of 13.8 for 64 rows of 50 keys; with that function inlined into the dispatcher every phase is a little longer
 // (one-row step of the 8B shape 1.2 %).
-enum AttKind : int { ATT_PAIRS = 0, ATT_TILES, ATT_DEC_CTA, ATT_DEC_STREAM };
+enum AttKind : int { ATT_PAIRS = 0, ATT_TILES, ATT_DEC_CTA, ATT_DEC_HALF, ATT_DEC_STREAM };
 
 // The step's work lists: once per step.
 __device__ __forceinline__ void att_lists(const DevCtx& c) {
   const SchedState* ss = c.ss;
   const int n = ss->cur_ndec;
-  if (threadIdx.x == 0) g_att_step = AttStep{n, ss->cur_TT, ss->cur_S, ss->cur_C, ss->cur_npf, ss->cur_npp, ss->cur_fuse};
+  if (threadIdx.x == 0) g_att_step = AttStep{n, ss->cur_TT, ss->cur_S, ss->cur_C, ss->cur_half, ss->cur_npf, ss->cur_npp, ss->cur_fuse};
   for (int i = threadIdx.x; i <= n; i += FWD_THREADS) {
     g_att_pre[i] = c.dec_kbpre[i];
     if (i < n) { g_att_bslot[i] = c.dec_bslot[i]; g_att_nctx[i] = c.dec_nctx[i]; g_att_row[i] = c.dec_row[i]; }
@@ -882,7 +899,8 @@ template <int HD, int NREP, bool PAIR>
 __device__ __forceinline__ void phase_attention_bf16(const DevCtx& c, int layer, int kind, float* smem_f) {
   char* tiles = tc_tiles(smem_f);   // 1024-byte aligned: the tiles are swizzled
   if (kind == ATT_DEC_STREAM) attn_decode_stream<HD, NREP>(c, layer);
-  else if (kind == ATT_DEC_CTA) attn_decode_cta<HD, NREP>(c, layer);
+  else if (kind == ATT_DEC_CTA) attn_decode_cta<HD, NREP, ATT_WARPS>(c, layer);
+  else if (kind == ATT_DEC_HALF) attn_decode_cta<HD, NREP, ATT_WARPS / 2>(c, layer);
   else if (kind == ATT_TILES) att_tiles<HD, NREP>(c, layer, smem_f);
   if constexpr (PAIR && HD == 128 && NREP == 4)
     if (kind == ATT_PAIRS) attn_prefill_pair(c, layer, tiles, g_att_step.npp);

@@ -37,7 +37,6 @@ struct AttPairShared {
     int r0;         // first of the unit's query rows in it
     int ids[32];    // block ids of its first four tiles
   } unit[2];        // the first unit, which is the same in all layers of a step, and any other
-  float2 ml[2][128];                   // maximum and sum of every row per stream
 };
 __shared__ __align__(16) AttPairShared g_ap;
 
@@ -381,13 +380,15 @@ static __device__ __noinline__ void attn_prefill_pair(const DevCtx& c, int layer
       }
     }
     // merge the streams: each of the two threads of a row takes half of the dims
-    g_ap.ml[s][q * 32 + lane] = make_float2(m, l);
+    // (maximum and sum of every row go where the stream's keys were: its scores are complete)
+    float2* ml = reinterpret_cast<float2*>(base + AP_K) + q * 32 + lane;
+    ml[s * 2048] = make_float2(m, l);
     const bool two = tiles > 1;
     ok = ok && mbar_wait_warp(c, &g_ap.o_full[0], no0 & 1u);
     if (two) ok = ok && mbar_wait_warp(c, &g_ap.o_full[1], no1 & 1u);
     tc_fence_after();
     __syncthreads();
-    const float2 a = g_ap.ml[0][q * 32 + lane], b = g_ap.ml[1][q * 32 + lane];
+    const float2 a = ml[0], b = ml[2048];
     const float M = two ? fmaxf(a.x, b.x) : a.x;
     float f0 = ap_ex2(a.x - M), f1 = two ? ap_ex2(b.x - M) : 0.f;   // (stream 0 has key 0, which every row sees: M is finite)
     const float inv = __fdividef(1.0f, two ? fmaf(f1, b.y, f0 * a.y) : a.y);
@@ -420,6 +421,7 @@ static __device__ __noinline__ void attn_prefill_pair(const DevCtx& c, int layer
                    : "memory");
     }
     tc_fence_before();
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // copies land there again for the next unit
     __syncthreads();
 #pragma unroll 2
     for (int k = 0; k < 8; ++k) {

@@ -150,6 +150,13 @@ __device__ __forceinline__ void block_exscan(int (&v)[N], int (&tot)[N]) {
   }
 }
 
+// Of the batch table while a step is composed; the attention's between the steps (attn_decode_cta).
+struct CtlScratch {
+  long long ticket[MAX_BATCH];
+  int phase[MAX_BATCH], rem[MAX_BATCH];
+};
+__shared__ __align__(16) CtlScratch g_ctl;
+
 // Query rows that a CTA pair takes at a time, and the requests that go to the pairs: a unit of a pair starts and ends in 7 us
 // where one of a single CTA takes 3, but goes through 128 keys of 64 rows in 2.6 us where that takes 5 for 32.  8B shape,
 // us a layer, single CTAs | pairs, for prompts x rows: 1 x 128 10.9 | 13.1, 1 x 256 16.7 | 15.4, 1 x 400 24.4 | 17, 1 x 512 27.6 |
@@ -397,9 +404,9 @@ static __device__ int schedule_step(const DevCtx& c, unsigned long long visible)
   SchedState* ss = c.ss;
   const int tid = threadIdx.x;
   const int MB = c.MB;
-  __shared__ int s_phase[MAX_BATCH];
-  __shared__ long long s_ticket[MAX_BATCH];
-  __shared__ int s_rem[MAX_BATCH];
+  int(&s_phase)[MAX_BATCH] = g_ctl.phase;
+  long long(&s_ticket)[MAX_BATCH] = g_ctl.ticket;
+  int(&s_rem)[MAX_BATCH] = g_ctl.rem;
   __shared__ int s_qstart[MAX_BATCH + 1];
   __shared__ int s_item_b[MAX_BATCH];
   __shared__ int s_n_admit;
@@ -709,9 +716,13 @@ static __device__ int schedule_step(const DevCtx& c, unsigned long long visible)
       const int U = n_dec_att * c.Hkv, maxkb = s_maxkb;
       const long long t_stream = 8 * S * ((((TT + S - 1) / S) + NW - 1) / NW) + 52;
       const long long t_unit = maxkb * ((U + NW - 1) / NW) * (5 * NW + 3 * min((long long)U, NW)) / NW + 14;
+      // More units than CTAs: half CTAs, one round, 6 a tile of their warps and 24 for a CTA's worth of units (fitted to 17 x 40 to
+      // 37 x 300: 24 x 40 11.4 us a layer against 9.9 with whole units per warp, 30 x 100 13.7 against 17.5 with two rounds of CTAs).
       int C = 0;
+      const int half = s_C > 0 && s_Citems > n_ctas;
       if (s_C > 0) {
-        const long long t_cta = ((s_Citems + n_ctas - 1) / n_ctas) * (6ll * ((min(s_C, maxkb) + 7) / 8) + 17) + (s_C < maxkb ? 14 : 0);
+        const int tiles = min(s_C, maxkb);
+        const long long t_cta = (half ? 6ll * ((tiles + 3) / 4) + 24ll * s_Citems / n_ctas + 1 : 6ll * ((tiles + 7) / 8) + 17) + (s_C < maxkb ? 14 : 0);
         if (t_cta <= t_stream && t_cta <= t_unit) C = s_C;
       }
       if (C == 0 && t_unit < t_stream) S = 0;
@@ -724,6 +735,7 @@ static __device__ int schedule_step(const DevCtx& c, unsigned long long visible)
       ss->cur_TT = (int)TT;
       ss->cur_S = (int)S;
       ss->cur_C = C;
+      ss->cur_half = half;
       ss->cur_npf = n_pf;
       ss->cur_npp = n_pp;
     }

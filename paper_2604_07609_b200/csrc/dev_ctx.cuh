@@ -97,6 +97,7 @@ struct SchedState {
   int cur_TT;     // attention: (row, kv head, KV block) tiles of those rows
   int cur_S;      // attention: tiles per sub-range of the flat tile sequence, 0 = a sub-range is a (row, kv head) unit
   int cur_C;      // attention: > 0: decode units are shared by the warps of a CTA, C tiles per part
+  int cur_half;   // attention: such units are shared by half of the warps of a CTA
   int cur_fuse;   // small decode step: the attention applies RoPE and writes K and V itself
   int cur_nuc;    // some row of the step samples from the nucleus of the whole row
   int cur_npf;    // attention: (request, query-row block) units of the multi-row requests that single CTAs take

@@ -51,7 +51,7 @@ __device__ __forceinline__ void make_plan(const DevCtx& c, const StepInfo& st) {
       const AttStep& a = g_att_step;
       if (a.npp > 0) g_plan[0][n++] = ph | ATT_PAIRS << 8;
       if (a.npf > 0) g_plan[0][n++] = ph | ATT_TILES << 8;
-      if (a.n_dec > 0) g_plan[0][n++] = ph | (a.C > 0 ? ATT_DEC_CTA : ATT_DEC_STREAM) << 8;
+      if (a.n_dec > 0) g_plan[0][n++] = ph | (a.C == 0 ? ATT_DEC_STREAM : a.half ? ATT_DEC_HALF : ATT_DEC_CTA) << 8;
       g_plan[0][n - 1] |= PLAN_BARRIER;
     } else if (c.E > 0 && (ph == PH_GU || ph == PH_DOWN)) {
       if (ph == PH_GU) g_plan[0][n++] = PH_MOE_GROUP | PLAN_BARRIER;   // routing lists and gathered rows first

@@ -53,6 +53,12 @@ def test_decode_attention_units_whole_and_cut(prompts):
     _check(MODELS[2048], prompts, 3, 512, B.WEIGHTS_STREAMING)
 
 
+@pytest.mark.parametrize("d, rows", [(2048, 38), (2048, 73), (1024, 75)])   # 152, 292 and 150 units: half CTAs take them
+def test_decode_attention_units_of_half_ctas(d, rows):
+    r = _check(MODELS[d], [100 + (37 * i) % 120 for i in range(rows)], 3, 16384, B.WEIGHTS_STREAMING if d == 2048 else B.WEIGHTS_ROW_MAJOR)
+    assert any(int(n) == rows for n in r["its"]["n_decode"])
+
+
 @pytest.mark.parametrize("tokens", [257, 300, 512, 513])
 def test_prefill_steps_of_several_token_passes(tokens):
     # 6144 QKV rows: 24 pairs of weight tiles, which three token passes divide evenly over 74 pairs of CTAs
