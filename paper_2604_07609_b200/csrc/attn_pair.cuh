@@ -77,9 +77,9 @@ __device__ __forceinline__ float ap_ex2(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-// 32 lanes x 32 consecutive 32-bit columns, without the wait
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
-  uint32_t* r = reinterpret_cast<uint32_t*>(v);
+// 32 lanes x 32 consecutive 32-bit columns, without the wait: the registers hold nothing before tmem_wait_ld() has named them, and
+// even a copy of one may not stand in between, so load and wait lie in one block of straight code.
+__device__ __forceinline__ void tmem_ld32_async(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, "
       "%18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
@@ -90,6 +90,15 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
       : "r"(taddr)
       : "memory");
 }
+#define BLINK_RW8(r, i) "+r"(r[i]), "+r"(r[i + 1]), "+r"(r[i + 2]), "+r"(r[i + 3]), "+r"(r[i + 4]), "+r"(r[i + 5]), "+r"(r[i + 6]), "+r"(r[i + 7])
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&a)[32], uint32_t (&b)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : BLINK_RW8(a, 0), BLINK_RW8(a, 8), BLINK_RW8(a, 16), BLINK_RW8(a, 24), BLINK_RW8(b, 0), BLINK_RW8(b, 8), BLINK_RW8(b, 16),
+                 BLINK_RW8(b, 24)
+               :
+               : "memory");
+}
+#undef BLINK_RW8
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float* v) {
   const uint32_t* r = reinterpret_cast<const uint32_t*>(v);
   asm volatile(
@@ -128,7 +137,10 @@ __device__ __forceinline__ void ap_probs(uint32_t t_s, uint32_t p_row, int swz, 
   const float2 scale2 = make_float2(qscale, qscale), neg2 = make_float2(neg, neg);
   float mx0 = -INFINITY, mx1 = -INFINITY;
   float2 s0 = make_float2(0.f, 0.f), s1 = s0;
-  auto quarter = [&](float(&v)[32], int k) {
+  auto quarter = [&](const uint32_t(&r)[32], int k) {
+    float v[32];
+#pragma unroll
+    for (int x = 0; x < 32; ++x) v[x] = __uint_as_float(r[x]);
     if constexpr (MASKED) {
 #pragma unroll
       for (int x = 0; x < 32; ++x) v[x] = 32 * k + x <= seen ? v[x] : -INFINITY;
@@ -155,19 +167,15 @@ __device__ __forceinline__ void ap_probs(uint32_t t_s, uint32_t p_row, int swz, 
     }
   };
   // (a wait for TMEM loads takes some 400 cycles: the second half is on its way while the first is worked on)
-  float va[32], vb[32], vc[32], vd[32];
-  tmem_ld32(t_s, va);
-  tmem_ld32(t_s + 32u, vb);
-  tmem_wait_ld();
-  regs_ready(va);
-  regs_ready(vb);
-  tmem_ld32(t_s + 64u, vc);
-  tmem_ld32(t_s + 96u, vd);
+  uint32_t va[32], vb[32], vc[32], vd[32];
+  tmem_ld32_async(t_s, va);
+  tmem_ld32_async(t_s + 32u, vb);
+  tmem_wait_ld(va, vb);
+  tmem_ld32_async(t_s + 64u, vc);
+  tmem_ld32_async(t_s + 96u, vd);
   quarter(va, 0);
   quarter(vb, 1);
-  tmem_wait_ld();
-  regs_ready(vc);
-  regs_ready(vd);
+  tmem_wait_ld(vc, vd);
   quarter(vc, 2);
   quarter(vd, 3);
   mx = fmaxf(mx0, mx1);
@@ -396,30 +404,29 @@ static __device__ __noinline__ void attn_prefill_pair(const DevCtx& c, int layer
     f1 *= inv;
     // through shared memory (where the probabilities were), so that rows leave whole
     const uint32_t o_row = b_s + AP_P + (uint32_t)((q * 32 + lane) * 256);
-    float o0[64], o1[64];
-    tmem_ld32(t_o + (uint32_t)(s * 64), o0);
-    tmem_ld32(t_o + (uint32_t)(s * 64 + 32), o0 + 32);
-    if (two) {
-      tmem_ld32(t_o + 128u + (uint32_t)(s * 64), o1);
-      tmem_ld32(t_o + 128u + (uint32_t)(s * 64 + 32), o1 + 32);
-    } else {
+    uint32_t a0[32], a1[32], b0[32], b1[32];   // (one stream: what the other's accumulator holds counts for nothing)
+    tmem_ld32_async(t_o + (uint32_t)(s * 64), a0);
+    tmem_ld32_async(t_o + (uint32_t)(s * 64 + 32), a1);
+    tmem_ld32_async(t_o + 128u + (uint32_t)(s * 64), b0);
+    tmem_ld32_async(t_o + 128u + (uint32_t)(s * 64 + 32), b1);
+    tmem_wait_ld(a0, a1);
+    tmem_wait_ld(b0, b1);
+    auto half_row = [&](const uint32_t(&r0)[32], const uint32_t(&r1)[32], int h) {
+      auto dim = [&](int x) { return fmaf(two ? __uint_as_float(r1[x]) : 0.f, f1, __uint_as_float(r0[x]) * f0); };
 #pragma unroll
-      for (int k = 0; k < 64; ++k) o1[k] = 0.f;
-    }
-    tmem_wait_ld();
-    regs_ready(o0);
-    regs_ready(o1);
+      for (int k = 0; k < 32; k += 8) {
+        uint32_t o[4];
 #pragma unroll
-    for (int k = 0; k < 64; k += 8) {
-      uint32_t o[4];
-#pragma unroll
-      for (int y = 0; y < 4; ++y) {
-        const __nv_bfloat162 b2 = __floats2bfloat162_rn(fmaf(o1[k + 2 * y], f1, o0[k + 2 * y] * f0), fmaf(o1[k + 2 * y + 1], f1, o0[k + 2 * y + 1] * f0));
-        o[y] = *reinterpret_cast<const uint32_t*>(&b2);
+        for (int y = 0; y < 4; ++y) {
+          const __nv_bfloat162 b2 = __floats2bfloat162_rn(dim(k + 2 * y), dim(k + 2 * y + 1));
+          o[y] = *reinterpret_cast<const uint32_t*>(&b2);
+        }
+        const uint32_t dst = o_row + (((s * 8 + h * 4 + (k >> 3)) ^ (lane & 7)) << 4);   // 16-byte pieces, swizzled by the row
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]) : "memory");
       }
-      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(o_row + (((s * 8 + (k >> 3)) ^ (lane & 7)) << 4)), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3])   // 16-byte pieces, swizzled by the row
-                   : "memory");
-    }
+    };
+    half_row(a0, b0, 0);
+    half_row(a1, b1, 1);
     tc_fence_before();
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // copies land there again for the next unit
     __syncthreads();

@@ -204,37 +204,19 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
 __device__ __forceinline__ void red_add_f32(float* p, float v) {
   asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "f"(v) : "memory");
 }
-// 32 lanes x 16 consecutive 32-bit columns -> 16 registers per thread
+// 32 lanes x 16 consecutive 32-bit columns -> 16 registers per thread.  The registers of a load hold nothing before the wait, and
+// even a copy of one may not stand between the two: here they are one statement.
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   uint32_t r[16];
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, "
-      "[%16];"
+      "[%16];\n\ttcgen05.wait::ld.sync.aligned;"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
         "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr)
       : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// The same without the wait: nothing may use the registers before tmem_wait_ld() and regs_ready().
-__device__ __forceinline__ void tmem_ld16_async(uint32_t taddr, float* v) {
-  uint32_t* r = reinterpret_cast<uint32_t*>(v);
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, "
-      "[%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
-}
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void regs_ready(float (&v)[N]) {   // no use of the registers moves in front of this
-#pragma unroll
-  for (int i = 0; i < N; ++i) asm volatile("" : "+f"(v[i]));
 }
 
 // Shared-memory matrix descriptor: K-major tile of rows x 64 bf16 (128-byte rows), 128-byte
@@ -410,23 +392,16 @@ struct TcEpiOut {
   int ilv_F;               // gate/up rows interleaved in the weight tiles: row n is output column (n & 1) * F + (n >> 1)
   __nv_bfloat16* act;      // non-null: a tile whose sums are complete goes straight to act = silu(gate) * up
 };
-// Columns [c_begin, c_end) of an accumulator (token rows t_base + column) -> out; lane = weight row n.  The next group of 16 is
-// on its way from TMEM (some 400 cycles) while one is stored.  An SM stores 32 bytes a cycle to L2 and reduces 25, whatever
-// the other SMs do: 128 columns are 4100 or 5200 cycles for eight warps.  plain: stores.  Else reductions, with row_map
-// into mapped rows, scaled.  Met once a phase, beyond the instruction cache: one copy of this code for all warps.
+// Columns [c_begin, c_end) of an accumulator (token rows t_base + column) -> out; lane = weight row n.  An SM stores 32 bytes a
+// cycle to L2 and reduces 25, whatever the other SMs do: 128 columns are 4100 or 5200 cycles for eight warps, which hide each
+// other's waits for TMEM (some 400 cycles): with the next group on its way while one is stored the GEMMs were longer (100 rows of
+// the 1B shape QKV 8.2 us against 7.8, gate/up 18.6 against 18.0).  plain: stores.  Else reductions, with row_map into mapped rows, scaled.  Met once a phase, beyond the instruction cache: one copy of this code for all warps.
 __device__ __forceinline__ void tc_epi_columns(const TcEpiOut& e, uint32_t taddr, int n, int t_base, int c_begin, int c_end, bool plain) {
-  if (c_begin >= c_end) return;
   const int n_out = e.ilv_F ? (n & 1) * e.ilv_F + (n >> 1) : n;
-  float next[16];
-  tmem_ld16_async(taddr + (uint32_t)c_begin, next);
 #pragma unroll 1
   for (int c0 = c_begin; c0 < c_end; c0 += 16) {
     float v[16];
-    tmem_wait_ld();
-    regs_ready(next);
-#pragma unroll
-    for (int j = 0; j < 16; ++j) v[j] = next[j];
-    if (c0 + 16 < c_end) tmem_ld16_async(taddr + (uint32_t)(c0 + 16), next);
+    tmem_ld16(taddr + (uint32_t)c0, v);
     const int t0 = t_base + c0;
     const int nv = n < e.N ? min(16, e.T - t0) : 0;   // token rows of this group that exist
     if (e.row_map != nullptr) {

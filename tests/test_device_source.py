@@ -43,3 +43,35 @@ def test_scheduler_and_phases_go_by_one_row_limit_for_small_steps():
     control, dec = _text("control.cuh"), _text("gemm_dec.cuh")
     assert re.search(r"const int fuse = c\.dec_small && T <= DEC_SMALL_ROWS\b", control)
     assert re.search(r"bool dec_small\(.*\{ return c\.dec_small && T <= DEC_SMALL_ROWS; \}", dec)
+
+
+def test_registers_of_a_tensor_memory_load_are_not_touched_before_the_wait():
+    """They hold nothing until tcgen05.wait::ld.  So the wait is part of the load's statement, or it names the registers (+r) and stands
+    behind the load in the same block: no branch, no way around a loop and no change of type between the two, each of which
+    may be a copy."""
+    texts = {f: re.sub(r"//[^\n]*", "", _text(f)) for f in sorted(os.listdir(CSRC)) if f.endswith((".cuh", ".cu"))}
+    wrappers, n_loads = [], 0
+    for text in texts.values():
+        for st in re.finditer(r"asm volatile\((.*?)\);", text, re.S):
+            code = st.group(1)
+            if "tcgen05.ld." in code:
+                n_loads += 1
+                if "tcgen05.wait::ld" in code:
+                    assert code.index("tcgen05.ld.") < code.index("tcgen05.wait::ld")
+                    continue
+                name, args = re.findall(r"void (\w+)\(([^{;]*)\) \{\s", text[:st.start()])[-1]
+                assert re.search(r"uint32_t \(&\w+\)\[\d+\]", args), f"{name}: destinations of another type than the instruction's"
+                wrappers.append(name)
+            elif "tcgen05.wait::ld" in code:
+                assert "+r" in code or "BLINK_RW" in code, "a wait that names no registers orders nothing that uses them"
+    assert n_loads >= 2
+    for name in wrappers:
+        for f, text in texts.items():
+            for call in re.finditer(r"\b%s\(([^;{]*), (\w+)\);" % name, text):
+                depth, i = 0, call.end()
+                while depth >= 0:   # to the end of the block that the load stands in
+                    depth += {"{": 1, "}": -1}.get(text[i], 0)
+                    i += 1
+                head = text[:call.start()].rstrip()
+                assert head[-1] in ";{}", f"{f}: {call.group(0)} under a condition"
+                assert re.search(r"tmem_wait_ld\w*\([^;]*\b%s\b[^;]*\);" % call.group(2), text[call.end():i]), f"{f}: {call.group(0)} is not waited for in its block"
