@@ -58,11 +58,6 @@ __device__ __forceinline__ void att_init(const DevCtx& c) {
   __syncthreads();
 }
 
-__device__ __forceinline__ float fast_ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
 __device__ __forceinline__ uint32_t pack_bf2(float lo, float hi) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&v);
@@ -435,7 +430,7 @@ constexpr int ATT_NSC = 2;   // ring stages per warp here
 constexpr int ATT_CTA_OFF = 65536;   // the space before it may be receiving weights of the O projection already
 struct AttCta {
   float m[ATT_WARPS][8], l[ATT_WARPS][8];   // maxima and sums of the warps
-  int last[2];
+  int last;
 };
 __shared__ AttCta g_att_cta;
 // GW: warps that share a unit, all of the CTA's or half of them (two groups, which go their own ways).
@@ -479,12 +474,13 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer) 
   const uint64_t kv_policy = l2_evict_first();
   uint32_t par = g_att_par[w];
 
-  // items in unit order; prefill tiles of a step sit on the first CTAs, so the decode items start from the last
+  // items in unit order, from the last CTA: prompt rows of a step sit on the first ones (those that single CTAs take only while no
+  // pair has any)
   for (int item = (int)gridDim.x - 1 - (int)blockIdx.x + grp * (int)gridDim.x; ; item += n_groups) {   // uniform over the group
-    int d = 0, rest = item, nkb = 0, ns = 1;
+    int d = 0, rest = item, nkb = 0, ns = 1;   // (the units of half CTAs are whole)
     for (; d < n_dec; ++d) {
       nkb = g_att_pre[d + 1] - g_att_pre[d];
-      ns = (nkb + C - 1) / C;
+      if constexpr (NG == 1) ns = (nkb + C - 1) / C;
       if (rest < Hkv * ns) break;
       rest -= Hkv * ns;
     }
@@ -642,7 +638,7 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer) 
         num.y = fmaf(f, a.y, num.y);
         den = fmaf(f, s_l[k][h], den);
       }
-      if (ns == 1) {
+      if (NG > 1 || ns == 1) {
         const float inv = __fdividef(1.0f, den);
         *reinterpret_cast<uint32_t*>(obase + i2 * 2) = pack_bf2(num.x * inv, num.y * inv);
       } else {
@@ -650,13 +646,13 @@ static __device__ __noinline__ void attn_decode_cta(const DevCtx& c, int layer) 
         if ((i2 * 2) % HD == 0) { rec[NREP * HD + h] = M; rec[NREP * HD + NREP + h] = den; }
       }
     }
-    if (ns > 1) {
+    if (NG == 1 && ns > 1) {
       const int unit = d * Hkv + g;
       __threadfence();
       group_sync();
-      if (tg == 0) g_att_cta.last[grp] = atomicAdd(&c.att_cnt[unit], 1) == ns - 1;
+      if (tg == 0) g_att_cta.last = atomicAdd(&c.att_cnt[unit], 1) == ns - 1;
       group_sync();
-      if (g_att_cta.last[grp]) {   // this group delivered the last part: merge in part order (records of a unit are consecutive)
+      if (g_att_cta.last) {   // this CTA delivered the last part: merge in part order (records of a unit are consecutive)
         __threadfence();
         const float* r0 = c.att_part + (size_t)(item - part) * REC;
         for (int i2 = tg; i2 < NREP * HD / 2; i2 += GT) {

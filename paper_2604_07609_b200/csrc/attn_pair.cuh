@@ -72,7 +72,7 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) {
       : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
   return d;
 }
-__device__ __forceinline__ float ap_ex2(float x) {
+__device__ __forceinline__ float fast_ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
@@ -156,8 +156,8 @@ __device__ __forceinline__ void ap_probs(uint32_t t_s, uint32_t p_row, int swz, 
 #pragma unroll
       for (int y = 0; y < 4; ++y) {
         float2 e = fma2(make_float2(v[x + 2 * y], v[x + 2 * y + 1]), scale2, neg2);
-        e.x = ap_ex2(e.x);
-        e.y = ap_ex2(e.y);
+        e.x = fast_ex2(e.x);
+        e.y = fast_ex2(e.y);
         if (y & 1) s1 = add2(s1, e); else s0 = add2(s0, e);
         const __nv_bfloat162 b2 = __floats2bfloat162_rn(e.x, e.y);
         o[y] = *reinterpret_cast<const uint32_t*>(&b2);
@@ -332,7 +332,7 @@ static __device__ __noinline__ void attn_prefill_pair(const DevCtx& c, int layer
         mx *= qscale;
         if (!__any_sync(0xffffffffu, mx > m + 8.f)) break;
         const float mn = fmaxf(m, mx);
-        const float f = mn == -INFINITY ? 1.f : ap_ex2(m - mn);
+        const float f = mn == -INFINITY ? 1.f : fast_ex2(m - mn);
         m = mn;
         l *= f;
         if (i > 0 && ok) {
@@ -398,7 +398,7 @@ static __device__ __noinline__ void attn_prefill_pair(const DevCtx& c, int layer
     __syncthreads();
     const float2 a = ml[0], b = ml[2048];
     const float M = two ? fmaxf(a.x, b.x) : a.x;
-    float f0 = ap_ex2(a.x - M), f1 = two ? ap_ex2(b.x - M) : 0.f;   // (stream 0 has key 0, which every row sees: M is finite)
+    float f0 = fast_ex2(a.x - M), f1 = two ? fast_ex2(b.x - M) : 0.f;   // (stream 0 has key 0, which every row sees: M is finite)
     const float inv = __fdividef(1.0f, two ? fmaf(f1, b.y, f0 * a.y) : a.y);
     f0 *= inv;
     f1 *= inv;

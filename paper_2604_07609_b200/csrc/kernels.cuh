@@ -231,7 +231,6 @@ __device__ __forceinline__ void run_phase(const DevCtx& c, int phase, int layer,
     case PH_ATTN:
       if constexpr (sizeof(WT) == 2) phase_attention_bf16<HD, NREP, PAIR>(c, layer, sub, smem);
       else phase_attention<WT, HD, NREP>(c, layer, smem);
-
       break;
     case PH_NORM2:
       if constexpr (!PAIR)
