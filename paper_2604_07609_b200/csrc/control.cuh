@@ -11,6 +11,7 @@
 #include "../../include/blink.h"
 #include "dev_ctx.cuh"
 #include "mailbox.h"
+#include "att_plan.h"
 
 namespace blink {
 
@@ -156,13 +157,6 @@ struct CtlScratch {
   int phase[MAX_BATCH], rem[MAX_BATCH];
 };
 __shared__ __align__(16) CtlScratch g_ctl;
-
-// Query rows that a CTA pair takes at a time, and the requests that go to the pairs: a unit of a pair starts and ends in 7 us
-// where one of a single CTA takes 3, but goes through 128 keys of 64 rows in 2.6 us where that takes 5 for 32.  8B shape,
-// us a layer, single CTAs | pairs, for prompts x rows: 1 x 128 10.9 | 13.1, 1 x 256 16.7 | 15.4, 1 x 400 24.4 | 17, 1 x 512 27.6 |
-// 19, 512 rows behind 3500 keys 177 | 63, 2 x 256 17.5 | 17.4, 3 x 170 15.4 | 17.5, 8 x 64 12.1 | 18.2, 24 x 20 17.0 | 34.2.
-constexpr int ATT_PAIR_ROWS = 64;
-__device__ __forceinline__ bool att_on_pairs(int keys) { return keys > 256; }
 
 __device__ __forceinline__ int32_t fake_token(unsigned long long ticket, int gen, int vocab) {
   // control-only stand-in sampler: a fixed hash of (ticket, index)
@@ -544,17 +538,25 @@ static __device__ int schedule_step(const DevCtx& c, unsigned long long visible)
   const int q_rows = 128 / c.n_rep;
   const int is_dec = f && take == 1;
   const int nkb_att = is_dec ? (new_len + c.bs - 1) / c.bs : 0;
-  const bool on_pairs = c.att_pair && take > 1 && att_on_pairs(new_len);
-  const int n_qb = (f && take > 1 && !on_pairs) ? (take + q_rows - 1) / q_rows : 0;
-  const int n_qp = (f && on_pairs) ? (take + ATT_PAIR_ROWS - 1) / ATT_PAIR_ROWS : 0;
+  const int n_blk = f && take > 1 ? (take + q_rows - 1) / q_rows : 0;
+  const bool pairs_ok = c.att_pair && take > 1 && att_on_pairs(new_len);
   // (entries 7 and 8: blocks that post_step may free at most, and tickets that may end, by completion or
-  // cancellation, for the trace space check)
-  int sc[10] = {f, take, want, sample, is_dec, nkb_att, n_qb, phase != PHASE_FREE ? have + want : 0, phase != PHASE_FREE ? 1 : 0, n_qp};
-  int sc_tot[10];
+  // cancellation, for the trace space check; 6, 9 and 10: blocks of query rows for single CTAs, for CTA pairs, the latter in blocks for
+  // single CTAs; the upper half of 8: requests for the pairs that have a long context)
+  const int is_long = pairs_ok && new_len > ATT_ONE_ROUND_KEYS;
+  int sc[11] = {f, take, want, sample, is_dec, nkb_att, pairs_ok ? 0 : n_blk, phase != PHASE_FREE ? have + want : 0, (phase != PHASE_FREE ? 1 : 0) | is_long << 16,
+                pairs_ok ? (take + ATT_PAIR_ROWS - 1) / ATT_PAIR_ROWS : 0, pairs_ok ? n_blk : 0};
+  int sc_tot[11];
   block_exscan(sc, sc_tot);
-  const int item = sc[0], qstart = sc[1], aoff = sc[2], row = sc[3], dec_idx = sc[4], kb_pre = sc[5], pf_off = n_qp > 0 ? sc[9] : sc_tot[9] + sc[6];
+  const int n_ctas = c.n_warps_grid / (CTRL_THREADS / 32);
+  const bool no_pairs = att_one_round_on_ctas(sc_tot[9] * c.Hkv, (sc_tot[6] + sc_tot[10]) * c.Hkv, n_ctas, sc_tot[8] >> 16 ? ATT_ONE_ROUND_KEYS + 1 : 0);
+  const bool on_pairs = pairs_ok && !no_pairs;
+  const int n_qp = on_pairs ? (take + ATT_PAIR_ROWS - 1) / ATT_PAIR_ROWS : 0, n_qb = on_pairs ? 0 : n_blk;
+  const int n_pp = no_pairs ? 0 : sc_tot[9], n_pf = sc_tot[6] + (no_pairs ? sc_tot[10] : 0);
+  const int item = sc[0], qstart = sc[1], aoff = sc[2], row = sc[3], dec_idx = sc[4], kb_pre = sc[5],
+            pf_off = on_pairs ? sc[9] : n_pp + sc[6] + (no_pairs ? sc[10] : 0);
   const int n_items = sc_tot[0], T = sc_tot[1], n_alloc = sc_tot[2], n_rows = sc_tot[3], n_dec_att = sc_tot[4], tot_kb = sc_tot[5],
-            n_pf = sc_tot[6], tot_may_free = sc_tot[7], n_live = sc_tot[8], n_pp = sc_tot[9];
+            tot_may_free = sc_tot[7], n_live = sc_tot[8] & 0xffff;
 
   if (T == 0) return 0;  // uniform: every thread sees the same T
 
@@ -640,7 +642,6 @@ static __device__ int schedule_step(const DevCtx& c, unsigned long long visible)
   // CTA-wide decode attention for few units: the smallest part size (of 32 candidates from a fair share up, at
   // least 24 tiles: a cut unit costs a merge through memory, about the time of three tiles per warp) whose parts fit
   // the grid at once; when none does, units stay whole
-  const int n_ctas = c.n_warps_grid / (CTRL_THREADS / 32);
   if (tid < 32 && c.dec_row != nullptr && n_dec_att > 0 && n_dec_att * c.Hkv <= 2 * n_ctas) {
     const int share = max(24, (tot_kb * c.Hkv + n_ctas - 1) / n_ctas);
     const int C = share + tid * ((share + 7) / 8);
@@ -690,52 +691,17 @@ static __device__ int schedule_step(const DevCtx& c, unsigned long long visible)
     ss->last_was_prefill = prefill_turn ? 1 : 0;
     if (c.dec_row != nullptr) {
       const long long TT = (long long)tot_kb * c.Hkv;
-      // Sub-ranges: k per warp of the grid.  Every cut of a unit costs a partial record and a merge,
-      // so a pure decode step takes one sub-range per warp up to 96 tiles; with prefill tiles in the
-      // step the CTAs reach their decode share at different times and smaller sub-ranges (up to 48
-      // tiles, the later ones handed out by the counter) even that out.
-      const long long NW = c.n_warps_grid;
-      const long long cap = n_pf + n_pp > 0 ? 48 : 96;
-      const long long k = (TT + cap * NW - 1) / (cap * NW) > 1 ? (TT + cap * NW - 1) / (cap * NW) : 1;
-      long long S = (TT + k * NW - 1) / (k * NW);
-      // at least 8 tiles per sub-range: a cut costs a partial record, a fence and a counter update (about the time of
-      // two tiles), and a unit cut into n parts is merged by one warp in n steps; with few long rows one tile per
-      // sub-range made a single 2048-token row take 120 us per layer, most of it the merge
-      if (S < 8) S = 8;
-      while ((TT + S - 1) / S > c.att_sub_max) S *= 2;   // cannot happen with the sizes set at create
-      // Three ways to run the decode units.  Estimates in units of 0.2 us, fitted to the measurements below: the streaming
-      // kernel cuts the flat sequence evenly, 8 a tile with all warps at work, 52 for the ends of cut units; whole units
-      // per warp need no cuts, a tile 5 with few warps at work and 8 with all; a CTA per part shares a unit between its
-      // eight warps, 6 a tile and 17 a round (start, merge in shared memory, two barriers).
-      // 8B shape, us a layer, streaming | whole units | CTA, for rows x keys:
-      //   17 x 40  17.9 | 11.9 | 10.2    17 x 300  26 | 30 | 12.7    17 x 1500  40 | 106 | 24    17 x 4000  70 | 280 | 50
-      //   24 x 40  18.0 | 11.7 | 15.2    24 x 300  26 | 29 | 19.9    24 x 1500  48 | 110 | 42    24 x 4000  87 | 285 | 90
-      //   37 x 40  18.1 | 12.0 | 20.1    37 x 300  27 | 30 | 25      37 x 1500  58 | 126 | 52    48 x 40  18.2 | 12.2
-      //   48 x 300  28 | 30    100 x 40  20 | 15.5    100 x 300  41 | 36    100 x 900  88 | 91    200 x 40  26.5 | 24.5
-      //   200 x 300  69 | 68    200 x 700  125 | 146    200 of 20 to 1500 keys  88 | 144
-      const int U = n_dec_att * c.Hkv, maxkb = s_maxkb;
-      const long long t_stream = 8 * S * ((((TT + S - 1) / S) + NW - 1) / NW) + 52;
-      const long long t_unit = maxkb * ((U + NW - 1) / NW) * (5 * NW + 3 * min((long long)U, NW)) / NW + 14;
-      // More units than CTAs: half CTAs, one round, 6 a tile of their warps and 24 for a CTA's worth of units (fitted to 17 x 40 to
-      // 37 x 300: 24 x 40 11.4 us a layer against 9.9 with whole units per warp, 30 x 100 13.7 against 17.5 with two rounds of CTAs).
-      int C = 0;
-      const int half = s_C > 0 && s_Citems > n_ctas;
-      if (s_C > 0) {
-        const int tiles = min(s_C, maxkb);
-        const long long t_cta = (half ? 6ll * ((tiles + 3) / 4) + 24ll * s_Citems / n_ctas + 1 : 6ll * ((tiles + 7) / 8) + 17) + (s_C < maxkb ? 14 : 0);
-        if (t_cta <= t_stream && t_cta <= t_unit) C = s_C;
-      }
-      if (C == 0 && t_unit < t_stream) S = 0;
+      const AttDecodeWay way =
+          att_decode_way({TT, n_dec_att * c.Hkv, s_maxkb, s_C, s_Citems, n_ctas, CTRL_THREADS / 32, n_pf + n_pp > 0, c.att_sub_max});
       // a decode step of few rows: the CTA-wide kernel also applies RoPE and writes the new keys and values
       const int fuse = c.dec_small && T <= DEC_SMALL_ROWS && n_pf + n_pp == 0 && s_C > 0;
-      if (fuse) C = s_C;
       ss->cur_fuse = fuse;
       c.dec_kbpre[n_dec_att] = tot_kb;
       ss->cur_ndec = n_dec_att;
       ss->cur_TT = (int)TT;
-      ss->cur_S = (int)S;
-      ss->cur_C = C;
-      ss->cur_half = half;
+      ss->cur_S = (int)way.S;
+      ss->cur_C = fuse ? s_C : way.C;
+      ss->cur_half = way.half;
       ss->cur_npf = n_pf;
       ss->cur_npp = n_pp;
     }

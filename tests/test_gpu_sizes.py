@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 import torch
 
+import att_plan
 from gpu_util import compare_with_oracle, gpu_run_forced
 from oracle import sampler as S
 from paper_2604_07609_b200 import binding as B
@@ -93,6 +94,14 @@ def test_prompt_attention_around_units_and_tiles(prompts, chunk):
 def test_prompt_attention_of_more_units_than_pairs():
     # 8 prompts x 5 units x 2 kv heads on 74 pairs, two layers: some pairs have a second unit in every layer
     _check(ModelCfg(2, 512, 8, 2, 128, 256, 1024), [290, 300, 310, 320, 257, 319, 288, 305], 2, 4096, B.WEIGHTS_STREAMING, relative=False)
+
+
+@pytest.mark.parametrize("heads, prompts", [((32, 8, 128), [270, 288]), ((8, 2, 128), [260, 20, 270, 288, 257, 30, 280, 265, 272, 288])], ids=str)
+def test_prompt_attention_that_would_take_the_pairs_a_second_round(heads, prompts):
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    assert att_plan.prompts_on_pairs([(0, p) for p in prompts], heads[1], n_sm) == 0
+    assert att_plan.prompts_on_pairs([(0, p) for p in prompts + [290]], heads[1], n_sm) > 0
+    _check(ModelCfg(1, 512, *heads, 256, 1024), prompts, 2, 4096, B.WEIGHTS_STREAMING, relative=False)
 
 
 def test_prompt_attention_leaves_the_pools_old_contents_alone():
