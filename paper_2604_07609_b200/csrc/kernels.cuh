@@ -21,7 +21,8 @@ struct StepInfo {
   bool dec;      // decode-sized: the GEMMs of gemm_dec.cuh
   bool small;    // of at most 16 rows: norms, SwiGLU and final norm run inside those GEMMs
   bool fuse;     // RoPE and the K/V write run inside the attention
-  bool fold;     // fp32: norms, RoPE, SwiGLU and final norm run inside the CUDA-core GEMMs
+  bool fold;     // fp32: norms, RoPE and SwiGLU run inside the CUDA-core GEMMs
+  bool fold_out; // and the final norm inside the LM head
   bool nuc;      // some row samples from the nucleus of its whole row
   bool att_cta;  // the attention phase leaves the first half of the weight ring alone
 };
@@ -37,7 +38,8 @@ __shared__ unsigned long long g_phase_t;                    // when the last pha
 // Phases that a step does not have because others do their work.
 __device__ __forceinline__ bool phase_absorbed(const DevCtx& c, const StepInfo& st, int ph) {
   if (c.fused) return ph == PH_ROPE || ph == PH_SILU;   // done by the epilogues of the QKV and gate/up GEMMs
-  if (st.fold) return ph == PH_NORM1 || ph == PH_ROPE || ph == PH_NORM2 || ph == PH_SILU || ph == PH_FNORM;
+  if (st.fold && ph != PH_FNORM) return ph == PH_NORM1 || ph == PH_ROPE || ph == PH_NORM2 || ph == PH_SILU;
+  if (st.fold_out) return ph == PH_FNORM;
   if (ph == PH_ROPE) return st.fuse;
   if (!st.small) return false;
   return ph == PH_NORM1 || ph == PH_FNORM || (c.E == 0 && (ph == PH_NORM2 || ph == PH_SILU));
@@ -87,7 +89,7 @@ static __device__ __noinline__ void step_begin(const DevCtx& c) {
     s.small = dec_small(c, s.T);
     s.dec = dec_step(c, s.T);
     s.fuse = fuse != 0;
-    s.fold = false;
+    s.fold = s.fold_out = false;
     s.att_cta = C > 0 && npf == 0;
     if (s.dec) dec_geometry<PAIR>(c, s.T, s.R);
     att_lists(c);
@@ -97,6 +99,7 @@ static __device__ __noinline__ void step_begin(const DevCtx& c) {
   } else {
     s.small = s.dec = s.fuse = s.att_cta = false;
     s.fold = fold_step(c, s.T);
+    s.fold_out = s.fold && fold_lm_head(c, s.R);
   }
   if (threadIdx.x < N_PHASE_TIMERS) g_phase_ns[threadIdx.x] = 0ull;
   if (threadIdx.x == 0) {
@@ -218,7 +221,7 @@ __device__ __forceinline__ void run_phase(const DevCtx& c, int phase, int layer,
     if (st.fold) {
       if (phase == PH_QKV) { phase_gemm_fold<FOLD_ROPE>(c, layer); return; }
       if (phase == PH_GU) { phase_gemm_fold<FOLD_SILU>(c, layer); return; }
-      if (phase == PH_LMHEAD) { phase_gemm_fold<FOLD_NORM>(c, 0); return; }
+      if (phase == PH_LMHEAD && st.fold_out) { phase_gemm_fold<FOLD_NORM>(c, 0); return; }
     }
   }
   switch (phase) {

@@ -14,6 +14,7 @@ from synth.configs import ModelCfg, SchedCfg
 from synth.workload import Request
 
 pytestmark = pytest.mark.gpu
+PH_FNORM = 9   # place of the final norm in a step's phase times
 
 # four query heads per kv head: the shape that runs its GEMMs on CTA pairs
 MODELS = {1024: ModelCfg(2, 1024, 8, 2, 128, 1024, 4096), 2048: ModelCfg(1, 2048, 16, 4, 64, 768, 4096),
@@ -80,6 +81,15 @@ def test_fp32_steps_with_and_without_element_wise_phases(rows, heads):
     sched = SchedCfg(max_batch=1, prefill_chunk_tokens=512, n_slots=16, max_prompt=rows, max_new=3, n_blocks=(rows + 18) // 16)
     r = compare_with_oracle(model, sched, _requests([rows], 3, model.vocab), make_weights(model, 5, "cpu", random_gains=True), 1e-4)
     assert int(r["its"]["n_tokens"][0]) == rows
+
+
+@pytest.mark.parametrize("rows, folded", [(24, True), (25, False)])   # 24 x 256 x 32400 products are the last below the limit
+def test_fp32_steps_with_and_without_the_final_norm_inside_the_lm_head(rows, folded):
+    model = ModelCfg(1, 256, 4, 2, 64, 512, 32400, dtype="fp32")
+    sched = SchedCfg(max_batch=rows, prefill_chunk_tokens=512, n_slots=32, max_prompt=8, max_new=3, n_blocks=rows)
+    r = compare_with_oracle(model, sched, _requests([3 + i % 5 for i in range(rows)], 3, model.vocab), make_weights(model, 5, "cpu", random_gains=True), 1e-4)
+    steps = [it for it in r["its"] if int(it["n_sample_rows"]) == rows]
+    assert steps and all((int(it["phase_ns"][PH_FNORM]) == 0) == folded for it in steps)
 
 
 # more than 256 keys: prompt attention on CTA pairs, in units of 64 rows and tiles of 128 keys
