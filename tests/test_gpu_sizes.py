@@ -14,7 +14,7 @@ from synth.configs import ModelCfg, SchedCfg
 from synth.workload import Request
 
 pytestmark = pytest.mark.gpu
-PH_FNORM = 9   # place of the final norm in a step's phase times
+PH_ROPE, PH_FNORM = 2, 9   # places in a step's phase times
 
 # four query heads per kv head: the shape that runs its GEMMs on CTA pairs
 MODELS = {1024: ModelCfg(2, 1024, 8, 2, 128, 1024, 4096), 2048: ModelCfg(1, 2048, 16, 4, 64, 768, 4096),
@@ -59,6 +59,41 @@ def test_decode_attention_units_whole_and_cut(prompts):
 def test_decode_attention_units_of_half_ctas(d, rows):
     r = _check(MODELS[d], [100 + (37 * i) % 120 for i in range(rows)], 3, 16384, B.WEIGHTS_STREAMING if d == 2048 else B.WEIGHTS_ROW_MAJOR)
     assert any(int(n) == rows for n in r["its"]["n_decode"])
+
+
+def _decode_keys(prompts, new):
+    """Contexts of the first step in which every request decodes (they are all there from the first step on)."""
+    return [p + 1 for p in prompts], [p + new - 1 for p in prompts]
+
+
+@pytest.mark.parametrize("heads", [(16, 16, 64), (32, 16, 64), (64, 16, 64), (128, 16, 64), (32, 8, 128), (64, 8, 128)], ids=str)
+def test_decode_attention_of_half_ctas_with_any_head_group(heads):
+    """One, two, four and eight query heads per kv head; the rule is asked that half CTAs take the decode steps."""
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    rows, new = n_sm // heads[1] + 3, 3
+    prompts = [100 + (37 * i) % 120 for i in range(rows)]
+    for keys in _decode_keys(prompts, new):
+        assert rows > 16 or heads[1] > 8
+        assert att_plan.decode_way(keys, heads[1], n_sm) == "half"
+    # The prompts' rows see up to 220 keys, whose probabilities the prefill kernel rounds (as below: rms 3 % above the oracles'
+    # distance); logits of d = 512, sigma 0.45, and the absolute bound of the small shapes
+    r = _check(ModelCfg(1, 512, *heads, 256, 1024), prompts, new, 8192, relative=False)
+    assert r["err_plain"] <= 2e-2
+    assert any(int(n) == rows for n in r["its"]["n_decode"])
+
+
+@pytest.mark.parametrize("heads", [(16, 16, 64), (32, 16, 64), (64, 16, 64), (128, 16, 64)], ids=str)
+@pytest.mark.parametrize("rows", [10, 16])
+def test_half_ctas_that_also_rotate_and_write_keys_and_values(rows, heads):
+    """Steps of at most 16 rows with more units than CTAs: RoPE and the K/V write run in the groups (no RoPE phase in those steps)."""
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    assert n_sm < rows * heads[1] <= 2 * n_sm
+    # CTA pairs (four query heads) at d = 1024; else d = 256, whose logits (sigma 0.32) the absolute bound was made for
+    pair = heads[0] == 4 * heads[1]
+    r = _check(ModelCfg(2, 1024 if pair else 256, *heads, 256, 1024), [3 + (37 * i) % 70 for i in range(rows)], 4, 4096, relative=pair)
+    assert r["err_plain"] <= 2e-2
+    steps = [it for it in r["its"] if int(it["n_tokens"]) == int(it["n_decode"]) == rows]
+    assert steps and all(int(it["phase_ns"][PH_ROPE]) == 0 for it in steps)
 
 
 @pytest.mark.parametrize("tokens", [257, 300, 512, 513])
