@@ -14,9 +14,9 @@
 //          (a smaller growth leaves probabilities above one, and their sum takes it up: nothing is lost)
 //     -> arrival in CTA 0, where a warp of the stream issues the next tile's scores and another the output MMAs
 //
-// What bounds it: of the 4900 cycles of a tile and stream (two streams side by side) the softmax takes 2600 (128 exponentials
-// a thread are 1024 cycles of a unit that both streams share; two warps per scheduler leave its latencies open), loads,
-// hand-overs and the scores' MMAs the rest.  512 rows behind 3500 keys: 177 us a layer with attn_prefill_tile, 63 here.
+// What bounds it: the softmax (128 exponentials a thread are 1024 cycles of a unit that both streams share; two warps per scheduler
+// leave its latencies open); loads, hand-overs and the scores' MMAs are the rest.  512 rows of 512 keys: 27.4 us a layer with
+// attn_prefill_tile, 14.4 here; behind 3500 keys 177 and 61.
 #pragma once
 #include "gemm_tc.cuh"
 
@@ -131,7 +131,7 @@ __device__ __forceinline__ uint64_t smem_desc_sw128_mn(uint32_t saddr) {
 
 // One row of a score tile -> probabilities (bf16, swizzled rows of 64 keys, two slabs), their sum, and the largest score.
 // One pass and no branch inside: with a pass for the maximum first and the accumulator's rescaling unrolled too, the body of a
-// tile was beyond the 32 KB instruction cache (10900 cycles a tile), and a conditional mask copies every value once more.
+// tile was beyond the 32 KB instruction cache (more than twice the time), and a conditional mask copies every value once more.
 template <bool MASKED>
 __device__ __forceinline__ void ap_probs(uint32_t t_s, uint32_t p_row, int swz, float qscale, float neg, int seen, float& mx, float2& sum) {
   const float2 scale2 = make_float2(qscale, qscale), neg2 = make_float2(neg, neg);
